@@ -210,6 +210,11 @@ __device__ __forceinline__ dd from_d<dd>(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
 }
+// 1 or 0 without a conversion (conversions from FP64 run on the slow FP64 pipe)
+template <typename R>
+__device__ __forceinline__ R unit(bool one) { return one ? R(1) : R(0); }
+template <>
+__device__ __forceinline__ dd unit<dd>(bool one) { return {one ? 1.f : 0.f, 0.f}; }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ dd rfma(dd a, dd b, dd c) { return dd_fma(a, b, c); }
@@ -219,9 +224,64 @@ __device__ __forceinline__ dd rmul(dd a, dd b) { return dd_mul(a, b); }
 __device__ __forceinline__ double radd(double a, double b) { return a + b; }
 __device__ __forceinline__ float radd(float a, float b) { return a + b; }
 __device__ __forceinline__ dd radd(dd a, dd b) { return dd_add(a, b); }
+__device__ __forceinline__ double rneg(double a) { return -a; }
+__device__ __forceinline__ float rneg(float a) { return -a; }
+__device__ __forceinline__ dd rneg(dd a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ double rsub(double a, double b) { return a - b; }
 __device__ __forceinline__ float rsub(float a, float b) { return a - b; }
 __device__ __forceinline__ dd rsub(dd a, dd b) { return dd_add(a, {-b.hi, -b.lo}); }
+
+// Type of the acceptance ratios and of the diagonal they come from: float pairs
+// where G is held in float pairs (an FP64 instruction of a warp holds its
+// scheduler's FP64 unit for 65 cycles, a dependent float-pair operation takes
+// about 30), FP64 otherwise.
+template <typename Real>
+struct RatioOf { using type = double; };
+template <>
+struct RatioOf<dd> { using type = dd; };
+__device__ __forceinline__ double to_ratio(double x, double) { return x; }
+__device__ __forceinline__ double to_ratio(float x, double) { return (double)x; }
+__device__ __forceinline__ dd to_ratio(dd x, dd) { return x; }
+template <typename Real>
+__device__ __forceinline__ Real ratio_to(double x) { return (Real)x; }
+template <typename Real>
+__device__ __forceinline__ Real ratio_to(dd x) { return x; }
+__device__ __forceinline__ bool is_neg(double x) { return x < 0.0; }
+__device__ __forceinline__ bool is_neg(dd x) { return x.hi < 0.f; }
+// Metropolis: u < min(1, |R|); a NaN ratio counts as 1
+__device__ __forceinline__ bool accepts(double u, double R) {
+  const double a = fabs(R);
+  // |R| >= 1 or NaN from the exponent bits, without an FP64 comparison
+  if ((__double2hiint(a) & 0x7fffffff) >= 0x3ff00000) return true;
+  return u < a;
+}
+__device__ __forceinline__ bool accepts(dd u, dd R) {
+  const float h = fabsf(R.hi), l = R.hi < 0.f ? -R.lo : R.lo;
+  if (!(h < 1.f || (h == 1.f && l < 0.f))) return true;
+  return u.hi < h || (u.hi == h && u.lo < l);
+}
+// a / b by one reciprocal estimate and Newton corrections of the quotient
+// (Markstein, IBM J. Res. Dev. 34, 1990): an error of a few units in the last
+// place in a quarter of the plain division's dependent FP64 instructions; values
+// outside the estimate's FP32 range take the plain division.
+__device__ __forceinline__ double quick_div(double a, double b) {
+  const int e = (__double2hiint(b) >> 20) & 0x7ff;
+  if (e < 1023 - 100 || e > 1023 + 100) return a / b;
+  const double r0 = (double)(1.0f / (float)b);
+  const double r = fma(r0, fma(-b, r0, 1.0), r0);
+  const double q = a * r;
+  return fma(fma(-b, q, a), r, q);
+}
+// float-pair quotient by long division with two correction steps
+__device__ __forceinline__ dd quick_div(dd a, dd b) {
+  const float r = 1.0f / b.hi;
+  const float q0 = a.hi * r;
+  dd t = dd_fma({-q0, 0.f}, b, a);
+  const float q1 = t.hi * r;
+  t = dd_fma({-q1, 0.f}, b, t);
+  const dd q = fast_two_sum(q0, q1);
+  return dd_add(q, {t.hi * r, 0.f});
+}
 
 // --------------------------------------------------------------------------
 // CTA-level dense product C = op(A) op(B), row-major, generic pointers
@@ -427,8 +487,6 @@ struct Smem {
   double* u2;       // [MV]
   double* delta;    // [MV]
   double* gam;      // [MV]
-  double* Rs;       // [2][MV] own-flavor ratios, double buffered (read by the peer CTA)
-  double* Rp;       // [MV] full ratio of the position a thread found accepted
   double* xdiag;    // [ld] exchange: diagonal of G for the potential energy
   double* spare;    // [ld] scratch (the float-pair QR's list of norms to recompute)
   double* xs;       // [8]  exchange: scalars
@@ -468,7 +526,7 @@ __host__ __device__ inline size_t smem_bytes_for(int ld, int MV) {
   size_t b = kSmemCounterBytes;
   b += kGemmRegionBytes;
   b += 6 * (size_t)ld * 8;        // v, ev, d, hv, xdiag, spare
-  b += 6 * (size_t)MV * 8;        // u2, delta, gam, Rs[2], Rp
+  b += 3 * (size_t)MV * 8;        // u2, delta, gam
   b += 8 * 8 + 32 * 8 + 32 * 4;   // xs, red, ired
   b += (size_t)MV * 4;            // qsite
   b += (size_t)ld * 4;            // qinv
@@ -502,8 +560,6 @@ __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   s.u2 = p; p += MV;
   s.delta = p; p += MV;
   s.gam = p; p += MV;
-  s.Rs = p; p += 2 * MV;
-  s.Rp = p; p += MV;
   s.xs = p; p += 8;
   s.red = p; p += 32;
   int* ip = reinterpret_cast<int*>(p);
@@ -989,9 +1045,6 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
 // sides) is staged in the shared GEMM buffer and finished there; everything
 // beyond it is updated by one accumulate-GEMM of depth PB.  PB is the largest
 // power of two <= 16 with PB (N + PB) elements fitting the buffer.
-__device__ __forceinline__ double rneg(double a) { return -a; }
-__device__ __forceinline__ dd rneg(dd a) { return {-a.hi, -a.lo}; }
-
 __device__ inline int lu_block_width(int N) {
   const int cap = 2 * 16 * kGemmMaxTile;
   int pb = 16;
@@ -1507,138 +1560,304 @@ __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const d
 }
 
 // Sequential single-field updates of one slice (Sec. 2.2.1) for this CTA's
-// flavor.  The ratios of every remaining position are evaluated in parallel
-// from the current diagonal of G; the first accepted position in visiting
-// order is found by a block reduction, which is exactly the sequential
-// Metropolis chain because rejected proposals leave G unchanged.  Accepted
-// flips are applied as delayed rank-1 updates (flushed every k accepts):
-//   a = -(delta/R_s) G_eff[:,i],  b = e_i - G_eff[i,:],  G_eff += a b^T.
+// flavor, in windows of kWin consecutive positions of the visiting order.
+//
+// Decisions: the acceptances of a window depend on G only through its kWin x kWin
+// block on the window's sites, for both flavors.  Each CTA publishes its flavor's
+// block of the effective G once per window; then both CTAs run the same chain of
+// decisions on both blocks, kept in registers and updated by a rank-1 step per
+// acceptance, so the flavors meet once per window instead of once per
+// acceptance.  The first acceptance in visiting order is found by a ballot over
+// the remaining positions' ratios, which is exactly the sequential Metropolis
+// chain because rejected proposals leave G unchanged.
+// Vectors: afterwards the accepted flips' delayed vectors
+//   a = -(delta/R_s) G_eff[:,i],  b = e_i - G_eff[i,:],  G_eff += a b^T
+// are formed for all N sites at once, each thread carrying kVecChunk flips'
+// sums of one column or row element through the earlier ones (no barrier between
+// flips: the elements of earlier vectors at the window's sites come from the
+// decisions).  They are flushed into G every delay_k acceptances.
+//
+// The bound is the serial chain per acceptance and the FP64 unit (a warp's FP64
+// instruction holds its scheduler's unit for 65 cycles): one warp per flavor
+// updates the ratios, in float pairs where G is.  Decisions and vectors of one
+// acceptance, measured on GB300: 12x12 float pairs, two CTAs per SM, 2.6 us (5.7 us
+// when every warp evaluated all N ratios and vectors between two cluster barriers
+// per acceptance); 8x8 float pairs 2.4 us (5.6); N = 72 FP64 2.35 us (2.85).
+constexpr int kWin = 32;       // positions per window: one warp lane each
+constexpr int kWinAcc = 16;    // acceptances per window (the vectors' shared memory)
+constexpr int kVecChunk = 8;   // flips whose vectors one thread forms together
+
+// Shared memory of a window: the idle product panels (S.gemm) and the QR's
+// partial sums (S.qred).
+template <typename Real>
+struct Window {
+  using Ratio = typename RatioOf<Real>::type;
+  Real* E;        // [kWin][kWin] this flavor's block of the effective G
+  Ratio* d;       // [kWin] its diagonal
+  Ratio* del;     // [kWin] exp(dv) - 1 of this flavor
+  Ratio* Rs;      // [kMaxFlavors][kWin] ratios
+  Ratio* dl;      // [kMaxFlavors][kWin] deltas of both flavors
+  Real* col;      // [kMaxFlavors][kWin] column of the accepted site
+  Real* row;      // [kMaxFlavors][kWin] its row
+  Real* a;        // [kMaxFlavors][kWin] its delayed vectors on the window
+  Real* b;
+  Real* mfa;      // [kWinAcc] this flavor's -(delta/R_s) per acceptance
+  int* ctl;       // [2] accepted position in the window (-1: none), R < 0
+  int* at;        // [kWinAcc] window positions of the acceptances
+  Real* sA;       // [kWinAcc][kWin] this flavor's a and b on the window, per acceptance
+  Real* sB;
+};
+template <typename Real>
+__device__ __forceinline__ Window<Real> window_of(const Smem& S) {
+  Window<Real> w;
+  double* p = S.gemm;
+  constexpr int blk = kWin * kWin;
+  static_assert((blk + 2 * kWin + 2 * kMaxFlavors * kWin + 4 * kMaxFlavors * kWin + 2 * kWinAcc + 1) * 8 <=
+                kGemmRegionBytes, "the window's block fits the product panels");
+  w.E = reinterpret_cast<Real*>(p); p += blk;
+  using Ratio = typename RatioOf<Real>::type;
+  w.d = reinterpret_cast<Ratio*>(p); p += kWin;
+  w.del = reinterpret_cast<Ratio*>(p); p += kWin;
+  w.Rs = reinterpret_cast<Ratio*>(p); p += kMaxFlavors * kWin;
+  w.dl = reinterpret_cast<Ratio*>(p); p += kMaxFlavors * kWin;
+  w.col = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
+  w.row = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
+  w.a = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
+  w.b = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
+  w.mfa = reinterpret_cast<Real*>(p); p += kWinAcc;
+  w.ctl = reinterpret_cast<int*>(p); p += 1;
+  w.at = reinterpret_cast<int*>(p);
+  static_assert(2 * kWinAcc * kWin <= 8 * 128, "the window's vectors fit the QR's partial sums");
+  w.sA = reinterpret_cast<Real*>(S.qred);
+  w.sB = w.sA + kWinAcc * kWin;
+  return w;
+}
+
+// One column (ROW = false: a) or row (ROW = true: b) element x of the vectors of
+// the nb <= kVecChunk acceptances j0..j0+nb-1 of the window whose first position
+// is pos; n0 vectors were pending before the window.  The sums run over the
+// earlier vectors in order.
+template <typename Real, bool ROW>
+__device__ __forceinline__ void window_vectors(const Real* G, int ld, int x, int pos, int n0, int j0, int nb, Real* A,
+                                               Real* B, const Window<Real>& w, const int* qsite) {
+  Real e[kVecChunk];
+  int f[kVecChunk], site[kVecChunk];
+#pragma unroll
+  for (int j = 0; j < kVecChunk; ++j) {
+    f[j] = w.at[j0 + (j < nb ? j : 0)];
+    site[j] = qsite[pos + f[j]];
+    e[j] = ROW ? G[(size_t)site[j] * ld + x] : G[(size_t)x * ld + site[j]];
+  }
+  for (int m = 0; m < n0; ++m) {
+    const Real v = ROW ? B[(size_t)m * ld + x] : A[(size_t)m * ld + x];
+    const Real* other = (ROW ? A : B) + (size_t)m * ld;
+#pragma unroll
+    for (int j = 0; j < kVecChunk; ++j) e[j] = rfma(v, other[site[j]], e[j]);
+  }
+  for (int q = 0; q < j0; ++q) {
+    const Real v = ROW ? B[(size_t)(n0 + q) * ld + x] : A[(size_t)(n0 + q) * ld + x];
+    const Real* other = (ROW ? w.sA : w.sB) + q * kWin;
+#pragma unroll
+    for (int j = 0; j < kVecChunk; ++j) e[j] = rfma(v, other[f[j]], e[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < kVecChunk; ++j) {
+    if (j >= nb) continue;
+    const Real v = ROW ? rsub(unit<Real>(x == site[j]), e[j]) : rmul(w.mfa[j0 + j], e[j]);
+    (ROW ? B : A)[(size_t)(n0 + j0 + j) * ld + x] = v;
+    const Real* other = (ROW ? w.sA : w.sB) + (j0 + j) * kWin;
+#pragma unroll
+    for (int q = j + 1; q < kVecChunk; ++q) e[q] = rfma(v, other[f[q]], e[q]);
+  }
+}
+
 template <typename Real>
 __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepParams& P, Smem& S,
-                             cg::cluster_group& cl, Real* G, Real* A, Real* B, int& sign, int& buf,
-                             long long* det) {
-  const int N = C.N, ld = C.ld, MV = C.MV, nfl = C.nfl, tid = threadIdx.x;
+                             cg::cluster_group& cl, Real* G, Real* A, Real* B, int& sign, long long* det) {
+  using Ratio = typename RatioOf<Real>::type;
+  const int N = C.N, ld = C.ld, MV = C.MV, nfl = C.nfl, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kRows = kWin / (kThreads / 32);  // window rows per warp: warp + 8 j
   long long t0 = clock64();
   const uint32_t key0 = (uint32_t)P.seed, key1 = (uint32_t)(P.seed >> 32) ^ C.chain_id;
+  Ratio* diag = reinterpret_cast<Ratio*>(S.d);
+  Ratio* u2_q = reinterpret_cast<Ratio*>(S.u2);
+  Ratio* delta_q = reinterpret_cast<Ratio*>(S.delta);
+  Ratio* gam_q = reinterpret_cast<Ratio*>(S.gam);
+  const Ratio one = unit<Ratio>(true);
+  for (int x = tid; x < N; x += kThreads) {
+    diag[x] = to_ratio(G[(size_t)x * ld + x], Ratio());
+    S.qinv[x] = -1;
+  }
+  __syncthreads();
   for (int q = tid; q < MV; q += kThreads) {
     const int k = dir ? MV - 1 - q : q;
     uint32_t ctr[4] = {(uint32_t)P.sweep, (uint32_t)(2 * tau + dir), (uint32_t)k, (uint32_t)(P.sweep >> 32)};
     philox4x32_10(ctr, key0, key1);
     const double u1 = uniform53(ctr[0], ctr[1]);
-    S.u2[q] = uniform53(ctr[2], ctr[3]);
+    u2_q[q] = from_d<Ratio>(uniform53(ctr[2], ctr[3]));
     const int f = S.fslice[k];
     const int fn = propose_field(C.ft, f, u1);
     const double dc = coupling(C.ft, C.cscale, fn) - coupling(C.ft, C.cscale, f);
-    S.delta[q] = exp(C.vsign[s * MV + k] * dc) - 1.0;
-    S.gam[q] = field_weight(C.ft, fn) / field_weight(C.ft, f);
+    delta_q[q] = from_d<Ratio>(exp(C.vsign[s * MV + k] * dc) - 1.0);
+    gam_q[q] = from_d<Ratio>(field_weight(C.ft, fn) / field_weight(C.ft, f));
     S.fnew[q] = (int8_t)fn;
     S.qsite[q] = C.site[k];
-  }
-  for (int x = tid; x < N; x += kThreads) {
-    S.d[x] = to_d(G[(size_t)x * ld + x]);
-    S.qinv[x] = -1;
-  }
-  // first accepted position of the current scan (two slots, alternating)
-  int* first_slot = S.ired + 16;
-  if (tid == 0) first_slot[0] = first_slot[1] = MV;
-  __syncthreads();
-  for (int q = tid; q < MV; q += kThreads) {
-    S.qinv[S.qsite[q]] = q;
-    S.Rs[buf * MV + q] = 1.0 + S.delta[q] * (1.0 - S.d[S.qsite[q]]);
+    S.qinv[C.site[k]] = q;
   }
   __syncthreads();
   tick(det, 0, t0);
+  const Window<Real> w = window_of<Real>(S);
   int pos = 0, nacc = 0;
   int64_t n_acc_slice = 0;
   const int kdel = P.delay_k;
-  // Barriers per acceptance: the cluster barrier (ratios of both flavors) and one
-  // CTA barrier after the scan.  The thread that owns site x updates the
-  // diagonal d_x and the next ratio of the vertex on x itself, so neither needs
-  // a barrier of its own; the flush is preceded by one.
-  while (true) {
-    double* Rs = S.Rs + buf * MV;
-    // the next position is accepted most of the time: start reading its column and
-    // row of G now, so that the cluster barrier covers the memory latency
-    const int ipre = (pos < MV) ? S.qsite[pos] : 0;
-    Real gc_pre = from_d<Real>(0.0), gr_pre = from_d<Real>(0.0);
-    if (tid < N) {
-      gc_pre = G[(size_t)tid * ld + ipre];
-      gr_pre = G[(size_t)ipre * ld + tid];
+  while (pos < MV) {
+    const int W = (MV - pos < kWin) ? MV - pos : kWin;
+    // ---- this flavor's block of the effective G, published to the peer
+    {
+      const int ic = S.qsite[pos + (lane < W ? lane : 0)];
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        const int r = warp + 8 * j;
+        const int ir = S.qsite[pos + (r < W ? r : 0)];
+        Real e = G[(size_t)ir * ld + ic];
+        for (int m = 0; m < nacc; ++m) e = rfma(A[(size_t)m * ld + ir], B[(size_t)m * ld + ic], e);
+        w.E[r * kWin + lane] = e;
+      }
+      if (warp == 0) {
+        w.d[lane] = diag[ic];
+        w.del[lane] = delta_q[pos + (lane < W ? lane : 0)];
+      }
     }
     cl.sync();
-    const double* Rr[kMaxFlavors];
-    for (int r = 0; r < nfl; ++r) Rr[r] = (r == s) ? Rs : cl.map_shared_rank(Rs, r);
-    for (int q = pos + tid; q < MV; q += kThreads) {
-      double R = S.gam[q];
-      for (int r = 0; r < nfl; ++r) R *= Rr[r][q];
-      const double aR = fabs(R);
-      if (S.u2[q] < (aR < 1.0 ? aR : 1.0)) {
-        S.Rp[q] = R;
-        atomicMin(first_slot + buf, q);
-        break;
+    Real e[kMaxFlavors][kRows];
+    Ratio dw = one, delw = one;  // warp r: diagonal and delta of flavor r
+#pragma unroll
+    for (int r = 0; r < kMaxFlavors; ++r) {
+      const bool live = r < nfl;
+      const Real* pe = (!live || r == s) ? w.E : cl.map_shared_rank(w.E, r);
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) e[r][j] = pe[(warp + 8 * j) * kWin + lane];
+      if (live && warp == r) {
+        dw = ((r == s) ? w.d : cl.map_shared_rank(w.d, r))[lane];
+        delw = ((r == s) ? w.del : cl.map_shared_rank(w.del, r))[lane];
+        w.dl[r * kWin + lane] = delw;
+        w.Rs[r * kWin + lane] = rfma(delw, rsub(one, dw), one);
       }
     }
-    __syncthreads();
-    const int first = first_slot[buf];
-    if (tid == 0) first_slot[buf ^ 1] = MV;
+    cl.sync();  // the peer has read this block; both flavors' ratios are in place
+    const Ratio u2 = u2_q[pos + (lane < W ? lane : 0)], gam = gam_q[pos + (lane < W ? lane : 0)];
+    const bool weighted = C.ft != 1;  // Ising fields: gamma = 1
+    int last = -1, na = 0;
+    // ---- decisions
+    while (true) {
+      if (warp == 0) {
+        Ratio R = w.Rs[lane];
+        if (weighted) R = rmul(gam, R);
+        if (nfl == 2) R = rmul(R, w.Rs[kWin + lane]);
+        const bool ok = lane > last && lane < W && accepts(u2, R);
+        const unsigned m = __ballot_sync(0xffffffffu, ok);
+        const int f = m ? __ffs(m) - 1 : -1;
+        if (lane == (m ? f : 0)) {
+          w.ctl[0] = f;
+          w.ctl[1] = is_neg(R);
+        }
+      }
+      __syncthreads();
+      const int f = w.ctl[0];
+      if (f < 0) break;
+      if (w.ctl[1]) sign = -sign;
+      // column f (every warp its rows) and row f (its warp) of both blocks
+      if (lane == f) {
+#pragma unroll
+        for (int r = 0; r < kMaxFlavors; ++r)
+#pragma unroll
+          for (int j = 0; j < kRows; ++j)
+            if (r < nfl) w.col[r * kWin + warp + 8 * j] = e[r][j];
+      }
+      if (warp == (f & 7)) {
+#pragma unroll
+        for (int r = 0; r < kMaxFlavors; ++r)
+#pragma unroll
+          for (int j = 0; j < kRows; ++j)
+            if (r < nfl && j == (f >> 3)) w.row[r * kWin + lane] = e[r][j];
+      }
+      // every lane of the flavor's warp divides for itself
+      Real mf = unit<Real>(false);
+      if (warp < nfl) {
+        const Ratio fac = quick_div(w.dl[warp * kWin + f], w.Rs[warp * kWin + f]);
+        mf = rneg(ratio_to<Real>(fac));
+        if (warp == s && lane == 0) {
+          w.mfa[na] = mf;
+          w.at[na] = f;
+        }
+      }
+      if (tid == 64) {
+        const int q = pos + f;
+        S.fslice[dir ? MV - 1 - q : q] = S.fnew[q];
+      }
+      __syncthreads();
+      if (warp < nfl) {
+        const Real ax = rmul(mf, w.col[warp * kWin + lane]);
+        const Real bx = rsub(unit<Real>(lane == f), w.row[warp * kWin + lane]);
+        w.a[warp * kWin + lane] = ax;
+        w.b[warp * kWin + lane] = bx;
+        if (warp == s) {
+          w.sA[na * kWin + lane] = ax;
+          w.sB[na * kWin + lane] = bx;
+        }
+        dw = rfma(to_ratio(ax, Ratio()), to_ratio(bx, Ratio()), dw);
+        w.Rs[warp * kWin + lane] = rfma(delw, rsub(one, dw), one);
+      }
+      last = f;
+      ++na;
+      __syncthreads();
+      if (na == kWinAcc || nacc + na == kdel) break;
+      // the rows after f of both blocks (earlier ones are not read again)
+#pragma unroll
+      for (int r = 0; r < kMaxFlavors; ++r) {
+        if (r >= nfl) continue;
+        const Real bc = w.b[r * kWin + lane];
+#pragma unroll
+        for (int j = 0; j < kRows; ++j)
+          if (warp + 8 * j > f) e[r][j] = rfma(w.a[r * kWin + warp + 8 * j], bc, e[r][j]);
+      }
+    }
+    // a window that stopped at its limit goes on behind its last acceptance
+    const int next = (na == kWinAcc || nacc + na == kdel) ? pos + last + 1 : pos + W;
     tick(det, 1, t0);
-    if (first >= MV) { buf ^= 1; break; }
-    const double R = S.Rp[first];
-    if (R < 0.0) sign = -sign;
-    const int k = dir ? MV - 1 - first : first;
-    const int i = S.qsite[first];
-    const double fac = S.delta[first] / Rs[first];
-    Real* a = A + (size_t)nacc * ld;
-    Real* b = B + (size_t)nacc * ld;
-    const Real mfac = from_d<Real>(-fac);
-    const bool hit = (first == pos);
-    double* Rs_next = S.Rs + (buf ^ 1) * MV;
-    // element x of column i (a) and of row i (b) of G_eff
-    for (int x = tid; x < N; x += kThreads) {
-      Real cx, ry;
-      if (hit && x == tid) {
-        cx = gc_pre;
-        ry = gr_pre;
-      } else {
-        cx = G[(size_t)x * ld + i];
-        ry = G[(size_t)i * ld + x];
+    // ---- the accepted flips' vectors on all sites: columns, then rows
+    if (na) {
+      const int Np = (N + 31) / 32 * 32;
+      for (int j0 = 0; j0 < na; j0 += kVecChunk) {
+        const int nb = (na - j0 < kVecChunk) ? na - j0 : kVecChunk;
+        for (int u = tid; u < 2 * Np; u += kThreads) {
+          if (u < Np) {
+            if (u < N) window_vectors<Real, false>(G, ld, u, pos, nacc, j0, nb, A, B, w, S.qsite);
+          } else if (u - Np < N) {
+            window_vectors<Real, true>(G, ld, u - Np, pos, nacc, j0, nb, A, B, w, S.qsite);
+          }
+        }
       }
-      // two independent accumulation chains each (even and odd m)
-      Real cx1 = from_d<Real>(0.0), ry1 = from_d<Real>(0.0);
-      int m = 0;
-      for (; m + 1 < nacc; m += 2) {
-        cx = rfma(A[(size_t)m * ld + x], B[(size_t)m * ld + i], cx);
-        ry = rfma(A[(size_t)m * ld + i], B[(size_t)m * ld + x], ry);
-        cx1 = rfma(A[(size_t)(m + 1) * ld + x], B[(size_t)(m + 1) * ld + i], cx1);
-        ry1 = rfma(A[(size_t)(m + 1) * ld + i], B[(size_t)(m + 1) * ld + x], ry1);
-      }
-      if (m < nacc) {
-        cx = rfma(A[(size_t)m * ld + x], B[(size_t)m * ld + i], cx);
-        ry = rfma(A[(size_t)m * ld + i], B[(size_t)m * ld + x], ry);
-      }
-      cx = radd(cx, cx1);
-      ry = radd(ry, ry1);
-      const Real ax = rmul(mfac, cx);
-      const Real bx = rsub(from_d<Real>(x == i ? 1.0 : 0.0), ry);
-      a[x] = ax;
-      b[x] = bx;
-      const double dx = S.d[x] + to_d(ax) * to_d(bx);
-      S.d[x] = dx;
-      const int qx = S.qinv[x];
-      if (qx >= 0) Rs_next[qx] = 1.0 + S.delta[qx] * (1.0 - dx);
+      __syncthreads();
+      // the diagonal on the sites still to be visited in this slice
+      for (int x = tid; x < N; x += kThreads)
+        if (S.qinv[x] >= next) {
+          Ratio dx = diag[x];
+          for (int m = nacc; m < nacc + na; ++m)
+            dx = rfma(to_ratio(A[(size_t)m * ld + x], Ratio()), to_ratio(B[(size_t)m * ld + x], Ratio()), dx);
+          diag[x] = dx;
+        }
+      nacc += na;
+      n_acc_slice += na;
     }
-    if (tid == 0) S.fslice[k] = S.fnew[first];
-    ++nacc;
-    ++n_acc_slice;
     tick(det, 2, t0);
     if (nacc == kdel) {
-      __syncthreads();
       flush_delayed<Real>(C, G, A, B, nacc, S);
       nacc = 0;
       tick(det, 3, t0);
     }
-    pos = first + 1;
-    buf ^= 1;
+    __syncthreads();
+    pos = next;
   }
   if (nacc) flush_delayed<Real>(C, G, A, B, nacc, S);
   tick(det, 3, t0);
@@ -2187,7 +2406,6 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(ChainDev* chains, Sw
   Real* B = P.ab_smem ? A + (size_t)P.delay_k * C.ld : (Real*)C.dB[s];
   const int L = C.L, nw = C.nw, MV = C.MV;
   int sign = C.sign;
-  int buf = 0;
   // thread 0's phase counters: cyc[0..3] per phase, det[0..7] per sub-phase
   long long* cyc = reinterpret_cast<long long*>(smem_raw);
   long long* det = cyc + 4;
@@ -2205,7 +2423,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(ChainDev* chains, Sw
     slice_potential_smem(C, s, S.fslice, S.v);
     v_wrap<Real>(C, G, S.v, +1.0, S);
     lap(1);
-    update_slice<Real>(C, s, tau, 0, P, S, cl, G, A, B, sign, buf, det);
+    update_slice<Real>(C, s, tau, 0, P, S, cl, G, A, B, sign, det);
     if (s == 0)
       for (int k = threadIdx.x; k < MV; k += kThreads) C.fields[(size_t)(tau - 1) * MV + k] = S.fslice[k];
     lap(0);
@@ -2229,7 +2447,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(ChainDev* chains, Sw
     __syncthreads();
     t_wrap<Real>(C, s, G, Gt, false, S);
     lap(1);
-    update_slice<Real>(C, s, tau, 1, P, S, cl, G, A, B, sign, buf, det);
+    update_slice<Real>(C, s, tau, 1, P, S, cl, G, A, B, sign, det);
     if (s == 0)
       for (int k = threadIdx.x; k < MV; k += kThreads) C.fields[(size_t)(tau - 1) * MV + k] = S.fslice[k];
     lap(0);
