@@ -24,11 +24,18 @@ using dqmc::host::symmetric_eigen;
 namespace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+size_t pad_to(size_t n, size_t q) { return (n + q - 1) / q * q; }
 
 // Site count from which chains of a DQMC_PREC_MIXED_TC context run their N^3
 // products on the tensor cores (smaller ones keep the float-pair SIMT tiles).
 constexpr int kDefaultTcMinSites = 96;
 int tc_min_sites(const dqmc_run_opts& o) { return o.tc_min_sites > 0 ? o.tc_min_sites : kDefaultTcMinSites; }
+// ... and from which FP64 products run on them, in every context (the FP64 kernels
+// serve all precisions): below it the FP64 pipe's N^3 / 1.65 cycles are less than
+// the split product's fixed cost.
+constexpr int kTc64MinSites = 32;
+bool pairs_on_tc(const dqmc_run_opts& o, int N) { return o.precision == DQMC_PREC_MIXED_TC && N >= tc_min_sites(o); }
+bool fp64_on_tc(int N) { return N >= kTc64MinSites; }
 
 
 struct ModelHost {
@@ -43,10 +50,10 @@ struct ModelHost {
   float *E32 = nullptr, *Einv32 = nullptr;
   float *Edd = nullptr, *Einvdd = nullptr;  // (hi, lo) pairs
   int* site_d = nullptr;
-  // split-product planes of the constant propagators (tensor-core products only)
-  void* cpl[dqmc::kMaxFlavors][5] = {};
-  int* cex[dqmc::kMaxFlavors][5] = {};
-  CUtensorMap tmc[dqmc::kMaxFlavors][5] = {};
+  // split-product planes of the constant propagators: exponents and tensor maps,
+  // [0] float pairs, [1] FP64
+  int* cex[2][dqmc::kMaxFlavors][dqmc::kCpSets] = {};
+  CUtensorMap tmc[2][dqmc::kMaxFlavors][dqmc::kCpSets] = {};
 };
 
 }  // namespace
@@ -60,6 +67,7 @@ struct dqmc_ctx {
   std::vector<int> chain_model;
   std::vector<ChainDev> chains_h;
   ChainDev* chains_d = nullptr;
+  dqmc::PlaneSet* planes_d = nullptr;
   int* order_d = nullptr;
   unsigned char* arena = nullptr;
   std::vector<void*> model_allocs;
@@ -156,28 +164,65 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// Tensor map of a digit-plane buffer of `bytes` bytes for the split products:
-// the 4D view [blocks][kPlaneDigits][rows][kPlaneK] of bf16 (k innermost,
-// contiguous) with a box of one whole block, so that a tiled copy at block
-// coordinate b moves the b-th block's bytes unchanged.  0 on success.
-int encode_plane_map(CUtensorMap* tm, void* base, int rows, size_t bytes) {
+// Tensor map of a digit-plane buffer of `bytes` bytes for the split products: the 2D
+// view [rows][kPlaneRowElems] of bf16 with a box of one whole block (digits x
+// tile_rows x kPlaneK, contiguous, a multiple of a row's 512 bytes as tile_rows is
+// one of 16), so that a tiled copy moves a block's bytes unchanged.  0 on success.
+int encode_plane_map(CUtensorMap* tm, void* base, int digits, int tile_rows, size_t bytes) {
   const PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
   if (!fn) return 1;
-  const uint64_t row_bytes = (uint64_t)dqmc::kPlaneK * 2;
-  const uint64_t blk = (uint64_t)dqmc::kPlaneDigits * rows * row_bytes;
-  if (bytes < blk || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return 2;
-  const cuuint64_t dims[4] = {(cuuint64_t)dqmc::kPlaneK, (cuuint64_t)rows, (cuuint64_t)dqmc::kPlaneDigits,
-                              (cuuint64_t)(bytes / blk)};
-  const cuuint64_t strides[3] = {row_bytes, (cuuint64_t)rows * row_bytes, blk};
-  const cuuint32_t box[4] = {(cuuint32_t)dqmc::kPlaneK, (cuuint32_t)rows, (cuuint32_t)dqmc::kPlaneDigits, 1u};
-  const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
-  const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+  const uint64_t row_bytes = (uint64_t)dqmc::kPlaneRowElems * 2;
+  const uint64_t blk = (uint64_t)digits * tile_rows * dqmc::kPlaneK * 2;
+  if (bytes < blk || blk % row_bytes != 0 || blk / row_bytes > 256 || (reinterpret_cast<uintptr_t>(base) & 15) != 0)
+    return 2;
+  const cuuint64_t dims[2] = {(cuuint64_t)dqmc::kPlaneRowElems, (cuuint64_t)(bytes / row_bytes)};
+  const cuuint64_t strides[1] = {row_bytes};
+  const cuuint32_t box[2] = {(cuuint32_t)dqmc::kPlaneRowElems, (cuuint32_t)(blk / row_bytes)};
+  const cuuint32_t es[2] = {1u, 1u};
+  const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, es,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : 3;
 }
 
-size_t pad_to(size_t n, size_t q) { return (n + q - 1) / q * q; }
+size_t plane_bytes(int digits, int N, bool right) { return dqmc::plane_elems(digits, N, N, right) * 2; }
+int plane_rows(int N, bool right) { return right ? dqmc::kPlaneRowsB : dqmc::umma_rows(N); }
+
+// The split products' buffers of one (chain, flavor) over the scratch `mem`: 0 on success.
+int fill_plane_set(const ModelHost& M, int s, bool fp64, void* mem, dqmc::PlaneSet& P) {
+  const int N = M.d.n_sites, nd = fp64 ? dqmc::kPlaneDigits64 : dqmc::kPlaneDigits;
+  const size_t a = plane_bytes(nd, N, false), b = plane_bytes(nd, N, true);
+  P.scratch = mem;
+  P.boff = a / 2;
+  int em = encode_plane_map(&P.tm_pl[0], mem, nd, plane_rows(N, false), a);
+  if (!em) em = encode_plane_map(&P.tm_pl[1], static_cast<unsigned char*>(mem) + a, nd, plane_rows(N, true), b);
+  for (int q = 0; q < dqmc::kCpSets; ++q) {
+    P.tm_cp[q] = M.tmc[fp64][s][q];
+    P.cex[q] = M.cex[fp64][s][q];
+  }
+  return em;
+}
+
+// Plane sets of chains laid out over their scratch planes, copied to the device;
+// the chains get the device addresses ([chain][flavor][float pairs, FP64]).
+dqmc_status plane_sets(dqmc_ctx* ctx, std::vector<ChainDev>& chains, const std::vector<int>& chain_model, bool pairs,
+                       dqmc::PlaneSet** out) {
+  std::vector<dqmc::PlaneSet> h(chains.size() * dqmc::kMaxFlavors * 2);
+  CUDA_TRY(ctx, cudaMalloc((void**)out, sizeof(dqmc::PlaneSet) * h.size()));
+  for (size_t c = 0; c < chains.size(); ++c) {
+    const ModelHost& M = ctx->models[chain_model[c]];
+    for (int s = 0; s < M.d.n_flavors; ++s)
+      for (int t = 0; t < 2; ++t) {
+        if (!(t ? fp64_on_tc(M.d.n_sites) : (pairs && pairs_on_tc(ctx->opts, M.d.n_sites)))) continue;
+        const size_t at = (c * dqmc::kMaxFlavors + s) * 2 + t;
+        const int em = fill_plane_set(M, s, t == 1, chains[c].planes[s], h[at]);
+        if (em) return fail(ctx, DQMC_ECUDA, "tensor map of the digit-plane scratch (code %d)", em);
+        (t ? chains[c].ps64 : chains[c].ps)[s] = *out + at;
+      }
+  }
+  CUDA_TRY(ctx, cudaMemcpyAsync(*out, h.data(), sizeof(dqmc::PlaneSet) * h.size(), cudaMemcpyHostToDevice, ctx->stream));
+  return DQMC_OK;
+}
 
 dqmc_status setup_model(dqmc_ctx* ctx, ModelHost& M) {
   const dqmc_model_desc& d = M.d;
@@ -233,40 +278,52 @@ dqmc_status setup_model(dqmc_ctx* ctx, ModelHost& M) {
   if ((st = upload(ctx, &M.ident, ident.data(), ident.size()))) return st;
   if ((st = upload(ctx, &M.site_d, M.site.data(), M.site.size()))) return st;
   if ((st = upload(ctx, &M.vsign_d, M.vsign.data(), M.vsign.size()))) return st;
-  if (ctx->opts.precision == DQMC_PREC_MIXED_TC && N >= tc_min_sites(ctx->opts)) {
-    // digit planes of e^-dtau K and e^+dtau K as the left and right factors of the
-    // wraps and of the B chain, split once per model (Sec. 3.1: the hopping
-    // propagator is a constant of the model)
-    struct { int which, right, tr; bool inv; } sets[5] = {{dqmc::kCpEA, 0, 0, false},
-                                                           {dqmc::kCpEtA, 0, 1, false},
-                                                           {dqmc::kCpEiA, 0, 0, true},
-                                                           {dqmc::kCpEiB, 1, 0, true},
-                                                           {dqmc::kCpEB, 1, 0, false}};
-    const size_t mat = (size_t)N * ld;
+  // digit planes of e^-dtau K and e^+dtau K as the left and right factors of the
+  // wraps and of the B chain, split once per model (Sec. 3.1: the hopping
+  // propagator is a constant of the model), all by one launch
+  struct { int which, right, tr; bool inv; } sets[dqmc::kCpSets] = {{dqmc::kCpEA, 0, 0, false},
+                                                                    {dqmc::kCpEtA, 0, 1, false},
+                                                                    {dqmc::kCpEiA, 0, 0, true},
+                                                                    {dqmc::kCpEiB, 1, 0, true},
+                                                                    {dqmc::kCpEB, 1, 0, false}};
+  const size_t mat = (size_t)N * ld;
+  dqmc::ConstPlaneJobs jobs{};
+  int n_jobs = 0;
+  for (int t = 0; t < 2; ++t) {
+    if (!(t ? fp64_on_tc(N) : pairs_on_tc(ctx->opts, N))) continue;
+    const int nd = t ? dqmc::kPlaneDigits64 : dqmc::kPlaneDigits;
+    size_t bytes = 0, ints = 0;
+    for (const auto& q : sets) {
+      bytes += align_up(plane_bytes(nd, N, q.right), 256);
+      ints += align_up(plane_bytes(1, N, q.right) / (2 * pad_to(N, dqmc::kPlaneK)), 64);
+    }
+    unsigned char* p = nullptr;
+    int* e = nullptr;
+    CUDA_TRY(ctx, cudaMalloc((void**)&p, bytes * nfl));
+    ctx->model_allocs.push_back(p);
+    CUDA_TRY(ctx, cudaMalloc((void**)&e, sizeof(int) * ints * nfl));
+    ctx->model_allocs.push_back(e);
     for (int f = 0; f < nfl; ++f)
       for (const auto& q : sets) {
-        void* p = nullptr;
-        int* e = nullptr;
-        CUDA_TRY(ctx, cudaMalloc(&p, dqmc::const_plane_bytes(N, q.right)));
-        ctx->model_allocs.push_back(p);
-        CUDA_TRY(ctx, cudaMalloc((void**)&e, sizeof(int) * dqmc::const_plane_exps(N, q.right)));
-        ctx->model_allocs.push_back(e);
-        const float* X = (q.inv ? M.Einvdd : M.Edd) + 2 * f * mat;
-        CUDA_TRY(ctx, dqmc::launch_const_planes(X, N, ld, q.right, q.tr, p, e, ctx->stream));
-        M.cpl[f][q.which] = p;
-        M.cex[f][q.which] = e;
-        const int em = encode_plane_map(&M.tmc[f][q.which], p, q.right ? dqmc::kPlaneRowsB : dqmc::kPlaneRowsA,
-                                        dqmc::const_plane_bytes(N, q.right));
+        const void* X = t ? (const void*)((q.inv ? M.Einv : M.E) + f * mat)
+                          : (const void*)((q.inv ? M.Einvdd : M.Edd) + 2 * f * mat);
+        jobs.job[n_jobs++] = {X, p, e, q.right, q.tr, t};
+        M.cex[t][f][q.which] = e;
+        const size_t pb = plane_bytes(nd, N, q.right);
+        const int em = encode_plane_map(&M.tmc[t][f][q.which], p, nd, plane_rows(N, q.right), pb);
         if (em) return fail(ctx, DQMC_ECUDA, "tensor map of the constant digit planes (code %d)", em);
+        p += align_up(pb, 256);
+        e += align_up(plane_bytes(1, N, q.right) / (2 * pad_to(N, dqmc::kPlaneK)), 64);
       }
   }
+  if (n_jobs) CUDA_TRY(ctx, dqmc::launch_const_planes(jobs, n_jobs, N, ld, ctx->stream));
   return DQMC_OK;
 }
 
 // Per-chain device memory, carved from one arena.  Returns the bytes needed
 // (ptrs filled when base != nullptr).
 size_t chain_layout(const ModelHost& M, int precision, int delay_k, unsigned char* base, ChainDev* C,
-                    int tc_min = 1) {
+                    bool pairs_tc = false) {
   const int N = M.d.n_sites, ld = M.ld, nfl = M.d.n_flavors, nst = M.d.L / M.d.n_wrap;
   const size_t rs = precision == DQMC_PREC_FP32 ? sizeof(float) : sizeof(double);  // FP64 or float pairs
   size_t off = 0;
@@ -295,9 +352,11 @@ size_t chain_layout(const ModelHost& M, int precision, int delay_k, unsigned cha
     if (C) C->work[s] = (double*)p;
     p = take((size_t)2 * ld * sizeof(int));
     if (C) C->iwork[s] = (int*)p;
-    if (precision == DQMC_PREC_MIXED_TC && N >= tc_min) {
-      // BF16 digit planes of the split tensor-core products (N x N x N at most)
-      p = take(dqmc::plane_bytes(N, N));
+    // BF16 digit planes of the split tensor-core products (N x N x N at most): both
+    // operand types use the same memory, never at the same time
+    const int nd = fp64_on_tc(N) ? dqmc::kPlaneDigits64 : pairs_tc ? dqmc::kPlaneDigits : 0;
+    if (nd) {
+      p = take(plane_bytes(nd, N, false) + plane_bytes(nd, N, true));
       if (C) C->planes[s] = p;
     }
   }
@@ -325,11 +384,6 @@ void fill_model_fields(const ModelHost& M, ChainDev& C) {
     C.Einv32[s] = M.Einv32 + s * mat;
     C.Edd[s] = M.Edd + 2 * s * mat;
     C.Einvdd[s] = M.Einvdd + 2 * s * mat;
-    for (int q = 0; q < 5; ++q) {
-      C.cpl[s][q] = M.cpl[s][q];
-      C.cex[s][q] = M.cex[s][q];
-      C.tm_cp[s][q] = M.tmc[s][q];
-    }
   }
   C.site = M.site_d;
   C.vsign = M.vsign_d;
@@ -455,7 +509,7 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   for (int i = 0; i < n_chains; ++i) {
     offs[i] = total;
     total += chain_layout(c->models[chain_model[i]], opts->precision, opts->delay_k, nullptr, nullptr,
-                          tc_min_sites(*opts));
+                          pairs_on_tc(*opts, models[chain_model[i]].n_sites));
   }
   if (cudaMalloc((void**)&c->arena, total) != cudaSuccess) {
     *out = ctx.release();
@@ -467,24 +521,8 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   for (int i = 0; i < n_chains; ++i) {
     ChainDev& C = c->chains_h[i];
     const ModelHost& M = c->models[chain_model[i]];
-    chain_layout(M, opts->precision, opts->delay_k, c->arena + offs[i], &C, tc_min_sites(*opts));
+    chain_layout(M, opts->precision, opts->delay_k, c->arena + offs[i], &C, pairs_on_tc(*opts, M.d.n_sites));
     fill_model_fields(M, C);
-    for (int s = 0; s < M.d.n_flavors; ++s) {
-      if (!C.planes[s]) continue;
-      // the scratch planes: the left operand's blocks first, the right operand's
-      // after them (the offset the kernels use)
-      const size_t N = (size_t)M.d.n_sites, kp = pad_to(N, dqmc::kPlaneK);
-      const size_t bytesA = (size_t)dqmc::kPlaneDigits * pad_to(N, dqmc::kPlaneRowsA) * kp * 2;
-      const size_t bytesB = (size_t)dqmc::kPlaneDigits * pad_to(N, dqmc::kPlaneRowsB) * kp * 2;
-      int em = encode_plane_map(&C.tm_pl[s][0], C.planes[s], dqmc::kPlaneRowsA, bytesA);
-      if (!em)
-        em = encode_plane_map(&C.tm_pl[s][1], static_cast<unsigned char*>(C.planes[s]) + bytesA, dqmc::kPlaneRowsB,
-                              bytesB);
-      if (em) {
-        *out = ctx.release();
-        return fail(*out, DQMC_ECUDA, "tensor map of the digit-plane scratch (code %d)", em);
-      }
-    }
     C.chain_id = (uint32_t)i;
     C.sign = 1;
     C.wait_cycles = opts->spin_limit;
@@ -508,6 +546,7 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   }
   *out = ctx.release();
   c = *out;
+  if ((st = plane_sets(c, c->chains_h, c->chain_model, true, &c->planes_d))) return st;
   CUDA_TRY(c, cudaMalloc((void**)&c->chains_d, sizeof(ChainDev) * n_chains));
   CUDA_TRY(c, cudaMemcpyAsync(c->chains_d, c->chains_h.data(), sizeof(ChainDev) * n_chains, cudaMemcpyHostToDevice,
                               c->stream));
@@ -525,23 +564,16 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   CUDA_TRY(c, cudaEventCreate(&c->ev0));
   CUDA_TRY(c, cudaEventCreate(&c->ev1));
   {
-    // the split tensor-core products stage their operands in a region of the
-    // dynamic shared memory; in the sweep it doubles as the delayed vectors A, B,
-    // kept in shared memory when they fit beside the rest
-    const int umma = opts->precision == DQMC_PREC_MIXED_TC;
-    const size_t base = dqmc::sweep_smem_bytes(c->maxN, c->maxld, c->maxMV, opts->delay_k, opts->precision);
+    // the split tensor-core products stage their operands over the SIMT products'
+    // panels and the delayed vectors A, B, which are kept in shared memory when they
+    // fit beside the rest
     const size_t rs = c->kprec == DQMC_PREC_FP32 ? sizeof(float) : sizeof(double);
     const size_t ab = (size_t)2 * opts->delay_k * c->maxld * rs;
-    c->smem = base + (umma ? dqmc::smem_tail(0, umma) : 0);
-    c->ab_smem = (base + dqmc::smem_tail(ab, umma) <= 200 * 1024) ? 1 : 0;
-    c->smem_sweep = base + dqmc::smem_tail(c->ab_smem ? ab : 0, umma);
-    if (umma) {
-      // every CTA of these kernels holds half of the SM's tensor
-      // memory (256 of 512 columns): at least 78 KB of shared memory per CTA keeps
-      // three of them from sharing an SM, so an allocation never waits
-      c->smem = std::max<size_t>(c->smem, 78 * 1024);
-      c->smem_sweep = std::max<size_t>(c->smem_sweep, 78 * 1024);
-    }
+    const int nd64 = fp64_on_tc(c->maxN) ? dqmc::kPlaneDigits64 : 0;
+    const int nd = c->kprec == DQMC_PREC_MIXED ? (pairs_on_tc(*opts, c->maxN) ? dqmc::kPlaneDigits : 0) : nd64;
+    c->smem = dqmc::smem_total(c->maxld, c->maxMV, 0, c->maxN, std::max(nd, nd64));
+    c->ab_smem = (dqmc::smem_total(c->maxld, c->maxMV, ab, c->maxN, nd) <= 200 * 1024) ? 1 : 0;
+    c->smem_sweep = dqmc::smem_total(c->maxld, c->maxMV, c->ab_smem ? ab : 0, c->maxN, nd);
   }
   if (!fields_or_null) CUDA_TRY(c, dqmc::launch_init_fields(c->chains_d, n_chains, opts->seed, 0, 0, c->stream));
   return initial_fill(c);
@@ -823,7 +855,11 @@ dqmc_status run_tau_measure(dqmc_ctx* ctx, int32_t n_tau, const double* site_pha
     st = download_chains(ctx);
     if (st) break;
     for (const ChainDev& C : ctx->chains_h)
-      if (C.error) { st = fail(ctx, DQMC_EUNSTABLE, "chain %u: singular matrix in the stabilisation", C.chain_id); break; }
+      if (C.error) {
+        st = (C.error & 2) ? timeout_message(ctx, C)
+                           : fail(ctx, DQMC_EUNSTABLE, "chain %u: singular matrix in the stabilisation", C.chain_id);
+        break;
+      }
   } while (false);
   cleanup();
   if (st) return st;
@@ -994,6 +1030,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
     ch[c].sign = 1;
   }
   ChainDev* ch_d = nullptr;
+  dqmc::PlaneSet* ps_d = nullptr;
   double *V_d = nullptr, *w_d = nullptr, *gK_d = nullptr, *gU_d = nullptr;
   std::vector<double> Vh((size_t)nfl * N * N), wh((size_t)nfl * N);
   for (int s = 0; s < nfl; ++s) {
@@ -1004,6 +1041,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   auto cleanup = [&]() {
     cudaFree(arena);
     cudaFree(ch_d);
+    cudaFree(ps_d);
     cudaFree(V_d);
     cudaFree(w_d);
     cudaFree(gK_d);
@@ -1022,6 +1060,10 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   for (int c = 0; c < n_cfg; ++c)
     GRAD_TRY(cudaMemcpyAsync(ch[c].fields, fields + (size_t)c * L * MV, (size_t)L * MV, cudaMemcpyHostToDevice,
                              ctx->stream));
+  if ((st = plane_sets(ctx, ch, std::vector<int>(n_cfg, model_index), false, &ps_d))) {
+    cleanup();
+    return st;
+  }
   GRAD_TRY(cudaMalloc((void**)&ch_d, sizeof(ChainDev) * n_cfg));
   GRAD_TRY(cudaMemcpyAsync(ch_d, ch.data(), sizeof(ChainDev) * n_cfg, cudaMemcpyHostToDevice, ctx->stream));
   GRAD_TRY(cudaMalloc((void**)&V_d, sizeof(double) * Vh.size()));
@@ -1030,7 +1072,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   GRAD_TRY(cudaMalloc((void**)&gU_d, sizeof(double) * (size_t)n_cfg * nfl));
   GRAD_TRY(cudaMemcpyAsync(V_d, Vh.data(), sizeof(double) * Vh.size(), cudaMemcpyHostToDevice, ctx->stream));
   GRAD_TRY(cudaMemcpyAsync(w_d, wh.data(), sizeof(double) * wh.size(), cudaMemcpyHostToDevice, ctx->stream));
-  dqmc::set_smem_bytes(dqmc::sweep_smem_bytes(N, M.ld, MV, 1, 0));
+  dqmc::set_smem_bytes(dqmc::smem_total(M.ld, MV, 0, N, fp64_on_tc(N) ? dqmc::kPlaneDigits64 : 0));
   GRAD_TRY(dqmc::launch_logdet_grad(ch_d, n_cfg, nfl, V_d, w_d, gK_d, gU_d, nullptr, ctx->stream));
   GRAD_TRY(cudaMemcpyAsync(grad_K, gK_d, sizeof(double) * (size_t)n_cfg * nfl * N * N, cudaMemcpyDeviceToHost,
                            ctx->stream));
@@ -1039,7 +1081,8 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   GRAD_TRY(cudaStreamSynchronize(ctx->stream));
 #undef GRAD_TRY
   for (int c = 0; c < n_cfg; ++c) {
-    if (ch[c].error) st = fail(ctx, DQMC_EUNSTABLE, "configuration %d: singular matrix in the stabilisation", c);
+    if (ch[c].error & 2) st = timeout_message(ctx, ch[c]);
+    else if (ch[c].error) st = fail(ctx, DQMC_EUNSTABLE, "configuration %d: singular matrix in the stabilisation", c);
     for (int s = 0; s < nfl; ++s) logdet[(size_t)c * nfl + s] = ch[c].logdet[s];
   }
   cleanup();
@@ -1064,12 +1107,14 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   std::vector<ChainDev> ch(n_cfg, ChainDev{});
   unsigned char* arena = nullptr;
   ChainDev* ch_d = nullptr;
+  dqmc::PlaneSet* ps_d = nullptr;
   double *V_d = nullptr, *w_d = nullptr, *G0_d = nullptr, *ew_d = nullptr, *gK_d = nullptr, *gU_d = nullptr,
          *ep_d = nullptr;
   dqmc_status st = DQMC_OK;
   auto cleanup = [&]() {
     cudaFree(arena);
     cudaFree(ch_d);
+    cudaFree(ps_d);
     cudaFree(V_d);
     cudaFree(w_d);
     cudaFree(G0_d);
@@ -1102,6 +1147,10 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
     std::copy(M.eigvec[s].begin(), M.eigvec[s].end(), Vh.begin() + (size_t)s * N * N);
     std::copy(M.eigval[s].begin(), M.eigval[s].end(), wh.begin() + (size_t)s * N);
   }
+  if ((st = plane_sets(ctx, ch, std::vector<int>(n_cfg, model_index), false, &ps_d))) {
+    cleanup();
+    return st;
+  }
   EGRAD_TRY(cudaMalloc((void**)&ch_d, sizeof(ChainDev) * n_cfg));
   EGRAD_TRY(cudaMemcpyAsync(ch_d, ch.data(), sizeof(ChainDev) * n_cfg, cudaMemcpyHostToDevice, ctx->stream));
   EGRAD_TRY(cudaMalloc((void**)&V_d, sizeof(double) * Vh.size()));
@@ -1113,7 +1162,7 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   EGRAD_TRY(cudaMalloc((void**)&gK_d, sizeof(double) * (size_t)n_cfg * nfl * N * N));
   EGRAD_TRY(cudaMalloc((void**)&gU_d, sizeof(double) * (size_t)n_cfg * nfl));
   EGRAD_TRY(cudaMalloc((void**)&ep_d, sizeof(double) * (size_t)n_cfg * nfl * 3));
-  dqmc::set_smem_bytes(dqmc::sweep_smem_bytes(N, ld, MV, 1, 0));
+  dqmc::set_smem_bytes(dqmc::smem_total(ld, MV, 0, N, fp64_on_tc(N) ? dqmc::kPlaneDigits64 : 0));
   EGRAD_TRY(dqmc::launch_energy_grad(ch_d, n_cfg, nfl, V_d, w_d, G0_d, ew_d, gK_d, gU_d, ep_d, ctx->stream));
   std::vector<double> gU((size_t)n_cfg * nfl), ep((size_t)n_cfg * nfl * 3);
   EGRAD_TRY(cudaMemcpyAsync(grad_K, gK_d, sizeof(double) * (size_t)n_cfg * nfl * N * N, cudaMemcpyDeviceToHost,
@@ -1124,7 +1173,8 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   EGRAD_TRY(cudaStreamSynchronize(ctx->stream));
 #undef EGRAD_TRY
   for (int c = 0; c < n_cfg; ++c) {
-    if (ch[c].error) st = fail(ctx, DQMC_EUNSTABLE, "configuration %d: singular matrix in the stabilisation", c);
+    if (ch[c].error & 2) st = timeout_message(ctx, ch[c]);
+    else if (ch[c].error) st = fail(ctx, DQMC_EUNSTABLE, "configuration %d: singular matrix in the stabilisation", c);
     double kin = 0.0, part = 0.0, pot = 0.0, gu = 0.0;
     for (int s = 0; s < nfl; ++s) {
       kin += ep[((size_t)c * nfl + s) * 3 + 0];
@@ -1149,6 +1199,7 @@ void dqmc_destroy(dqmc_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
   cudaFree(ctx->arena);
   cudaFree(ctx->chains_d);
+  cudaFree(ctx->planes_d);
   cudaFree(ctx->order_d);
   cudaFree(ctx->scratch);
   cudaFree(ctx->tau_work);

@@ -283,17 +283,24 @@ __device__ __forceinline__ dd quick_div(dd a, dd b) {
   return dd_add(q, {t.hi * r, 0.f});
 }
 
+// A pointer known to lie in shared memory, in a function that is not inlined and
+// could not tell (generic loads of the panels cost the products a quarter).
+template <typename T>
+__device__ __forceinline__ T* as_shared(T* p) {
+  return reinterpret_cast<T*>(__cvta_shared_to_generic(__cvta_generic_to_shared(p)));
+}
+
 // --------------------------------------------------------------------------
 // CTA-level dense product C = op(A) op(B), row-major, generic pointers
-// (global or shared).  Output tiles of 16R x 16R (R = 3, 4, 5 outputs per
-// thread and dimension; R is picked per size so that N = 144 or 400 need no
-// padding), 16-deep K panels staged in shared memory.  C must not alias A or B.
+// (global or shared).  Output tiles of 16R x 16R (R = 1..5 outputs per thread and
+// dimension; R is picked per size so that N = 16, 144 or 400 need no padding),
+// 16-deep K panels staged in shared memory.  C must not alias A or B.
 // --------------------------------------------------------------------------
 constexpr int kGemmMaxTile = 80;  // 16 * 5
 
 __host__ __device__ inline int gemm_pick_r(int n) {
   int best_r = 4, best = 1 << 30;
-  for (int r = 5; r >= 3; --r) {
+  for (int r = 5; r >= 1; --r) {
     const int t = 16 * r;
     const int padded = ((n + t - 1) / t) * t;
     if (padded < best) { best = padded; best_r = r; }
@@ -305,8 +312,8 @@ template <typename T, bool TA, bool TB, int R, bool ACC = false>
 __device__ void cta_gemm_r(int M, int Nc, int Kd, const T* __restrict__ A, int lda, const T* __restrict__ B,
                            int ldb, T* __restrict__ C, int ldc, T* sm) {
   constexpr int TT = 16 * R;
-  T* As = sm;            // [16][TT]
-  T* Bs = sm + 16 * TT;  // [16][TT]
+  T* As = as_shared(sm);  // [16][TT]
+  T* Bs = As + 16 * TT;   // [16][TT]
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += TT)
     for (int n0 = 0; n0 < Nc; n0 += TT) {
@@ -363,11 +370,15 @@ __device__ void cta_gemm_r(int M, int Nc, int Kd, const T* __restrict__ A, int l
   __syncthreads();
 }
 
+// One copy per kernel and operand form (a call costs nothing beside the product;
+// inlined copies at every call site took minutes to compile and spilled).
 template <typename T, bool TA, bool TB>
-__device__ void cta_gemm(int M, int Nc, int Kd, const T* __restrict__ A, int lda, const T* __restrict__ B,
+__device__ __noinline__ void cta_gemm(int M, int Nc, int Kd, const T* __restrict__ A, int lda, const T* __restrict__ B,
                          int ldb, T* __restrict__ C, int ldc, T* sm) {
   const int r = gemm_pick_r(M > Nc ? M : Nc);
-  if (r == 3) cta_gemm_r<T, TA, TB, 3>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
+  if (r == 1) cta_gemm_r<T, TA, TB, 1>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
+  else if (r == 2) cta_gemm_r<T, TA, TB, 2>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
+  else if (r == 3) cta_gemm_r<T, TA, TB, 3>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
   else if (r == 5) cta_gemm_r<T, TA, TB, 5>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
   else cta_gemm_r<T, TA, TB, 4>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
 }
@@ -380,8 +391,8 @@ template <bool TA, bool TB, int R, bool ACC = false>
 __device__ void cta_gemm_dd_r(int M, int Nc, int Kd, const dd* __restrict__ A, int lda, const dd* __restrict__ B,
                               int ldb, dd* __restrict__ C, int ldc, dd* sm) {
   constexpr int TT = 16 * R;
-  dd* As = sm;            // [16][TT]
-  dd* Bs = sm + 16 * TT;  // [16][TT]
+  dd* As = as_shared(sm);  // [16][TT]
+  dd* Bs = As + 16 * TT;   // [16][TT]
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += TT)
     for (int n0 = 0; n0 < Nc; n0 += TT) {
@@ -479,7 +490,7 @@ __device__ __forceinline__ void cta_copy(int N, int ld, const T* src, T* dst) {
 // --------------------------------------------------------------------------
 struct Smem {
   double* gemm;     // kGemmRegionBytes: 2*16*kGemmMaxTile doubles of the SIMT GEMM panels (also
-                    // float / float-pair), or a staging buffer of the tensor-core products
+                    // float / float-pair)
   double* v;        // [ld] slice potential / exp factors
   double* ev;       // [ld]
   double* d;        // [ld] current diagonal of the effective G
@@ -501,7 +512,9 @@ struct Smem {
   double* ab;       // delayed vectors A, B [2][k][ld] when they fit in shared memory
   int flavor;       // the CTA's flavor
   double* qred;     // [8][128] partial sums of the QR trailing update
-  Umma um;          // tensor-core products: barriers and TMEM slot, staging aliased with ab
+  Umma um;          // tensor-core products: barriers and TMEM slot, staging over gemm and ab
+  const PlaneSet* ps;    // split products of float pairs (null: SIMT tiles)
+  const PlaneSet* ps64;  // split products of FP64 operands (null: the FP64 pipe)
   int dd_tile;      // register tile of the float-pair SIMT products (0: by padding, 3, 4)
 };
 
@@ -509,22 +522,17 @@ struct Smem {
 // cycle counters of the sweep kernel (fixed addresses, no registers).
 constexpr int kSmemCounterBytes = 16 * 8;
 
-// exponent entries per operand of the split products: rows padded to the tile height
-__host__ __device__ inline int exp_len(int ld) {
-  const int a = umma_pad(ld, kUmmaM), b = umma_pad(ld, kUmmaNT);
-  return a > b ? a : b;
-}
+// exponent entries per operand of the split products: rows padded to whole tiles
+__host__ __device__ inline int exp_len(int ld) { return ld + kPlaneMaxRows; }
 
-// Shared memory of the fresh-G, measurement and adjoint kernels.  The sweep
-// kernel adds the delayed vectors at the end; with the tensor-core products
-// the same region (s.ab) holds their two staging buffers, which are only live
-// inside a product, never while delayed vectors are pending.
-constexpr int kGemmRegionBytes =
-    (2 * 16 * kGemmMaxTile * 8 > kUmmaStageBytes) ? 2 * 16 * kGemmMaxTile * 8 : kUmmaStageBytes;
+// Layout: the vectors and barriers, then (128-byte aligned) the SIMT products'
+// panels and, in the sweep kernel, the delayed vectors.  The tensor-core products
+// stage their operands over both: neither is live inside a product (a flush has
+// cut its delayed vectors into digits before the first copy lands).
+constexpr int kGemmRegionBytes = 2 * 16 * kGemmMaxTile * 8;
 
-__host__ __device__ inline size_t smem_bytes_for(int ld, int MV) {
+__host__ __device__ inline size_t smem_stage_offset(int ld, int MV) {
   size_t b = kSmemCounterBytes;
-  b += kGemmRegionBytes;
   b += 6 * (size_t)ld * 8;        // v, ev, d, hv, xdiag, spare
   b += 3 * (size_t)MV * 8;        // u2, delta, gam
   b += 8 * 8 + 32 * 8 + 32 * 4;   // xs, red, ired
@@ -536,21 +544,15 @@ __host__ __device__ inline size_t smem_bytes_for(int ld, int MV) {
   b += 2 * (size_t)exp_len(ld) * 4;  // expA, expB
   b = (b + 15) / 16 * 16;
   b += 128;                       // mbarriers and the TMEM slot of the tensor-core products
-  return b;
+  return (b + 127) / 128 * 128 + 128;  // room to align the panels
 }
-// Bytes of the region at s.ab (start 128-byte aligned by carve_smem): the
-// delayed vectors, or the second and third staging buffers of the tensor-core
-// products (the first is the GEMM region).
-__host__ __device__ inline size_t smem_tail_bytes(size_t ab_bytes, bool umma) {
-  const size_t st = umma ? (size_t)(kUmmaStages - 1) * kUmmaStageBytes : 0;
-  return 128 + (ab_bytes > st ? ab_bytes : st);
-}
+__host__ __device__ inline size_t smem_bytes_for(int ld, int MV) { return smem_stage_offset(ld, MV) + kGemmRegionBytes; }
 
 __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   Smem s;
+  unsigned char* const start = base;
   base += kSmemCounterBytes;
   double* p = reinterpret_cast<double*>(base);
-  s.gemm = p; p += kGemmRegionBytes / 8;
   s.v = p; p += ld;
   s.ev = p; p += ld;
   s.d = p; p += ld;
@@ -581,43 +583,63 @@ __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   s.um.err = nullptr;
   s.um.where = nullptr;
   s.dd_tile = 0;
+  s.ps = nullptr;
+  s.ps64 = nullptr;
   s.um.limit = kUmmaWaitCycles;
   s.um.stall = 0;
-  s.um.tmA = nullptr;
-  s.um.tmB = nullptr;
-  s.um.boff = 0;
   q += 128;
-  // base is 16-byte aligned (kSmemCounterBytes past the start); align s.ab to 128
-  const uintptr_t qa = (reinterpret_cast<uintptr_t>(q) + 127) & ~(uintptr_t)127;
-  s.ab = reinterpret_cast<double*>(qa);
-  s.um.stage0 = reinterpret_cast<unsigned char*>(s.gemm);
-  s.um.stage1 = reinterpret_cast<unsigned char*>(qa);
+  q = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(q) + 127) & ~(uintptr_t)127);
+  s.gemm = reinterpret_cast<double*>(q);
+  s.ab = reinterpret_cast<double*>(q + kGemmRegionBytes);
+  uint32_t dyn;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+  s.um.stage = q;
+  s.um.stage_bytes = dyn - (uint32_t)(q - start);
   return s;
 }
 
+// The split products of this CTA: float pairs (want_dd) and / or FP64 operands,
+// where the chain has plane buffers.  Returns whether tensor memory was allocated
+// (every path out of the kernel then calls umma_free).
+__device__ __forceinline__ bool umma_begin(ChainDev& C, int s, Smem& S, bool want_dd, bool want_64) {
+  S.dd_tile = C.dd_tile;
+  S.um.err = &C.error;
+  // the caller's wait limit and the test hook concern the float-pair products; FP64
+  // ones keep the default limit
+  S.um.limit = (want_dd && C.wait_cycles > 0) ? C.wait_cycles : kUmmaWaitCycles;
+  S.um.stall = want_dd ? C.test_stall : 0;
+  S.um.where = C.wait_where[s];
+  S.ps = want_dd ? C.ps[s] : nullptr;
+  S.ps64 = want_64 ? C.ps64[s] : nullptr;
+  const bool on = S.ps != nullptr || S.ps64 != nullptr;
+  if (on) umma_alloc(S.um);
+  return on;
+}
+
 // Float-pair product of the mixed path: exact-split tensor-core products when
-// the chain has digit-plane scratch, the float-pair SIMT tiles otherwise.
+// the chain has plane buffers, the float-pair SIMT tiles otherwise.  constA /
+// constB: index of a prepared constant operand (kCpEA ...), -1: split here.
 template <bool TA, bool TB, bool ACC>
 __device__ void gemm_dd(const ChainDev& C, int s, Smem& S, int M, int Nc, int Kd, const dd* A, int lda, const dd* B,
                         int ldb, dd* Cm, int ldc, int constA = -1, int constB = -1) {
 #if DQMC_WITH_UMMA
-  if (C.planes[s]) {
-    // constA / constB: index of a prepared constant operand (kCpEA ...), -1: split here
-    const UmmaOperand cA = constA >= 0 ? UmmaOperand{(const __nv_bfloat16*)C.cpl[s][constA], C.cex[s][constA],
-                                                     &C.tm_cp[s][constA]}
-                                       : UmmaOperand{nullptr, nullptr, nullptr};
-    const UmmaOperand cB = constB >= 0 ? UmmaOperand{(const __nv_bfloat16*)C.cpl[s][constB], C.cex[s][constB],
-                                                     &C.tm_cp[s][constB]}
-                                       : UmmaOperand{nullptr, nullptr, nullptr};
-    gemm_umma<TA, TB, ACC>(M, Nc, Kd, A, lda, B, ldb, Cm, ldc, (__nv_bfloat16*)C.planes[s], S.expA, S.expB, S.um,
-                           cA, cB);
+  if (S.ps) {
+    gemm_umma<dd>(TA, TB, ACC, M, Nc, Kd, A, lda, B, ldb, Cm, ldc, S.ps, S.expA, S.expB, S.um, constA, constB);
     return;
   }
-#else
-  (void)constA;
-  (void)constB;
 #endif
   gemm_dd_tiles<TA, TB, ACC>(M, Nc, Kd, A, lda, B, ldb, Cm, ldc, reinterpret_cast<dd*>(S.gemm), S.dd_tile);
+}
+
+// FP64 product: exact-split tensor-core products when the chain has plane buffers
+// (its N from kTc64MinSites), the FP64 pipe's tiles otherwise.
+template <bool TA, bool TB>
+__device__ void gemm_64(Smem& S, int M, int Nc, int Kd, const double* A, int lda, const double* B, int ldb, double* Cm,
+                        int ldc, int constA = -1, int constB = -1) {
+  if (S.ps64)
+    gemm_umma<double>(TA, TB, false, M, Nc, Kd, A, lda, B, ldb, Cm, ldc, S.ps64, S.expA, S.expB, S.um, constA, constB);
+  else
+    cta_gemm<double, TA, TB>(M, Nc, Kd, A, lda, B, ldb, Cm, ldc, S.gemm);
 }
 
 // Slice potential v^s_i of slice tau (1-based) from global fields.
@@ -948,7 +970,7 @@ template <typename T>
 __device__ int lu_factor_blk(int N, int ld, T* A, int* piv, T* tmp, double& logdet, int& sign, Smem& S);
 
 __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, UDV src, Smem& S,
-                      long long* det = nullptr) {
+                                       long long* det = nullptr) {
   long long t0 = clock64();
   const int N = C.N, ld = C.ld;
   double* X = wmat(C, s, 0);
@@ -965,12 +987,12 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
         X[(size_t)x * ld + y] *= S.ev[x];
       }
       __syncthreads();
-      cta_gemm<double, false, false>(N, N, N, E, ld, X, ld, Y, ld, S.gemm);
+      gemm_64<false, false>(S, N, N, N, E, ld, X, ld, Y, ld, kCpEA, -1);
       double* t_ = X; X = Y; Y = t_;
     }
   } else {
     for (int t = t2; t >= t1 + 1; --t) {
-      cta_gemm<double, true, false>(N, N, N, E, ld, X, ld, Y, ld, S.gemm);
+      gemm_64<true, false>(S, N, N, N, E, ld, X, ld, Y, ld, kCpEtA, -1);
       slice_potential_global(C, s, t, S.v);
       for (int x = threadIdx.x; x < N; x += kThreads) S.ev[x] = exp(S.v[x]);
       __syncthreads();
@@ -1006,7 +1028,7 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
     int detq = 1;
     if (lu_factor_blk(N, ld, Ucp, C.iwork[s] + ld, wmat(C, s, 9), ldu, detq, S)) detq = 1;
     tick(det, 5, t0);
-    cta_gemm<double, true, false>(N, N, N, V, ld, src.T, ld, wmat(C, s, 5), ld, S.gemm);
+    gemm_64<true, false>(S, N, N, N, V, ld, src.T, ld, wmat(C, s, 5), ld);
     tick(det, 6, t0);
     return detq;
   }
@@ -1027,7 +1049,7 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
     Rt[(size_t)x * ld + y] = (y >= x && Dn[x] > 0.0) ? X[(size_t)x * ld + y] / Dn[x] : 0.0;
   }
   __syncthreads();
-  cta_gemm<double, false, false>(N, N, N, Rt, ld, PT, ld, wmat(C, s, 5), ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, Rt, ld, PT, ld, wmat(C, s, 5), ld);
   tick(det, 6, t0);
   return detq;
 }
@@ -1053,10 +1075,12 @@ __device__ inline int lu_block_width(int N) {
 }
 
 // C += A B (row-major, no transposes) on the register-tiled CTA products.
-__device__ inline void gemm_acc(int M, int Nc, int Kd, const double* A, int lda, const double* B, int ldb, double* C,
+__device__ __noinline__ void gemm_acc(int M, int Nc, int Kd, const double* A, int lda, const double* B, int ldb, double* C,
                                 int ldc, Smem& S) {
   const int r = gemm_pick_r(M > Nc ? M : Nc);
-  if (r == 3) cta_gemm_r<double, false, false, 3, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  if (r == 1) cta_gemm_r<double, false, false, 1, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  else if (r == 2) cta_gemm_r<double, false, false, 2, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  else if (r == 3) cta_gemm_r<double, false, false, 3, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
   else if (r == 5) cta_gemm_r<double, false, false, 5, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
   else cta_gemm_r<double, false, false, 4, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
 }
@@ -1232,8 +1256,8 @@ __device__ int green_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, double* G
   const int N = C.N, ld = C.ld;
   double* W0 = wmat(C, s, 0);
   double* W1 = wmat(C, s, 1);
-  cta_gemm<double, true, false>(N, N, N, R.Q, ld, Lf.Q, ld, W0, ld, S.gemm);
-  cta_gemm<double, false, true>(N, N, N, R.T, ld, Lf.T, ld, W1, ld, S.gemm);
+  gemm_64<true, false>(S, N, N, N, R.Q, ld, Lf.Q, ld, W0, ld);
+  gemm_64<false, true>(S, N, N, N, R.T, ld, Lf.T, ld, W1, ld);
   // 1/Db and Ds of both chains (vectors 5..7 of the workspace)
   double* ibR = wvec(C, s, 5);
   double* ibL = wvec(C, s, 6);
@@ -1268,7 +1292,7 @@ __device__ int green_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, double* G
     W1[(size_t)i * ld + j] *= ibL[i];
   }
   __syncthreads();
-  cta_gemm<double, false, false>(N, N, N, Lf.Q, ld, W1, ld, Gout, ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, Lf.Q, ld, W1, ld, Gout, ld);
   double part = 0.0;
   for (int i = threadIdx.x; i < N; i += kThreads) {
     const double dR = R.D[i], dL = Lf.D[i];
@@ -1354,17 +1378,8 @@ __global__ void __launch_bounds__(kThreads) fresh_green_kernel(ChainDev* chains,
   if (mode == 1 && c != out_chain) return;
   ChainDev& C = chains[c];
   Smem S = carve_smem(smem_raw, C.ld, C.MV);
-  // the working precision's tensor-core products need the CTA's tensor memory
-  const bool umma = DQMC_WITH_UMMA && std::is_same<Real, dd>::value && mode == 0 && C.planes[s] != nullptr;
-  S.um.err = &C.error;
-  S.dd_tile = C.dd_tile;
-  S.um.limit = C.wait_cycles > 0 ? C.wait_cycles : kUmmaWaitCycles;
-  S.um.stall = C.test_stall;
-  S.um.tmA = &C.tm_pl[s][0];
-  S.um.tmB = &C.tm_pl[s][1];
-  S.um.boff = (size_t)kUmmaDig * umma_pad(C.N, kUmmaM) * umma_pad(C.N, kUmmaK);
-  S.um.where = C.wait_where[s];
-  if (umma) umma_alloc(S.um);
+  const bool pairs = std::is_same<Real, dd>::value && mode == 0;
+  const bool umma = umma_begin(C, s, S, DQMC_WITH_UMMA && pairs, !pairs);
   double logdet;
   int sign;
   const int bad = (mode == 0) ? fill_left_chain_working<Real>(C, s, S, logdet, sign)
@@ -1419,16 +1434,7 @@ __global__ void __launch_bounds__(kThreads) green_tau_kernel(ChainDev* chains, i
   const int N = C.N, ld = C.ld, nw = C.nw, nst = C.L / nw;
   const int j0 = tau / nw;
   constexpr bool mixed = std::is_same<Real, dd>::value;
-  const bool umma = DQMC_WITH_UMMA && mixed && C.planes[s] != nullptr;
-  S.um.err = &C.error;
-  S.dd_tile = C.dd_tile;
-  S.um.limit = C.wait_cycles > 0 ? C.wait_cycles : kUmmaWaitCycles;
-  S.um.stall = C.test_stall;
-  S.um.tmA = &C.tm_pl[s][0];
-  S.um.tmB = &C.tm_pl[s][1];
-  S.um.boff = (size_t)kUmmaDig * umma_pad(C.N, kUmmaM) * umma_pad(C.N, kUmmaK);
-  S.um.where = C.wait_where[s];
-  if (umma) umma_alloc(S.um);
+  const bool umma = umma_begin(C, s, S, DQMC_WITH_UMMA && mixed, !mixed);
   int dq = 1;
   for (int j = 1; j <= j0; ++j) {
     const UDV src = (j == 1) ? ident_udv(C) : work_udv(C, s, dq);
@@ -1505,8 +1511,8 @@ __device__ void t_wrap<double>(const ChainDev& C, int s, double* G, double* Gt, 
   const int N = C.N, ld = C.ld;
   const double* X = up ? C.E[s] : C.Einv[s];
   const double* Y = up ? C.Einv[s] : C.E[s];
-  cta_gemm<double, false, false>(N, N, N, X, ld, G, ld, Gt, ld, S.gemm);
-  cta_gemm<double, false, false>(N, N, N, Gt, ld, Y, ld, G, ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, X, ld, G, ld, Gt, ld, up ? kCpEA : kCpEiA, -1);
+  gemm_64<false, false>(S, N, N, N, Gt, ld, Y, ld, G, ld, -1, up ? kCpEiB : kCpEB);
 }
 template <>
 __device__ void t_wrap<float>(const ChainDev& C, int s, float* G, float* Gt, bool up, Smem& S) {
@@ -1536,8 +1542,17 @@ template <>
 __device__ void flush_delayed<double>(const ChainDev& C, double* G, const double* A, const double* B, int nacc,
                                       Smem& S) {
   const int N = C.N, ld = C.ld;
+  // depth nacc <= 64: the FP64 pipe's N^2 nacc / 1.65 cycles against the split
+  // product's cost per output (N = 64, 16 vectors: 19 us on the pipe, 22 us split;
+  // N = 144: 97 and 60 us)
+  if (S.ps64 && N >= 96) {
+    gemm_umma<double>(true, false, true, N, N, nacc, A, ld, B, ld, G, ld, S.ps64, S.expA, S.expB, S.um, -1, -1);
+    return;
+  }
   const int r = gemm_pick_r(N);
-  if (r == 3) cta_gemm_r<double, true, false, 3, true>(N, N, nacc, A, ld, B, ld, G, ld, S.gemm);
+  if (r == 1) cta_gemm_r<double, true, false, 1, true>(N, N, nacc, A, ld, B, ld, G, ld, S.gemm);
+  else if (r == 2) cta_gemm_r<double, true, false, 2, true>(N, N, nacc, A, ld, B, ld, G, ld, S.gemm);
+  else if (r == 3) cta_gemm_r<double, true, false, 3, true>(N, N, nacc, A, ld, B, ld, G, ld, S.gemm);
   else if (r == 5) cta_gemm_r<double, true, false, 5, true>(N, N, nacc, A, ld, B, ld, G, ld, S.gemm);
   else cta_gemm_r<double, true, false, 4, true>(N, N, nacc, A, ld, B, ld, G, ld, S.gemm);
 }
@@ -1547,14 +1562,16 @@ __device__ void flush_delayed<float>(const ChainDev& C, float* G, const float* A
   const int N = C.N, ld = C.ld;
   float* sm = reinterpret_cast<float*>(S.gemm);
   const int r = gemm_pick_r(N);
-  if (r == 3) cta_gemm_r<float, true, false, 3, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
+  if (r == 1) cta_gemm_r<float, true, false, 1, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
+  else if (r == 2) cta_gemm_r<float, true, false, 2, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
+  else if (r == 3) cta_gemm_r<float, true, false, 3, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
   else if (r == 5) cta_gemm_r<float, true, false, 5, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
   else cta_gemm_r<float, true, false, 4, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
 }
 template <>
 __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const dd* B, int nacc, Smem& S) {
-  // a rank-k update (k <= 64): the float-pair SIMT tiles beat the split
-  // tensor-core product, whose digit split and recombination cost O(N^2 k_dig)
+  // a rank-k update (k <= 64): the float-pair SIMT tiles beat the split tensor-core
+  // product, whose digit split and recombination cost O(N^2) whatever k
   gemm_dd_tiles<true, false, true>(C.N, C.N, nacc, A, C.ld, B, C.ld, G, C.ld, reinterpret_cast<dd*>(S.gemm),
                                    S.dd_tile);
 }
@@ -2118,7 +2135,7 @@ __device__ inline void dd_to_d_inplace(int N, int ld, void* buf) {
 }
 
 __device__ int chain_step_mixed(const ChainDev& C, int s, int t1, int t2, bool left, UDV src, Smem& S,
-                      long long* det = nullptr) {
+                                             long long* det = nullptr) {
   long long t0 = clock64();
   const int N = C.N, ld = C.ld;
   dd* X = reinterpret_cast<dd*>(wmat(C, s, 0));
@@ -2388,18 +2405,9 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(ChainDev* chains, Sw
   ChainDev& C = chains[c];
   Smem S = carve_smem(smem_raw, C.ld, C.MV);
   S.flavor = s;
-  // the split tensor-core products (float-pair path with digit planes) need the
-  // CTA's tensor memory for the whole sweep
-  const bool umma = DQMC_WITH_UMMA && std::is_same<Real, dd>::value && C.planes[s] != nullptr;
-  S.um.err = &C.error;
-  S.dd_tile = C.dd_tile;
-  S.um.limit = C.wait_cycles > 0 ? C.wait_cycles : kUmmaWaitCycles;
-  S.um.stall = C.test_stall;
-  S.um.tmA = &C.tm_pl[s][0];
-  S.um.tmB = &C.tm_pl[s][1];
-  S.um.boff = (size_t)kUmmaDig * umma_pad(C.N, kUmmaM) * umma_pad(C.N, kUmmaK);
-  S.um.where = C.wait_where[s];
-  if (umma) umma_alloc(S.um);
+  // the split tensor-core products need the CTA's tensor memory for the whole sweep
+  const bool umma = umma_begin(C, s, S, DQMC_WITH_UMMA && std::is_same<Real, dd>::value,
+                               !std::is_same<Real, dd>::value);
   Real* G = (Real*)C.G[s];
   Real* Gt = (Real*)C.Gtmp[s];
   Real* A = P.ab_smem ? reinterpret_cast<Real*>(S.ab) : (Real*)C.dA[s];
@@ -2536,8 +2544,8 @@ __device__ int displaced_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, doubl
   double* W1 = wmat(C, s, 1);
   double* W7 = wmat(C, s, 7);
   double* W8 = wmat(C, s, 8);
-  cta_gemm<double, true, false>(N, N, N, R.Q, ld, Lf.Q, ld, W0, ld, S.gemm);
-  cta_gemm<double, false, true>(N, N, N, R.T, ld, Lf.T, ld, W1, ld, S.gemm);
+  gemm_64<true, false>(S, N, N, N, R.Q, ld, Lf.Q, ld, W0, ld);
+  gemm_64<false, true>(S, N, N, N, R.T, ld, Lf.T, ld, W1, ld);
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     const double dR = R.D[i], dL = Lf.D[j];
@@ -2567,10 +2575,10 @@ __device__ int displaced_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, doubl
     W8[(size_t)i * ld + j] = (dLi > 1.0 ? 1.0 : dLi) * m / (dRj > 1.0 ? dRj : 1.0);
   }
   __syncthreads();
-  cta_gemm<double, false, false>(N, N, N, Lf.Q, ld, W7, ld, W0, ld, S.gemm);
-  cta_gemm<double, false, false>(N, N, N, W0, ld, R.T, ld, Gt0, ld, S.gemm);
-  cta_gemm<double, true, false>(N, N, N, Lf.T, ld, W8, ld, W0, ld, S.gemm);
-  cta_gemm<double, false, true>(N, N, N, W0, ld, R.Q, ld, G0t, ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, Lf.Q, ld, W7, ld, W0, ld);
+  gemm_64<false, false>(S, N, N, N, W0, ld, R.T, ld, Gt0, ld);
+  gemm_64<true, false>(S, N, N, N, Lf.T, ld, W8, ld, W0, ld);
+  gemm_64<false, true>(S, N, N, N, W0, ld, R.Q, ld, G0t, ld);
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     G0t[(size_t)i * ld + j] = -G0t[(size_t)i * ld + j];

@@ -12,10 +12,12 @@ __global__ void __launch_bounds__(kThreads) green0_kernel(ChainDev* chains, int 
   if (c >= n_cfg) return;
   ChainDev& C = chains[c];
   Smem S = carve_smem(smem_raw, C.ld, C.MV);
+  const bool umma = umma_begin(C, s, S, false, true);
   double logdet;
   int sign;
   if (fill_left_chain(C, s, S, logdet, sign)) {
     if (threadIdx.x == 0) C.error = 1;
+    if (umma) umma_free(S.um);
     return;
   }
   const double* Gf = wmat(C, s, 6);
@@ -24,6 +26,7 @@ __global__ void __launch_bounds__(kThreads) green0_kernel(ChainDev* chains, int 
     const int x = e / C.N, y = e - x * C.N;
     out[e] = Gf[(size_t)x * C.ld + y];
   }
+  if (umma) umma_free(S.um);
   if (threadIdx.x == 0) { C.logdet[s] = logdet; C.fresh_sign[s] = sign; }
 }
 
@@ -46,6 +49,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
   if (c >= n_cfg) return;
   ChainDev& C = chains[c];
   Smem S = carve_smem(smem_raw, C.ld, C.MV);
+  const bool umma = umma_begin(C, s, S, false, true);
   const int N = C.N, ld = C.ld, L = C.L, nw = C.nw, nst = L / nw;
   const size_t mat = (size_t)N * ld;
   double* ew = ework_all + ((size_t)c * nfl + s) * 6 * mat;
@@ -59,6 +63,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
   int sign;
   if (fill_left_chain(C, s, S, logdet, sign)) {  // storage slots: left chains; W6 = G(0)
     if (threadIdx.x == 0) C.error = 1;
+    if (umma) umma_free(S.um);
     return;
   }
   const double* G0 = G0all + ((size_t)c * nfl + s) * N * N;
@@ -104,6 +109,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
       const UDV Lf = (j == nst) ? ident_udv(C) : slot_udv(C, s, j);
       if (displaced_from_udv(C, s, work_udv(C, s, dq), Lf, T2, G0t, S)) {
         if (threadIdx.x == 0) C.error = 1;
+        if (umma) umma_free(S.um);
         return;
       }
       copy_udv_to_slot(C, s, j, dq);
@@ -114,12 +120,12 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
         G0t[(size_t)x * ld + y] *= S.hv[y];
       }
       __syncthreads();
-      cta_gemm<double, false, false>(N, N, N, G0t, ld, C.Einv[s], ld, T1, ld, S.gemm);
+      gemm_64<false, false>(S, N, N, N, G0t, ld, C.Einv[s], ld, T1, ld, -1, kCpEiB);
       double* t_ = G0t; G0t = T1; T1 = t_;
     }
     // Z = G(tau-1,0) Gamma^T G(0,tau)
-    cta_gemm<double, false, false>(N, N, N, Gt0, ld, Gam, ld, T1, ld, S.gemm);
-    cta_gemm<double, false, false>(N, N, N, T1, ld, G0t, ld, Z, ld, S.gemm);
+    gemm_64<false, false>(S, N, N, N, Gt0, ld, Gam, ld, T1, ld);
+    gemm_64<false, false>(S, N, N, N, T1, ld, G0t, ld, Z, ld);
     for (int e = threadIdx.x; e < N * N; e += kThreads) {
       const int x = e / N, y = e - x * N;
       SE[(size_t)x * ld + y] += S.ev[x] * Z[(size_t)x * ld + y];
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
         Gt0[(size_t)x * ld + y] *= S.ev[x];
       }
       __syncthreads();
-      cta_gemm<double, false, false>(N, N, N, C.E[s], ld, Gt0, ld, T1, ld, S.gemm);
+      gemm_64<false, false>(S, N, N, N, C.E[s], ld, Gt0, ld, T1, ld, kCpEA, -1);
       double* t_ = Gt0; Gt0 = T1; T1 = t_;
     }
   }
@@ -158,8 +164,8 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
     W3[(size_t)x * ld + y] = Vs[e];
   }
   __syncthreads();
-  cta_gemm<double, true, false>(N, N, N, SE, ld, W3, ld, W1, ld, S.gemm);
-  cta_gemm<double, true, false>(N, N, N, W3, ld, W1, ld, W2, ld, S.gemm);
+  gemm_64<true, false>(S, N, N, N, SE, ld, W3, ld, W1, ld);
+  gemm_64<true, false>(S, N, N, N, W3, ld, W1, ld, W2, ld);
   const double dt = C.dtau;
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int a = e / N, b = e - a * N;
@@ -169,8 +175,8 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
     W2[(size_t)a * ld + b] *= -dt * exp(-0.5 * dt * (la + lb)) * shc;
   }
   __syncthreads();
-  cta_gemm<double, false, false>(N, N, N, W3, ld, W2, ld, W1, ld, S.gemm);
-  cta_gemm<double, false, true>(N, N, N, W1, ld, W3, ld, W0, ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, W3, ld, W2, ld, W1, ld);
+  gemm_64<false, true>(S, N, N, N, W1, ld, W3, ld, W0, ld);
   double* out = gK + ((size_t)c * nfl + s) * N * N;
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int x = e / N, y = e - x * N;
@@ -186,6 +192,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
     ep[1] = part;
     ep[2] = (s == 0) ? pot : 0.0;
   }
+  if (umma) umma_free(S.um);
 }
 
 cudaError_t launch_energy_grad(ChainDev* chains, int n_cfg, int nfl, const double* eigvec, const double* eigval,

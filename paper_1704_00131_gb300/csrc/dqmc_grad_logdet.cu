@@ -18,11 +18,13 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
   if (c >= n_cfg) return;
   ChainDev& C = chains[c];
   Smem S = carve_smem(smem_raw, C.ld, C.MV);
+  const bool umma = umma_begin(C, s, S, false, true);
   const int N = C.N, ld = C.ld, L = C.L, nw = C.nw, nst = L / nw;
   double logdet;
   int sign;
   if (fill_left_chain(C, s, S, logdet, sign)) {
     if (threadIdx.x == 0) C.error = 1;
+    if (umma) umma_free(S.um);
     return;
   }
   if (threadIdx.x == 0) { C.logdet[s] = logdet; C.fresh_sign[s] = sign; }
@@ -52,8 +54,8 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
       gu += (1.0 - Gc[(size_t)i * ld + i]) * C.vsign[s * C.MV + k] *
             coupling_dU(C.ft, C.dtau, C.U, C.cscale, C.fields[(size_t)(tau - 1) * C.MV + k]);
     }
-    cta_gemm<double, false, false>(N, N, N, C.E[s], ld, Gc, ld, Wt, ld, S.gemm);
-    cta_gemm<double, false, false>(N, N, N, Wt, ld, C.Einv[s], ld, Gc, ld, S.gemm);
+    gemm_64<false, false>(S, N, N, N, C.E[s], ld, Gc, ld, Wt, ld, kCpEA, -1);
+    gemm_64<false, false>(S, N, N, N, Wt, ld, C.Einv[s], ld, Gc, ld, -1, kCpEiB);
     if (tau % nw == 0 && tau < L) {
       const int j = tau / nw;
       const UDV src = (j == 1) ? ident_udv(C) : slot_udv(C, s, j - 1);
@@ -63,6 +65,7 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
       int sgt;
       if (green_from_udv(C, s, work_udv(C, s, dq), Lf, wmat(C, s, 6), ldt, sgt, S)) {
         if (threadIdx.x == 0) C.error = 1;
+        if (umma) umma_free(S.um);
         return;
       }
       cta_copy(N, ld, (const double*)wmat(C, s, 6), Gc);
@@ -78,15 +81,15 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
   double* W3 = wmat(C, s, 3);
   const double* Vs = V + (size_t)s * N * N;
   const double* ws = w + (size_t)s * N;
-  cta_gemm<double, false, false>(N, N, N, Sacc, ld, C.Einv[s], ld, W0, ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, Sacc, ld, C.Einv[s], ld, W0, ld, -1, kCpEiB);
   // V is dense [N][N] (ld = N); use a copy with the chain's ld
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int x = e / N, y = e - x * N;
     W3[(size_t)x * ld + y] = Vs[e];
   }
   __syncthreads();
-  cta_gemm<double, true, false>(N, N, N, W0, ld, W3, ld, W1, ld, S.gemm);
-  cta_gemm<double, true, false>(N, N, N, W3, ld, W1, ld, W2, ld, S.gemm);
+  gemm_64<true, false>(S, N, N, N, W0, ld, W3, ld, W1, ld);
+  gemm_64<true, false>(S, N, N, N, W3, ld, W1, ld, W2, ld);
   const double dt = C.dtau;
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int a = e / N, b = e - a * N;
@@ -96,14 +99,15 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
     W2[(size_t)a * ld + b] *= -dt * exp(-0.5 * dt * (la + lb)) * shc;
   }
   __syncthreads();
-  cta_gemm<double, false, false>(N, N, N, W3, ld, W2, ld, W1, ld, S.gemm);
-  cta_gemm<double, false, true>(N, N, N, W1, ld, W3, ld, W0, ld, S.gemm);
+  gemm_64<false, false>(S, N, N, N, W3, ld, W2, ld, W1, ld);
+  gemm_64<false, true>(S, N, N, N, W1, ld, W3, ld, W0, ld);
   double* out = gK + ((size_t)c * nfl + s) * N * N;
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int x = e / N, y = e - x * N;
     const double gxy = W0[(size_t)x * ld + y];
     out[e] = (x == y) ? gxy : gxy + W0[(size_t)y * ld + x];
   }
+  if (umma) umma_free(S.um);
 }
 
 cudaError_t launch_logdet_grad(ChainDev* chains, int n_cfg, int nfl, const double* eigvec, const double* eigval,

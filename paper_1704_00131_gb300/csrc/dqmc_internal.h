@@ -9,11 +9,41 @@ namespace dqmc {
 
 constexpr int kThreads = 256;      // threads per CTA of every kernel
 constexpr int kMaxFlavors = 2;
-// Digit planes of the split tensor-core products: blocks of kPlaneDigits digits
-// x rows x kPlaneK bf16 (rows: kPlaneRowsA for a left operand, kPlaneRowsB for
-// a right one), one block per (tile, 16-wide K chunk), copied to shared memory
-// by one tiled tensor copy each.
-constexpr int kPlaneDigits = 7, kPlaneRowsA = 64, kPlaneRowsB = 48, kPlaneK = 16;
+// Digit planes of the split tensor-core products: blocks of digits x rows x kPlaneK
+// bf16, one block per (tile, 16-wide K chunk), copied to shared memory by one
+// tiled tensor copy each.  Float pairs have kPlaneDigits digits, FP64 operands
+// kPlaneDigits64; a right operand's tiles have kPlaneRowsB rows, a left operand's
+// umma_rows(N).
+constexpr int kPlaneDigits = 7, kPlaneDigits64 = 8, kPlaneMaxRows = 128, kPlaneRowsB = 32, kPlaneK = 16;
+constexpr int kPlaneRowElems = 256;  // bf16 per row of the copies' 2D view of a plane buffer
+// row tiles of an N-row left operand: equal, at most kPlaneMaxRows, rounded to 16
+__host__ __device__ inline int umma_row_tiles(int n) { return (n + kPlaneMaxRows - 1) / kPlaneMaxRows; }
+__host__ __device__ inline int umma_rows(int n) {
+  const int t = umma_row_tiles(n);
+  return ((n + t - 1) / t + 15) / 16 * 16;
+}
+// bf16 elements of the left and right operands' planes of N x K matrices
+__host__ __device__ inline size_t plane_elems(int digits, int n, int k, bool right) {
+  const size_t rows = right ? (size_t)(n + kPlaneRowsB - 1) / kPlaneRowsB * kPlaneRowsB
+                            : (size_t)umma_rows(n) * umma_row_tiles(n);
+  return (size_t)digits * rows * ((k + kPlaneK - 1) / kPlaneK * kPlaneK);
+}
+
+enum { kCpEA = 0, kCpEtA = 1, kCpEiA = 2, kCpEiB = 3, kCpEB = 4, kCpSets = 5 };
+
+// The split products' buffers of one (chain, flavor) and operand type: scratch
+// planes of the left operand, those of the right one `boff` elements behind them;
+// digit planes and row exponents of the constant operands, prepared once per
+// model: kCpEA = E as left factor, kCpEtA = E^T left, kCpEiA = E^-1 left, kCpEiB =
+// E^-1 right, kCpEB = E right; and the tensor maps (2D views with a box of one block)
+// of the scratch as left [0] and right [1] operand and of the constant planes.
+struct alignas(64) PlaneSet {
+  CUtensorMap tm_pl[2];
+  CUtensorMap tm_cp[kCpSets];
+  void* scratch;
+  size_t boff;
+  const int* cex[kCpSets];
+};
 
 // Device-resident description and state of one Markov chain.  One CTA per
 // (chain, flavor) works on it; the CTAs of a chain form one thread-block
@@ -41,17 +71,9 @@ struct ChainDev {
   double* slots[kMaxFlavors];     // FP64 [nst+1] x {Q [N][ld], T [N][ld], D [ld]}
   int* slot_detq[kMaxFlavors];    // [nst+1]
   double* work[kMaxFlavors];      // FP64 stabilisation workspace, kWorkMats matrices + vectors
-  void* planes[kMaxFlavors];      // BF16 digit planes of the split tensor-core products (mixed path)
-  // digit planes and row exponents of the constant split operands, prepared once
-  // per model: kCpEA = E as left factor, kCpEtA = E^T left, kCpEiA = E^-1 left,
-  // kCpEiB = E^-1 right, kCpEB = E right (null without tensor-core products)
-  const void* cpl[kMaxFlavors][5];
-  const int* cex[kMaxFlavors][5];
-  // tensor maps (4D views [blocks][digits][rows][k] with a box of one block) of
-  // the scratch planes as left [0] and right [1] operand, and of the constant
-  // operands' planes
-  CUtensorMap tm_pl[kMaxFlavors][2];
-  CUtensorMap tm_cp[kMaxFlavors][5];
+  void* planes[kMaxFlavors];      // scratch of the split products' digit planes (shared by both operand types)
+  const PlaneSet* ps[kMaxFlavors];    // split products of float pairs (null: register tiles)
+  const PlaneSet* ps64[kMaxFlavors];  // split products of FP64 operands (null: register tiles)
   int* iwork[kMaxFlavors];        // [2*ld]
   uint32_t chain_id;
   int sign;                       // sign of the current weight (written by rank 0)
@@ -88,7 +110,6 @@ struct ChainDev {
 };
 
 constexpr int kWorkMats = 10;     // N x ld FP64 matrices per flavor in `work`
-enum { kCpEA = 0, kCpEtA = 1, kCpEiA = 2, kCpEiB = 3, kCpEB = 4 };
 
 __host__ __device__ inline size_t slot_stride(int N, int ld) { return (size_t)2 * N * ld + ld; }
 __host__ __device__ inline size_t work_elems(int N, int ld) { return (size_t)kWorkMats * N * ld + 8 * (size_t)ld; }
@@ -110,19 +131,21 @@ cudaError_t launch_fresh_green(ChainDev* chains, int n_chains, int nfl, int prec
                                double* out, int out_chain, cudaStream_t st);
 cudaError_t launch_sweep(ChainDev* chains, const SweepParams& p, int nfl, int precision, size_t smem,
                          cudaStream_t st);
-size_t sweep_smem_bytes(int maxN, int maxld, int maxMV, int delay_k, int precision);
-// bytes of the shared-memory region behind the base (delayed vectors and/or the
-// staging buffers of the split tensor-core products)
-size_t smem_tail(size_t ab_bytes, int umma);
-// bytes of the BF16 digit planes of one CTA's split products up to N x N x kmax
-size_t plane_bytes(int N, int kmax);
-// digit planes of a constant N x N float-pair operand: as the left factor
-// (right = 0; tr = 1 for its transpose) or as the right factor (right = 1);
-// bytes of the planes and entries of the exponent vector
-size_t const_plane_bytes(int N, int right);
-int const_plane_exps(int N, int right);
-cudaError_t launch_const_planes(const void* X, int N, int ld, int right, int tr, void* planes, int* ex,
-                                cudaStream_t st);
+// dynamic shared memory with `ab_bytes` of delayed vectors; digits > 0: also room to
+// stage the split products of matrices of up to maxN sites
+size_t smem_total(int maxld, int maxMV, size_t ab_bytes, int maxN, int digits);
+// One constant operand's planes: an N x N FP64 or float-pair matrix as the left
+// (right = 0; tr = 1 for its transpose) or right factor.
+struct ConstPlaneJob {
+  const void* X;
+  void* planes;
+  int* ex;
+  int right, tr, fp64;
+};
+struct ConstPlaneJobs {
+  ConstPlaneJob job[2 * kMaxFlavors * kCpSets];
+};
+cudaError_t launch_const_planes(const ConstPlaneJobs& jobs, int n_jobs, int N, int ld, cudaStream_t st);
 cudaError_t launch_copy_green(ChainDev* chains, int chain, int flavor, int precision, double* out,
                               cudaStream_t st);
 cudaError_t launch_green_tau(ChainDev* chains, int chain, int nfl, int precision, int tau, double* out,

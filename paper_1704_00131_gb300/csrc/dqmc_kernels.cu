@@ -111,39 +111,54 @@ __global__ void corr_kernel(ChainDev* chains, int n_chains, const int* csr_all, 
 // --------------------------------------------------------------------------
 // Launchers.
 // --------------------------------------------------------------------------
-size_t sweep_smem_bytes(int maxN, int maxld, int maxMV, int delay_k, int precision) {
-  (void)maxN; (void)delay_k; (void)precision;
-  return smem_bytes_for(maxld, maxMV);
+// The split products want three stages; two where three would leave room for one
+// CTA per SM instead of two (a second CTA hides more than a third stage).
+size_t smem_total(int maxld, int maxMV, size_t ab_bytes, int maxN, int digits) {
+  const size_t plain = smem_bytes_for(maxld, maxMV) + ab_bytes;
+  if (!digits) return plain;
+  size_t stage = 0;  // the tile height is not monotonic in N
+  for (int n = 1; n <= maxN; ++n) {
+    const size_t b = (size_t)digits * kPlaneK * 2 * (umma_rows(n) + kPlaneRowsB);
+    stage = b > stage ? b : stage;
+  }
+  const size_t off = smem_stage_offset(maxld, maxMV), half = 113 * 1024;
+  const size_t two = off + 2 * stage > plain ? off + 2 * stage : plain;
+  const size_t three = off + 3 * stage > plain ? off + 3 * stage : plain;
+  // every CTA of these kernels holds half of the SM's tensor memory (256 of 512
+  // columns): at least 78 KB of shared memory per CTA keeps three of them from
+  // sharing an SM, so an allocation never waits
+  const size_t need = (three <= half || two > half) ? three : two;
+  return need > 78 * 1024 ? need : 78 * 1024;
 }
 
-size_t smem_tail(size_t ab_bytes, int umma) { return smem_tail_bytes(ab_bytes, umma != 0); }
-
-size_t plane_bytes(int N, int kmax) { return umma_plane_elems(N, kmax) * sizeof(__nv_bfloat16); }
-
-// Digit planes and row exponents of a constant operand of the split products
-// (one CTA): the left factor's rows (tiles of kUmmaM) or the right factor's
-// columns (tiles of kUmmaNT), laid out as gemm_umma stages them.
-__global__ void __launch_bounds__(kThreads) const_planes_kernel(const dd* X, int N, int ld, int right, int tr,
-                                                                __nv_bfloat16* P, int* ex) {
-  const int rows = right ? kUmmaNT : kUmmaM;
-  const int Rp = umma_pad(N, rows), Kp = umma_pad(N, kUmmaK);
+// Digit planes and row exponents of a model's constant operands of the split
+// products, one CTA each: a left factor's rows (tiles of umma_rows(N)) or a right
+// factor's columns (tiles of kUmmaNT), laid out as gemm_umma stages them.
+template <typename T>
+__device__ void const_planes(const ConstPlaneJob& J, int N, int ld, int* ex) {
+  const int rows = J.right ? kUmmaNT : umma_rows(N);
+  const int Rp = J.right ? umma_pad(N, kUmmaNT) : rows * umma_row_tiles(N), Kp = umma_pad(N, kUmmaK);
+  const T* X = (const T*)J.X;
   // logical row r of the operand: row r of X, or column r (transpose / right factor)
-  const bool colwise = right ? !tr : tr;
+  const bool colwise = J.right ? !J.tr : J.tr;
   if (colwise) umma_row_exponents<true>(N, N, X, ld, Rp, ex);
   else umma_row_exponents<false>(N, N, X, ld, Rp, ex);
-  __syncthreads();
-  if (colwise) umma_planes<true>(N, N, X, ld, Rp, Kp, rows, ex, P);
-  else umma_planes<false>(N, N, X, ld, Rp, Kp, rows, ex, P);
+  for (int r = threadIdx.x; r < Rp; r += kThreads) J.ex[r] = ex[r];
+  if (colwise) umma_planes<true>(N, N, X, ld, Rp, Kp, rows, ex, (__nv_bfloat16*)J.planes);
+  else umma_planes<false>(N, N, X, ld, Rp, Kp, rows, ex, (__nv_bfloat16*)J.planes);
+}
+__global__ void __launch_bounds__(kThreads) const_planes_kernel(ConstPlaneJobs jobs, int N, int ld) {
+  extern __shared__ int const_planes_ex[];
+  const ConstPlaneJob& J = jobs.job[blockIdx.x];
+  if (J.fp64) const_planes<double>(J, N, ld, const_planes_ex);
+  else const_planes<dd>(J, N, ld, const_planes_ex);
 }
 
-size_t const_plane_bytes(int N, int right) {
-  return (size_t)kUmmaDig * umma_pad(N, right ? kUmmaNT : kUmmaM) * umma_pad(N, kUmmaK) * sizeof(__nv_bfloat16);
-}
-int const_plane_exps(int N, int right) { return umma_pad(N, right ? kUmmaNT : kUmmaM); }
-
-cudaError_t launch_const_planes(const void* X, int N, int ld, int right, int tr, void* planes, int* ex,
-                                cudaStream_t st) {
-  const_planes_kernel<<<1, kThreads, 0, st>>>((const dd*)X, N, ld, right, tr, (__nv_bfloat16*)planes, ex);
+cudaError_t launch_const_planes(const ConstPlaneJobs& jobs, int n_jobs, int N, int ld, cudaStream_t st) {
+  const size_t smem = sizeof(int) * exp_len(ld);
+  const cudaError_t e = set_smem((const void*)const_planes_kernel, smem);
+  if (e != cudaSuccess) return e;
+  const_planes_kernel<<<n_jobs, kThreads, smem, st>>>(jobs, N, ld);
   return cudaGetLastError();
 }
 

@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
   if (c >= n_chains) return;
   ChainDev& C = chains[c];
   Smem S = carve_smem(smem_raw, C.ld, C.MV);
+  const bool umma = umma_begin(C, s, S, false, true);
   const int N = C.N, ld = C.ld, nw = C.nw, nst = C.L / nw;
   const int ntc = n_tau < C.L ? n_tau : C.L;
   const size_t mat = (size_t)N * ld;
@@ -57,6 +58,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
   double* Gf = wmat(C, s, 6);
   if (green_from_udv(C, s, ident_udv(C), slot_udv(C, s, 0), Gf, logdet, sg, S)) {
     if (threadIdx.x == 0) C.error = 1;
+    if (umma) umma_free(S.um);
     return;
   }
   if (threadIdx.x == 0) sign_out[(size_t)c * nfl + s] = sg;
@@ -85,12 +87,12 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
         Gtt[(size_t)x * ld + y] *= S.ev[x] * S.hv[y];
       }
       __syncthreads();
-      cta_gemm<double, false, false>(N, N, N, C.E[s], ld, Gt0, ld, T1, ld, S.gemm);
+      gemm_64<false, false>(S, N, N, N, C.E[s], ld, Gt0, ld, T1, ld, kCpEA, -1);
       { double* t_ = Gt0; Gt0 = T1; T1 = t_; }
-      cta_gemm<double, false, false>(N, N, N, G0t, ld, C.Einv[s], ld, T1, ld, S.gemm);
+      gemm_64<false, false>(S, N, N, N, G0t, ld, C.Einv[s], ld, T1, ld, -1, kCpEiB);
       { double* t_ = G0t; G0t = T1; T1 = t_; }
-      cta_gemm<double, false, false>(N, N, N, C.E[s], ld, Gtt, ld, T1, ld, S.gemm);
-      cta_gemm<double, false, false>(N, N, N, T1, ld, C.Einv[s], ld, Gtt, ld, S.gemm);
+      gemm_64<false, false>(S, N, N, N, C.E[s], ld, Gtt, ld, T1, ld, kCpEA, -1);
+      gemm_64<false, false>(S, N, N, N, T1, ld, C.Einv[s], ld, Gtt, ld, -1, kCpEiB);
       if (tau % nw == 0) {
         const int j = tau / nw;
         dq = chain_step(C, s, (j - 1) * nw, j * nw, false, (j == 1) ? ident_udv(C) : work_udv(C, s, dq), S);
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
         if (!bad) bad = green_from_udv(C, s, R, Lf, Gf, logdet, sg, S);
         if (bad) {
           if (threadIdx.x == 0) C.error = 1;
+          if (umma) umma_free(S.um);
           return;
         }
         double mx = 0.0, sm = 0.0;
@@ -167,6 +170,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
     pr[1] = ev_max;
     pr[2] = (double)events;
   }
+  if (umma) umma_free(S.um);
 }
 
 // Time-displaced correlation functions per class from the flavors' shares (two

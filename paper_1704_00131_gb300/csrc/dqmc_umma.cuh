@@ -1,94 +1,102 @@
-// Exact-split BF16 products of float-pair matrices on the fifth-generation
+// Exact-split BF16 products of FP64 or float-pair matrices on the fifth-generation
 // tensor cores (tcgen05.mma, accumulators in tensor memory, operands staged in
 // shared memory by tiled tensor copies).  Included by dqmc_device.cuh inside its
 // namespace, after the float-pair arithmetic.
 //
 // Scheme (Ozaki, Ogita, Oishi & Rump, Numer. Algorithms 59, 2012, on BF16
 // digits): every row i of op(A) and column j of op(B) is scaled by a power of
-// two so that its entries satisfy |x| < 2^(e-1), then cut into kUmmaDig
-// balanced 8-bit digits,
-//     x = 2^(e-8) sum_t q_t 2^(-8t),   q_t integer, |q_t| <= 128.
-// The digit planes hold q_t 2^(-8t) as BF16 (exact: eight significant bits and
-// a power-of-two scale), so the product of digits t and u carries the weight of
-// its diagonal d = t + u:
+// two, rounded to a fixed-point integer and cut into ND balanced 8-bit digits,
+//     x = 2^(e-8) sum_t q_t 2^(-8t),   q_t integer, |q_t| <= 128,
+// ND = 7 for float pairs (|x| < 2^(e-1): 56 bits under the row's largest entry)
+// and ND = 8 for FP64 (|x| < 2^(e-2): 63 bits).  The digit planes hold
+// q_t 2^(-8t) as BF16 (exact), so the product of digits t and u carries the
+// weight of its diagonal d = t + u:
 //     (op(A) op(B))_ij = 2^(eA_i + eB_j - 16) sum_{t,u} sum_k qA_t qB_u 2^(-8(t+u)).
-// Diagonals 0..3 are accumulated in FP32 tensor-memory accumulators of their
-// own: their terms are multiples of 2^(-8d) below 2^(14-8d), and (d+1) K 2^14 <=
-// 2^24 keeps every partial sum exact for K <= 256 (the segment length
-// kUmmaKSeg).  Diagonals 4..6 share one accumulator whose FP32 rounding is
-// 2^-24 of a term already 2^-32 below the result.  Pairs with t + u > 6
-// (weight < 2^-56) are dropped.  The five accumulators are summed in float
-// pairs, scaled, and stored (or added) into C.
+// Each diagonal d < ND has an FP32 tensor-memory accumulator of its own: its terms
+// are multiples of 2^(-8d) below 2^(14-8d), so every partial sum is exact while
+// (d+1) K <= 1024, for d <= 3 up to the segment length K = 256; later diagonals
+// round at 2^-24 of terms already 2^-32 below the result.  Pairs with t + u >= ND
+// are dropped (below 2^-56 and 2^-64 of the scale).  The diagonals are summed as
+// float pairs, or for FP64 as one integer that is rounded once.
 //
-// Tiles: UM = 64 rows (one MMA M) x NT = 48 columns (MMA N), K in chunks of 16
-// (one MMA K).  A chunk stages all digits of an A tile and a B tile: the digit
-// planes are laid out in global memory (per-chain scratch, L2-resident; the
-// constant propagators' planes are prepared once per model) in the order
-// (tile, k chunk, digit) with each 16-wide block in the canonical K-major layout
-// without swizzle.  The host describes each plane buffer by a tensor map, a 4D
-// view [blocks][7 digits][rows][16 k] whose box is one whole block, so one chunk
-// is two tiled tensor copies (cp.async.bulk.tensor) of 14 KB and 10.5 KB that
-// reproduce the blocks byte for byte in shared memory.  The chunks of
-// all tiles form one sequence streamed through three stages: while the 28 MMAs
-// of chunk g run, the copies of chunks g+1 and g+2 are in flight, across tile
-// boundaries too.  One thread issues the copies and the MMAs; completion is
-// tracked with mbarriers whose waits give up after ~1 s (the chain's error
-// word records it).
+// Largest error over |A||B| against 80-bit sums (normal A, log-normal B): FP64
+// operands 1.0e-16 at N = 64 and 5.6e-16 at N = 144, where a chain of FP64 FMAs has
+// 1.0e-15 and 1.4e-15.
+//
+// Cost per product on GB300 (one CTA of two per SM, cycles): FP64 N = 64 44k, 72 69k,
+// 144 298k, where the FP64 pipe's tiles need 159k, 280k and 1.8M per CTA and SM
+// (half of it with one CTA); float pairs N = 144 274k (the float-pair register tiles
+// 560k).  Cutting the operands and recombining the diagonals take about half of it,
+// the chunk pipeline the rest.
+//
+// Tiles: 128 x 32 outputs (MMA M = 128).  The B digits of a tile are staged as one
+// 32 ND-row operand, so digit t of A meets the digits 0..ND-1-t of B in one MMA of
+// N = 32 (ND - t) whose accumulators t..ND-1 are adjacent columns: ND MMAs per
+// 16-deep chunk instead of ND (ND+1) / 2, each reading A from shared memory once.
+// A matrix of N rows is cut into ceil(N / 128) equal row tiles, rounded to 16 rows
+// (rows past a tile read whatever follows it in the staging area: their outputs
+// are not used).  The digit planes are laid out in global memory (per-chain
+// scratch, L2-resident; the constant propagators' planes are prepared once per
+// model) in the order (tile, k chunk, digit) with each 16-wide block in the
+// canonical K-major layout without swizzle; a tensor map describes each plane
+// buffer as 512-byte rows with a box of one whole (tile, k chunk), so one chunk is
+// two tiled tensor copies (cp.async.bulk.tensor).  The chunks of all
+// tiles form one sequence streamed through two or three stages: warp 1 issues the
+// copies, warp 0 the MMAs, each through one elected thread (one thread doing both
+// spent 1300 cycles a chunk on issue and bookkeeping, the MMAs take 450 - 580).
+// Completion is tracked with mbarriers whose waits give up after ~1 s (the chain's
+// error word records it).
 #pragma once
 
-constexpr int kUmmaDig = 7;                 // digits per operand
-constexpr int kUmmaSlots = 5;               // accumulators: diagonals 0, 1, 2, 3 and 4..6
-constexpr int kUmmaM = 64;                  // tile rows (MMA M)
-constexpr int kUmmaNT = 48;                 // tile columns (MMA N)
-constexpr int kUmmaK = 16;                  // MMA K and staged chunk
-static_assert(kUmmaDig == kPlaneDigits && kUmmaM == kPlaneRowsA && kUmmaNT == kPlaneRowsB && kUmmaK == kPlaneK,
-              "the host's tensor maps describe these plane blocks");
+constexpr int kUmmaNT = kPlaneRowsB;        // tile columns
+constexpr int kUmmaK = kPlaneK;             // MMA K and staged chunk
+constexpr int kUmmaM = kPlaneMaxRows;       // MMA M
 constexpr int kUmmaKSeg = 256;              // k per exactly accumulated segment
 constexpr int kUmmaCols = 256;              // tensor-memory columns allocated per CTA
-constexpr int kUmmaBlockA = kUmmaM * kUmmaK * 2;    // bytes of one digit block of A
-constexpr int kUmmaBlockB = kUmmaNT * kUmmaK * 2;   // ... of B
-constexpr int kUmmaStageBytes = kUmmaDig * (kUmmaBlockA + kUmmaBlockB);
-constexpr int kUmmaStages = 3;                             // copy pipeline depth
+constexpr int kUmmaStages = 3;              // copy pipeline depth (at most)
+constexpr int kUmmaNonFinite = 1 << 20;     // exponent of a row that holds an Inf or NaN
 constexpr long long kUmmaWaitCycles = 2000000000LL;        // default wait limit, ~1 s
+static_assert(kPlaneDigits64 * kUmmaNT <= kUmmaCols && kPlaneDigits64 * kUmmaNT <= 256,
+              "one MMA spans every diagonal's accumulator");
+
+// digits of an operand type
+template <typename T>
+struct UmmaDigits { static constexpr int n = kPlaneDigits64; };
+template <>
+struct UmmaDigits<dd> { static constexpr int n = kPlaneDigits; };
 
 __host__ __device__ inline int umma_pad(int n, int q) { return (n + q - 1) / q * q; }
-// bf16 elements of the digit planes of one CTA for products up to n x n x kmax
-__host__ __device__ inline size_t umma_plane_elems(int n, int kmax) {
-  const size_t kp = (size_t)umma_pad(kmax, kUmmaK);
-  return (size_t)kUmmaDig * ((size_t)umma_pad(n, kUmmaM) + (size_t)umma_pad(n, kUmmaNT)) * kp;
-}
 
 // State of the tensor-core products of one CTA.  Nothing in it is indexed at
 // run time (that would push the kernel's whole shared-memory descriptor into
-// local memory): the stages are found by umma_stage, and thread 0's
-// bookkeeping lives in the 128-byte shared barrier area.
+// local memory): thread 0's bookkeeping lives in the 128-byte shared barrier area.
 struct Umma {
-  const CUtensorMap* tmA; // tensor maps of the scratch planes as left / right operand
-  const CUtensorMap* tmB;
-  size_t boff;            // elements from the scratch planes to the right operand's planes
-  unsigned char* stage0;  // first staging buffer (kUmmaStageBytes, the GEMM region)
-  unsigned char* stage1;  // second; the third follows it
+  unsigned char* stage;   // staging area (nothing else is live there during a product)
+  uint32_t stage_bytes;   // its bytes
   uint64_t* bar;          // shared, 128 bytes: [0, 48) the 2 kUmmaStages mbarriers (copies landed
-                          // per stage, then MMAs done per stage); [48, 96) thread 0's counters
-                          // of copies and MMA commits issued and waited per stage; [96, 100)
-                          // the TMEM slot; [100, 104) thread 0's count of products; [104, 112)
-                          // a barrier that nothing arrives on (the test_stall hook)
+                          // per stage, then MMAs done per stage); [48, 56) accumulators complete;
+                          // [56, 64) a barrier that nothing arrives on (the test_stall hook);
+                          // [64, 68) the parities of the seven barriers' next phases; [68, 76)
+                          // chunks copied and multiplied by a product that gave up; [96, 100) the
+                          // TMEM slot; [100, 104) the count of products
   uint32_t* tmem_slot;    // tcgen05.alloc writes the accumulator base here
   int* err;               // chain error word (nonzero: a wait gave up)
   long long limit;        // SM cycles after which a wait gives up
   int stall;              // test hook: the first wait of a product waits on the barrier at
-                          // [104, 112), which gives up after `limit`
+                          // [56, 64), which gives up after `limit`
   int* where;             // [6] or null: the first wait that gave up (kind, chunk, chunks,
                           // product ordinal, barrier word)
 };
 
-__device__ __forceinline__ unsigned char* umma_stage(const Umma& U, int st) {
-  return st == 0 ? U.stage0 : U.stage1 + (size_t)(st - 1) * kUmmaStageBytes;
-}
-// thread 0's counters (shared): copies issued / waited, commits issued / waited, per stage
-__device__ __forceinline__ uint32_t* umma_book(const Umma& U) { return reinterpret_cast<uint32_t*>(U.bar + 2 * kUmmaStages); }
+__device__ __forceinline__ uint64_t* umma_acc(const Umma& U) { return U.bar + 2 * kUmmaStages; }
+__device__ __forceinline__ uint64_t* umma_never(const Umma& U) { return U.bar + 2 * kUmmaStages + 1; }
+__device__ __forceinline__ uint32_t* umma_book(const Umma& U) { return reinterpret_cast<uint32_t*>(U.bar + 8); }
 __device__ __forceinline__ uint32_t* umma_calls(const Umma& U) { return U.tmem_slot + 1; }
-__device__ __forceinline__ uint64_t* umma_never(const Umma& U) { return U.bar + 2 * kUmmaStages + 7; }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0u;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -129,14 +137,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     if (clock64() - t0 > limit) return false;
   }
 }
-// One block of digit planes (all seven digits of a tile x 16-wide K chunk)
-// into shared memory: a tiled tensor copy of box (16, rows, 7, 1) at block
-// coordinate `block` of the 4D view [blocks][7][rows][16] the map describes.
-__device__ __forceinline__ void tma_load_block(void* dst, const CUtensorMap* tm, int block, uint64_t* bar) {
+// One block of digit planes (all digits of a tile x 16-wide K chunk, contiguous in
+// the plane buffer) into shared memory: a tiled tensor copy of the block's rows of
+// the buffer's 2D view [rows][kPlaneRowElems] the map describes.  The copy engine
+// works row by row: 512-byte rows move a chunk in a third of the cycles that the
+// 32-byte rows of a [digits][rows][16] view took (1400 a chunk of 25 KB).
+__device__ __forceinline__ void tma_load_block(void* dst, const CUtensorMap* tm, int row, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-      "[%6];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(0), "r"(0), "r"(0), "r"(block), "r"(smem_u32(bar))
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(0), "r"(row), "r"(smem_u32(bar))
       : "memory");
 }
 __device__ __forceinline__ void umma_bf16(uint32_t dtm, uint64_t ad, uint64_t bd, uint32_t id, uint32_t acc) {
@@ -150,13 +160,13 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 #pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
+  for (int q = 0; q < 4; ++q) v[q] = __uint_as_float(r[q]);
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -173,16 +183,14 @@ __device__ inline void umma_alloc(const Umma& U) {
   // the copy and MMA barriers live for the whole kernel: initialised once here,
   // never re-initialised while an arrival could still be on its way
   if (threadIdx.x == 0) {
-    for (int q = 0; q < 2 * kUmmaStages; ++q) mbar_init(U.bar + q);
-    mbar_init(umma_never(U));
-    uint32_t* book = umma_book(U);
-    for (int q = 0; q < 4 * kUmmaStages; ++q) book[q] = 0u;
+    for (int q = 0; q < 2 * kUmmaStages + 2; ++q) mbar_init(U.bar + q);
+    *umma_book(U) = 0u;
     *umma_calls(U) = 0u;
   }
   // tiled tensor copies need 128-byte aligned shared destinations: a staging
   // buffer that is not marks the products void (they are then skipped and the
   // call reports it) instead of issuing a copy the hardware would reject
-  if (threadIdx.x == 0 && (((smem_u32(U.stage0) | smem_u32(U.stage1)) & 127u) != 0u)) {
+  if (threadIdx.x == 0 && ((smem_u32(U.stage) & 127u) != 0u)) {
     if (U.where && U.where[0] == 0) U.where[0] = 9;
     if (U.err) atomicOr(U.err, 2);
   }
@@ -206,28 +214,68 @@ __device__ inline void umma_free(const Umma& U) {
 // groups 256 bytes apart.
 __device__ __forceinline__ int umma_core_off(int r, int k) { return (r >> 3) * 128 + (k >> 3) * 64 + (r & 7) * 8 + (k & 7); }
 
-// Eight consecutive k of one row (or column) cut into digits: writes one
-// 16-byte core row per digit, blocks `bstride` elements apart.
-__device__ __forceinline__ void umma_split8(const dd* x, int e, __nv_bfloat16* out, size_t bstride) {
-  float h[8], l[8];
+// ---- operands to digits -------------------------------------------------------
+// |x| as an ordered integer whose top bits are the exponent, and the row exponent
+// e from the largest one (|x| < 2^(e-2) FP64, 2^(e-1) float pairs; 0: a zero row)
+__device__ __forceinline__ int umma_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int umma_mag(dd x) { return __float_as_int(x.hi) & 0x7fffffff; }
+__device__ __forceinline__ int umma_exp_of(int mag, double) {
+  const int ex = mag >> 20;
+  return ex == 0x7ff ? kUmmaNonFinite : ex == 0 ? 0 : ex - 1023 + 3;
+}
+__device__ __forceinline__ int umma_exp_of(int mag, dd) {
+  const int ex = mag >> 23;
+  return ex == 0xff ? kUmmaNonFinite : ex == 0 ? 0 : ex - 127 + 2;
+}
+// x 2^(8 ND - e) rounded to an integer
+__device__ __forceinline__ long long umma_fixed(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  const unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
+  const int sh = (ex ? ex : 1) - 1075 + 64 - e;
+  unsigned long long v = 0;
+  if (sh >= 0) v = m << (sh & 63);
+  else if (sh > -64) v = (m + (1ull << (-sh - 1))) >> (-sh);
+  return (long long)b < 0 ? -(long long)v : (long long)v;
+}
+__device__ __forceinline__ long long umma_fixed_f(float x, int e) {
+  const uint32_t b = __float_as_uint(x);
+  const int ex = (int)(b >> 23) & 0xff;
+  const uint32_t m = (b & 0x7fffffu) | (ex ? 0x800000u : 0u);
+  const int sh = (ex ? ex : 1) - 150 + 56 - e;
+  unsigned long long v = 0;
+  if (sh >= 0) v = (unsigned long long)m << (sh & 63);
+  else if (sh > -32) v = (m + (1u << (-sh - 1))) >> (-sh);
+  return (int)b < 0 ? -(long long)v : (long long)v;
+}
+__device__ __forceinline__ long long umma_fixed(dd x, int e) { return umma_fixed_f(x.hi, e) + umma_fixed_f(x.lo, e); }
+
+// Eight consecutive k of one row (or column) cut into digits: writes one 16-byte
+// core row per digit, blocks `bstride` elements apart.  The balanced digits are the
+// bytes of X + sum 128 256^b, less 128; a byte under the exponent bits of a power
+// of two is a float after one subtraction, already scaled by 2^(-8t).
+template <typename T>
+__device__ __forceinline__ void umma_split8(const T* x, int e, __nv_bfloat16* out, size_t bstride) {
+  constexpr int ND = UmmaDigits<T>::n;
+  uint32_t lo[8], hi[8];
+  const bool ok = e != kUmmaNonFinite;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    h[q] = ldexpf(x[q].hi, -e);
-    l[q] = ldexpf(x[q].lo, -e);
+    const unsigned long long y = (unsigned long long)(ok ? umma_fixed(x[q], e) : 0ll) +
+                                 (ND == 8 ? 0x8080808080808080ull : 0x0080808080808080ull);
+    lo[q] = (uint32_t)y;
+    hi[q] = (uint32_t)(y >> 32);
   }
 #pragma unroll
-  for (int t = 0; t < kUmmaDig; ++t) {
+  for (int t = 0; t < ND; ++t) {
+    const int byte = ND - 1 - t;                       // of X: its top digit first
+    const uint32_t magic = (uint32_t)(150 - 8 * t) << 23;
+    // 2^23 2^(-8t) + byte 2^(-8t); the top digit of seven may need a ninth bit
+    const uint32_t sel = (ND == 7 && t == 0) ? 0x7632u : (0x7640u | (uint32_t)(byte & 3));
+    const float off = __uint_as_float(magic) * (1.0f + 128.0f / 8388608.0f);
     float dg[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      h[q] *= 256.f;
-      l[q] *= 256.f;
-      const float qt = rintf(h[q]);
-      dg[q] = ldexpf(qt, -8 * t);
-      const dd r = two_sum(h[q] - qt, l[q]);
-      h[q] = r.hi;
-      l[q] = r.lo;
-    }
+    for (int q = 0; q < 8; ++q) dg[q] = __uint_as_float(__byte_perm(byte >= 4 ? hi[q] : lo[q], magic, sel)) - off;
     uint32_t w[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -238,83 +286,186 @@ __device__ __forceinline__ void umma_split8(const dd* x, int e, __nv_bfloat16* o
   }
 }
 
-// Exponents of the logical rows of an operand (R x Kd, padded to Rp rows):
-// |x| < 2^(e-1) for every entry of the row (0 for an all-zero or padding row).
-// TR: logical row r is column r of X (X[k * ldx + r]); else row r.
-template <bool TR>
-__device__ void umma_row_exponents(int R, int Kd, const dd* X, int ldx, int Rp, int* ex) {
+// Exponents of the logical rows of an operand (R x Kd, padded to Rp rows).  TR:
+// logical row r is column r of X (X[k * ldx + r]); else row r.  Ends with a barrier.
+template <bool TR, typename T>
+__device__ void umma_row_exponents(int R, int Kd, const T* X, int ldx, int Rp, int* ex) {
   const int tid = threadIdx.x, warp_id = tid >> 5, lane_id = tid & 31;
-  auto expo = [](float amax) { return amax > 0.f ? ilogbf(amax) + 2 : 0; };
+  constexpr int nw = kThreads / 32;
   if (!TR) {
-    for (int r = warp_id; r < Rp; r += kThreads / 32) {
-      float amax = 0.f;
+    for (int r = warp_id; r < Rp; r += nw) {
+      int mag = 0;
       if (r < R)
-        for (int k = lane_id; k < Kd; k += 32) amax = fmaxf(amax, fabsf(X[(size_t)r * ldx + k].hi));
-#pragma unroll
-      for (int o = 16; o; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      if (lane_id == 0) ex[r] = expo(amax);
+        for (int k = lane_id; k < Kd; k += 32) mag = max(mag, umma_mag(X[(size_t)r * ldx + k]));
+      mag = __reduce_max_sync(0xffffffffu, mag);
+      if (lane_id == 0) ex[r] = umma_exp_of(mag, T());
     }
   } else {
-    for (int r = tid; r < Rp; r += kThreads) {
-      float amax = 0.f;
-      if (r < R)
-        for (int k = 0; k < Kd; ++k) amax = fmaxf(amax, fabsf(X[(size_t)k * ldx + r].hi));
-      ex[r] = expo(amax);
+    // the warps share the k range, each thread one column of a 32-wide strip
+    for (int r = tid; r < Rp; r += kThreads) ex[r] = 0;
+    __syncthreads();
+    for (int r0 = 0; r0 < R; r0 += 32) {
+      const int r = r0 + lane_id;
+      int mag = 0;
+      if (r < R) {
+        int k = warp_id;
+        for (; k + 7 * nw < Kd; k += 8 * nw) {
+          int m[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) m[q] = umma_mag(X[(size_t)(k + q * nw) * ldx + r]);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) mag = max(mag, m[q]);
+        }
+#pragma unroll 4
+        for (; k < Kd; k += nw) mag = max(mag, umma_mag(X[(size_t)k * ldx + r]));
+        if (mag) atomicMax(ex + r, mag);
+      }
     }
+    __syncthreads();
+    for (int r = tid; r < Rp; r += kThreads) ex[r] = umma_exp_of(ex[r], T());
   }
+  __syncthreads();
 }
 
-// A split operand prepared once (the constant propagators e^-+dtau K): its digit
-// planes in the product's layout and its row exponents; null planes: split the
-// operand inside the product.
-struct UmmaOperand {
-  const __nv_bfloat16* planes;
-  const int* ex;
-  const CUtensorMap* tm;  // its tensor map (the 4D block view of `planes`)
-};
-
-// Digit planes of op(A) (rows of tile height UM) or of op(B)^T (rows = columns
-// of op(B), tile height NT): P[(tile * nkc + kc) * kUmmaDig + t] is a block of
+// Digit planes of op(A) (row tiles of umma_rows(M) rows) or of op(B)^T (rows =
+// columns of op(B), tiles of kUmmaNT): P[(tile * nkc + kc) * ND + t] is a block of
 // `tile_rows` x 16.  TR: the logical row r of the operand is column r of X
-// (X[k * ldx + r]); else row r (X[r * ldx + k]).
-template <bool TR>
-__device__ void umma_planes(int R, int Kd, const dd* X, int ldx, int Rp, int Kp, int tile_rows, const int* ex,
+// (X[k * ldx + r]); else row r (X[r * ldx + k]).  Eight neighbouring threads write
+// one 128-byte core matrix.
+template <bool TR, typename T>
+__device__ void umma_planes(int R, int Kd, const T* X, int ldx, int Rp, int Kp, int tile_rows, const int* ex,
                             __nv_bfloat16* P) {
+  constexpr int ND = UmmaDigits<T>::n;
   const int nkc = Kp / kUmmaK, kg8 = Kp / 8;
   const size_t blk = (size_t)tile_rows * kUmmaK;
   const int items = Rp * kg8;
-  for (int e = threadIdx.x; e < items; e += kThreads) {
-    int r, g;
-    if (TR) { g = e / Rp; r = e - g * Rp; } else { r = e / kg8; g = e - r * kg8; }
-    const int k0 = 8 * g;
-    dd x[8];
+  auto where = [&](int e, int& r, int& g) {
+    if (TR) {
+      g = e / Rp;
+      r = e - g * Rp;
+    } else {
+      const int h = e >> 3;
+      g = h % kg8;
+      r = (h / kg8) * 8 + (e & 7);
+    }
+  };
+  auto fetch = [&](int r, int g, T (&x)[8]) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int k = k0 + q;
-      x[q] = (r < R && k < Kd) ? (TR ? X[(size_t)k * ldx + r] : X[(size_t)r * ldx + k]) : dd{0.f, 0.f};
+      const int k = 8 * g + q;
+      x[q] = (r < R && k < Kd) ? (TR ? X[(size_t)k * ldx + r] : X[(size_t)r * ldx + k]) : T{};
     }
-    const int tile = r / tile_rows, rr = r - tile * tile_rows, kc = k0 / kUmmaK;
-    __nv_bfloat16* out = P + ((size_t)tile * nkc + kc) * kUmmaDig * blk + umma_core_off(rr, k0 - kc * kUmmaK);
-    umma_split8(x, ex[r], out, blk);
+  };
+  // the next item's loads are in flight while this one is cut
+  int e = threadIdx.x, r = 0, g = 0;
+  T x[8];
+  if (e < items) {
+    where(e, r, g);
+    fetch(r, g, x);
+  }
+  while (e < items) {
+    T y[8];
+    const int en = e + kThreads;
+    int rn = 0, gn = 0;
+    if (en < items) {
+      where(en, rn, gn);
+      fetch(rn, gn, y);
+    }
+    const int tile = r / tile_rows, rr = r - tile * tile_rows, kc = g >> 1;
+    __nv_bfloat16* out = P + ((size_t)tile * nkc + kc) * ND * blk + umma_core_off(rr, (g & 1) * 8);
+    umma_split8<T>(x, ex[r], out, blk);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = y[q];
+    e = en;
+    r = rn;
+    g = gn;
   }
 }
 
-// TMEM lane of tile row r for an M = 64 accumulator: rows 16q..16q+15 sit in
-// lanes 32q..32q+15 (the four 32-lane sub-partitions, first half each).
-__device__ __forceinline__ int umma_lane_of_row64(int r) { return ((r >> 4) << 5) + (r & 15); }
+// ---- diagonals to results ------------------------------------------------------
+// sum_d v_d 2^e
+__device__ __forceinline__ dd umma_combine(const float (&v)[kPlaneDigits], int e) {
+  const dd s1 = two_sum(v[0], v[1]), s2 = two_sum(v[2], v[3]);
+  const float tail = v[4] + (v[5] + v[6]);
+  dd s = two_sum(s1.hi, s2.hi);
+  s = two_sum(s.hi, s.lo + ((s1.lo + s2.lo) + tail));
+  // 2^e as two float factors
+  const int ec = max(-250, min(250, e)), e1 = ec / 2, e2 = ec - e1;
+  const float f1 = __int_as_float((127 + e1) << 23), f2 = __int_as_float((127 + e2) << 23);
+  s.hi = s.hi * f1 * f2;
+  s.lo = s.lo * f1 * f2;
+  if (e > 2000) s = {__int_as_float(0x7fc00000), 0.f};
+  return s;
+}
+// For FP64 the eight diagonals make one integer T = sum_d V_d 2^(8 (7-d)), V_d =
+// v_d 2^(8d), of at most 82 bits; it is normalised and rounded to 53 bits in
+// integer arithmetic (a warp's FP64 instruction costs 65 cycles of its scheduler's
+// FP64 unit, these thirty integer ones about as many issue slots).
+__device__ __forceinline__ double umma_combine(const float (&v)[kPlaneDigits64], int e) {
+  long long h = __float2int_rn(v[0]), l = __float2int_rn(v[4] * 4294967296.f);
+  h = h * 256 + __float2int_rn(v[1] * 256.f);
+  h = h * 256 + __float2int_rn(v[2] * 65536.f);
+  h = h * 256 + __float2int_rn(v[3] * 16777216.f);
+  l = l * 256 + __float2int_rn(v[5] * 1099511627776.f);
+  l = l * 256 + __float2int_rn(v[6] * 281474976710656.f);
+  l = l * 256 + __float2int_rn(v[7] * 72057594037927936.f);
+  h += l >> 32;
+  uint32_t w = (uint32_t)l;
+  const bool neg = h < 0;
+  if (neg) {
+    h = ~h;
+    w = 0u - w;
+    if (w == 0u) ++h;
+  }
+  unsigned long long m = (unsigned long long)h;
+  int ex = e - 56 + 32 + 63 + 1023;  // biased exponent of bit 63 of m
+  if (!(m >> 32)) {
+    m = (m << 32) | w;
+    w = 0u;
+    ex -= 32;
+    if (!(m >> 32)) { m <<= 32; ex -= 32; }
+  }
+  const int s = __clz((int)(m >> 32));
+  m = s ? (m << s) | (w >> (32 - s)) : m;
+  ex -= s;
+  m += 0x400ull;                        // round at bit 11
+  if (m < 0x400ull) { m = 0x8000000000000000ull | (m >> 1); ++ex; }
+  unsigned long long bits = ((unsigned long long)(uint32_t)ex << 52) | ((m >> 11) & 0xfffffffffffffull);
+  if (ex <= 0 || !(m >> 63)) bits = 0ull;
+  else if (ex >= 2047) bits = 0x7ff0000000000000ull;
+  if (e > 8000) bits = 0x7ff8000000000000ull;
+  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
 
-// C (+)= op(A) op(B), M x Nc, inner dimension Kd, float-pair operands (global
-// or L2-resident), on the tensor cores.  All threads of the CTA call it.
-// planes: the chain's scratch (left operand's planes at the start, the right
-// operand's at U.boff; U.tmA / U.tmB their tensor maps); expA, expB: shared
-// [roundup(M,64)], [roundup(Nc,48)] ints.  C must not alias A or B.
-template <bool TA, bool TB, bool ACC>
-__device__ void gemm_umma(int M, int Nc, int Kd, const dd* __restrict__ A, int lda, const dd* __restrict__ B, int ldb,
-                          dd* __restrict__ C, int ldc, __nv_bfloat16* planes, int* expA_s, int* expB_s, const Umma U,
-                          UmmaOperand cA = {nullptr, nullptr, nullptr}, UmmaOperand cB = {nullptr, nullptr, nullptr}) {
+__device__ __forceinline__ uint4 umma_pack(double a, double b) {
+  return make_uint4((uint32_t)__double2loint(a), (uint32_t)__double2hiint(a), (uint32_t)__double2loint(b),
+                    (uint32_t)__double2hiint(b));
+}
+__device__ __forceinline__ uint4 umma_pack(dd a, dd b) {
+  return make_uint4(__float_as_uint(a.hi), __float_as_uint(a.lo), __float_as_uint(b.hi), __float_as_uint(b.lo));
+}
+
+// C (+)= op(A) op(B), M x Nc, inner dimension Kd, FP64 or float-pair operands
+// (global, shared or L2-resident), on the tensor cores.  All threads of the CTA
+// call it.  ps: the plane buffers and tensor maps, made for M rows; ca, cb: a
+// prepared constant operand (kCpEA ...) or -1; expA, expB: shared, umma_pad'ed M and
+// Nc ints.  C must not alias A or B.
+template <typename T>
+__device__ __noinline__ void gemm_umma(bool ta, bool tb, bool acc, int M, int Nc, int Kd, const T* A, int lda,
+                                       const T* B, int ldb, T* C, int ldc, const PlaneSet* ps, int* expA_s,
+                                       int* expB_s, Umma U, int ca, int cb) {
+  constexpr int ND = UmmaDigits<T>::n;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int Mp = umma_pad(M, kUmmaM), Np = umma_pad(Nc, kUmmaNT), Kp = umma_pad(Kd, kUmmaK);
-  const int nmt = Mp / kUmmaM, nnt = Np / kUmmaNT, nkc = Kp / kUmmaK;
+  expA_s = as_shared(expA_s);
+  expB_s = as_shared(expB_s);
+  U.bar = as_shared(U.bar);
+  U.tmem_slot = as_shared(U.tmem_slot);
+  const int R = umma_rows(M), nmt = umma_row_tiles(M);
+  const int Mp = R * nmt, Np = umma_pad(Nc, kUmmaNT), Kp = umma_pad(Kd, kUmmaK);
+  const int nnt = Np / kUmmaNT, nkc = Kp / kUmmaK;
+  const uint32_t blockA = (uint32_t)R * kUmmaK * 2, blockB = kUmmaNT * kUmmaK * 2;
+  const uint32_t stage_bytes = ND * (blockA + blockB);
+  const int nst = min(kUmmaStages, (int)(U.stage_bytes / stage_bytes));
   // after a wait gave up (in this or an earlier product of the kernel) the
   // products are skipped: the results are void and the host reports it
   // (the chain's error word is shared with the peer flavor's CTA: thread 0
@@ -324,48 +475,49 @@ __device__ void gemm_umma(int M, int Nc, int Kd, const dd* __restrict__ A, int l
   // earlier generic writes of the staging area (other products) before the
   // copies of this one
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  const CUtensorMap* tmA = cA.planes ? cA.tm : U.tmA;
-  const CUtensorMap* tmB = cB.planes ? cB.tm : U.tmB;
-  const int* expA = cA.planes ? cA.ex : expA_s;
-  const int* expB = cB.planes ? cB.ex : expB_s;
-  if (!cA.planes) umma_row_exponents<TA>(M, Kd, A, lda, Mp, expA_s);
-  if (!cB.planes) umma_row_exponents<!TB>(Nc, Kd, B, ldb, Np, expB_s);
-  __syncthreads();
-  if (!cA.planes) {
-    umma_planes<TA>(M, Kd, A, lda, Mp, Kp, kUmmaM, expA_s, planes);
-  }
-  if (!cB.planes) {
-    __nv_bfloat16* pb = planes + U.boff;
-    umma_planes<!TB>(Nc, Kd, B, ldb, Np, Kp, kUmmaNT, expB_s, pb);
+  const CUtensorMap* tmA = ca >= 0 ? &ps->tm_cp[ca] : &ps->tm_pl[0];
+  const CUtensorMap* tmB = cb >= 0 ? &ps->tm_cp[cb] : &ps->tm_pl[1];
+  const int* expA = ca >= 0 ? ps->cex[ca] : expA_s;
+  const int* expB = cb >= 0 ? ps->cex[cb] : expB_s;
+  // both operands by the same code (a right operand's logical rows are its columns)
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    if ((side ? cb : ca) >= 0) continue;
+    const T* X = side ? B : A;
+    const int n = side ? Nc : M, ldx = side ? ldb : lda, np = side ? Np : Mp, tile = side ? kUmmaNT : R;
+    int* ex = side ? expB_s : expA_s;
+    __nv_bfloat16* P = (__nv_bfloat16*)ps->scratch + (side ? ps->boff : 0);
+    if (side ? !tb : ta) {
+      umma_row_exponents<true>(n, Kd, X, ldx, np, ex);
+      umma_planes<true>(n, Kd, X, ldx, np, Kp, tile, ex, P);
+    } else {
+      umma_row_exponents<false>(n, Kd, X, ldx, np, ex);
+      umma_planes<false>(n, Kd, X, ldx, np, Kp, tile, ex, P);
+    }
   }
   // the planes are read by the bulk copies (async proxy)
   asm volatile("fence.proxy.async.global;" ::: "memory");
   __syncthreads();
   const uint32_t tmem = *U.tmem_slot;
-  constexpr uint32_t idesc = umma_idesc(kUmmaM, kUmmaNT);
-  // chunk sequence: tiles (mt, nt) in order, within a tile its k chunks; a tile's
-  // chunks are accumulated in segments of kUmmaKSeg
-  const int segc = kUmmaKSeg / kUmmaK;
-  const int nch = nmt * nnt * nkc;
-  // Thread 0's bookkeeping (U.cpy_*, U.mma_*: copies and MMA commits issued and
-  // waited per stage, continued across the products of the kernel).  Every
-  // barrier has at most one phase in flight when it is waited on (a stage is
-  // refilled only after its MMAs are done, its MMAs issued only after its copy
-  // landed, and every product ends with all of them waited), so parity waits are
-  // sound.  live: no wait has given up; once one has, nothing more is issued and
-  // the end of the product drains what is in flight before the tensor memory and
-  // the staging buffers are used again.
-  uint32_t* cpy_n = umma_book(U);
-  uint32_t* cpy_w = cpy_n + kUmmaStages;
-  uint32_t* mma_n = cpy_n + 2 * kUmmaStages;
-  uint32_t* mma_w = cpy_n + 3 * kUmmaStages;
-  bool live = true;
-  auto gave_up = [&](int kind, int g) {
-    if (live && U.where && U.where[0] == 0) {
-      const int st = g % kUmmaStages;
+  // 16-byte stores of two neighbouring outputs where C's rows allow them
+  const bool vec = ((reinterpret_cast<uintptr_t>(C) | ((uintptr_t)ldc * sizeof(T))) & 15) == 0;
+  // Chunk sequence: tiles (mt, nt) in order, within a tile its k chunks; a tile's
+  // chunks are accumulated in segments of kUmmaKSeg.  Chunk c uses stage c % nst for
+  // the (c / nst)-th time in this product; every barrier has at most one phase in
+  // flight when it is waited on (a stage is refilled only after its MMAs are done,
+  // multiplied only after its copy landed), and a product ends with all of them
+  // complete, so parity waits are sound.  par: the barriers' next parities (shared,
+  // continued across products): bits 0..2 copies, 3..5 MMAs, 6 accumulators.
+  const int segc = kUmmaKSeg / kUmmaK, nseg = (nkc + segc - 1) / segc;
+  const int nch = nmt * nnt * nkc, n_seg = nmt * nnt * nseg;
+  const uint32_t par = *umma_book(U);
+  uint64_t* bar_full = U.bar;
+  uint64_t* bar_mma = U.bar + kUmmaStages;
+  bool live = true;  // no wait of this warp has given up
+  auto gave_up = [&](int kind, int g, uint64_t* bar) {
+    if (live && lane == 0 && U.where && atomicCAS(U.where, 0, kind) == 0) {
       unsigned long long w = 0;
-      asm volatile("ld.shared.b64 %0, [%1];" : "=l"(w) : "r"(smem_u32(U.bar + (kind == 1 ? st : kUmmaStages + st))));
-      U.where[0] = kind;
+      asm volatile("ld.shared.b64 %0, [%1];" : "=l"(w) : "r"(smem_u32(bar)));
       U.where[1] = g;
       U.where[2] = nch;
       U.where[3] = (int)*umma_calls(U);
@@ -374,120 +526,153 @@ __device__ void gemm_umma(int M, int Nc, int Kd, const dd* __restrict__ A, int l
     }
     live = false;
   };
-  uint64_t* bar_full = U.bar;
-  uint64_t* bar_mma = U.bar + kUmmaStages;
-  auto wait_mma = [&](int st, long long lim) {
-    if (mma_w[st] == mma_n[st]) return true;
-    if (!mbar_wait(bar_mma + st, (mma_n[st] - 1) & 1, lim)) return false;
-    mma_w[st] = mma_n[st];
-    return true;
-  };
-  auto wait_copy = [&](int st, long long lim) {
-    if (cpy_w[st] == cpy_n[st]) return true;
-    if (!mbar_wait(bar_full + st, (cpy_n[st] - 1) & 1, lim)) return false;
-    cpy_w[st] = cpy_n[st];
-    return true;
-  };
-  auto issue_copy = [&](int g) {  // thread 0: chunk g into stage g % kUmmaStages
-    if (!live || g >= nch) return;
-    const int st = g % kUmmaStages;
-    if (!wait_mma(st, U.limit)) { gave_up(2, g); return; }
-    const int tile = g / nkc, kc = g - tile * nkc, mt = tile / nnt, nt = tile - mt * nnt;
-    mbar_expect_tx(bar_full + st, kUmmaStageBytes);
-    unsigned char* dst = umma_stage(U, st);
-    tma_load_block(dst, tmA, mt * nkc + kc, bar_full + st);
-    tma_load_block(dst + kUmmaDig * kUmmaBlockA, tmB, nt * nkc + kc, bar_full + st);
-    ++cpy_n[st];
-  };
-  if (tid == 0)
-    for (int g = 0; g < kUmmaStages - 1; ++g) issue_copy(g);
-  uint32_t written = 0u;
-  for (int g = 0; g < nch; ++g) {
-    const int st = g % kUmmaStages;
-    const int tile = g / nkc, kc = g - tile * nkc, mt = tile / nnt, nt = tile - mt * nnt;
-    if (kc % segc == 0) written = 0u;
-    if (tid == 0 && live) {
-      bool landed = wait_copy(st, U.limit);
-      // test hook: a wait that cannot end (its barrier's phase 0 never completes)
-      if (landed && U.stall && g == 0) landed = mbar_wait(umma_never(U), 0u, U.limit);
-      if (!landed) {
-        gave_up(1, g);
-      } else {
+  int c = 0, cst = 0, cuse = 0;          // warp 1: next chunk to copy, its stage and use
+  int crowA = 0, crowB = 0, ckc = 0, cnt = 0;  // ... its rows in the planes, k chunk and column tile
+  int m = 0, mst = 0, muse = 0;          // warp 0: next chunk to multiply
+  const int rowsA = (int)(ND * blockA / (2 * kPlaneRowElems)), rowsB = (int)(ND * blockB / (2 * kPlaneRowElems));
+  const uint32_t stage0 = smem_u32(U.stage);
+  bool dead = false;
+  int mt = 0, nt = 0, seg = 0;
+  for (int sg = 0; sg < n_seg && !dead; ++sg) {
+    const int kc0 = seg * segc, kc1 = min(nkc, kc0 + segc);
+    const int end = (mt * nnt + nt) * nkc + kc1;  // chunks up to the end of this segment
+    if (warp == 1) {
+      // copies of this segment and, while its MMAs drain, of the next one's first chunks
+      const int ahead = min(nch, end + nst);
+      while (live && c < ahead) {
+        if (cuse > 0 && !mbar_wait(bar_mma + cst, ((par >> (3 + cst)) ^ (cuse - 1)) & 1, U.limit)) {
+          gave_up(2, c, bar_mma + cst);
+          break;
+        }
+        unsigned char* dst = U.stage + (size_t)cst * stage_bytes;
+        if (elect_one()) {
+          mbar_expect_tx(bar_full + cst, stage_bytes);
+          tma_load_block(dst, tmA, crowA, bar_full + cst);
+          tma_load_block(dst + ND * blockA, tmB, crowB, bar_full + cst);
+        }
+        __syncwarp();
+        ++c;
+        if (++cst == nst) { cst = 0; ++cuse; }
+        crowA += rowsA;
+        crowB += rowsB;
+        if (++ckc == nkc) {
+          ckc = 0;
+          if (++cnt == nnt) { cnt = 0; crowB = 0; }
+          else crowA -= nkc * rowsA;  // the next column tile reads the same row tile again
+        }
+      }
+    } else if (warp == 0) {
+      for (int kc = kc0; live && kc < kc1; ++kc) {
+        bool landed = mbar_wait(bar_full + mst, ((par >> mst) ^ muse) & 1, U.limit);
+        // test hook: a wait that cannot end (its barrier's phase 0 never completes)
+        if (landed && U.stall && m == 0) landed = mbar_wait(umma_never(U), 0u, U.limit);
+        if (!landed) {
+          gave_up(1, m, bar_full + mst);
+          break;
+        }
         tc_fence_after();
-        const uint32_t sa = smem_u32(umma_stage(U, st));
-        const uint32_t sb = sa + kUmmaDig * kUmmaBlockA;
+        const uint32_t sa = stage0 + (uint32_t)mst * stage_bytes;
+        const uint64_t ad = umma_sdesc(sa, 128, 256), bd = umma_sdesc(sa + ND * blockA, 128, 256);
+        if (elect_one()) {
 #pragma unroll
-        for (int t = 0; t < kUmmaDig; ++t)
-#pragma unroll
-          for (int u = 0; t + u < kUmmaDig; ++u) {
-            const int d = (t + u < kUmmaSlots - 1) ? t + u : kUmmaSlots - 1;
-            const uint64_t ad = umma_sdesc(sa + t * kUmmaBlockA, 128, 256);
-            const uint64_t bd = umma_sdesc(sb + u * kUmmaBlockB, 128, 256);
-            umma_bf16(tmem + d * kUmmaNT, ad, bd, idesc, (written >> d) & 1u);
-            written |= 1u << d;
-          }
-        umma_commit(bar_mma + st);
-        ++mma_n[st];
+          for (int t = 0; t < ND; ++t)
+            umma_bf16(tmem + t * kUmmaNT, ad + (uint64_t)(t * (blockA >> 4)), bd,
+                      umma_idesc(kUmmaM, kUmmaNT * (ND - t)), !(kc == kc0 && t == 0));
+          umma_commit(bar_mma + mst);
+          if (kc + 1 == kc1) umma_commit(umma_acc(U));
+        }
+        __syncwarp();
+        ++m;
+        if (++mst == nst) { mst = 0; ++muse; }
       }
     }
-    // keep two chunks in flight: chunk g+2 goes where chunk g-1 was, whose MMAs
-    // were issued before chunk g's (waiting for them does not drain the pipe)
-    if (tid == 0) issue_copy(g + kUmmaStages - 1);
-    const bool seg_end = (kc + 1 == nkc) || ((kc + 1) % segc == 0);
-    if (!seg_end) continue;
-    // epilogue of a tile segment: all its MMAs done (the last commit covers
-    // every MMA issued before it); thread 0 waits, then releases the CTA
-    if (tid == 0 && live && !wait_mma(st, U.limit)) gave_up(3, g);
-    tc_fence_before();
-    __syncthreads();
+    // epilogue of a tile segment: all its MMAs done
+    if (live && !mbar_wait(umma_acc(U), ((par >> 6) ^ sg) & 1, U.limit)) gave_up(3, end - 1, umma_acc(U));
     tc_fence_after();
-    const int ks = kc - kc % segc;
-    // warp w reads sub-partition w % 4 (rows 16 (w % 4) .. + 15 in its lanes
-    // 0..15) and the column half w / 4 of the tile
-    const int rloc = (warp & 3) * 16 + (lane & 15);
-    const int row = mt * kUmmaM + rloc;
-    const bool live_row = (lane < 16) && row < M;
-    const int eA = live_row ? expA[row] : 0;
-    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    for (int c0 = (warp >> 2) * (kUmmaNT / 2); c0 < (warp >> 2) * (kUmmaNT / 2) + kUmmaNT / 2; c0 += 8) {
-      float v[kUmmaSlots][8];
+    if (live) {
+      const bool add = acc || seg > 0;
+      // warp w reads lanes 32 (w % 4) .. + 31 (tile rows) and the column half w / 4
+      const int rloc = (warp & 3) * 32 + lane;
+      const int row = mt * R + rloc;
+      const bool live_row = rloc < R && row < M;
+      if ((warp & 3) * 32 < R) {
+        const int eA = live_row ? expA[row] : 0;
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+#pragma unroll 1
+        for (int c0 = (warp >> 2) * (kUmmaNT / 2); c0 < (warp >> 2) * (kUmmaNT / 2) + kUmmaNT / 2; c0 += 4) {
+          if (nt * kUmmaNT + c0 >= Nc) break;
+          T* cp = C + (size_t)row * ldc + nt * kUmmaNT + c0;
+          T old[4];
+          if (add && live_row) {
 #pragma unroll
-      for (int d = 0; d < kUmmaSlots; ++d) tmem_ld8(tmem + lane_base + d * kUmmaNT + c0, v[d]);
-      tmem_ld_wait();
-      if (live_row) {
+            for (int q = 0; q < 4; ++q) old[q] = (nt * kUmmaNT + c0 + q < Nc) ? cp[q] : T{};
+          }
+          float v[ND][4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int col = nt * kUmmaNT + c0 + q;
-          if (col < Nc) {
-            dd sum = {v[kUmmaSlots - 1][q], 0.f};
+          for (int d = 0; d < ND; ++d) tmem_ld4(tmem + lane_base + d * kUmmaNT + c0, v[d]);
+          tmem_ld_wait();
+          if (live_row) {
+            T sum[4];
 #pragma unroll
-            for (int d = kUmmaSlots - 2; d >= 0; --d) sum = dd_add(sum, {v[d][q], 0.f});
-            const int e = eA + expB[col] - 16;
-            sum.hi = ldexpf(sum.hi, e);
-            sum.lo = ldexpf(sum.lo, e);
-            dd* cp = C + (size_t)row * ldc + col;
-            *cp = (ACC || ks > 0) ? dd_add(*cp, sum) : sum;
+            for (int q = 0; q < 4; ++q) {
+              const int col = nt * kUmmaNT + c0 + q;
+              float d[ND];
+#pragma unroll
+              for (int t = 0; t < ND; ++t) d[t] = v[t][q];
+              sum[q] = umma_combine(d, eA + expB[col] - 16);
+              if (add) sum[q] = radd(old[q], sum[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q += 2) {
+              const int col = nt * kUmmaNT + c0 + q;
+              if (vec && col + 1 < Nc) {
+                *reinterpret_cast<uint4*>(cp + q) = umma_pack(sum[q], sum[q + 1]);
+              } else {
+                if (col < Nc) cp[q] = sum[q];
+                if (col + 1 < Nc) cp[q + 1] = sum[q + 1];
+              }
+            }
           }
         }
       }
     }
+    if (++seg == nseg) {
+      seg = 0;
+      if (++nt == nnt) { nt = 0; ++mt; }
+    }
     // the accumulators are overwritten by the next segment's first MMAs
     tc_fence_before();
-    __syncthreads();
+    dead = __syncthreads_or(!live);
     tc_fence_after();
   }
-  if (tid == 0) {
-    // every copy and every MMA commit of the product waited for (all complete
-    // already unless a wait gave up: then with the default limit, a drain)
-    for (int st = 0; st < kUmmaStages; ++st) {
-      const long long lim = live ? U.limit : kUmmaWaitCycles;
-      if (!wait_copy(st, lim) && live) gave_up(4, st);
-      if (!wait_mma(st, lim) && live) gave_up(5, st);
+  // A wait gave up: what is in flight is drained (with the default limit) before the
+  // staging buffers and the tensor memory are used again.
+  if (dead) {
+    uint32_t* book = umma_book(U);
+    if (warp == 1 && lane == 0) book[1] = (uint32_t)c;
+    if (warp == 0 && lane == 0) book[2] = (uint32_t)m;
+    __syncthreads();
+    if (tid == 0) {
+      for (int q = max(0, (int)book[1] - nst); q < (int)book[1]; ++q)
+        mbar_wait(bar_full + q % nst, ((par >> (q % nst)) ^ (q / nst)) & 1, kUmmaWaitCycles);
+      for (int q = max(0, (int)book[2] - nst); q < (int)book[2]; ++q)
+        mbar_wait(bar_mma + q % nst, ((par >> (3 + q % nst)) ^ (q / nst)) & 1, kUmmaWaitCycles);
+      // the products after a wait gave up are skipped: the parities are not used again
+      if (U.err) atomicOr(U.err, 2);
     }
+  } else if (tid == 0) {
+    // every copy and MMA of the product is complete: next parities
+    uint32_t p = par ^ ((uint32_t)(n_seg & 1) << 6);
+    bool done = true;
+    for (int q = 0; q < nst && q < nch; ++q) {
+      const uint32_t uses = (uint32_t)((nch - q + nst - 1) / nst);
+      done = done && mbar_wait(bar_mma + q, ((par >> (3 + q)) ^ (uses - 1)) & 1, kUmmaWaitCycles);
+      p ^= ((uses & 1u) << q) | ((uses & 1u) << (3 + q));
+    }
+    *umma_book(U) = p;
+    if (!done && U.err) atomicOr(U.err, 2);
   }
-  const bool ok = live;
   // the staging buffers are reused by generic loads and stores after the product
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  if (!ok && U.err) atomicOr(U.err, 2);
   __syncthreads();
 }
