@@ -210,6 +210,8 @@ __device__ __forceinline__ dd from_d<dd>(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
 }
+template <typename R>
+__device__ __forceinline__ R from_zero() { return R{}; }
 // 1 or 0 without a conversion (conversions from FP64 run on the slow FP64 pipe)
 template <typename R>
 __device__ __forceinline__ R unit(bool one) { return one ? R(1) : R(0); }
@@ -529,7 +531,12 @@ __host__ __device__ inline int exp_len(int ld) { return ld + kPlaneMaxRows; }
 // panels and, in the sweep kernel, the delayed vectors.  The tensor-core products
 // stage their operands over both: neither is live inside a product (a flush has
 // cut its delayed vectors into digits before the first copy lands).
+// (The panels also hold the QR's, two of kPanel columns.)
 constexpr int kGemmRegionBytes = 2 * 16 * kGemmMaxTile * 8;
+__host__ __device__ inline size_t gemm_region_bytes(int ld) {
+  const size_t qr = (size_t)2 * 4 * (ld + 1) * 8;
+  return ((qr > (size_t)kGemmRegionBytes ? qr : (size_t)kGemmRegionBytes) + 127) / 128 * 128;
+}
 
 __host__ __device__ inline size_t smem_stage_offset(int ld, int MV) {
   size_t b = kSmemCounterBytes;
@@ -546,7 +553,7 @@ __host__ __device__ inline size_t smem_stage_offset(int ld, int MV) {
   b += 128;                       // mbarriers and the TMEM slot of the tensor-core products
   return (b + 127) / 128 * 128 + 128;  // room to align the panels
 }
-__host__ __device__ inline size_t smem_bytes_for(int ld, int MV) { return smem_stage_offset(ld, MV) + kGemmRegionBytes; }
+__host__ __device__ inline size_t smem_bytes_for(int ld, int MV) { return smem_stage_offset(ld, MV) + gemm_region_bytes(ld); }
 
 __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   Smem s;
@@ -590,7 +597,7 @@ __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   q += 128;
   q = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(q) + 127) & ~(uintptr_t)127);
   s.gemm = reinterpret_cast<double*>(q);
-  s.ab = reinterpret_cast<double*>(q + kGemmRegionBytes);
+  s.ab = reinterpret_cast<double*>(q + gemm_region_bytes(ld));
   uint32_t dyn;
   asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
   s.um.stage = q;
@@ -697,198 +704,754 @@ __device__ inline UDV slot_udv(const ChainDev& C, int s, int j) {
   return u;
 }
 
-// M[k:, j] -= bk v (v^T M[k:, j]) for the columns j0 <= j < N, v = hv[k:].
-// 8 row groups x 32 columns: rows are read coalesced along j; the partial dot
-// products of the row groups are summed in shared memory in a fixed order.
-__device__ void householder_apply(int N, int ld, double* M, int k, int j0, double bk, const double* hv,
-                                  double* qred) {
-  const int tid = threadIdx.x, lane = tid & 31, rg = tid >> 5;
-  for (int c0 = j0; c0 < N; c0 += 128) {
-    double w[4] = {0.0, 0.0, 0.0, 0.0};
-    int i = k + rg;
-    // four rows per iteration with all loads issued first (memory-level parallelism)
-    for (; i + 24 < N; i += 32) {
-      double x[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = c0 + lane + 32 * q;
-          x[r][q] = (j < N) ? M[(size_t)(i + 8 * r) * ld + j] : 0.0;
-        }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const double vi = hv[i + 8 * r];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[q] = fma(vi, x[r][q], w[q]);
+__device__ inline void to_dd_mat(int N, int ld, const double* src, dd* dst) {
+  for (int e = threadIdx.x; e < N * N; e += kThreads) {
+    const int x = e / N, y = e - x * N;
+    dst[(size_t)x * ld + y] = from_d<dd>(src[(size_t)x * ld + y]);
+  }
+  __syncthreads();
+}
+
+// dd -> double in place (same 8-byte slot)
+__device__ inline void dd_to_d_inplace(int N, int ld, void* buf) {
+  dd* a = reinterpret_cast<dd*>(buf);
+  double* b = reinterpret_cast<double*>(buf);
+  for (int e = threadIdx.x; e < N * N; e += kThreads) {
+    const int x = e / N, y = e - x * N;
+    const dd v = a[(size_t)x * ld + y];
+    b[(size_t)x * ld + y] = to_d(v);
+  }
+  __syncthreads();
+}
+
+// ---- pivoted QR in panels, LU and solves, on FP64 or float-pair matrices --------
+// Scalars of the reflectors and the LU in the matrix's own type.
+__device__ __forceinline__ double rsqrt_of_sum(double x) { return sqrt(x); }
+// sqrt of a float pair: FP32 root and one Newton step (Heron) on the pair
+__device__ __forceinline__ dd rsqrt_of_sum(dd x) {
+  if (!(x.hi > 0.f)) return {0.f, 0.f};
+  const float r = sqrtf(x.hi);
+  const dd e = dd_fma({-r, 0.f}, {r, 0.f}, x);
+  return fast_two_sum(r, e.hi / (2.f * r));
+}
+__device__ __forceinline__ bool is_pos(double x) { return x > 0.0; }
+__device__ __forceinline__ bool is_pos(dd x) { return x.hi > 0.f; }
+__device__ __forceinline__ double rabs(double x) { return fabs(x); }
+__device__ __forceinline__ dd rabs(dd x) { return x.hi < 0.f ? dd{-x.hi, -x.lo} : x; }
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ dd shfl_xor(dd v, int o) {
+  return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ double shfl(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ dd shfl(dd v, int l) {
+  return {__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
+}
+
+// Panels in shared memory, column-major with an odd column stride (neighbouring
+// threads' rows and columns fall into different banks).
+__device__ __forceinline__ int panel_ld(int N) { return N | 1; }
+// Columns per panel of the QR.  Wider panels save passes over the matrix, but the
+// products of more reflectors lose the small rows of Q: with 16 columns the wrapped
+// G's drift on 4 x 4 lattices is four times the unblocked factorisation's, with 4
+// the same (FP64, U = 4: mean 1.4e-11, 3.7e-12 and 3.5e-12).
+constexpr int kPanel = 4;  // gemm_region_bytes counts two such panels
+// Columns per panel of the LU and the solves: the largest power of two <= 16 of which
+// two panels fit the product area.
+__device__ inline int panel_width(int N, const Smem& S) {
+  const int cap = (int)(S.um.stage_bytes / 16);
+  int w = 16;
+  while (w > 1 && w * panel_ld(N) > cap) w >>= 1;
+  return w;
+}
+
+// log2 of a positive FP64 number in FP32 (an order for the columns, not a value)
+__device__ __forceinline__ float log2_rough(double x) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  const float m = __int_as_float(((hi & 0xfffff) << 3) | 0x3f800000);
+  return ex == 0 ? -3.0e38f : (float)(ex - 1023) + __log2f(m);
+}
+// order of a column: log2 of its norm (from the square) and scale, NaN last
+__device__ __forceinline__ float column_key(float norm2, float lsc) {
+  const float k = 0.5f * log2f(norm2) + lsc;
+  return k == k ? k : -3.4e38f;
+}
+__device__ __forceinline__ float column_key(double norm2, float lsc) {
+  const float k = norm2 > 0.0 ? 0.5f * log2_rough(norm2) + lsc : -3.3e38f;
+  return k == k ? k : -3.4e38f;
+}
+__device__ __forceinline__ float column_key(dd norm2, float lsc) { return column_key(fmaxf(norm2.hi, 0.f), lsc); }
+__device__ __forceinline__ float as_float(double x) { return (float)x; }
+__device__ __forceinline__ float as_float(dd x) { return x.hi; }
+
+// Keys (log2 of the scaled column norms, by list position) of the columns of M = X
+// diag(dsc), and log2 dsc (by column).  The sums of squares stay in FP32: X is a
+// product of n_wrap slices with an orthogonal matrix, far inside its range, and the
+// keys only order the columns (NaN last).
+template <typename T>
+__device__ void column_keys(int N, int ld, const T* X, const double* dsc, float* key, float* lsc, Smem& S) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int nw = kThreads / 32;
+  float* part = reinterpret_cast<float*>(S.qred);   // [nw][32] partial sums of squares
+  for (int j0 = 0; j0 < N; j0 += 32) {
+    const int j = j0 + lane;
+    float a0 = 0.f, a1 = 0.f;
+    if (j < N) {
+      int i = warp;
+      for (; i + nw < N; i += 2 * nw) {
+        const float x = as_float(X[(size_t)i * ld + j]), y = as_float(X[(size_t)(i + nw) * ld + j]);
+        a0 = fmaf(x, x, a0);
+        a1 = fmaf(y, y, a1);
+      }
+      if (i < N) {
+        const float x = as_float(X[(size_t)i * ld + j]);
+        a0 = fmaf(x, x, a0);
       }
     }
-    for (; i < N; i += 8) {
-      const double vi = hv[i];
-      const double* row = M + (size_t)i * ld;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = c0 + lane + 32 * q;
-        if (j < N) w[q] = fma(vi, row[j], w[q]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) qred[rg * 128 + lane + 32 * q] = w[q];
+    part[warp * 32 + lane] = a0 + a1;
     __syncthreads();
-    double wt[4];
+    if (warp == 0 && j < N) {
+      float a = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      double t = 0.0;
-#pragma unroll
-      for (int r = 0; r < 8; ++r) t += qred[r * 128 + lane + 32 * q];
-      wt[q] = bk * t;
-    }
-    i = k + rg;
-    for (; i + 24 < N; i += 32) {
-      double x[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = c0 + lane + 32 * q;
-          x[r][q] = (j < N) ? M[(size_t)(i + 8 * r) * ld + j] : 0.0;
-        }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const double vi = hv[i + 8 * r];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = c0 + lane + 32 * q;
-          if (j < N) M[(size_t)(i + 8 * r) * ld + j] = x[r][q] - wt[q] * vi;
-        }
-      }
-    }
-    for (; i < N; i += 8) {
-      const double vi = hv[i];
-      double* row = M + (size_t)i * ld;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = c0 + lane + 32 * q;
-        if (j < N) row[j] -= wt[q] * vi;
-      }
+      for (int w = 0; w < nw; ++w) a += part[w * 32 + lane];
+      lsc[j] = log2_rough(dsc[j]);
+      key[j] = column_key(a, lsc[j]);
     }
     __syncthreads();
   }
 }
 
-// Householder QR with column pivoting of M (N x N, in place): on return the
-// upper triangle holds R, the strict lower triangle the Householder vectors
-// (their leading entries in vk0), beta[k] the reflector coefficients,
-// perm[k] the original column at position k.  Returns det(Q) = (-1)^#reflectors.
-// Pivot = remaining column of largest norm (ties to the lowest index); norms
-// are downdated and recomputed when cancellation sets in (LAPACK xGEQP3 rule).
-__device__ int qr_pivoted(int N, int ld, double* M, double* beta, double* vk0, double* cn, double* cn0,
-                          int* perm, Smem& S) {
-  const int tid = threadIdx.x;
-  for (int j = tid; j < N; j += kThreads) {
-    double acc = 0.0;
-    for (int i = 0; i < N; ++i) acc = fma(M[(size_t)i * ld + j], M[(size_t)i * ld + j], acc);
-    cn[j] = sqrt(acc);
-    cn0[j] = cn[j];
-    perm[j] = j;
-  }
-  __syncthreads();
-  const double tol3z = sqrt(2.220446049250313e-16);
-  int detq = 1;
-  for (int k = 0; k < N; ++k) {
-    // pivot
-    double bv = -1.0;
-    int bi = N;
-    for (int j = k + tid; j < N; j += kThreads)
-      if (cn[j] > bv) { bv = cn[j]; bi = j; }
-    int p = block_argmax(bv, bi, S.red, S.ired);
-    if (p >= N) p = k;  // no finite candidate (NaN input): keep the column order
-    if (p != k) {
-      for (int i = tid; i < N; i += kThreads) {
-        const double t = M[(size_t)i * ld + k];
-        M[(size_t)i * ld + k] = M[(size_t)i * ld + p];
-        M[(size_t)i * ld + p] = t;
+// A[r0:, j0:] -= V (W^T A[r0:, j0:]) with the N - r0 rows of V and W in shared
+// panels of `nb` <= kPanel columns: one column of A per thread (and G threads, one row
+// class each, where the columns leave threads over), the nb sums in registers.
+// FLIP: the roles of V and W exchanged.  LIST: position j stands for column list[j],
+// and the keys of the rows below the panel are renewed.
+template <typename T, bool FLIP, bool LIST>
+__device__ void panel_apply(int N, int ld, T* A, int r0, int j0, int nb, const T* Vp, const T* Wp, Smem& S,
+                            const int* list, float* key, const float* lsc) {
+  constexpr int PW = kPanel;
+  const int tid = threadIdx.x, ldp = panel_ld(N);
+  const T* Lp = FLIP ? Wp : Vp;  // left factor of the update
+  const T* Rp = FLIP ? Vp : Wp;  // the sums' factor
+  T* red = reinterpret_cast<T*>(S.qred);  // [G][4][cw] <= 1024
+  for (int c0 = j0; c0 < N; c0 += kThreads) {
+    const int nc = (N - c0 < kThreads) ? N - c0 : kThreads;
+    const int cw = (nc + 31) / 32 * 32, G = kThreads / cw;
+    const int g = tid / cw, jj = tid - g * cw;
+    const bool act = g < G && jj < nc;
+    const int j = act ? (LIST ? list[c0 + jj] : c0 + jj) : 0;
+    float n2 = 0.f;
+    T y[PW];
+#pragma unroll
+    for (int q = 0; q < PW; ++q) y[q] = from_zero<T>();
+    if (act) {
+      // four rows at a time, their loads issued together
+      int i = r0 + g;
+      for (; i + 3 * G < N; i += 4 * G) {
+        T x[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) x[b] = A[(size_t)(i + b * G) * ld + j];
+        const T* r = Rp + (i - r0);
+#pragma unroll
+        for (int q = 0; q < PW; ++q)
+          if (q < nb) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) y[q] = rfma(r[q * ldp + b * G], x[b], y[q]);
+          }
       }
-      if (tid == 0) {
-        const int tp = perm[k]; perm[k] = perm[p]; perm[p] = tp;
-        double t = cn[k]; cn[k] = cn[p]; cn[p] = t;
-        t = cn0[k]; cn0[k] = cn0[p]; cn0[p] = t;
+      for (; i < N; i += G) {
+        const T x = A[(size_t)i * ld + j];
+        const T* r = Rp + (i - r0);
+#pragma unroll
+        for (int q = 0; q < PW; ++q)
+          if (q < nb) y[q] = rfma(r[q * ldp], x, y[q]);
       }
-      __syncthreads();
     }
-    // reflector from column k, rows k..N-1
-    double part = 0.0;
-    for (int i = k + tid; i < N; i += kThreads) {
-      const double x = M[(size_t)i * ld + k];
-      part = fma(x, x, part);
-      S.hv[i] = x;
+    if (G > 1) {
+      // the row classes' sums in rounds of four, each summed by one class
+#pragma unroll
+      for (int b = 0; b < PW; b += 4) {
+        if (b >= nb) continue;
+        if (act) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) red[(g * 4 + q) * cw + jj] = y[b + q];
+        }
+        __syncthreads();
+        if (act) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q % G == g) {
+              T t = red[q * cw + jj];
+              for (int h = 1; h < G; ++h) t = radd(t, red[(h * 4 + q) * cw + jj]);
+              red[q * cw + jj] = t;
+            }
+        }
+        __syncthreads();
+        if (act) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) y[b + q] = red[q * cw + jj];
+        }
+        __syncthreads();
+      }
     }
-    const double xn2 = block_sum(part, S.red);
-    const double xnorm = sqrt(xn2);
-    const double x0 = S.hv[k];
-    double bk = 0.0;
-    double alpha = 0.0;
-    if (xnorm > 0.0) {
-      alpha = (x0 >= 0.0) ? -xnorm : xnorm;
-      const double v0 = x0 - alpha;
-      const double vtv = xn2 - x0 * x0 + v0 * v0;
-      bk = (vtv > 0.0) ? 2.0 / vtv : 0.0;
-      __syncthreads();
-      if (tid == 0) S.hv[k] = v0;
-      __syncthreads();
-    }
-    if (tid == 0) {
-      beta[k] = bk;
-      vk0[k] = S.hv[k];
-    }
-    if (bk != 0.0) detq = -detq;
-    // apply H = I - bk v v^T to the trailing columns j > k
-    if (bk != 0.0) householder_apply(N, ld, M, k, k + 1, bk, S.hv, S.qred);
-    __syncthreads();
-    if (tid == 0) M[(size_t)k * ld + k] = (xnorm > 0.0) ? alpha : x0;
-    // downdate the trailing column norms
-    for (int j = k + 1 + tid; j < N; j += kThreads) {
-      if (cn[j] != 0.0) {
-        double t = fabs(M[(size_t)k * ld + j]) / cn[j];
-        t = fmax(0.0, (1.0 + t) * (1.0 - t));
-        const double r = cn[j] / cn0[j];
-        if (t * r * r <= tol3z) {
-          double acc = 0.0;
-          for (int i = k + 1; i < N; ++i) acc = fma(M[(size_t)i * ld + j], M[(size_t)i * ld + j], acc);
-          cn[j] = sqrt(acc);
-          cn0[j] = cn[j];
-        } else {
-          cn[j] *= sqrt(t);
+    if (act) {
+#pragma unroll
+      for (int q = 0; q < PW; ++q) y[q] = rneg(y[q]);
+      int i = r0 + g;
+      for (; i + 3 * G < N; i += 4 * G) {
+        T x[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) x[b] = A[(size_t)(i + b * G) * ld + j];
+        const T* l = Lp + (i - r0);
+#pragma unroll
+        for (int q = 0; q < PW; ++q)
+          if (q < nb) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) x[b] = rfma(l[q * ldp + b * G], y[q], x[b]);
+          }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          A[(size_t)(i + b * G) * ld + j] = x[b];
+          if (LIST && i + b * G >= r0 + nb) {
+            const float f = as_float(x[b]);
+            n2 = fmaf(f, f, n2);
+          }
+        }
+      }
+      for (; i < N; i += G) {
+        T x = A[(size_t)i * ld + j];
+        const T* l = Lp + (i - r0);
+#pragma unroll
+        for (int q = 0; q < PW; ++q)
+          if (q < nb) x = rfma(l[q * ldp], y[q], x);
+        A[(size_t)i * ld + j] = x;
+        if (LIST && i >= r0 + nb) {
+          const float f = as_float(x);
+          n2 = fmaf(f, f, n2);
         }
       }
     }
-    __syncthreads();
+    if (LIST) {
+      float* part = reinterpret_cast<float*>(S.qred);
+      if (act) part[g * cw + jj] = n2;
+      __syncthreads();
+      if (act && g == 0) {
+        for (int h = 1; h < G; ++h) n2 += part[h * cw + jj];
+        key[c0 + jj] = column_key(n2, lsc[j]);
+      }
+      __syncthreads();
+    }
   }
+  __syncthreads();
+}
+
+// Wp = Vp Tm (nb x nb, row stride kPanel)
+template <typename T>
+__device__ void panel_times_t(int rows, int ldp, int nb, const T* Vp, const T* Tm, T* Wp) {
+  const int q = threadIdx.x % kPanel;
+  if (q < nb)
+    for (int i = threadIdx.x / kPanel; i < rows; i += kThreads / kPanel) {
+      T a = from_zero<T>();
+      for (int j = 0; j < nb; ++j) a = rfma(Vp[j * ldp + i], Tm[j * kPanel + q], a);
+      Wp[q * ldp + i] = a;
+    }
+  __syncthreads();
+}
+
+// alpha = -sign(x_0) |x|, v_0 = x_0 - alpha and beta = 2 / v^T v from x_0 and |x|^2.
+template <typename T>
+__device__ __forceinline__ void reflector_scalars(T x0, T xn2, T& alpha, T& v0, T& beta) {
+  const T xn = rsqrt_of_sum(xn2);
+  alpha = is_neg(x0) ? xn : rneg(xn);
+  v0 = rsub(x0, alpha);
+  beta = quick_div(unit<T>(true), rfma(rabs(x0), xn, xn2));  // v^T v = 2 (|x|^2 + |x_0| |x|)
+}
+
+// T of the panel at hand, behind qr_blocked's other entries of S.qred.
+template <typename T>
+__device__ __forceinline__ T* panel_tri(const Smem& S) { return reinterpret_cast<T*>(S.qred) + 256; }
+
+// Pivoted Householder QR of M = X diag(dsc), X N x N, in panels: reflections act on rows
+// and commute with the column scales, so the factors are X's, R_M = R_X diag(dsc[perm]).
+// Columns do not move: perm[k] is the column at position k, R_kj sits at X[k][perm[j]],
+// reflector k's vector below row k of column perm[k] (its leading entry in vk0[k]).
+// tri[panel][kPanel][kPanel]: the triangular factors T of the panels' products H_0 .. H_{nb-1} =
+// 1 - V T V^T (compact WY, Schreiber & Van Loan 1989).  Returns det(Q) = (-1)^#reflectors.
+//
+// Pivoting: a panel takes the columns of largest remaining scaled norm, renewed from the
+// updated matrix, and orders them by their downdated norms while it is factorised: the
+// order of Businger and Golub's pivoting but for a column that overtakes a panel's
+// last ones within the panel.  (Sorting the columns once before an unpivoted
+// factorisation is cheaper still, but made the wrapped G's drift up to 3.5 times
+// larger: the first block of a chain has no graded scales to sort by.)
+//
+// A panel is factorised in shared memory, one reduction per column: the products of
+// the column with every column of the panel give its norm, the update's coefficients
+// and T's next column at once.  One warp forms the scalars and the next pivot (a warp's
+// FP64 instruction holds its scheduler's unit for 65 cycles; eight warps computing the
+// same square root and quotients cost most of a column before).  The rest of the matrix
+// is updated once per panel, from registers.
+template <typename T>
+__device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* vk0, T* tri, Smem& S) {
+  constexpr int pw = kPanel, RG = kThreads / pw, nwarp = kThreads / 32;
+  static_assert(32 / pw == nwarp, "one lane group of the scalar warp per warp's partial products");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = tid % pw, rg = tid / pw;
+  const int ldp = panel_ld(N);
+  T* Vp = reinterpret_cast<T*>(S.gemm);
+  T* Wp = Vp + pw * ldp;
+  T* red = reinterpret_cast<T*>(S.qred);        // [nwarp][pw] partial products
+  T* wq = red + nwarp * pw;                     // [pw] update coefficients of the columns to come
+  T* zq = wq + pw;                              // [2][pw] products with the earlier vectors
+  T* sc = zq + 2 * pw;                          // [2][2] leading entry of v, beta
+  T* Tm = panel_tri<T>(S);                      // [pw][pw], by panel column
+  float* key = reinterpret_cast<float*>(S.hv);  // [N] by position
+  float* lsc = key + N;                         // [N] by column
+  int* list = S.qinv;                           // [N] columns by position
+  int* rank = reinterpret_cast<int*>(S.spare);  // [N]
+  int* pos_of = S.ired + 16;                    // [pw] position in the panel of its columns (-1: to come)
+  int* next_p = S.ired;                         // [2] pivot of the next step
+  int detq = 1;
+  column_keys<T>(N, ld, X, dsc, key, lsc, S);
+  for (int j = tid; j < N; j += kThreads) list[j] = j;
+  __syncthreads();
+  for (int k0 = 0; k0 < N; k0 += pw) {
+    const int nb = (N - k0 < pw) ? N - k0 : pw, rows = N - k0;
+    // the panel's columns: the nb largest keys, in order; the others keep theirs
+    for (int t = tid; t < rows; t += kThreads) {
+      const float kt = key[k0 + t];
+      int r = 0;
+      for (int u = 0; u < rows; ++u) {
+        const float ku = key[k0 + u];
+        r += (ku > kt || (ku == kt && u < t)) ? 1 : 0;
+      }
+      rank[t] = r;
+    }
+    __syncthreads();
+    {
+      int at[9], cj[9];  // N <= 9 kThreads positions (the shared vectors allow fewer)
+      float kk[9];
+#pragma unroll
+      for (int b = 0; b < 9; ++b) {
+        const int t = tid + b * kThreads;
+        at[b] = -1;
+        if (t < rows) {
+          const int r = rank[t];
+          int idx = r;
+          if (r >= nb) {
+            idx = nb + t;
+            for (int u = 0; u < t; ++u) idx -= rank[u] < nb ? 1 : 0;
+          }
+          at[b] = k0 + idx;
+          cj[b] = list[k0 + t];
+          kk[b] = key[k0 + t];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int b = 0; b < 9; ++b)
+        if (at[b] >= 0) {
+          list[at[b]] = cj[b];
+          key[at[b]] = kk[b];
+        }
+      __syncthreads();
+    }
+    for (int e = tid; e < rows * pw; e += kThreads) {
+      const int r = e / pw, c = e - r * pw;
+      if (c < nb) Vp[c * ldp + r] = X[(size_t)(k0 + r) * ld + list[k0 + c]];
+    }
+    if (tid < pw * pw) Tm[tid] = from_zero<T>();
+    if (tid < 2 * pw) zq[tid] = from_zero<T>();
+    if (tid < pw) pos_of[tid] = -1;
+    if (tid == 0) next_p[0] = 0;  // the selection is in order
+    __syncthreads();
+    // squared norms of the panel's columns (warp 0, lane q), downdated step by step
+    T nrm2 = from_zero<T>();
+    const float lscq = (q < nb) ? lsc[list[k0 + q]] : 0.f;
+    auto over_groups = [](T v) {  // the sum over a warp's lanes of the same q
+#pragma unroll
+      for (int o = 16; o >= pw; o >>= 1) v = radd(v, shfl_xor(v, o));
+      return v;
+    };
+    {
+      T a = from_zero<T>();
+      if (q < nb)
+        for (int r = rg; r < rows; r += RG) a = rfma(Vp[q * ldp + r], Vp[q * ldp + r], a);
+      a = over_groups(a);
+      if (lane < pw) red[warp * pw + lane] = a;
+      __syncthreads();
+      if (warp == 0) nrm2 = over_groups(red[lane]);
+      __syncthreads();
+    }
+    for (int c = 0; c < nb; ++c) {
+      const int p = next_p[c & 1];
+      const T* x = Vp + p * ldp;
+      T a = from_zero<T>();
+      if (q < nb) {
+        const T* y = Vp + q * ldp;
+        for (int r = c + rg; r < rows; r += RG) a = rfma(x[r], y[r], a);
+      }
+      a = over_groups(a);
+      if (lane < pw) red[warp * pw + lane] = a;
+      __syncthreads();
+      if (warp == 0) {
+        const T t = over_groups(red[lane]);  // lane group w holds warp w's sums
+        const T xn2 = shfl(t, p);
+        const T x0 = x[c];
+        T alpha = x0, v0 = x0, beta = from_zero<T>();
+        if (is_pos(xn2)) reflector_scalars(x0, xn2, alpha, v0, beta);
+        // v_q^T v (earlier columns), v^T y_q (columns to come)
+        const int pq = pos_of[q];
+        const bool done = q >= nb || pq >= 0 || q == p;
+        const T yc = (q < nb) ? Vp[q * ldp + c] : from_zero<T>();
+        const T z = rfma(rneg(alpha), yc, t);
+        const T w = rneg(rmul(beta, z));
+        if (lane < pw) {
+          if (pq >= 0) zq[(c & 1) * pw + q] = z;
+          wq[q] = done ? from_zero<T>() : w;
+        }
+        // the next pivot: largest downdated norm among the columns to come
+        const T rc = rfma(w, v0, yc);
+        nrm2 = rfma(rneg(rc), rc, nrm2);
+        float k = done ? -3.5e38f : column_key(nrm2, lscq);
+        int kp = q;
+#pragma unroll
+        for (int o = pw / 2; o; o >>= 1) {
+          const float ok = __shfl_xor_sync(0xffffffffu, k, o);
+          const int op = __shfl_xor_sync(0xffffffffu, kp, o);
+          if (ok > k || (ok == k && op < kp)) { k = ok; kp = op; }
+        }
+        __syncwarp();
+        if (lane == 0) {
+          sc[(c & 1) * 2] = v0;
+          sc[(c & 1) * 2 + 1] = beta;
+          pos_of[p] = c;
+          next_p[(c & 1) ^ 1] = kp;
+          X[(size_t)(k0 + c) * ld + list[k0 + p]] = alpha;  // R's diagonal
+          vk0[k0 + c] = v0;
+        }
+      }
+      __syncthreads();
+      const T v0 = sc[(c & 1) * 2], beta = sc[(c & 1) * 2 + 1];
+      if (is_pos(beta)) detq = -detq;
+      if (q < nb && pos_of[q] < 0) {
+        const T w = wq[q];
+        T* y = Vp + q * ldp;
+        for (int r = c + rg; r < rows; r += RG) y[r] = rfma(w, (r == c) ? v0 : x[r], y[r]);
+      }
+      // T's next column (last warp): -beta T (V^T v) over the earlier ones, beta itself
+      if (warp == nwarp - 1 && lane < pw) {
+        T t = from_zero<T>();
+        for (int j = 0; j < nb; ++j) t = rfma(Tm[lane * pw + j], zq[(c & 1) * pw + j], t);
+        t = rneg(rmul(beta, t));
+        __syncwarp((1u << pw) - 1u);
+        Tm[lane * pw + p] = lane == p ? beta : t;
+      }
+      __syncthreads();
+      if (tid == 0) Vp[p * ldp + c] = v0;
+    }
+    __syncthreads();
+    // R's strict upper part and the vectors back to X; V gets its zeros above the diagonal
+    for (int e = tid; e < rows * pw; e += kThreads) {
+      const int r = e / pw, c = e - r * pw;
+      if (c < nb && r != pos_of[c]) X[(size_t)(k0 + r) * ld + list[k0 + c]] = Vp[c * ldp + r];
+    }
+    int col = 0, pc = 0;
+    if (q < nb) { col = list[k0 + q]; pc = pos_of[q]; }
+    const int tr = rg;  // row of T (threads below pw * pw)
+    const T tv = (tid < pw * pw) ? Tm[tid] : from_zero<T>();
+    __syncthreads();
+    // (a position is below kPanel, so one row per thread covers the zeros)
+    if (q < nb && rg < pc) Vp[q * ldp + rg] = from_zero<T>();
+    if (tid < nb) list[k0 + pc] = col;  // the panel's columns by position
+    // T by position: in global memory, or in place for a single panel
+    T* tg = N > pw ? tri + (size_t)(k0 / pw) * pw * pw : Tm;
+    if (tid < pw * pw && tr < nb && q < nb) tg[pos_of[tr] * pw + pc] = tv;
+    __syncthreads();
+    if (k0 + nb < N) {
+      panel_times_t<T>(rows, ldp, nb, Vp, Tm, Wp);
+      // Q^T A = A - V T^T V^T A = A - V (V T)^T A
+      panel_apply<T, false, true>(N, ld, X, k0, k0 + nb, nb, Vp, Wp, S, list, key, lsc);
+    }
+  }
+  for (int j = tid; j < N; j += kThreads) perm[j] = list[j];
+  __syncthreads();
   return detq;
 }
 
-// Q = H_0 H_1 ... H_{N-1} from the reflectors left in M by qr_pivoted.
-__device__ void form_q(int N, int ld, const double* M, const double* beta, const double* vk0, double* Q,
-                       Smem& S) {
+// Q = H_0 H_1 ... H_{N-1} from qr_blocked's vectors, panel by panel from the last:
+// Q A = A - (V T) (V^T A).
+template <typename T>
+__device__ void form_q_blk(int N, int ld, const T* X, const int* perm, const T* vk0, const T* tri, T* Q, Smem& S) {
   const int tid = threadIdx.x;
+  constexpr int pw = kPanel;
+  const int ldp = panel_ld(N);
+  T* Vp = reinterpret_cast<T*>(S.gemm);
+  T* Wp = Vp + pw * ldp;
   for (int e = tid; e < N * N; e += kThreads) {
     const int x = e / N, y = e - x * N;
-    Q[(size_t)x * ld + y] = (x == y) ? 1.0 : 0.0;
+    Q[(size_t)x * ld + y] = unit<T>(x == y);
   }
   __syncthreads();
-  for (int k = N - 1; k >= 0; --k) {
-    const double bk = beta[k];
-    if (bk == 0.0) continue;
-    for (int i = k + tid; i < N; i += kThreads) S.hv[i] = (i == k) ? vk0[k] : M[(size_t)i * ld + k];
+  for (int k0 = (N - 1) / pw * pw; k0 >= 0; k0 -= pw) {
+    const int nb = (N - k0 < pw) ? N - k0 : pw, rows = N - k0;
+    for (int e = tid; e < rows * pw; e += kThreads) {
+      const int r = e / pw, c = e - r * pw;
+      if (c < nb)
+        Vp[c * ldp + r] = r < c ? from_zero<T>() : r == c ? vk0[k0 + c] : X[(size_t)(k0 + r) * ld + perm[k0 + c]];
+    }
     __syncthreads();
-    householder_apply(N, ld, Q, k, k, bk, S.hv, S.qred);
+    panel_times_t<T>(rows, ldp, nb, Vp, N > pw ? tri + (size_t)(k0 / pw) * pw * pw : panel_tri<T>(S), Wp);
+    panel_apply<T, true, false>(N, ld, Q, k0, k0, nb, Vp, Wp, S, nullptr, nullptr, nullptr);
   }
 }
 
-// One step of a UDV chain (Sec. 2.3): X = Bcal Q_src, M = X D_src, M P = Q R,
-// D = |diag R|, T = D^-1 R P^T T_src.  Right chain (left == false): Bcal =
-// B_t2 ... B_t1+1.  Left chain: Bcal = B_t1+1^T ... B_t2^T.  Result in
-// (W2, wvec 0, W5); returns det(Q).
+// LU and solves of the middle matrix, blocked, templated on double and float
+// pairs.  On the mixed path they run in float pairs on the FP32 pipes: every
+// row of Mid has an entry of order one (for each i either Db_R,i = 1 or
+// Ds_R,i = 1, and likewise for the columns), so Mid, its LU factors and the
+// solution X = Mid^-1 Db_R^-1 Q_R^T stay inside the float range; entries that
+// underflow are below 1e-38 of their row and change G by less than that in
+// absolute value.
+//
+// Blocking: a panel of columns (or a block of rows of the right-hand sides) is
+// staged in shared memory and finished there; everything beyond it is updated by
+// one accumulate-GEMM.  Pivots are chosen on the top 32 bits of |a| (a pivot within
+// 2^-20 of the largest); one warp forms each pivot's reciprocal, log|det| is summed
+// once at the end.
+
+// C += A B (row-major, no transposes) on the register-tiled CTA products.
+__device__ __noinline__ void gemm_acc(int M, int Nc, int Kd, const double* A, int lda, const double* B, int ldb, double* C, int ldc,
+                                Smem& S) {
+  const int r = gemm_pick_r(M > Nc ? M : Nc);
+  if (r == 1) cta_gemm_r<double, false, false, 1, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  else if (r == 2) cta_gemm_r<double, false, false, 2, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  else if (r == 3) cta_gemm_r<double, false, false, 3, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  else if (r == 5) cta_gemm_r<double, false, false, 5, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+  else cta_gemm_r<double, false, false, 4, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
+}
+__device__ inline void gemm_acc(int M, int Nc, int Kd, const dd* A, int lda, const dd* B, int ldb, dd* C, int ldc,
+                                Smem& S) {
+  gemm_dd_tiles<false, false, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, reinterpret_cast<dd*>(S.gemm), S.dd_tile);
+}
+
+// order of |a| for the pivot search: its top 32 bits; -1 for NaN, 1 for what they miss
+__device__ __forceinline__ int pivot_key(double a) {
+  const int k = umma_mag(a);
+  return a != a ? -1 : (k == 0 && a != 0.0) ? 1 : k;
+}
+__device__ __forceinline__ int pivot_key(dd a) { return a.hi != a.hi ? -1 : umma_mag(a); }
+
+// P A = L U in place (unit L below the diagonal, rows interchanged whole); rowof[i] =
+// the row of A now at row i, diag[k] = 1 / U_kk.  tmp: 16 x N scratch (ld).  Returns 1
+// if a pivot column has no finite nonzero entry.
+template <typename T>
+__device__ int lu_factor_blk(int N, int ld, T* A, int* rowof, T* diag, T* tmp, double& logdet, int& sign, Smem& S) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int PB = panel_width(N, S), ldp = panel_ld(N);
+  T* P = reinterpret_cast<T*>(S.gemm);  // [PB][ldp], column-major
+  T* U = P + PB * ldp;                  // [PB][<= N] rows of U12
+  T* ud = reinterpret_cast<T*>(S.spare);  // [N] diagonal of U
+  int* piv = S.ired + 16;               // [16] the panel's interchanges
+  T* dinv_s = reinterpret_cast<T*>(S.xs + 6);
+  int sg = 1;
+  for (int i = tid; i < N; i += kThreads) rowof[i] = i;
+  for (int k0 = 0; k0 < N; k0 += PB) {
+    const int nb = (N - k0 < PB) ? N - k0 : PB, rows = N - k0, n2 = N - k0 - nb;
+    for (int e = tid; e < rows * nb; e += kThreads) {
+      const int r = e / nb, q = e - r * nb;
+      P[q * ldp + r] = A[(size_t)(k0 + r) * ld + k0 + q];
+    }
+    __syncthreads();
+    for (int c = 0; c < nb; ++c) {
+      int bk = -1, bi = rows;
+      for (int r = c + tid; r < rows; r += kThreads) {
+        const int k = pivot_key(P[c * ldp + r]);
+        if (k > bk) { bk = k; bi = r; }
+      }
+      const int wk = __reduce_max_sync(0xffffffffu, bk);
+      const int wi = __reduce_min_sync(0xffffffffu, bk == wk ? bi : rows);
+      if (lane == 0) { S.ired[warp] = wk; S.ired[8 + warp] = wi; }
+      __syncthreads();
+      int key = -1, p = rows;
+#pragma unroll
+      for (int w = 0; w < kThreads / 32; ++w) {
+        const int k = S.ired[w], i = S.ired[8 + w];
+        if (k > key || (k == key && i < p)) { key = k; p = i; }
+      }
+      if (key <= 0) return 1;
+      const T d = P[c * ldp + p];
+      if (p != c) sg = -sg;
+      if (is_neg(d)) sg = -sg;
+      __syncthreads();
+      if (warp == 0) {
+        if (lane == 0) {
+          *dinv_s = quick_div(unit<T>(true), d);
+          ud[k0 + c] = d;
+        }
+      } else if (warp == 1) {
+        if (lane == 0) piv[c] = p;
+        if (p != c) {
+          for (int q = lane; q < nb; q += 32) {
+            const T t = P[q * ldp + c];
+            P[q * ldp + c] = P[q * ldp + p];
+            P[q * ldp + p] = t;
+          }
+          if (lane == 0) {
+            const int t = rowof[k0 + c];
+            rowof[k0 + c] = rowof[k0 + p];
+            rowof[k0 + p] = t;
+          }
+        }
+      }
+      __syncthreads();
+      const T dinv = *dinv_s;
+      if (tid == 0) diag[k0 + c] = dinv;
+      for (int r = c + 1 + tid; r < rows; r += kThreads) {
+        const T l = rmul(P[c * ldp + r], dinv);
+        P[c * ldp + r] = l;
+        const T ml = rneg(l);
+        for (int q = c + 1; q < nb; ++q) P[q * ldp + r] = rfma(ml, P[q * ldp + c], P[q * ldp + r]);
+      }
+      __syncthreads();
+    }
+    for (int e = tid; e < rows * nb; e += kThreads) {
+      const int r = e / nb, q = e - r * nb;
+      A[(size_t)(k0 + r) * ld + k0 + q] = P[q * ldp + r];
+    }
+    // the panel's interchanges on the columns outside it (one thread per column)
+    for (int j = tid; j < N; j += kThreads) {
+      if (j >= k0 && j < k0 + nb) continue;
+      for (int c = 0; c < nb; ++c) {
+        const int p = k0 + piv[c];
+        if (p != k0 + c) {
+          const T t = A[(size_t)(k0 + c) * ld + j];
+          A[(size_t)(k0 + c) * ld + j] = A[(size_t)p * ld + j];
+          A[(size_t)p * ld + j] = t;
+        }
+      }
+    }
+    __syncthreads();
+    if (n2 > 0) {
+      // U12 = L11^-1 A12 column by column (L11 = P rows 0..nb-1)
+      for (int jj = tid; jj < n2; jj += kThreads) {
+        const int j = k0 + nb + jj;
+        for (int q = 0; q < nb; ++q) {
+          T u = A[(size_t)(k0 + q) * ld + j];
+          for (int p2 = 0; p2 < q; ++p2) u = rfma(rneg(P[p2 * ldp + q]), U[p2 * n2 + jj], u);
+          U[q * n2 + jj] = u;
+          A[(size_t)(k0 + q) * ld + j] = u;
+          tmp[(size_t)q * ld + jj] = rneg(u);
+        }
+      }
+      __syncthreads();
+      // A22 -= L21 U12
+      gemm_acc(rows - nb, n2, nb, A + (size_t)(k0 + nb) * ld + k0, ld, tmp, ld, A + (size_t)(k0 + nb) * ld + k0 + nb,
+               ld, S);
+    }
+  }
+  double lg = 0.0;
+  for (int k = tid; k < N; k += kThreads) lg += log(fabs(to_d(ud[k])));
+  logdet = block_sum(lg, S.red);
+  sign = sg;
+  return 0;
+}
+
+// Solve (LU) X = B for all N columns of B, B already in interchanged row order
+// (B <- X).  Blocks of PB rows are solved in shared memory, one thread per
+// column; the rows beyond a block are updated by one accumulate-GEMM.  tmp: PB x N.
+template <typename T>
+__device__ void lu_solve_blk(int N, int ld, const T* LU, const T* diag, T* B, T* tmp, Smem& S) {
+  const int tid = threadIdx.x;
+  const int PB = panel_width(N, S);
+  T* Y = reinterpret_cast<T*>(S.gemm);   // [PB][N] block of right-hand sides
+  T* Lb = Y + PB * N;                    // [PB][PB] diagonal block
+  for (int pass = 0; pass < 2; ++pass) {
+    const int nblk = (N + PB - 1) / PB;
+    for (int bi = 0; bi < nblk; ++bi) {
+      // forward: blocks top to bottom; backward: bottom to top
+      const int r0 = pass == 0 ? bi * PB : (nblk - 1 - bi) * PB;
+      const int nb = (N - r0 < PB) ? N - r0 : PB;
+      for (int e = tid; e < nb * nb; e += kThreads) {
+        const int q = e / nb, p2 = e - q * nb;
+        Lb[q * PB + p2] = rneg(LU[(size_t)(r0 + q) * ld + r0 + p2]);
+      }
+      for (int e = tid; e < nb * N; e += kThreads) {
+        const int q = e / N, j = e - q * N;
+        Y[q * N + j] = B[(size_t)(r0 + q) * ld + j];
+      }
+      __syncthreads();
+      for (int j = tid; j < N; j += kThreads) {
+        if (pass == 0) {
+          for (int q = 1; q < nb; ++q) {
+            T y = Y[q * N + j];
+            for (int p2 = 0; p2 < q; ++p2) y = rfma(Lb[q * PB + p2], Y[p2 * N + j], y);
+            Y[q * N + j] = y;
+          }
+        } else {
+          for (int q = nb - 1; q >= 0; --q) {
+            T y = Y[q * N + j];
+            for (int p2 = q + 1; p2 < nb; ++p2) y = rfma(Lb[q * PB + p2], Y[p2 * N + j], y);
+            Y[q * N + j] = rmul(y, diag[r0 + q]);
+          }
+        }
+        for (int q = 0; q < nb; ++q) {
+          const T y = Y[q * N + j];
+          B[(size_t)(r0 + q) * ld + j] = y;
+          tmp[(size_t)q * ld + j] = rneg(y);
+        }
+      }
+      __syncthreads();
+      if (pass == 0 && r0 + nb < N)
+        gemm_acc(N - r0 - nb, N, nb, LU + (size_t)(r0 + nb) * ld + r0, ld, tmp, ld, B + (size_t)(r0 + nb) * ld, ld, S);
+      if (pass == 1 && r0 > 0) gemm_acc(r0, N, nb, LU + r0, ld, tmp, ld, B, ld, S);
+    }
+  }
+}
+
+// The decomposition M = Q D T of M = X diag(src.D) src.T (X the product of a block of
+// slices with src.Q, in W0 or W1): pivoted QR of X, D = |diag R_M|,
+// T = D^-1 R_M P^T T_src with R_M,ij = R_X,ij dsc_j.  Result in (W2, wvec 0, W5), FP64;
+// returns det(Q).
+template <typename T>
+__device__ int udv_of_product(const ChainDev& C, int s, T* X, UDV src, Smem& S, long long* det, long long t0) {
+  const int N = C.N, ld = C.ld;
+  double* Dn = wvec(C, s, 0);
+  T* vk0 = reinterpret_cast<T*>(wvec(C, s, 2));
+  double* dsc = wvec(C, s, 5);
+  double* invr = wvec(C, s, 6);
+  int* perm = C.iwork[s];
+  T* tri = reinterpret_cast<T*>(wmat(C, s, 3));  // W3 and W4: about kPanel N entries
+  const int detq = qr_blocked<T>(N, ld, X, src.D, perm, vk0, tri, S);
+  T* Qn = reinterpret_cast<T*>(wmat(C, s, 2));
+  form_q_blk<T>(N, ld, X, perm, vk0, tri, Qn, S);
+  if constexpr (std::is_same<T, dd>::value) dd_to_d_inplace(N, ld, Qn);
+  tick(det, 5, t0);
+  T* PT = reinterpret_cast<T*>(wmat(C, s, 3));
+  T* Rt = reinterpret_cast<T*>(wmat(C, s, 4));
+  for (int x = threadIdx.x; x < N; x += kThreads) dsc[x] = src.D[perm[x]];
+  __syncthreads();  // src.D may be the vector that takes the new D
+  for (int x = threadIdx.x; x < N; x += kThreads) {
+    const double rkk = fabs(to_d(X[(size_t)x * ld + perm[x]]));
+    Dn[x] = rkk * dsc[x];
+    invr[x] = (rkk > 0.0 && dsc[x] > 0.0) ? 1.0 / (rkk * dsc[x]) : 0.0;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < N * N; e += kThreads) {
+    const int x = e / N, y = e - x * N;
+    PT[(size_t)x * ld + y] = from_d<T>(src.T[(size_t)perm[x] * ld + y]);
+    Rt[(size_t)x * ld + y] = y >= x ? rmul(X[(size_t)x * ld + perm[y]], from_d<T>(invr[x] * dsc[y])) : from_zero<T>();
+  }
+  __syncthreads();
+  T* Tn = reinterpret_cast<T*>(wmat(C, s, 5));
+  if constexpr (std::is_same<T, dd>::value) {
+    gemm_dd<false, false, false>(C, s, S, N, N, N, Rt, ld, PT, ld, Tn, ld);
+    dd_to_d_inplace(N, ld, Tn);
+  } else {
+    gemm_64<false, false>(S, N, N, N, Rt, ld, PT, ld, Tn, ld);
+  }
+  tick(det, 6, t0);
+  return detq;
+}
+
 // One-sided Jacobi SVD (Hestenes) of M = U S V^T, N x N in place: column
 // pairs of M are rotated until mutually orthogonal (|m_p . m_q| <= 1e-15
 // |m_p| |m_q| for every pair, at most 60 sweeps); then S_j = |m_j|, the
@@ -966,9 +1529,10 @@ __device__ void svd_jacobi(int N, int ld, double* M, double* V, double* Sv) {
   __syncthreads();
 }
 
-template <typename T>
-__device__ int lu_factor_blk(int N, int ld, T* A, int* piv, T* tmp, double& logdet, int& sign, Smem& S);
-
+// One step of a UDV chain (Sec. 2.3): X = Bcal Q_src, M = X D_src, M P = Q R,
+// D = |diag R|, T = D^-1 R P^T T_src.  Right chain (left == false): Bcal =
+// B_t2 ... B_t1+1.  Left chain: Bcal = B_t1+1^T ... B_t2^T.  Result in
+// (W2, wvec 0, W5); returns det(Q).
 __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, UDV src, Smem& S,
                                        long long* det = nullptr) {
   long long t0 = clock64();
@@ -1005,14 +1569,14 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
     }
   }
   tick(det, 4, t0);
-  // M = X D_src
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    X[(size_t)x * ld + y] *= src.D[y];
-  }
-  __syncthreads();
   double* Dn = wvec(C, s, 0);
   if (C.stab_svd) {
+    // M = X D_src
+    for (int e = threadIdx.x; e < N * N; e += kThreads) {
+      const int x = e / N, y = e - x * N;
+      X[(size_t)x * ld + y] *= src.D[y];
+    }
+    __syncthreads();
     // M = U S V^T: Q = U, D = S, T = V^T T_src, det Q from an LU of U
     double* V = Y;
     svd_jacobi(N, ld, X, V, Dn);
@@ -1026,222 +1590,13 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
     __syncthreads();
     double ldu;
     int detq = 1;
-    if (lu_factor_blk(N, ld, Ucp, C.iwork[s] + ld, wmat(C, s, 9), ldu, detq, S)) detq = 1;
+    if (lu_factor_blk(N, ld, Ucp, S.qinv, S.hv, wmat(C, s, 9), ldu, detq, S)) detq = 1;
     tick(det, 5, t0);
     gemm_64<true, false>(S, N, N, N, V, ld, src.T, ld, wmat(C, s, 5), ld);
     tick(det, 6, t0);
     return detq;
   }
-  double* beta = wvec(C, s, 1);
-  double* vk0 = wvec(C, s, 2);
-  int* perm = C.iwork[s];
-  const int detq = qr_pivoted(N, ld, X, beta, vk0, wvec(C, s, 3), wvec(C, s, 4), perm, S);
-  double* Qn = wmat(C, s, 2);
-  form_q(N, ld, X, beta, vk0, Qn, S);
-  tick(det, 5, t0);
-  double* PT = wmat(C, s, 3);
-  double* Rt = wmat(C, s, 4);
-  for (int x = threadIdx.x; x < N; x += kThreads) Dn[x] = fabs(X[(size_t)x * ld + x]);
-  __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    PT[(size_t)x * ld + y] = src.T[(size_t)perm[x] * ld + y];
-    Rt[(size_t)x * ld + y] = (y >= x && Dn[x] > 0.0) ? X[(size_t)x * ld + y] / Dn[x] : 0.0;
-  }
-  __syncthreads();
-  gemm_64<false, false>(S, N, N, N, Rt, ld, PT, ld, wmat(C, s, 5), ld);
-  tick(det, 6, t0);
-  return detq;
-}
-
-// LU and solves of the middle matrix, blocked, templated on double and float
-// pairs.  On the mixed path they run in float pairs on the FP32 pipes: every
-// row of Mid has an entry of order one (for each i either Db_R,i = 1 or
-// Ds_R,i = 1, and likewise for the columns), so Mid, its LU factors and the
-// solution X = Mid^-1 Db_R^-1 Q_R^T stay inside the float range; entries that
-// underflow are below 1e-38 of their row and change G by less than that in
-// absolute value.  Pivots are chosen on |hi + lo| in FP64 and divisions use the
-// FP64 reciprocal of the pivot.
-//
-// Blocking: a panel of PB columns (or a block of PB rows of the right-hand
-// sides) is staged in the shared GEMM buffer and finished there; everything
-// beyond it is updated by one accumulate-GEMM of depth PB.  PB is the largest
-// power of two <= 16 with PB (N + PB) elements fitting the buffer.
-__device__ inline int lu_block_width(int N) {
-  const int cap = 2 * 16 * kGemmMaxTile;
-  int pb = 16;
-  while (pb > 1 && pb * (N + pb) > cap) pb >>= 1;
-  return pb;
-}
-
-// C += A B (row-major, no transposes) on the register-tiled CTA products.
-__device__ __noinline__ void gemm_acc(int M, int Nc, int Kd, const double* A, int lda, const double* B, int ldb, double* C,
-                                int ldc, Smem& S) {
-  const int r = gemm_pick_r(M > Nc ? M : Nc);
-  if (r == 1) cta_gemm_r<double, false, false, 1, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
-  else if (r == 2) cta_gemm_r<double, false, false, 2, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
-  else if (r == 3) cta_gemm_r<double, false, false, 3, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
-  else if (r == 5) cta_gemm_r<double, false, false, 5, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
-  else cta_gemm_r<double, false, false, 4, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, S.gemm);
-}
-__device__ inline void gemm_acc(int M, int Nc, int Kd, const dd* A, int lda, const dd* B, int ldb, dd* C, int ldc,
-                                Smem& S) {
-  gemm_dd_tiles<false, false, true>(M, Nc, Kd, A, lda, B, ldb, C, ldc, reinterpret_cast<dd*>(S.gemm), S.dd_tile);
-}
-
-// P A = L U in place (unit L below the diagonal, rows interchanged whole);
-// piv[k] = row interchanged with row k.  tmp: PB x N scratch (ld).  Returns 1 if
-// a pivot column has no finite nonzero entry.
-template <typename T>
-__device__ int lu_factor_blk(int N, int ld, T* A, int* piv, T* tmp, double& logdet, int& sign, Smem& S) {
-  const int tid = threadIdx.x;
-  const int PB = lu_block_width(N);
-  T* P = reinterpret_cast<T*>(S.gemm);
-  double ld_ = 0.0;
-  int sg = 1;
-  for (int k0 = 0; k0 < N; k0 += PB) {
-    const int nb = (N - k0 < PB) ? N - k0 : PB, rows = N - k0, n2 = N - k0 - nb;
-    for (int e = tid; e < rows * nb; e += kThreads) {
-      const int r = e / nb, q = e - r * nb;
-      P[r * PB + q] = A[(size_t)(k0 + r) * ld + k0 + q];
-    }
-    __syncthreads();
-    for (int c = 0; c < nb; ++c) {
-      double bv = -1.0;
-      int bi = rows;
-      for (int r = c + tid; r < rows; r += kThreads) {
-        const double a = fabs(to_d(P[r * PB + c]));
-        if (a > bv) { bv = a; bi = r; }
-      }
-      const int p = block_argmax(bv, bi, S.red, S.ired);
-      if (p >= rows) return 1;
-      if (tid == 0) piv[k0 + c] = k0 + p;
-      const double pv = to_d(P[p * PB + c]);
-      if (!(pv != 0.0)) return 1;
-      if (p != c) {
-        for (int q = tid; q < nb; q += kThreads) {
-          const T t = P[c * PB + q];
-          P[c * PB + q] = P[p * PB + q];
-          P[p * PB + q] = t;
-        }
-        sg = -sg;
-      }
-      __syncthreads();
-      const double d = to_d(P[c * PB + c]);
-      ld_ += log(fabs(d));
-      if (d < 0.0) sg = -sg;
-      const T dinv = from_d<T>(1.0 / d);
-      for (int r = c + 1 + tid; r < rows; r += kThreads) {
-        const T l = rmul(P[r * PB + c], dinv);
-        P[r * PB + c] = l;
-        const T ml = rneg(l);
-        for (int q = c + 1; q < nb; ++q) P[r * PB + q] = rfma(ml, P[c * PB + q], P[r * PB + q]);
-      }
-      __syncthreads();
-    }
-    for (int e = tid; e < rows * nb; e += kThreads) {
-      const int r = e / nb, q = e - r * nb;
-      A[(size_t)(k0 + r) * ld + k0 + q] = P[r * PB + q];
-    }
-    // the panel's interchanges on the columns outside it (one thread per column)
-    for (int j = tid; j < N; j += kThreads) {
-      if (j >= k0 && j < k0 + nb) continue;
-      for (int c = 0; c < nb; ++c) {
-        const int p = piv[k0 + c];
-        if (p != k0 + c) {
-          const T t = A[(size_t)(k0 + c) * ld + j];
-          A[(size_t)(k0 + c) * ld + j] = A[(size_t)p * ld + j];
-          A[(size_t)p * ld + j] = t;
-        }
-      }
-    }
-    __syncthreads();
-    if (n2 > 0) {
-      // U12 = L11^-1 A12 column by column (L11 = P rows 0..nb-1, staging after it)
-      T* U = P + PB * PB;
-      for (int jj = tid; jj < n2; jj += kThreads) {
-        const int j = k0 + nb + jj;
-        for (int q = 0; q < nb; ++q) {
-          T u = A[(size_t)(k0 + q) * ld + j];
-          for (int p2 = 0; p2 < q; ++p2) u = rfma(rneg(P[q * PB + p2]), U[p2 * n2 + jj], u);
-          U[q * n2 + jj] = u;
-          A[(size_t)(k0 + q) * ld + j] = u;
-          tmp[(size_t)q * ld + jj] = rneg(u);
-        }
-      }
-      __syncthreads();
-      // A22 -= L21 U12
-      gemm_acc(rows - nb, n2, nb, A + (size_t)(k0 + nb) * ld + k0, ld, tmp, ld, A + (size_t)(k0 + nb) * ld + k0 + nb,
-               ld, S);
-    }
-  }
-  logdet = ld_;
-  sign = sg;
-  return 0;
-}
-
-// Solve (LU) X = B for all N columns of B, B already in interchanged row order
-// (B <- X).  Blocks of PB rows are solved in shared memory, one thread per
-// column; the rows beyond a block are updated by one accumulate-GEMM.  tmp: PB x N.
-template <typename T>
-__device__ void lu_solve_blk(int N, int ld, const T* LU, T* B, T* tmp, Smem& S) {
-  const int tid = threadIdx.x;
-  const int PB = lu_block_width(N);
-  T* Lb = reinterpret_cast<T*>(S.gemm);  // [PB][PB] diagonal block
-  T* Y = Lb + PB * PB;                   // [PB][N] block of right-hand sides
-  for (int pass = 0; pass < 2; ++pass) {
-    const int nblk = (N + PB - 1) / PB;
-    for (int bi = 0; bi < nblk; ++bi) {
-      // forward: blocks top to bottom; backward: bottom to top
-      const int r0 = pass == 0 ? bi * PB : (nblk - 1 - bi) * PB;
-      const int nb = (N - r0 < PB) ? N - r0 : PB;
-      for (int e = tid; e < nb * nb; e += kThreads) {
-        const int q = e / nb, p2 = e - q * nb;
-        Lb[q * PB + p2] = LU[(size_t)(r0 + q) * ld + r0 + p2];
-      }
-      for (int e = tid; e < nb * N; e += kThreads) {
-        const int q = e / N, j = e - q * N;
-        Y[q * N + j] = B[(size_t)(r0 + q) * ld + j];
-      }
-      __syncthreads();
-      for (int j = tid; j < N; j += kThreads) {
-        if (pass == 0) {
-          for (int q = 1; q < nb; ++q) {
-            T y = Y[q * N + j];
-            for (int p2 = 0; p2 < q; ++p2) y = rfma(rneg(Lb[q * PB + p2]), Y[p2 * N + j], y);
-            Y[q * N + j] = y;
-          }
-        } else {
-          for (int q = nb - 1; q >= 0; --q) {
-            T y = Y[q * N + j];
-            for (int p2 = q + 1; p2 < nb; ++p2) y = rfma(rneg(Lb[q * PB + p2]), Y[p2 * N + j], y);
-            Y[q * N + j] = rmul(y, from_d<T>(1.0 / to_d(Lb[q * PB + q])));
-          }
-        }
-        for (int q = 0; q < nb; ++q) {
-          const T y = Y[q * N + j];
-          B[(size_t)(r0 + q) * ld + j] = y;
-          tmp[(size_t)q * ld + j] = rneg(y);
-        }
-      }
-      __syncthreads();
-      if (pass == 0 && r0 + nb < N)
-        gemm_acc(N - r0 - nb, N, nb, LU + (size_t)(r0 + nb) * ld + r0, ld, tmp, ld, B + (size_t)(r0 + nb) * ld, ld, S);
-      if (pass == 1 && r0 > 0) gemm_acc(r0, N, nb, LU + r0, ld, tmp, ld, B, ld, S);
-    }
-  }
-}
-
-// Row map of the LU row interchanges: row i of P b is row rowof[i] of b.
-__device__ void lu_row_map(int N, const int* piv, int* rowof) {
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < N; ++i) rowof[i] = i;
-    for (int k = 0; k < N; ++k) {
-      const int p = piv[k];
-      const int t = rowof[k]; rowof[k] = rowof[p]; rowof[p] = t;
-    }
-  }
-  __syncthreads();
+  return udv_of_product<double>(C, s, X, src, S, det, t0);
 }
 
 // Stable G from a right chain R (B(tau,0) = Q_R D_R T_R) and a left chain Lf
@@ -1275,18 +1630,17 @@ __device__ int green_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, double* G
   __syncthreads();
   double ldm;
   int sm;
-  int* piv = C.iwork[s] + ld;
+  int* rowof = S.qinv;
+  double* udiag = S.hv;
   double* tmp = wmat(C, s, 9);
-  if (lu_factor_blk(N, ld, W0, piv, tmp, ldm, sm, S)) return 1;
-  int* rowof = C.iwork[s];
-  lu_row_map(N, piv, rowof);
+  if (lu_factor_blk(N, ld, W0, rowof, udiag, tmp, ldm, sm, S)) return 1;
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     const int r = rowof[i];
     W1[(size_t)i * ld + j] = R.Q[(size_t)j * ld + r] * ibR[r];
   }
   __syncthreads();
-  lu_solve_blk(N, ld, W0, W1, tmp, S);
+  lu_solve_blk(N, ld, W0, udiag, W1, tmp, S);
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     W1[(size_t)i * ld + j] *= ibL[i];
@@ -1884,256 +2238,11 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
   }
 }
 
-// ---- float-pair Householder QR with FP64 column scales (mixed path) -------
-// M = X diag(dsc) with X the float-pair product Bcal Q (entries O(1)) and dsc
-// the FP64 scales D of the previous decomposition, which may exceed the float
-// range.  Householder reflections act on rows and commute with the column
-// scaling, so the pivoted QR of M is the QR of X with the pivot chosen by the
-// scaled norm dsc_j ||X[k:, j]|| (Businger-Golub on M); R_M = R_X diag(dsc[perm]).
-__device__ void householder_apply_dd(int N, int ld, dd* M, int k, int j0, dd bk, const dd* hv, dd* qred) {
-  const int tid = threadIdx.x, lane = tid & 31, rg = tid >> 5;
-  for (int c0 = j0; c0 < N; c0 += 128) {
-    dd w[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    int i = k + rg;
-    for (; i + 24 < N; i += 32) {
-      dd x[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = c0 + lane + 32 * q;
-          x[r][q] = (j < N) ? M[(size_t)(i + 8 * r) * ld + j] : dd{0.f, 0.f};
-        }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const dd vi = hv[i + 8 * r];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[q] = dd_fma(vi, x[r][q], w[q]);
-      }
-    }
-    for (; i < N; i += 8) {
-      const dd vi = hv[i];
-      const dd* row = M + (size_t)i * ld;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = c0 + lane + 32 * q;
-        if (j < N) w[q] = dd_fma(vi, row[j], w[q]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) qred[rg * 128 + lane + 32 * q] = w[q];
-    __syncthreads();
-    dd wt[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      dd t = {0.f, 0.f};
-#pragma unroll
-      for (int r = 0; r < 8; ++r) t = dd_add(t, qred[r * 128 + lane + 32 * q]);
-      const dd bw = dd_mul(bk, t);
-      wt[q] = {-bw.hi, -bw.lo};
-    }
-    i = k + rg;
-    for (; i + 24 < N; i += 32) {
-      dd x[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = c0 + lane + 32 * q;
-          x[r][q] = (j < N) ? M[(size_t)(i + 8 * r) * ld + j] : dd{0.f, 0.f};
-        }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const dd vi = hv[i + 8 * r];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = c0 + lane + 32 * q;
-          if (j < N) M[(size_t)(i + 8 * r) * ld + j] = dd_fma(wt[q], vi, x[r][q]);
-        }
-      }
-    }
-    for (; i < N; i += 8) {
-      const dd vi = hv[i];
-      dd* row = M + (size_t)i * ld;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = c0 + lane + 32 * q;
-        if (j < N) row[j] = dd_fma(wt[q], vi, row[j]);
-      }
-    }
-    __syncthreads();
-  }
-}
-
-__device__ int qr_pivoted_dd(int N, int ld, dd* X, double* dsc, double* beta, dd* vk0, double* cn_g, double* cn0_g,
-                             int* perm_g, Smem& S) {
-  // Per-column state in shared memory (the sweep's slice buffers, idle during
-  // the stabilisation): norms cn / cn0, scales, pivot order, recompute list.
-  // The reflector's scalars are formed by thread 0 and broadcast; the norms are
-  // downdated with LAPACK's xGEQPF rule and those that cancel below its
-  // threshold are recomputed in FP64 by one warp each.
-  (void)cn_g;
-  (void)cn0_g;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  dd* hv = reinterpret_cast<dd*>(S.hv);
-  dd* qred = reinterpret_cast<dd*>(S.qred);
-  double* cn = S.d;
-  double* cn0 = S.xdiag;
-  double* sd = S.ev;
-  int* perm = S.qinv;
-  int* flag = reinterpret_cast<int*>(S.spare);
-  int* nflag = S.ired + 24;
-  double* sc = S.xs + 4;
-  for (int j = tid; j < N; j += kThreads) {
-    double acc = 0.0;
-    for (int i = 0; i < N; ++i) {
-      const double x = to_d(X[(size_t)i * ld + j]);
-      acc = fma(x, x, acc);
-    }
-    cn[j] = sqrt(acc);
-    cn0[j] = cn[j];
-    perm[j] = j;
-    sd[j] = dsc[j];
-  }
-  __syncthreads();
-  const double tol3z = sqrt(2.220446049250313e-16);
-  int detq = 1;
-  for (int k = 0; k < N; ++k) {
-    double bv = -1.0;
-    int bi = N;
-    for (int j = k + tid; j < N; j += kThreads) {
-      const double sn = sd[j] * cn[j];
-      if (sn > bv) { bv = sn; bi = j; }
-    }
-    int p = block_argmax(bv, bi, S.red, S.ired);
-    if (p >= N) p = k;
-    if (p != k) {
-      for (int i = tid; i < N; i += kThreads) {
-        const dd t = X[(size_t)i * ld + k];
-        X[(size_t)i * ld + k] = X[(size_t)i * ld + p];
-        X[(size_t)i * ld + p] = t;
-      }
-      if (tid == 0) {
-        const int tp = perm[k]; perm[k] = perm[p]; perm[p] = tp;
-        double t = cn[k]; cn[k] = cn[p]; cn[p] = t;
-        t = cn0[k]; cn0[k] = cn0[p]; cn0[p] = t;
-        t = sd[k]; sd[k] = sd[p]; sd[p] = t;
-      }
-      __syncthreads();
-    }
-    double part = 0.0;
-    for (int i = k + tid; i < N; i += kThreads) {
-      const dd x = X[(size_t)i * ld + k];
-      const double xd = to_d(x);
-      part = fma(xd, xd, part);
-      hv[i] = x;
-    }
-    const double xn2 = block_sum(part, S.red);
-    if (tid == 0) {
-      const double xnorm = sqrt(xn2);
-      const dd x0 = hv[k];
-      double bk = 0.0;
-      if (xnorm > 0.0) {
-        const double x0d = to_d(x0);
-        const double alpha = (x0d >= 0.0) ? -xnorm : xnorm;
-        const dd v0 = dd_add(x0, from_d<dd>(-alpha));
-        const double v0d = to_d(v0);
-        const double vtv = xn2 - x0d * x0d + v0d * v0d;
-        bk = (vtv > 0.0) ? 2.0 / vtv : 0.0;
-        hv[k] = v0;
-        X[(size_t)k * ld + k] = from_d<dd>(alpha);
-      }
-      beta[k] = bk;
-      vk0[k] = hv[k];
-      sc[0] = bk;
-      *nflag = 0;
-    }
-    __syncthreads();
-    const double bk = sc[0];
-    if (bk != 0.0) {
-      detq = -detq;
-      householder_apply_dd(N, ld, X, k, k + 1, from_d<dd>(bk), hv, qred);
-    }
-    for (int j = k + 1 + tid; j < N; j += kThreads) {
-      if (cn[j] != 0.0) {
-        double t = fabs(to_d(X[(size_t)k * ld + j])) / cn[j];
-        t = fmax(0.0, (1.0 + t) * (1.0 - t));
-        const double r = cn[j] / cn0[j];
-        if (t * r * r <= tol3z) flag[atomicAdd(nflag, 1)] = j;
-        else cn[j] *= sqrt(t);
-      }
-    }
-    __syncthreads();
-    const int nf = *nflag;
-    if (nf) {
-      for (int q = warp; q < nf; q += kThreads / 32) {
-        const int j = flag[q];
-        double acc = 0.0;
-        for (int i = k + 1 + lane; i < N; i += 32) {
-          const double x = to_d(X[(size_t)i * ld + j]);
-          acc = fma(x, x, acc);
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) {
-          cn[j] = sqrt(acc);
-          cn0[j] = cn[j];
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (int j = tid; j < N; j += kThreads) {
-    perm_g[j] = perm[j];
-    dsc[j] = sd[j];
-  }
-  __syncthreads();
-  return detq;
-}
-
-__device__ void form_q_dd(int N, int ld, const dd* X, const double* beta, const dd* vk0, dd* Q, Smem& S) {
-  const int tid = threadIdx.x;
-  dd* hv = reinterpret_cast<dd*>(S.hv);
-  dd* qred = reinterpret_cast<dd*>(S.qred);
-  for (int e = tid; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    Q[(size_t)x * ld + y] = {(x == y) ? 1.f : 0.f, 0.f};
-  }
-  __syncthreads();
-  for (int k = N - 1; k >= 0; --k) {
-    const double bk = beta[k];
-    if (bk == 0.0) continue;
-    for (int i = k + tid; i < N; i += kThreads) hv[i] = (i == k) ? vk0[k] : X[(size_t)i * ld + k];
-    __syncthreads();
-    householder_apply_dd(N, ld, Q, k, k, from_d<dd>(bk), hv, qred);
-  }
-}
-
 // ---- stabilisation with float-float products (mixed path) ----------------
 // Same steps as chain_step / green_from_udv; the dense products (the B chain,
 // T = D^-1 R P^T T, Q_R^T Q_L, T_R T_L^T, Q_L Y) run as float-float GEMMs on the
 // FP32 pipes, the pivoted QR, Q accumulation, LU and triangular solves stay
 // FP64.  Storage matrices (Q, T) remain FP64.
-__device__ inline void to_dd_mat(int N, int ld, const double* src, dd* dst) {
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    dst[(size_t)x * ld + y] = from_d<dd>(src[(size_t)x * ld + y]);
-  }
-  __syncthreads();
-}
-
-// dd -> double in place (same 8-byte slot)
-__device__ inline void dd_to_d_inplace(int N, int ld, void* buf) {
-  dd* a = reinterpret_cast<dd*>(buf);
-  double* b = reinterpret_cast<double*>(buf);
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    const dd v = a[(size_t)x * ld + y];
-    b[(size_t)x * ld + y] = to_d(v);
-  }
-  __syncthreads();
-}
-
 __device__ int chain_step_mixed(const ChainDev& C, int s, int t1, int t2, bool left, UDV src, Smem& S,
                                              long long* det = nullptr) {
   long long t0 = clock64();
@@ -2171,41 +2280,7 @@ __device__ int chain_step_mixed(const ChainDev& C, int s, int t1, int t2, bool l
     }
   }
   tick(det, 4, t0);
-  double* Dn = wvec(C, s, 0);
-  double* beta = wvec(C, s, 1);
-  dd* vk0 = reinterpret_cast<dd*>(wvec(C, s, 2));
-  double* dsc = wvec(C, s, 5);
-  double* invr = wvec(C, s, 6);
-  int* perm = C.iwork[s];
-  for (int j = threadIdx.x; j < N; j += kThreads) dsc[j] = src.D[j];
-  __syncthreads();
-  const int detq = qr_pivoted_dd(N, ld, X, dsc, beta, vk0, wvec(C, s, 3), wvec(C, s, 4), perm, S);
-  dd* Qd = reinterpret_cast<dd*>(wmat(C, s, 2));
-  form_q_dd(N, ld, X, beta, vk0, Qd, S);
-  dd_to_d_inplace(N, ld, Qd);
-  tick(det, 5, t0);
-  dd* PT = reinterpret_cast<dd*>(wmat(C, s, 3));
-  dd* Rt = reinterpret_cast<dd*>(wmat(C, s, 4));
-  // D = |diag R_M| = |R_X,kk| dsc_k;  R~_ij = R_X,ij dsc_j / (|R_X,ii| dsc_i), |R~_ij| <= 1
-  for (int x = threadIdx.x; x < N; x += kThreads) {
-    const double rkk = fabs(to_d(X[(size_t)x * ld + x]));
-    Dn[x] = rkk * dsc[x];
-    invr[x] = (rkk > 0.0 && dsc[x] > 0.0) ? 1.0 / (rkk * dsc[x]) : 0.0;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    PT[(size_t)x * ld + y] = from_d<dd>(src.T[(size_t)perm[x] * ld + y]);
-    dd r = {0.f, 0.f};
-    if (y >= x) r = dd_mul(X[(size_t)x * ld + y], from_d<dd>(invr[x] * dsc[y]));
-    Rt[(size_t)x * ld + y] = r;
-  }
-  __syncthreads();
-  dd* Tn = reinterpret_cast<dd*>(wmat(C, s, 5));
-  gemm_dd<false, false, false>(C, s, S, N, N, N, Rt, ld, PT, ld, Tn, ld);
-  dd_to_d_inplace(N, ld, Tn);
-  tick(det, 6, t0);
-  return detq;
+  return udv_of_product<dd>(C, s, X, src, S, det, t0);
 }
 
 __device__ int green_from_udv_mixed(const ChainDev& C, int s, UDV R, UDV Lf, double* Gout, double& logdet,
@@ -2242,19 +2317,18 @@ __device__ int green_from_udv_mixed(const ChainDev& C, int s, UDV R, UDV Lf, dou
   __syncthreads();
   double ldm;
   int smi;
-  int* piv = C.iwork[s] + ld;
+  int* rowof = S.qinv;
+  dd* udiag = reinterpret_cast<dd*>(S.hv);
   dd* tmpd = reinterpret_cast<dd*>(wmat(C, s, 9));
-  if (lu_factor_blk(N, ld, W0d, piv, tmpd, ldm, smi, S)) return 1;
+  if (lu_factor_blk(N, ld, W0d, rowof, udiag, tmpd, ldm, smi, S)) return 1;
   // right-hand side Db_R^-1 Q_R^T with the LU row interchanges applied
-  int* rowof = C.iwork[s];
-  lu_row_map(N, piv, rowof);
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     const int r = rowof[i];
     W1d[(size_t)i * ld + j] = from_d<dd>(R.Q[(size_t)j * ld + r] * ibR[r]);
   }
   __syncthreads();
-  lu_solve_blk(N, ld, W0d, W1d, tmpd, S);
+  lu_solve_blk(N, ld, W0d, udiag, W1d, tmpd, S);
   dd* Yd = reinterpret_cast<dd*>(wmat(C, s, 9));
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
@@ -2556,17 +2630,16 @@ __device__ int displaced_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, doubl
   __syncthreads();
   double ldm;
   int smi;
-  int* piv = C.iwork[s] + ld;
+  int* rowof = S.qinv;
+  double* udiag = S.hv;
   double* tmp = wmat(C, s, 9);
-  if (lu_factor_blk(N, ld, W0, piv, tmp, ldm, smi, S)) return 1;
-  int* rowof = C.iwork[s];
-  lu_row_map(N, piv, rowof);
+  if (lu_factor_blk(N, ld, W0, rowof, udiag, tmp, ldm, smi, S)) return 1;
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     W1[(size_t)i * ld + j] = (rowof[i] == j) ? 1.0 : 0.0;
   }
   __syncthreads();
-  lu_solve_blk(N, ld, W0, W1, tmp, S);  // W1 = Mid^-1
+  lu_solve_blk(N, ld, W0, udiag, W1, tmp, S);  // W1 = Mid^-1
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     const double m = W1[(size_t)i * ld + j];
