@@ -1936,11 +1936,13 @@ __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const d
 // Decisions: the acceptances of a window depend on G only through its kWin x kWin
 // block on the window's sites, for both flavors.  Each CTA publishes its flavor's
 // block of the effective G once per window; then both CTAs run the same chain of
-// decisions on both blocks, kept in registers and updated by a rank-1 step per
+// decisions on both blocks in shared memory, updated by a rank-1 step per
 // acceptance, so the flavors meet once per window instead of once per
 // acceptance.  The first acceptance in visiting order is found by a ballot over
 // the remaining positions' ratios, which is exactly the sequential Metropolis
-// chain because rejected proposals leave G unchanged.
+// chain because rejected proposals leave G unchanged.  One warp per flavor follows
+// the chain (the ratios of all lanes are renewed from the accepted flip's vectors
+// alone, so it finds the next acceptance while the other warps renew the blocks).
 // Vectors: afterwards the accepted flips' delayed vectors
 //   a = -(delta/R_s) G_eff[:,i],  b = e_i - G_eff[i,:],  G_eff += a b^T
 // are formed for all N sites at once, each thread carrying kVecChunk flips'
@@ -1949,28 +1951,25 @@ __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const d
 // decisions).  They are flushed into G every delay_k acceptances.
 //
 // The bound is the serial chain per acceptance and the FP64 unit (a warp's FP64
-// instruction holds its scheduler's unit for 65 cycles): one warp per flavor
-// updates the ratios, in float pairs where G is.  Decisions and vectors of one
-// acceptance, measured on GB300: 12x12 float pairs, two CTAs per SM, 2.6 us (5.7 us
-// when every warp evaluated all N ratios and vectors between two cluster barriers
-// per acceptance); 8x8 float pairs 2.4 us (5.6); N = 72 FP64 2.35 us (2.85).
+// instruction holds its scheduler's unit for 65 cycles).  Per acceptance on GB300, one
+// CTA per SM, N = 64: the decisions 1130 cycles in float pairs and 2460 in FP64, the
+// vectors 580 and 920, the window's exchange 240; two cluster barriers, FP64 ratios,
+// quotients and vectors of all N sites by every warp took 11000 and 5900.
 constexpr int kWin = 32;       // positions per window: one warp lane each
 constexpr int kWinAcc = 16;    // acceptances per window (the vectors' shared memory)
 constexpr int kVecChunk = 8;   // flips whose vectors one thread forms together
+constexpr int kWinLd = kWin + 1;  // row stride of a block: rows and columns without bank conflicts
 
 // Shared memory of a window: the idle product panels (S.gemm) and the QR's
 // partial sums (S.qred).
 template <typename Real>
 struct Window {
   using Ratio = typename RatioOf<Real>::type;
-  Real* E;        // [kWin][kWin] this flavor's block of the effective G
-  Ratio* d;       // [kWin] its diagonal
+  Real* E;        // [kMaxFlavors][kWin][kWinLd] the flavors' blocks of the effective G
+  Ratio* d;       // [kWin] this flavor's diagonal
   Ratio* del;     // [kWin] exp(dv) - 1 of this flavor
   Ratio* Rs;      // [kMaxFlavors][kWin] ratios
-  Ratio* dl;      // [kMaxFlavors][kWin] deltas of both flavors
-  Real* col;      // [kMaxFlavors][kWin] column of the accepted site
-  Real* row;      // [kMaxFlavors][kWin] its row
-  Real* a;        // [kMaxFlavors][kWin] its delayed vectors on the window
+  Real* a;        // [kMaxFlavors][kWin] the accepted site's delayed vectors on the window
   Real* b;
   Real* mfa;      // [kWinAcc] this flavor's -(delta/R_s) per acceptance
   int* ctl;       // [2] accepted position in the window (-1: none), R < 0
@@ -1982,17 +1981,14 @@ template <typename Real>
 __device__ __forceinline__ Window<Real> window_of(const Smem& S) {
   Window<Real> w;
   double* p = S.gemm;
-  constexpr int blk = kWin * kWin;
-  static_assert((blk + 2 * kWin + 2 * kMaxFlavors * kWin + 4 * kMaxFlavors * kWin + 2 * kWinAcc + 1) * 8 <=
-                kGemmRegionBytes, "the window's block fits the product panels");
+  constexpr int blk = kMaxFlavors * kWin * kWinLd;
+  static_assert((blk + 2 * kWin + 3 * kMaxFlavors * kWin + 2 * kWinAcc + 1) * 8 <= kGemmRegionBytes,
+                "the window's blocks fit the product panels");
   w.E = reinterpret_cast<Real*>(p); p += blk;
   using Ratio = typename RatioOf<Real>::type;
   w.d = reinterpret_cast<Ratio*>(p); p += kWin;
   w.del = reinterpret_cast<Ratio*>(p); p += kWin;
   w.Rs = reinterpret_cast<Ratio*>(p); p += kMaxFlavors * kWin;
-  w.dl = reinterpret_cast<Ratio*>(p); p += kMaxFlavors * kWin;
-  w.col = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
-  w.row = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
   w.a = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
   w.b = reinterpret_cast<Real*>(p); p += kMaxFlavors * kWin;
   w.mfa = reinterpret_cast<Real*>(p); p += kWinAcc;
@@ -2047,7 +2043,6 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
                              cg::cluster_group& cl, Real* G, Real* A, Real* B, int& sign, long long* det) {
   using Ratio = typename RatioOf<Real>::type;
   const int N = C.N, ld = C.ld, MV = C.MV, nfl = C.nfl, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kRows = kWin / (kThreads / 32);  // window rows per warp: warp + 8 j
   long long t0 = clock64();
   const uint32_t key0 = (uint32_t)P.seed, key1 = (uint32_t)(P.seed >> 32) ^ C.chain_id;
   Ratio* diag = reinterpret_cast<Ratio*>(S.d);
@@ -2086,112 +2081,108 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
     // ---- this flavor's block of the effective G, published to the peer
     {
       const int ic = S.qsite[pos + (lane < W ? lane : 0)];
+      Real e[kWin / 8];
+      int ir[kWin / 8];
 #pragma unroll
-      for (int j = 0; j < kRows; ++j) {
+      for (int j = 0; j < kWin / 8; ++j) {
         const int r = warp + 8 * j;
-        const int ir = S.qsite[pos + (r < W ? r : 0)];
-        Real e = G[(size_t)ir * ld + ic];
-        for (int m = 0; m < nacc; ++m) e = rfma(A[(size_t)m * ld + ir], B[(size_t)m * ld + ic], e);
-        w.E[r * kWin + lane] = e;
+        ir[j] = S.qsite[pos + (r < W ? r : 0)];
+        e[j] = G[(size_t)ir[j] * ld + ic];
       }
+      for (int m = 0; m < nacc; ++m) {
+        const Real bm = B[(size_t)m * ld + ic];
+#pragma unroll
+        for (int j = 0; j < kWin / 8; ++j) e[j] = rfma(A[(size_t)m * ld + ir[j]], bm, e[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < kWin / 8; ++j) w.E[(s * kWin + warp + 8 * j) * kWinLd + lane] = e[j];
       if (warp == 0) {
         w.d[lane] = diag[ic];
         w.del[lane] = delta_q[pos + (lane < W ? lane : 0)];
       }
     }
     cl.sync();
-    Real e[kMaxFlavors][kRows];
     Ratio dw = one, delw = one;  // warp r: diagonal and delta of flavor r
+    for (int r = 0; r < nfl; ++r) {
+      if (r != s) {
+        const Real* pe = cl.map_shared_rank(w.E, r) + r * kWin * kWinLd;
+        Real* me = w.E + r * kWin * kWinLd;
 #pragma unroll
-    for (int r = 0; r < kMaxFlavors; ++r) {
-      const bool live = r < nfl;
-      const Real* pe = (!live || r == s) ? w.E : cl.map_shared_rank(w.E, r);
-#pragma unroll
-      for (int j = 0; j < kRows; ++j) e[r][j] = pe[(warp + 8 * j) * kWin + lane];
-      if (live && warp == r) {
+        for (int j = 0; j < kWin / 8; ++j) me[(warp + 8 * j) * kWinLd + lane] = pe[(warp + 8 * j) * kWinLd + lane];
+      }
+      if (warp == r) {
         dw = ((r == s) ? w.d : cl.map_shared_rank(w.d, r))[lane];
         delw = ((r == s) ? w.del : cl.map_shared_rank(w.del, r))[lane];
-        w.dl[r * kWin + lane] = delw;
         w.Rs[r * kWin + lane] = rfma(delw, rsub(one, dw), one);
       }
     }
-    cl.sync();  // the peer has read this block; both flavors' ratios are in place
+    cl.sync();  // the peer has read this block; both flavors' blocks and ratios are in place
     const Ratio u2 = u2_q[pos + (lane < W ? lane : 0)], gam = gam_q[pos + (lane < W ? lane : 0)];
     const bool weighted = C.ft != 1;  // Ising fields: gamma = 1
     int last = -1, na = 0;
     // ---- decisions
     while (true) {
-      if (warp == 0) {
-        Ratio R = w.Rs[lane];
+      // the flavors' warps: the next acceptance (both find the same) and its factor
+      Real mf = unit<Real>(false);
+      int f = -1;
+      if (warp < nfl) {
+        const Ratio Rw = w.Rs[warp * kWin + lane];
+        Ratio R = (warp == 0) ? Rw : w.Rs[lane];
         if (weighted) R = rmul(gam, R);
-        if (nfl == 2) R = rmul(R, w.Rs[kWin + lane]);
+        if (nfl == 2) R = rmul(R, (warp == 1) ? Rw : w.Rs[kWin + lane]);
         const bool ok = lane > last && lane < W && accepts(u2, R);
         const unsigned m = __ballot_sync(0xffffffffu, ok);
-        const int f = m ? __ffs(m) - 1 : -1;
-        if (lane == (m ? f : 0)) {
+        f = m ? __ffs(m) - 1 : -1;
+        const unsigned negs = __ballot_sync(0xffffffffu, is_neg(R));
+        if (warp == 0 && lane == 0) {
           w.ctl[0] = f;
-          w.ctl[1] = is_neg(R);
+          w.ctl[1] = f >= 0 ? (int)((negs >> f) & 1u) : 0;
+        }
+        if (f >= 0) {
+          // every lane the accepted position's quotient
+          const Ratio df = shfl(delw, f), Rf = shfl(Rw, f);
+          mf = rneg(ratio_to<Real>(quick_div(df, Rf)));
+        }
+      } else if (last >= 0) {
+        // the other warps meanwhile: the rows after the last acceptance of both blocks
+        for (int r = 0; r < nfl; ++r) {
+          const Real bc = w.b[r * kWin + lane];
+          Real* blk = w.E + r * kWin * kWinLd + lane;
+#pragma unroll
+          for (int j = 0; j < 6; ++j) {
+            const int row = last + 1 + (warp - 2) + 6 * j;
+            if (row < kWin) blk[row * kWinLd] = rfma(w.a[r * kWin + row], bc, blk[row * kWinLd]);
+          }
         }
       }
       __syncthreads();
-      const int f = w.ctl[0];
+      if (warp >= nfl) f = w.ctl[0];
       if (f < 0) break;
       if (w.ctl[1]) sign = -sign;
-      // column f (every warp its rows) and row f (its warp) of both blocks
-      if (lane == f) {
-#pragma unroll
-        for (int r = 0; r < kMaxFlavors; ++r)
-#pragma unroll
-          for (int j = 0; j < kRows; ++j)
-            if (r < nfl) w.col[r * kWin + warp + 8 * j] = e[r][j];
-      }
-      if (warp == (f & 7)) {
-#pragma unroll
-        for (int r = 0; r < kMaxFlavors; ++r)
-#pragma unroll
-          for (int j = 0; j < kRows; ++j)
-            if (r < nfl && j == (f >> 3)) w.row[r * kWin + lane] = e[r][j];
-      }
-      // every lane of the flavor's warp divides for itself
-      Real mf = unit<Real>(false);
       if (warp < nfl) {
-        const Ratio fac = quick_div(w.dl[warp * kWin + f], w.Rs[warp * kWin + f]);
-        mf = rneg(ratio_to<Real>(fac));
-        if (warp == s && lane == 0) {
-          w.mfa[na] = mf;
-          w.at[na] = f;
-        }
-      }
-      if (tid == 64) {
-        const int q = pos + f;
-        S.fslice[dir ? MV - 1 - q : q] = S.fnew[q];
-      }
-      __syncthreads();
-      if (warp < nfl) {
-        const Real ax = rmul(mf, w.col[warp * kWin + lane]);
-        const Real bx = rsub(unit<Real>(lane == f), w.row[warp * kWin + lane]);
+        const Real* blk = w.E + warp * kWin * kWinLd;
+        const Real ax = rmul(mf, blk[lane * kWinLd + f]);
+        const Real bx = rsub(unit<Real>(lane == f), blk[f * kWinLd + lane]);
         w.a[warp * kWin + lane] = ax;
         w.b[warp * kWin + lane] = bx;
         if (warp == s) {
           w.sA[na * kWin + lane] = ax;
           w.sB[na * kWin + lane] = bx;
+          if (lane == 0) {
+            w.mfa[na] = mf;
+            w.at[na] = f;
+          }
         }
         dw = rfma(to_ratio(ax, Ratio()), to_ratio(bx, Ratio()), dw);
         w.Rs[warp * kWin + lane] = rfma(delw, rsub(one, dw), one);
+      } else if (tid == 64) {
+        const int q = pos + f;
+        S.fslice[dir ? MV - 1 - q : q] = S.fnew[q];
       }
       last = f;
       ++na;
       __syncthreads();
       if (na == kWinAcc || nacc + na == kdel) break;
-      // the rows after f of both blocks (earlier ones are not read again)
-#pragma unroll
-      for (int r = 0; r < kMaxFlavors; ++r) {
-        if (r >= nfl) continue;
-        const Real bc = w.b[r * kWin + lane];
-#pragma unroll
-        for (int j = 0; j < kRows; ++j)
-          if (warp + 8 * j > f) e[r][j] = rfma(w.a[r * kWin + warp + 8 * j], bc, e[r][j]);
-      }
     }
     // a window that stopped at its limit goes on behind its last acceptance
     const int next = (na == kWinAcc || nacc + na == kdel) ? pos + last + 1 : pos + W;
