@@ -85,6 +85,36 @@ __device__ __forceinline__ double2 block_zsum(double2 v, double* red) {
   return make_double2(re, im);
 }
 
+// a / b without the scaling of zdiv, for |b| of order one (ratios, pivots of Mid)
+__device__ __forceinline__ double2 zdiv_unit(double2 a, double2 b) {
+  return zscal(quick_div(1.0, zabs2(b)), zmul(a, zconj(b)));
+}
+// |a| where the squares neither overflow nor vanish
+__device__ __forceinline__ double zabs_unit(double2 a) { return sqrt(zabs2(a)); }
+
+// A warp's FP64 instruction holds its scheduler's FP64 unit for 65 cycles whatever its
+// active lanes: scalars that all threads need (reflector norms, pivots' inverses,
+// update factors) are formed by one warp and passed through shared memory, pivot
+// searches compare the top 32 bits as integers, and logarithms and arguments are
+// taken once per column after the elimination instead of by every thread in it.
+
+// Position of the largest key over the block (ties to the lowest index; N if none).
+__device__ __forceinline__ int block_argmax_key(int key, int idx, int N, int* ired) {
+  const int wk = __reduce_max_sync(0xffffffffu, key);
+  const int wi = __reduce_min_sync(0xffffffffu, key == wk ? idx : N);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) { ired[threadIdx.x >> 5] = wk; ired[8 + (threadIdx.x >> 5)] = wi; }
+  __syncthreads();
+  int bk = -1, bi = N;
+#pragma unroll
+  for (int w = 0; w < kThreads / 32; ++w)
+    if (ired[w] > bk || (ired[w] == bk && ired[8 + w] < bi)) { bk = ired[w]; bi = ired[8 + w]; }
+  return bk < 0 ? N : bi;
+}
+// order of a nonnegative number / of a complex pivot's larger component (NaN: -1)
+__device__ __forceinline__ int top_bits(double x) { return x != x ? -1 : __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int pivot_key(double2 a) { return max(pivot_key(a.x), pivot_key(a.y)); }
+
 // ---- shared memory of a chain's CTA ----------------------------------------
 constexpr int kZgTile = 32;  // C tile of the complex products
 constexpr int kZgK = 16;     // K step
@@ -107,12 +137,13 @@ struct Sm {
   int* first;           // [1] first accepted position of a scan
   int8_t* fsl;          // [MV] fields of the current slice (sites, then bonds)
   int8_t* fn;           // [N] proposed fields
+  double2* tab;         // [2] exp(i g eta(l)) for l = 1, 2 (conjugate for -1, -2)
 };
 
 __host__ __device__ inline size_t su2_smem_layout(int N, int MV) {
   return (size_t)kZgBytes + (size_t)8 * N * sizeof(double2) + 256 * sizeof(double2) + (size_t)N * sizeof(double) +
          32 * sizeof(double) + 32 * sizeof(int) + 16 /* alignment */ + sizeof(double2) + 16 +
-         (size_t)((MV + 15) / 16 * 16) + (size_t)((N + 15) / 16 * 16);
+         (size_t)((MV + 15) / 16 * 16) + (size_t)((N + 15) / 16 * 16) + 2 * sizeof(double2);
 }
 
 __device__ inline Sm su2_carve(unsigned char* base, int N, int MV) {
@@ -133,6 +164,7 @@ __device__ inline Sm su2_carve(unsigned char* base, int N, int MV) {
   s.ired = reinterpret_cast<int*>(q); q += 32 * sizeof(int);
   q = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(q) + 15) & ~(uintptr_t)15);
   s.P = reinterpret_cast<double2*>(q); q += sizeof(double2);
+  s.tab = reinterpret_cast<double2*>(q); q += 2 * sizeof(double2);
   s.first = reinterpret_cast<int*>(q); q += 16;
   s.fsl = reinterpret_cast<int8_t*>(q); q += (size_t)((MV + 15) / 16 * 16);
   s.fn = reinterpret_cast<int8_t*>(q);
@@ -144,9 +176,48 @@ __device__ inline Sm su2_carve(unsigned char* base, int N, int MV) {
 // is, 1 transpose, 2 conjugate transpose; A and B real (double) or complex
 // (double2).  Tiles of 32 x 32 outputs, 2 x 2 per thread, K in steps of 16
 // staged in shared memory.  C must not alias A or B.
+// Matrices of up to 16 x 16: one output per thread, a 32 x 32 tile would leave three
+// quarters of the FP64 pipe's work to padding.
+template <int OPA, int OPB, bool ACC, typename TA, typename TB>
+__device__ void zgemm16(int M, int Nc, int Kd, const TA* A, int lda, const TB* B, int ldb, double2* C, int ldc,
+                        unsigned char* smem) {
+  TA* As = reinterpret_cast<TA*>(smem);                                           // [16][17] (k, m)
+  TB* Bs = reinterpret_cast<TB*>(smem + kZgK * (kZgTile + 1) * sizeof(double2));  // [16][17] (k, n)
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  double2 acc = make_double2(0.0, 0.0);
+  for (int k0 = 0; k0 < Kd; k0 += 16) {
+    {
+      const int mm = (OPA == 0) ? ty : tx, kk = (OPA == 0) ? tx : ty, gk = k0 + kk;
+      TA v = zzero<TA>();
+      if (mm < M && gk < Kd) v = (OPA == 0) ? A[(size_t)mm * lda + gk] : zop<OPA>(A[(size_t)gk * lda + mm]);
+      As[kk * 17 + mm] = v;
+    }
+    {
+      const int nn = (OPB == 0) ? tx : ty, kk = (OPB == 0) ? ty : tx, gk = k0 + kk;
+      TB v = zzero<TB>();
+      if (nn < Nc && gk < Kd) v = (OPB == 0) ? B[(size_t)gk * ldb + nn] : zop<OPB>(B[(size_t)nn * ldb + gk]);
+      Bs[kk * 17 + nn] = v;
+    }
+    __syncthreads();
+    const int ke = Kd - k0 < 16 ? Kd - k0 : 16;
+#pragma unroll 4
+    for (int kk = 0; kk < ke; ++kk) acc = zmac(acc, As[kk * 17 + ty], Bs[kk * 17 + tx]);
+    __syncthreads();
+  }
+  if (ty < M && tx < Nc) {
+    double2* cp = C + (size_t)ty * ldc + tx;
+    *cp = ACC ? zadd(*cp, acc) : acc;
+  }
+  __syncthreads();
+}
+
 template <int OPA, int OPB, bool ACC, typename TA, typename TB>
 __device__ void zgemm(int M, int Nc, int Kd, const TA* A, int lda, const TB* B, int ldb, double2* C, int ldc,
                       unsigned char* smem) {
+  if (M <= 16 && Nc <= 16) {
+    zgemm16<OPA, OPB, ACC>(M, Nc, Kd, A, lda, B, ldb, C, ldc, smem);
+    return;
+  }
   TA* As = reinterpret_cast<TA*>(smem);                                     // [kZgK][33] (k, m)
   TB* Bs = reinterpret_cast<TB*>(smem + kZgK * (kZgTile + 1) * sizeof(double2));  // [kZgK][33] (k, n)
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -239,9 +310,18 @@ __device__ void z_store_slot(const Su2Dev& C, int j, int detq) {
   __syncthreads();
 }
 
+// The field's phase factor exp(i g eta(l)) from the CTA's table.
+__device__ __forceinline__ double2 field_phase(const Sm& S, int l) {
+  const double2 t = S.tab[(l == 1 || l == -1) ? 0 : 1];
+  return l > 0 ? t : zconj(t);
+}
+__device__ inline void fill_phase_table(const Su2Dev& C, Sm& S) {
+  if (threadIdx.x < 2) S.tab[threadIdx.x] = zexpi(C.g * hs_eta(threadIdx.x + 1));
+  __syncthreads();
+}
 // exp(s i g eta(l)) of slice tau for every site, into ph (s = +1 or -1)
-__device__ inline void slice_phases(const Su2Dev& C, const int8_t* f, double s, double2* ph) {
-  for (int x = threadIdx.x; x < C.N; x += kThreads) ph[x] = zexpi(s * C.g * hs_eta(f[x]));
+__device__ inline void slice_phases(const Su2Dev& C, const int8_t* f, double s, const Sm& S) {
+  for (int x = threadIdx.x; x < C.N; x += kThreads) S.ph[x] = field_phase(S, s > 0.0 ? f[x] : -f[x]);
   __syncthreads();
 }
 
@@ -280,10 +360,14 @@ __device__ void zhouse_apply(int N, int ld, double2* X, int k, int j0, double b,
       for (int i = k + rg; i < N; i += 8) w = zmac(w, zconj(hv[i]), X[(size_t)i * ld + j]);
     qred[rg * 32 + lane] = w;
     __syncthreads();
-    double2 s = make_double2(0.0, 0.0);
+    if (rg == 0) {
+      double2 t = w;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) s = zadd(s, qred[r * 32 + lane]);
-    s = zscal(b, s);
+      for (int r = 1; r < 8; ++r) t = zadd(t, qred[r * 32 + lane]);
+      qred[lane] = zscal(b, t);
+    }
+    __syncthreads();
+    const double2 s = qred[lane];
     if (j < N)
       for (int i = k + rg; i < N; i += 8) {
         double2* xp = X + (size_t)i * ld + j;
@@ -299,26 +383,28 @@ __device__ void zhouse_apply(int N, int ld, double2* X, int k, int j0, double b,
 // alpha = -(x_0/|x_0|) |x| (Hermitian, unitary, det -1).  The pivot is the
 // column of largest remaining norm (ties: lowest index), the norms downdated
 // as in LAPACK's xGEQPF and recomputed when cancellation would spoil them.
-// perm[k] = the original column now at position k.  Returns det Q.
+// perm[k] = the original column now at position k.  Returns det Q.  cn, cn0: the
+// remaining columns' squared norms, downdated, and their last full values.
 __device__ int zqr_pivoted(int N, int ld, double2* X, double* beta, double2* vk0, double* cn, double* cn0, int* perm,
                            Sm& S) {
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   for (int j = tid; j < N; j += kThreads) {
     double acc = 0.0;
     for (int i = 0; i < N; ++i) acc += zabs2(X[(size_t)i * ld + j]);
-    cn[j] = sqrt(acc);
-    cn0[j] = cn[j];
+    cn[j] = acc;
+    cn0[j] = acc;
     perm[j] = j;
   }
   __syncthreads();
-  const double tol3z = sqrt(2.220446049250313e-16);
+  const double tol3z = 1.4901161193847656e-08;  // sqrt(2^-52)
   int detq = 1;
   for (int k = 0; k < N; ++k) {
-    double bv = -1.0;
-    int bi = N;
-    for (int j = k + tid; j < N; j += kThreads)
-      if (cn[j] > bv) { bv = cn[j]; bi = j; }
-    int p = block_argmax(bv, bi, S.red, S.ired);
+    int bv = -1, bi = N;
+    for (int j = k + tid; j < N; j += kThreads) {
+      const int key = top_bits(fmax(cn[j], 0.0));
+      if (key > bv) { bv = key; bi = j; }
+    }
+    int p = block_argmax_key(bv, bi, N, S.ired);
     if (p >= N) p = k;
     if (p != k) {
       for (int i = tid; i < N; i += kThreads) {
@@ -333,50 +419,51 @@ __device__ int zqr_pivoted(int N, int ld, double2* X, double* beta, double2* vk0
       }
       __syncthreads();
     }
-    double part = 0.0;
-    for (int i = k + tid; i < N; i += kThreads) {
-      const double2 x = X[(size_t)i * ld + k];
-      part += zabs2(x);
-      S.hv[i] = x;
+    if (tid < 32) {
+      double part = 0.0;
+      for (int i = k + lane; i < N; i += 32) {
+        const double2 x = X[(size_t)i * ld + k];
+        part += zabs2(x);
+        S.hv[i] = x;
+      }
+      const double xn2 = warp_sum(part);
+      __syncwarp();
+      const double2 x0 = S.hv[k];
+      double bk = 0.0;
+      double2 alpha = x0;
+      if (xn2 > 0.0) {
+        const double xnorm = sqrt(xn2), a2 = zabs2(x0);
+        alpha = (a2 > 0.0) ? zscal(-xnorm * rsqrt(a2), x0) : make_double2(-xnorm, 0.0);
+        const double2 v0 = zsub(x0, alpha);
+        const double vhv = xn2 - a2 + zabs2(v0);
+        bk = (vhv > 0.0) ? quick_div(2.0, vhv) : 0.0;
+        __syncwarp();
+        if (lane == 0) S.hv[k] = v0;
+      }
+      if (lane == 0) {
+        beta[k] = bk;
+        vk0[k] = S.hv[k];
+        X[(size_t)k * ld + k] = alpha;
+        S.red[0] = bk;
+      }
     }
-    const double xn2 = block_sum(part, S.red);
-    const double xnorm = sqrt(xn2);
-    const double2 x0 = S.hv[k];
-    double bk = 0.0;
-    double2 alpha = make_double2(0.0, 0.0);
-    if (xnorm > 0.0) {
-      const double a0 = zabs(x0);
-      alpha = (a0 > 0.0) ? zscal(-xnorm / a0, x0) : make_double2(-xnorm, 0.0);
-      const double2 v0 = zsub(x0, alpha);
-      const double vhv = xn2 - zabs2(x0) + zabs2(v0);
-      bk = (vhv > 0.0) ? 2.0 / vhv : 0.0;
-      __syncthreads();
-      if (tid == 0) S.hv[k] = v0;
-      __syncthreads();
-    }
-    if (tid == 0) {
-      beta[k] = bk;
-      vk0[k] = S.hv[k];
-    }
+    __syncthreads();
+    const double bk = S.red[0];
     if (bk != 0.0) {
       detq = -detq;
       zhouse_apply(N, ld, X, k, k + 1, bk, S.hv, S.qred);
     }
     __syncthreads();
-    if (tid == 0) X[(size_t)k * ld + k] = (xnorm > 0.0) ? alpha : x0;
+    // |x_j|^2 less the new row's entry; renewed where cancellation sets in
     for (int j = k + 1 + tid; j < N; j += kThreads) {
-      if (cn[j] != 0.0) {
-        double t = zabs(X[(size_t)k * ld + j]) / cn[j];
-        t = fmax(0.0, (1.0 + t) * (1.0 - t));
-        const double r = cn[j] / cn0[j];
-        if (t * r * r <= tol3z) {
-          double acc = 0.0;
-          for (int i = k + 1; i < N; ++i) acc += zabs2(X[(size_t)i * ld + j]);
-          cn[j] = sqrt(acc);
-          cn0[j] = cn[j];
-        } else {
-          cn[j] *= sqrt(t);
-        }
+      const double t = cn[j] - zabs2(X[(size_t)k * ld + j]);
+      if (!(t > tol3z * cn0[j])) {
+        double acc = 0.0;
+        for (int i = k + 1; i < N; ++i) acc += zabs2(X[(size_t)i * ld + j]);
+        cn[j] = acc;
+        cn0[j] = acc;
+      } else {
+        cn[j] = t;
       }
     }
     __syncthreads();
@@ -415,7 +502,7 @@ __device__ int z_chain_step(const Su2Dev& C, int t1, int t2, bool left, ZUdv src
     const int t = left ? t2 - q : t1 + 1 + q;
     const int8_t* f = C.fields + (size_t)(t - 1) * C.MV;
     if (!left) {
-      slice_phases(C, f, +1.0, S.ph);
+      slice_phases(C, f, +1.0, S);
       for (int e = threadIdx.x; e < N * N; e += kThreads) {
         const int x = e / N, y = e - x * N;
         X[(size_t)x * ld + y] = zmul(S.ph[x], X[(size_t)x * ld + y]);
@@ -426,7 +513,7 @@ __device__ int z_chain_step(const Su2Dev& C, int t1, int t2, bool left, ZUdv src
     } else {
       zgemm<0, 0, false>(N, N, N, C.E, ld, X, ld, Y, ld, S.gemm);
       for (int b = 0; b < C.nb; ++b) bond_rows(N, ld, Y, C.bi[b], C.bj[b], C.a0 * f[N + b]);
-      slice_phases(C, f, -1.0, S.ph);
+      slice_phases(C, f, -1.0, S);
       for (int e = threadIdx.x; e < N * N; e += kThreads) {
         const int x = e / N, y = e - x * N;
         Y[(size_t)x * ld + y] = zmul(S.ph[x], Y[(size_t)x * ld + y]);
@@ -447,19 +534,69 @@ __device__ int z_chain_step(const Su2Dev& C, int t1, int t2, bool left, ZUdv src
   int* perm = C.iwork;
   const int detq = zqr_pivoted(N, ld, X, beta, vk0, dvec(C, 2), dvec(C, 3), perm, S);
   zform_q(N, ld, X, beta, vk0, zmat(C, 2), S);
-  for (int k = threadIdx.x; k < N; k += kThreads) Dn[k] = zabs(X[(size_t)k * ld + k]);
+  for (int k = threadIdx.x; k < N; k += kThreads) {
+    Dn[k] = zabs(X[(size_t)k * ld + k]);
+    dvec(C, 1)[k] = Dn[k] > 0.0 ? 1.0 / Dn[k] : 0.0;
+  }
   __syncthreads();
   // Y = D^-1 R (upper triangle), Rt = P^T src.T (row k = row perm[k] of src.T)
   double2* Rt = zmat(C, 7);
   for (int e = threadIdx.x; e < N * N; e += kThreads) {
     const int x = e / N, y = e - x * N;
-    const double dinv = Dn[x] > 0.0 ? 1.0 / Dn[x] : 0.0;
-    Y[(size_t)x * ld + y] = (y >= x) ? zscal(dinv, X[(size_t)x * ld + y]) : make_double2(0.0, 0.0);
+    Y[(size_t)x * ld + y] = (y >= x) ? zscal(dvec(C, 1)[x], X[(size_t)x * ld + y]) : make_double2(0.0, 0.0);
     Rt[(size_t)x * ld + y] = src.T[(size_t)perm[x] * ld + y];
   }
   __syncthreads();
   zgemm<0, 0, false>(N, N, N, (const double2*)Y, ld, (const double2*)Rt, ld, zmat(C, 3), ld, S.gemm);
   return detq;
+}
+
+// X <- Mid^-1 X by Gauss-Jordan with partial pivoting (Mid is used up); piv[k] = the
+// k-th pivot (shared), swaps counts the row interchanges.  Returns 1 on a singular Mid.
+__device__ int z_gauss_jordan(int N, int ld, double2* Mid, double2* X, double2* piv, int& swaps, Sm& S) {
+  const int tid = threadIdx.x;
+  for (int k = 0; k < N; ++k) {
+    int bv = -1, bi = N;
+    for (int i = k + tid; i < N; i += kThreads) {
+      const int key = pivot_key(Mid[(size_t)i * ld + k]);
+      if (key > bv) { bv = key; bi = i; }
+    }
+    const int p = block_argmax_key(bv, bi, N, S.ired);
+    if (p >= N) return 1;
+    const double2 d = Mid[(size_t)p * ld + k];
+    if (d.x == 0.0 && d.y == 0.0) return 1;
+    if (p != k) ++swaps;
+    if (tid < 32) {
+      const double2 dinv = zdiv(make_double2(1.0, 0.0), d);
+      if (tid == 0) {
+        S.qred[0] = dinv;
+        piv[k] = d;
+      }
+    }
+    // row k takes row p's place (after the barrier; its factors are zero there)
+    for (int i = tid; i < N; i += kThreads)
+      S.hv[i] = (i == k) ? make_double2(0.0, 0.0) : Mid[(size_t)(i == p ? k : i) * ld + k];
+    __syncthreads();
+    const double2 dinv = S.qred[0];
+    for (int j = tid; j < 2 * N; j += kThreads) {
+      double2* M = j < N ? Mid : X;
+      const int c = j < N ? j : j - N;
+      const double2 t = M[(size_t)p * ld + c];
+      if (p != k) M[(size_t)p * ld + c] = M[(size_t)k * ld + c];
+      M[(size_t)k * ld + c] = zmul(t, dinv);
+    }
+    __syncthreads();
+    // the columns of Mid up to k are not read again
+    for (int e = tid; e < N * N; e += kThreads) {
+      const int i = e / N, j = e - i * N;
+      if (i == k) continue;
+      const double2 f = S.hv[i], mf = make_double2(-f.x, -f.y);
+      if (j > k) Mid[(size_t)i * ld + j] = zmac(Mid[(size_t)i * ld + j], mf, Mid[(size_t)k * ld + j]);
+      X[(size_t)i * ld + j] = zmac(X[(size_t)i * ld + j], mf, X[(size_t)k * ld + j]);
+    }
+    __syncthreads();
+  }
+  return 0;
 }
 
 // G = (1 + B(tau,0) B(beta,tau))^-1 from the right chain R = B(tau,0) and the
@@ -475,11 +612,12 @@ __device__ int z_green(const Su2Dev& C, ZUdv R, ZUdv Lf, double2* Gout, double& 
   double *dbR = dvec(C, 4), *dsR = dvec(C, 5), *dbL = dvec(C, 6), *dsL = dvec(C, 7);
   double lsum = 0.0;
   for (int i = tid; i < N; i += kThreads) {
-    dbR[i] = fmax(R.D[i], 1.0);
+    // dbR, dbL hold 1 / Db
+    dbR[i] = 1.0 / fmax(R.D[i], 1.0);
     dsR[i] = fmin(R.D[i], 1.0);
-    dbL[i] = fmax(Lf.D[i], 1.0);
+    dbL[i] = 1.0 / fmax(Lf.D[i], 1.0);
     dsL[i] = fmin(Lf.D[i], 1.0);
-    lsum += log(dbR[i]) + log(dbL[i]);
+    lsum += log(fmax(R.D[i], 1.0)) + log(fmax(Lf.D[i], 1.0));
   }
   lsum = block_sum(lsum, S.red);
   double2* Mid = zmat(C, 4);
@@ -489,55 +627,27 @@ __device__ int z_green(const Su2Dev& C, ZUdv R, ZUdv Lf, double2* Gout, double& 
   for (int e = tid; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
     const double2 qq = Mid[(size_t)i * ld + j], tt = X[(size_t)i * ld + j];
-    Mid[(size_t)i * ld + j] = zadd(zscal(1.0 / (dbR[i] * dbL[j]), qq), zscal(dsR[i] * dsL[j], tt));
+    Mid[(size_t)i * ld + j] = zadd(zscal(dbR[i] * dbL[j], qq), zscal(dsR[i] * dsL[j], tt));
   }
   __syncthreads();
   for (int e = tid; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
-    X[(size_t)i * ld + j] = zscal(1.0 / dbR[i], zconj(R.Q[(size_t)j * ld + i]));  // Db_R^-1 Q_R^H
+    X[(size_t)i * ld + j] = zscal(dbR[i], zconj(R.Q[(size_t)j * ld + i]));  // Db_R^-1 Q_R^H
   }
   __syncthreads();
+  int swaps = 0;
+  if (z_gauss_jordan(N, ld, Mid, X, S.col, swaps, S)) return 1;
   double la = 0.0, ar = 0.0;
-  for (int k = 0; k < N; ++k) {
-    double bv = -1.0;
-    int bi = N;
-    for (int i = k + tid; i < N; i += kThreads) {
-      const double a = zabs(Mid[(size_t)i * ld + k]);
-      if (a > bv) { bv = a; bi = i; }
-    }
-    const int p = block_argmax(bv, bi, S.red, S.ired);
-    if (p >= N || zabs(Mid[(size_t)p * ld + k]) == 0.0) return 1;
-    if (p != k) {
-      for (int j = tid; j < N; j += kThreads) {
-        double2 t = Mid[(size_t)k * ld + j]; Mid[(size_t)k * ld + j] = Mid[(size_t)p * ld + j]; Mid[(size_t)p * ld + j] = t;
-        t = X[(size_t)k * ld + j]; X[(size_t)k * ld + j] = X[(size_t)p * ld + j]; X[(size_t)p * ld + j] = t;
-      }
-      ar += 3.14159265358979323846;
-      __syncthreads();
-    }
-    const double2 d = Mid[(size_t)k * ld + k];
+  for (int k = tid; k < N; k += kThreads) {
+    const double2 d = S.col[k];
     la += log(zabs(d));
     ar += atan2(d.y, d.x);
-    const double2 dinv = zdiv(make_double2(1.0, 0.0), d);
-    __syncthreads();
-    for (int j = tid; j < N; j += kThreads) {
-      Mid[(size_t)k * ld + j] = zmul(Mid[(size_t)k * ld + j], dinv);
-      X[(size_t)k * ld + j] = zmul(X[(size_t)k * ld + j], dinv);
-    }
-    for (int i = tid; i < N; i += kThreads) S.hv[i] = (i == k) ? make_double2(0.0, 0.0) : Mid[(size_t)i * ld + k];
-    __syncthreads();
-    for (int e = tid; e < N * N; e += kThreads) {
-      const int i = e / N, j = e - i * N;
-      if (i == k) continue;
-      const double2 f = S.hv[i];
-      Mid[(size_t)i * ld + j] = zsub(Mid[(size_t)i * ld + j], zmul(f, Mid[(size_t)k * ld + j]));
-      X[(size_t)i * ld + j] = zsub(X[(size_t)i * ld + j], zmul(f, X[(size_t)k * ld + j]));
-    }
-    __syncthreads();
   }
+  la = block_sum(la, S.red);
+  ar = block_sum(ar, S.red) + 3.14159265358979323846 * swaps;
   for (int e = tid; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
-    X[(size_t)i * ld + j] = zscal(1.0 / dbL[i], X[(size_t)i * ld + j]);
+    X[(size_t)i * ld + j] = zscal(dbL[i], X[(size_t)i * ld + j]);
   }
   __syncthreads();
   zgemm<0, 0, false>(N, N, N, Lf.Q, ld, (const double2*)X, ld, Gout, ld, S.gemm);
@@ -574,39 +684,8 @@ __device__ int z_displaced(const Su2Dev& C, ZUdv R, ZUdv Lf, double2* Gt0, doubl
     MI[(size_t)i * ld + j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
   }
   __syncthreads();
-  for (int k = 0; k < N; ++k) {
-    double bv = -1.0;
-    int bi = N;
-    for (int i = k + tid; i < N; i += kThreads) {
-      const double a = zabs(Mid[(size_t)i * ld + k]);
-      if (a > bv) { bv = a; bi = i; }
-    }
-    const int p = block_argmax(bv, bi, S.red, S.ired);
-    if (p >= N || zabs(Mid[(size_t)p * ld + k]) == 0.0) return 1;
-    if (p != k) {
-      for (int j = tid; j < N; j += kThreads) {
-        double2 t = Mid[(size_t)k * ld + j]; Mid[(size_t)k * ld + j] = Mid[(size_t)p * ld + j]; Mid[(size_t)p * ld + j] = t;
-        t = MI[(size_t)k * ld + j]; MI[(size_t)k * ld + j] = MI[(size_t)p * ld + j]; MI[(size_t)p * ld + j] = t;
-      }
-      __syncthreads();
-    }
-    const double2 dinv = zdiv(make_double2(1.0, 0.0), Mid[(size_t)k * ld + k]);
-    __syncthreads();
-    for (int j = tid; j < N; j += kThreads) {
-      Mid[(size_t)k * ld + j] = zmul(Mid[(size_t)k * ld + j], dinv);
-      MI[(size_t)k * ld + j] = zmul(MI[(size_t)k * ld + j], dinv);
-    }
-    for (int i = tid; i < N; i += kThreads) S.hv[i] = (i == k) ? make_double2(0.0, 0.0) : Mid[(size_t)i * ld + k];
-    __syncthreads();
-    for (int e = tid; e < N * N; e += kThreads) {
-      const int i = e / N, j = e - i * N;
-      if (i == k) continue;
-      const double2 f = S.hv[i];
-      Mid[(size_t)i * ld + j] = zsub(Mid[(size_t)i * ld + j], zmul(f, Mid[(size_t)k * ld + j]));
-      MI[(size_t)i * ld + j] = zsub(MI[(size_t)i * ld + j], zmul(f, MI[(size_t)k * ld + j]));
-    }
-    __syncthreads();
-  }
+  int swaps = 0;
+  if (z_gauss_jordan(N, ld, Mid, MI, S.col, swaps, S)) return 1;
   // G(tau,0) = Q_L (Db_L^-1 MI Ds_R) T_R
   for (int e = tid; e < N * N; e += kThreads) {
     const int i = e / N, j = e - i * N;
@@ -689,10 +768,11 @@ __device__ void z_update_slice(Su2Dev& C, int tau, int dir, const Su2SweepParams
     S.u2[q] = uniform53(ctr[2], ctr[3]);
     const int f = S.fsl[k];
     const int fn = propose_field(2, f, u1);
-    const double dth = C.g * (hs_eta(fn) - hs_eta(f));
-    const double2 e = zexpi(dth);
+    const double2 e = zmul(field_phase(S, fn), zconj(field_phase(S, f)));  // e^{i g (eta(l') - eta(l))}
     S.delta[q] = make_double2(e.x - 1.0, e.y);
-    S.gr[q] = zscal(hs_gamma(fn) / hs_gamma(f), zconj(e));
+    const bool one_n = fn == 1 || fn == -1, one_o = f == 1 || f == -1;
+    const double up = (1.0 + sqrt(6.0) / 3.0) / (1.0 - sqrt(6.0) / 3.0), dn = (1.0 - sqrt(6.0) / 3.0) / (1.0 + sqrt(6.0) / 3.0);
+    S.gr[q] = zscal(one_n == one_o ? 1.0 : one_n ? up : dn, zconj(e));  // gamma(l') / gamma(l)
     S.fn[q] = (int8_t)fn;
   }
   for (int x = tid; x < N; x += kThreads) S.d[x] = G[(size_t)x * ld + x];
@@ -707,8 +787,9 @@ __device__ void z_update_slice(Su2Dev& C, int tau, int dir, const Su2SweepParams
       const int k = dir ? N - 1 - q : q;
       const double2 r1 = zadd(make_double2(1.0, 0.0), zmul(S.delta[q], zsub(make_double2(1.0, 0.0), S.d[k])));
       const double2 R = zmul(S.gr[q], zmul(r1, r1));
-      const double ratio = fabs(zmul(Pc, R).x) / fabs(Pc.x);
-      if (S.u2[q] < (ratio < 1.0 ? ratio : 1.0)) {
+      // u < min(1, |Re(P R)| / |Re P|) without the quotient
+      const double a = fabs(zmul(Pc, R).x), b = fabs(Pc.x);
+      if (!(a < b) || S.u2[q] * b < a) {
         atomicMin(S.first, q);
         break;
       }
@@ -717,26 +798,38 @@ __device__ void z_update_slice(Su2Dev& C, int tau, int dir, const Su2SweepParams
     const int first = *S.first;
     if (first >= N) break;
     const int k = dir ? N - 1 - first : first;
-    const double2 r1 = zadd(make_double2(1.0, 0.0), zmul(S.delta[first], zsub(make_double2(1.0, 0.0), S.d[k])));
-    const double2 coef = zdiv(S.delta[first], r1);
-    for (int x = tid; x < N; x += kThreads) {
-      S.col[x] = G[(size_t)x * ld + k];
-      const double2 gkx = G[(size_t)k * ld + x];
-      S.row[x] = make_double2((x == k ? 1.0 : 0.0) - gkx.x, -gkx.y);
+    // warp 0: the update's factor; warp 1: the new phase
+    if (tid < 64) {
+      const double2 r1 = zadd(make_double2(1.0, 0.0), zmul(S.delta[first], zsub(make_double2(1.0, 0.0), S.d[k])));
+      if (tid < 32) {
+        const double2 coef = zdiv(S.delta[first], r1);
+        if (tid == 0) S.qred[0] = coef;
+      } else {
+        const double2 PR = zmul(Pc, zmul(S.gr[first], zmul(r1, r1)));
+        const double2 Pn = zscal(rsqrt(zabs2(PR)), PR);
+        if (tid == 32) S.qred[1] = Pn;
+      }
     }
     __syncthreads();
-    if (tid == 0) {
-      const double2 R = zmul(S.gr[first], zmul(r1, r1));
-      const double2 PR = zmul(Pc, R);
-      *S.P = zscal(1.0 / zabs(PR), PR);
+    const double2 coef = S.qred[0];
+    for (int x = tid; x < N; x += kThreads) {
+      const double2 c = zmul(coef, G[(size_t)x * ld + k]);
+      const double2 gkx = G[(size_t)k * ld + x];
+      const double2 r = make_double2((x == k ? 1.0 : 0.0) - gkx.x, -gkx.y);
+      S.col[x] = make_double2(-c.x, -c.y);
+      S.row[x] = r;
+      S.d[x] = zmac(S.d[x], S.col[x], r);
+    }
+    if (tid == 32) {
+      *S.P = S.qred[1];
       S.fsl[k] = S.fn[first];
     }
+    __syncthreads();
     for (int e = tid; e < N * N; e += kThreads) {
       const int x = e / N, y = e - x * N;
       double2* gp = G + (size_t)x * ld + y;
-      *gp = zsub(*gp, zmul(zmul(coef, S.col[x]), S.row[y]));
+      *gp = zmac(*gp, S.col[x], S.row[y]);
     }
-    for (int x = tid; x < N; x += kThreads) S.d[x] = zsub(S.d[x], zmul(zmul(coef, S.col[x]), S.row[x]));
     ++nacc;
     pos = first + 1;
     __syncthreads();
@@ -963,12 +1056,13 @@ __global__ void __launch_bounds__(kThreads) su2_sweep_kernel(Su2Dev* chains, Su2
   Su2Dev& C = chains[blockIdx.x];
   if (blockIdx.x >= P.n_chains) return;
   Sm S = su2_carve(smem_raw, C.N, C.MV);
+  fill_phase_table(C, S);
   const int L = C.L, nw = C.nw;
   if (threadIdx.x == 0) *S.P = C.P;
   __syncthreads();
   for (int tau = 1; tau <= L; ++tau) {
     load_slice(C, tau, S);
-    slice_phases(C, S.fsl, +1.0, S.ph);
+    slice_phases(C, S.fsl, +1.0, S);
     z_v_wrap(C, C.G, S.ph);
     z_update_slice(C, tau, 0, P, S);
     for (int b = C.nb - 1; b >= 0; --b) {
@@ -989,7 +1083,7 @@ __global__ void __launch_bounds__(kThreads) su2_sweep_kernel(Su2Dev* chains, Su2
     }
     z_update_slice(C, tau, 1, P, S);
     store_slice(C, tau, S);
-    slice_phases(C, S.fsl, -1.0, S.ph);
+    slice_phases(C, S.fsl, -1.0, S);
     z_v_wrap(C, C.G, S.ph);
     if ((tau - 1) % nw == 0) z_stabilise(C, (tau - 1) / nw, false, S);
     if (P.measure && tau - 1 >= P.meas_first && tau - 1 <= P.meas_last) z_measure(C, S);
@@ -1010,6 +1104,7 @@ __global__ void __launch_bounds__(kThreads) su2_fresh_kernel(Su2Dev* chains, int
   if (c >= n_chains || (mode == 1 && c != only)) return;
   Su2Dev& C = chains[c];
   Sm S = su2_carve(smem_raw, C.N, C.MV);
+  fill_phase_table(C, S);
   double la = 0.0, ar = 0.0;
   if (z_fill_left(C, S, la, ar)) {
     if (threadIdx.x == 0) C.error |= 1;
@@ -1090,6 +1185,7 @@ __global__ void __launch_bounds__(kThreads) su2_tau_kernel(Su2Dev* chains, int n
   if (c >= n_chains || (only >= 0 && c != only)) return;
   Su2Dev& C = chains[c];
   Sm S = su2_carve(smem_raw, C.N, C.MV);
+  fill_phase_table(C, S);
   const int N = C.N, ld = C.ld, nw = C.nw, nst = C.L / nw;
   double2* Gt0 = zmat(C, 8);
   double2* G0t = zmat(C, 9);
@@ -1112,7 +1208,7 @@ __global__ void __launch_bounds__(kThreads) su2_tau_kernel(Su2Dev* chains, int n
       const int8_t* f = C.fields + (size_t)(tau - 1) * C.MV;
       double2* W = zmat(C, 0);
       // G(tau,0) = E X_0 .. X_{nb-1} e^{V} G(tau-1,0)
-      slice_phases(C, f, +1.0, S.ph);
+      slice_phases(C, f, +1.0, S);
       for (int e = threadIdx.x; e < N * N; e += kThreads) {
         const int x = e / N, y = e - x * N;
         Gt0[(size_t)x * ld + y] = zmul(S.ph[x], Gt0[(size_t)x * ld + y]);
@@ -1122,7 +1218,7 @@ __global__ void __launch_bounds__(kThreads) su2_tau_kernel(Su2Dev* chains, int n
       zgemm<0, 0, false>(N, N, N, C.E, ld, (const double2*)Gt0, ld, W, ld, S.gemm);
       zcopy(N, ld, W, Gt0);
       // G(0,tau) = G(0,tau-1) e^{-V} X_{nb-1}^-1 .. X_0^-1 E^-1
-      slice_phases(C, f, -1.0, S.ph);
+      slice_phases(C, f, -1.0, S);
       for (int e = threadIdx.x; e < N * N; e += kThreads) {
         const int x = e / N, y = e - x * N;
         G0t[(size_t)x * ld + y] = zmul(G0t[(size_t)x * ld + y], S.ph[y]);
