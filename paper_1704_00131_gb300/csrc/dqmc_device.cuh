@@ -595,7 +595,9 @@ __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   s.um.limit = kUmmaWaitCycles;
   s.um.stall = 0;
   q += 128;
-  q = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(q) + 127) & ~(uintptr_t)127);
+  // (offsets from the 128-byte aligned start, no pointer-to-integer casts: the compiler
+  // then knows that the panels are shared memory)
+  q = start + ((size_t)(q - start) + 127) / 128 * 128;
   s.gemm = reinterpret_cast<double*>(q);
   s.ab = reinterpret_cast<double*>(q + gemm_region_bytes(ld));
   uint32_t dyn;
@@ -844,7 +846,7 @@ __device__ void panel_apply(int N, int ld, T* A, int r0, int j0, int nb, const T
 #pragma unroll
     for (int q = 0; q < PW; ++q) y[q] = from_zero<T>();
     if (act) {
-      // four rows at a time, their loads issued together
+      // four rows at a time, their loads issued together (eight were slower)
       int i = r0 + g;
       for (; i + 3 * G < N; i += 4 * G) {
         T x[4];
@@ -1725,7 +1727,7 @@ __device__ int fill_left_chain_working(const ChainDev& C, int s, Smem& S, double
 template <typename Real>
 __global__ void __launch_bounds__(kThreads) fresh_green_kernel(ChainDev* chains, int n_chains, int mode,
                                                                double* out, int out_chain) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nfl = chains[0].nfl;
   const int c = blockIdx.x / nfl, s = blockIdx.x % nfl;
   if (c >= n_chains) return;
@@ -1779,7 +1781,7 @@ __device__ void t_wrap(const ChainDev& C, int s, Real* G, Real* Gt, bool up, Sme
 // the work matrices W0..W8; out: [nfl][N][N] FP64.
 template <typename Real>
 __global__ void __launch_bounds__(kThreads) green_tau_kernel(ChainDev* chains, int chain, int tau, double* out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   ChainDev& C = chains[chain];
   const int s = blockIdx.x;
   if (s >= C.nfl) return;
@@ -1887,6 +1889,65 @@ __device__ void t_wrap<dd>(const ChainDev& C, int s, dd* G, dd* Gt, bool up, Sme
   gemm_dd<false, false, false>(C, s, S, N, N, N, Gt, ld, Y, ld, G, ld, -1, up ? kCpEiB : kCpEB);
 }
 
+// G += sum_m a_m b_m^T in float pairs: 16R x 16R tiles of G in registers, the vectors read
+// where they are (shared memory, or the chain's arena).  The sums start from G, whose
+// loads are the tile's only global reads, and keep its value and their error terms
+// apart until the end (the products' scheme).  Instruction issue is the bound: 12 FP32
+// operations per product and output, N^2 k 12 / 128 cycles per CTA.
+template <int R>
+__device__ void rank_update_dd(int N, int ld, dd* G, const dd* A, const dd* B, int nacc) {
+  constexpr int TT = 16 * R;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  for (int m0 = 0; m0 < N; m0 += TT)
+    for (int n0 = 0; n0 < N; n0 += TT) {
+      int row[R], col[R];
+      float h[R][R], l[R][R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        row[i] = min(m0 + ty * R + i, N - 1);
+        col[i] = min(n0 + tx * R + i, N - 1);
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          const dd g = G[(size_t)row[i] * ld + col[j]];
+          h[i][j] = g.hi;
+          l[i][j] = g.lo;
+        }
+#pragma unroll 2
+      for (int m = 0; m < nacc; ++m) {
+        dd a[R], b[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) a[i] = A[(size_t)m * ld + row[i]];
+#pragma unroll
+        for (int j = 0; j < R; ++j) b[j] = B[(size_t)m * ld + col[j]];
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < R; ++j) {
+            const float p = a[i].hi * b[j].hi;
+            const float pe = fmaf(a[i].hi, b[j].hi, -p);
+            const float t = h[i][j] + p;
+            const float bb = t - h[i][j];
+            const float te = (h[i][j] - (t - bb)) + (p - bb);
+            h[i][j] = t;
+            float lo = l[i][j] + (te + pe);
+            lo = fmaf(a[i].hi, b[j].lo, lo);
+            l[i][j] = fmaf(a[i].lo, b[j].hi, lo);
+          }
+      }
+      // (clamped rows and columns repeat another thread's outputs and are not stored)
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+          if (m0 + ty * R + i < N && n0 + tx * R + j < N)
+            G[(size_t)row[i] * ld + col[j]] = fast_two_sum(h[i][j], l[i][j]);
+    }
+  __syncthreads();
+}
+
 // G <- G + sum_m a_m b_m^T  (flush of the delayed rank-k update), a register-
 // blocked product G += A^T B with A, B stored as rows a_m, b_m.
 template <typename Real>
@@ -1924,10 +1985,18 @@ __device__ void flush_delayed<float>(const ChainDev& C, float* G, const float* A
 }
 template <>
 __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const dd* B, int nacc, Smem& S) {
-  // a rank-k update (k <= 64): the float-pair SIMT tiles beat the split tensor-core
+  // a rank-k update (k <= 64): the float-pair register tiles beat the split tensor-core
   // product, whose digit split and recombination cost O(N^2) whatever k
-  gemm_dd_tiles<true, false, true>(C.N, C.N, nacc, A, C.ld, B, C.ld, G, C.ld, reinterpret_cast<dd*>(S.gemm),
-                                   S.dd_tile);
+  int r = S.dd_tile;
+  if (r != 3 && r != 4) {
+    r = 4;
+    for (int q = 3; q >= 1; --q)
+      if (umma_pad(C.N, 16 * q) < umma_pad(C.N, 16 * r)) r = q;
+  }
+  if (r == 1) rank_update_dd<1>(C.N, C.ld, G, A, B, nacc);
+  else if (r == 2) rank_update_dd<2>(C.N, C.ld, G, A, B, nacc);
+  else if (r == 3) rank_update_dd<3>(C.N, C.ld, G, A, B, nacc);
+  else rank_update_dd<4>(C.N, C.ld, G, A, B, nacc);
 }
 
 // Sequential single-field updates of one slice (Sec. 2.2.1) for this CTA's
@@ -2462,7 +2531,7 @@ __device__ int close_event(ChainDev& C, int s, Smem& S, cg::cluster_group& cl, d
 // One sweep of every chain (Algorithm 1, upward then downward).
 template <typename Real>
 __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(ChainDev* chains, SweepParams P) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
   const int nfl = (int)cl.num_blocks();
   const int s = (int)cl.block_rank();

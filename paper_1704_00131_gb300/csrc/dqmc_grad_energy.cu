@@ -6,7 +6,7 @@ namespace dqmc {
 
 // G(0) of every (configuration, flavor) into G0all [n_cfg][nfl][N][N] (FP64).
 __global__ void __launch_bounds__(kThreads) green0_kernel(ChainDev* chains, int n_cfg, double* G0all) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nfl = chains[0].nfl;
   const int c = blockIdx.x / nfl, s = blockIdx.x % nfl;
   if (c >= n_cfg) return;
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kThreads) green0_kernel(ChainDev* chains, int 
 __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains, int n_cfg, const double* V,
                                                                const double* w, const double* G0all, double* ework_all,
                                                                double* gK, double* gU, double* eparts) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nfl = chains[0].nfl;
   const int c = blockIdx.x / nfl, s = blockIdx.x % nfl;
   if (c >= n_cfg) return;

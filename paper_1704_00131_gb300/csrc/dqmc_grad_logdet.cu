@@ -12,7 +12,7 @@ namespace dqmc {
 // F of exp(-dtau x) over the eigenvalues of K (Frechet derivative).
 __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains, int n_cfg, const double* V,
                                                                const double* w, double* gK, double* gU) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nfl = chains[0].nfl;
   const int c = blockIdx.x / nfl, s = blockIdx.x % nfl;
   if (c >= n_cfg) return;

@@ -49,7 +49,7 @@ __device__ int left_chain_running(const ChainDev& C, int s, Smem& S, double& log
 __global__ void __launch_bounds__(kThreads) fresh_green_noalloc_kernel(ChainDev C, double* scratch,
                                                                        double* out, double* logdet_out,
                                                                        int* sign_out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int s = blockIdx.x;
   const int N = C.N, ld = C.ld;
   // carve this flavor's part of the scratch array

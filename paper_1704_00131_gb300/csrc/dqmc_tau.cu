@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
                                                                const double* phase, int phase_ld, double* tw_all,
                                                                size_t tw_stride, double* obs, double* prec,
                                                                int* sign_out, TauCorrArgs tc) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nfl = chains[0].nfl;
   const int c = blockIdx.x / nfl, s = blockIdx.x % nfl;
   if (c >= n_chains) return;

@@ -301,6 +301,19 @@ __device__ void umma_row_exponents(int R, int Kd, const T* X, int ldx, int Rp, i
       if (lane_id == 0) ex[r] = umma_exp_of(mag, T());
     }
   } else {
+    if (Kd <= 32) {
+      // few k (a rank-k update): one thread per row, no exchange between warps
+      for (int r = tid; r < Rp; r += kThreads) {
+        int mag = 0;
+        if (r < R) {
+#pragma unroll 8
+          for (int k = 0; k < Kd; ++k) mag = max(mag, umma_mag(X[(size_t)k * ldx + r]));
+        }
+        ex[r] = umma_exp_of(mag, T());
+      }
+      __syncthreads();
+      return;
+    }
     // the warps share the k range, each thread one column of a 32-wide strip
     for (int r = tid; r < Rp; r += kThreads) ex[r] = 0;
     __syncthreads();
