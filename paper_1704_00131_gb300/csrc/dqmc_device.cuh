@@ -478,13 +478,45 @@ __device__ void gemm_dd_tiles(int M, int Nc, int Kd, const dd* A, int lda, const
   else cta_gemm_dd_r<TA, TB, 4, ACC>(M, Nc, Kd, A, lda, B, ldb, C, ldc, sm);
 }
 
-template <typename T>
-__device__ __forceinline__ void cta_copy(int N, int ld, const T* src, T* dst) {
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    dst[(size_t)x * ld + y] = src[(size_t)x * ld + y];
+// store(x, y, load(x, y)) for every element of an N x N matrix, four per thread in
+// flight (the matrices come from L2: a loop of one load and one store at a time waits
+// out its latency N^2 / 256 times, a tenth of a slice at N = 64).  In place is fine:
+// every element is loaded and stored by one thread.  Ends with a barrier.
+template <typename L, typename F>
+__device__ __forceinline__ void each_element(int N, L load, F store) {
+  constexpr int U = 4;
+  const int n = N * N, dq = kThreads / N, dr = kThreads - dq * N;
+  int e = threadIdx.x, x = e / N, y = e - x * N;
+  if (n <= kThreads) {
+    if (e < n) store(x, y, load(x, y));
+    e = n;
+  }
+  while (e < n) {
+    decltype(load(0, 0)) v[U];
+    int xs[U], ys[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool ok = e < n;
+      xs[u] = ok ? x : -1;
+      ys[u] = y;
+      v[u] = load(ok ? x : 0, ok ? y : 0);
+      e += kThreads;
+      x += dq;
+      y += dr;
+      if (y >= N) { y -= N; ++x; }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (xs[u] >= 0) store(xs[u], ys[u], v[u]);
   }
   __syncthreads();
+}
+
+template <typename T>
+__device__ __forceinline__ void cta_copy(int N, int ld, const T* src, T* dst) {
+  each_element(
+      N, [&](int x, int y) { return src[(size_t)x * ld + y]; },
+      [&](int x, int y, T v) { dst[(size_t)x * ld + y] = v; });
 }
 
 // --------------------------------------------------------------------------
@@ -707,23 +739,18 @@ __device__ inline UDV slot_udv(const ChainDev& C, int s, int j) {
 }
 
 __device__ inline void to_dd_mat(int N, int ld, const double* src, dd* dst) {
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    dst[(size_t)x * ld + y] = from_d<dd>(src[(size_t)x * ld + y]);
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int x, int y) { return src[(size_t)x * ld + y]; },
+      [&](int x, int y, double v) { dst[(size_t)x * ld + y] = from_d<dd>(v); });
 }
 
 // dd -> double in place (same 8-byte slot)
 __device__ inline void dd_to_d_inplace(int N, int ld, void* buf) {
   dd* a = reinterpret_cast<dd*>(buf);
   double* b = reinterpret_cast<double*>(buf);
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    const dd v = a[(size_t)x * ld + y];
-    b[(size_t)x * ld + y] = to_d(v);
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int x, int y) { return a[(size_t)x * ld + y]; },
+      [&](int x, int y, dd v) { b[(size_t)x * ld + y] = to_d(v); });
 }
 
 // ---- pivoted QR in panels, LU and solves, on FP64 or float-pair matrices --------
@@ -1437,12 +1464,14 @@ __device__ int udv_of_product(const ChainDev& C, int s, T* X, UDV src, Smem& S, 
     invr[x] = (rkk > 0.0 && dsc[x] > 0.0) ? 1.0 / (rkk * dsc[x]) : 0.0;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    PT[(size_t)x * ld + y] = from_d<T>(src.T[(size_t)perm[x] * ld + y]);
-    Rt[(size_t)x * ld + y] = y >= x ? rmul(X[(size_t)x * ld + perm[y]], from_d<T>(invr[x] * dsc[y])) : from_zero<T>();
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int x, int y) { return src.T[(size_t)perm[x] * ld + y]; },
+      [&](int x, int y, double v) { PT[(size_t)x * ld + y] = from_d<T>(v); });
+  each_element(
+      N, [&](int x, int y) { return X[(size_t)x * ld + perm[y]]; },
+      [&](int x, int y, T v) {
+        Rt[(size_t)x * ld + y] = y >= x ? rmul(v, from_d<T>(invr[x] * dsc[y])) : from_zero<T>();
+      });
   T* Tn = reinterpret_cast<T*>(wmat(C, s, 5));
   if constexpr (std::is_same<T, dd>::value) {
     gemm_dd<false, false, false>(C, s, S, N, N, N, Rt, ld, PT, ld, Tn, ld);
@@ -1548,11 +1577,9 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
       slice_potential_global(C, s, t, S.v);
       for (int x = threadIdx.x; x < N; x += kThreads) S.ev[x] = exp(S.v[x]);
       __syncthreads();
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        X[(size_t)x * ld + y] *= S.ev[x];
-      }
-      __syncthreads();
+      each_element(
+          N, [&](int x, int y) { return X[(size_t)x * ld + y]; },
+          [&](int x, int y, double v) { X[(size_t)x * ld + y] = v * S.ev[x]; });
       gemm_64<false, false>(S, N, N, N, E, ld, X, ld, Y, ld, kCpEA, -1);
       double* t_ = X; X = Y; Y = t_;
     }
@@ -1562,11 +1589,9 @@ __device__ int chain_step(const ChainDev& C, int s, int t1, int t2, bool left, U
       slice_potential_global(C, s, t, S.v);
       for (int x = threadIdx.x; x < N; x += kThreads) S.ev[x] = exp(S.v[x]);
       __syncthreads();
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        Y[(size_t)x * ld + y] *= S.ev[x];
-      }
-      __syncthreads();
+      each_element(
+          N, [&](int x, int y) { return Y[(size_t)x * ld + y]; },
+          [&](int x, int y, double v) { Y[(size_t)x * ld + y] = v * S.ev[x]; });
       double* t_ = X; X = Y; Y = t_;
     }
   }
@@ -1623,31 +1648,26 @@ __device__ int green_from_udv(const ChainDev& C, int s, UDV R, UDV Lf, double* G
     ibL[i] = 1.0 / (Lf.D[i] > 1.0 ? Lf.D[i] : 1.0);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    const double dR = R.D[i], dL = Lf.D[j];
-    const double dsR = dR > 1.0 ? 1.0 : dR, dsL = dL > 1.0 ? 1.0 : dL;
-    W0[(size_t)i * ld + j] = W0[(size_t)i * ld + j] * (ibR[i] * ibL[j]) + dsR * W1[(size_t)i * ld + j] * dsL;
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int i, int j) { return make_double2(W0[(size_t)i * ld + j], W1[(size_t)i * ld + j]); },
+      [&](int i, int j, double2 v) {
+        const double dR = R.D[i], dL = Lf.D[j];
+        const double dsR = dR > 1.0 ? 1.0 : dR, dsL = dL > 1.0 ? 1.0 : dL;
+        W0[(size_t)i * ld + j] = v.x * (ibR[i] * ibL[j]) + dsR * v.y * dsL;
+      });
   double ldm;
   int sm;
   int* rowof = S.qinv;
   double* udiag = S.hv;
   double* tmp = wmat(C, s, 9);
   if (lu_factor_blk(N, ld, W0, rowof, udiag, tmp, ldm, sm, S)) return 1;
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    const int r = rowof[i];
-    W1[(size_t)i * ld + j] = R.Q[(size_t)j * ld + r] * ibR[r];
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int i, int j) { return R.Q[(size_t)j * ld + rowof[i]]; },
+      [&](int i, int j, double v) { W1[(size_t)i * ld + j] = v * ibR[rowof[i]]; });
   lu_solve_blk(N, ld, W0, udiag, W1, tmp, S);
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    W1[(size_t)i * ld + j] *= ibL[i];
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int i, int j) { return W1[(size_t)i * ld + j]; },
+      [&](int i, int j, double v) { W1[(size_t)i * ld + j] = v * ibL[i]; });
   gemm_64<false, false>(S, N, N, N, Lf.Q, ld, W1, ld, Gout, ld);
   double part = 0.0;
   for (int i = threadIdx.x; i < N; i += kThreads) {
@@ -1851,11 +1871,9 @@ __device__ void v_wrap(const ChainDev& C, Real* G, const double* v, double a, Sm
     evi[x] = from_d<Real>(exp(-a * v[x]));
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    G[(size_t)x * ld + y] = rmul(rmul(G[(size_t)x * ld + y], evr[x]), evi[y]);
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int x, int y) { return G[(size_t)x * ld + y]; },
+      [&](int x, int y, Real g) { G[(size_t)x * ld + y] = rmul(rmul(g, evr[x]), evi[y]); });
 }
 
 // Hopping wrap: up  G <- E G E^-1;  down  G <- E^-1 G E.
@@ -2161,7 +2179,8 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
       for (int m = 0; m < nacc; ++m) {
         const Real bm = B[(size_t)m * ld + ic];
 #pragma unroll
-        for (int j = 0; j < kWin / 8; ++j) e[j] = rfma(A[(size_t)m * ld + ir[j]], bm, e[j]);
+        for (int j = 0; j < kWin / 8; ++j)
+          if (warp + 8 * j < W) e[j] = rfma(A[(size_t)m * ld + ir[j]], bm, e[j]);
       }
 #pragma unroll
       for (int j = 0; j < kWin / 8; ++j) w.E[(s * kWin + warp + 8 * j) * kWinLd + lane] = e[j];
@@ -2220,7 +2239,7 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
 #pragma unroll
           for (int j = 0; j < 6; ++j) {
             const int row = last + 1 + (warp - 2) + 6 * j;
-            if (row < kWin) blk[row * kWinLd] = rfma(w.a[r * kWin + row], bc, blk[row * kWinLd]);
+            if (row < W) blk[row * kWinLd] = rfma(w.a[r * kWin + row], bc, blk[row * kWinLd]);
           }
         }
       }
@@ -2317,11 +2336,9 @@ __device__ int chain_step_mixed(const ChainDev& C, int s, int t1, int t2, bool l
       slice_potential_global(C, s, t, S.v);
       for (int x = threadIdx.x; x < N; x += kThreads) evr[x] = from_d<dd>(exp(S.v[x]));
       __syncthreads();
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        X[(size_t)x * ld + y] = dd_mul(X[(size_t)x * ld + y], evr[x]);
-      }
-      __syncthreads();
+      each_element(
+          N, [&](int x, int y) { return X[(size_t)x * ld + y]; },
+          [&](int x, int y, dd v) { X[(size_t)x * ld + y] = dd_mul(v, evr[x]); });
       gemm_dd<false, false, false>(C, s, S, N, N, N, E, ld, X, ld, Y, ld, kCpEA, -1);
       dd* t_ = X; X = Y; Y = t_;
     }
@@ -2331,11 +2348,9 @@ __device__ int chain_step_mixed(const ChainDev& C, int s, int t1, int t2, bool l
       slice_potential_global(C, s, t, S.v);
       for (int x = threadIdx.x; x < N; x += kThreads) evr[x] = from_d<dd>(exp(S.v[x]));
       __syncthreads();
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        Y[(size_t)x * ld + y] = dd_mul(Y[(size_t)x * ld + y], evr[x]);
-      }
-      __syncthreads();
+      each_element(
+          N, [&](int x, int y) { return Y[(size_t)x * ld + y]; },
+          [&](int x, int y, dd v) { Y[(size_t)x * ld + y] = dd_mul(v, evr[x]); });
       dd* t_ = X; X = Y; Y = t_;
     }
   }
@@ -2366,15 +2381,14 @@ __device__ int green_from_udv_mixed(const ChainDev& C, int s, UDV R, UDV Lf, dou
   }
   __syncthreads();
   // Mid (float pairs, scale factors applied in FP64) in W0; right-hand side in W1
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    const double dR = R.D[i], dL = Lf.D[j];
-    const double dsR = dR > 1.0 ? 1.0 : dR, dsL = dL > 1.0 ? 1.0 : dL;
-    const double qq = to_d(W0d[(size_t)i * ld + j]);
-    const double tt = to_d(W1d[(size_t)i * ld + j]);
-    W0d[(size_t)i * ld + j] = from_d<dd>(qq * (ibR[i] * ibL[j]) + dsR * tt * dsL);
-  }
-  __syncthreads();
+  struct Pair { dd q, t; };
+  each_element(
+      N, [&](int i, int j) { return Pair{W0d[(size_t)i * ld + j], W1d[(size_t)i * ld + j]}; },
+      [&](int i, int j, Pair v) {
+        const double dR = R.D[i], dL = Lf.D[j];
+        const double dsR = dR > 1.0 ? 1.0 : dR, dsL = dL > 1.0 ? 1.0 : dL;
+        W0d[(size_t)i * ld + j] = from_d<dd>(to_d(v.q) * (ibR[i] * ibL[j]) + dsR * to_d(v.t) * dsL);
+      });
   double ldm;
   int smi;
   int* rowof = S.qinv;
@@ -2382,19 +2396,14 @@ __device__ int green_from_udv_mixed(const ChainDev& C, int s, UDV R, UDV Lf, dou
   dd* tmpd = reinterpret_cast<dd*>(wmat(C, s, 9));
   if (lu_factor_blk(N, ld, W0d, rowof, udiag, tmpd, ldm, smi, S)) return 1;
   // right-hand side Db_R^-1 Q_R^T with the LU row interchanges applied
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    const int r = rowof[i];
-    W1d[(size_t)i * ld + j] = from_d<dd>(R.Q[(size_t)j * ld + r] * ibR[r]);
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int i, int j) { return R.Q[(size_t)j * ld + rowof[i]]; },
+      [&](int i, int j, double v) { W1d[(size_t)i * ld + j] = from_d<dd>(v * ibR[rowof[i]]); });
   lu_solve_blk(N, ld, W0d, udiag, W1d, tmpd, S);
   dd* Yd = reinterpret_cast<dd*>(wmat(C, s, 9));
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    Yd[(size_t)i * ld + j] = from_d<dd>(to_d(W1d[(size_t)i * ld + j]) * ibL[i]);
-  }
-  __syncthreads();
+  each_element(
+      N, [&](int i, int j) { return W1d[(size_t)i * ld + j]; },
+      [&](int i, int j, dd v) { Yd[(size_t)i * ld + j] = from_d<dd>(to_d(v) * ibL[i]); });
   gemm_dd<false, false, false>(C, s, S, N, N, N, QLd, ld, Yd, ld, reinterpret_cast<dd*>(Gout), ld);
   dd_to_d_inplace(N, ld, Gout);
   double part = 0.0;
@@ -2442,14 +2451,15 @@ __device__ void stabilise(ChainDev& C, int s, int j, bool up, Real* G, Smem& S, 
   }
   tick(det, 7, t0);
   double mx = 0.0, sm = 0.0;
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int x = e / N, y = e - x * N;
-    const double gf = Gf[(size_t)x * ld + y];
-    const double dg = fabs(gf - to_d(G[(size_t)x * ld + y]));
-    mx = fmax(mx, dg);
-    sm += dg;
-    G[(size_t)x * ld + y] = from_d<Real>(gf);
-  }
+  struct Both { double fresh; Real wrapped; };
+  each_element(
+      N, [&](int x, int y) { return Both{Gf[(size_t)x * ld + y], G[(size_t)x * ld + y]}; },
+      [&](int x, int y, Both v) {
+        const double dg = fabs(v.fresh - to_d(v.wrapped));
+        mx = fmax(mx, dg);
+        sm += dg;
+        G[(size_t)x * ld + y] = from_d<Real>(v.fresh);
+      });
   ev_max = block_max(mx, S.red);
   ev_sum = block_sum(sm, S.red);
   fresh_sign = sg;

@@ -115,21 +115,18 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
       copy_udv_to_slot(C, s, j, dq);
     } else {
       // G(0,tau) = G(0,tau-1) e^{-V} E^-1
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        G0t[(size_t)x * ld + y] *= S.hv[y];
-      }
-      __syncthreads();
+      each_element(
+          N, [&](int x, int y) { return G0t[(size_t)x * ld + y]; },
+          [&](int x, int y, double v) { G0t[(size_t)x * ld + y] = v * S.hv[y]; });
       gemm_64<false, false>(S, N, N, N, G0t, ld, C.Einv[s], ld, T1, ld, -1, kCpEiB);
       double* t_ = G0t; G0t = T1; T1 = t_;
     }
     // Z = G(tau-1,0) Gamma^T G(0,tau)
     gemm_64<false, false>(S, N, N, N, Gt0, ld, Gam, ld, T1, ld);
     gemm_64<false, false>(S, N, N, N, T1, ld, G0t, ld, Z, ld);
-    for (int e = threadIdx.x; e < N * N; e += kThreads) {
-      const int x = e / N, y = e - x * N;
-      SE[(size_t)x * ld + y] += S.ev[x] * Z[(size_t)x * ld + y];
-    }
+    each_element(
+        N, [&](int x, int y) { return make_double2(SE[(size_t)x * ld + y], Z[(size_t)x * ld + y]); },
+        [&](int x, int y, double2 v) { SE[(size_t)x * ld + y] = fma(S.ev[x], v.y, v.x); });
     for (int k = threadIdx.x; k < C.MV; k += kThreads) {
       const int i = C.site[k];
       double acc = 0.0;
@@ -142,11 +139,9 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
     if (stab) {
       double* t_ = Gt0; Gt0 = T2; T2 = t_;
     } else {
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        Gt0[(size_t)x * ld + y] *= S.ev[x];
-      }
-      __syncthreads();
+      each_element(
+          N, [&](int x, int y) { return Gt0[(size_t)x * ld + y]; },
+          [&](int x, int y, double v) { Gt0[(size_t)x * ld + y] = v * S.ev[x]; });
       gemm_64<false, false>(S, N, N, N, C.E[s], ld, Gt0, ld, T1, ld, kCpEA, -1);
       double* t_ = Gt0; Gt0 = T1; T1 = t_;
     }

@@ -80,13 +80,17 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
         S.hv[x] = exp(-S.v[x]);
       }
       __syncthreads();
-      for (int e = threadIdx.x; e < N * N; e += kThreads) {
-        const int x = e / N, y = e - x * N;
-        Gt0[(size_t)x * ld + y] *= S.ev[x];
-        G0t[(size_t)x * ld + y] *= S.hv[y];
-        Gtt[(size_t)x * ld + y] *= S.ev[x] * S.hv[y];
-      }
-      __syncthreads();
+      struct Three { double a, b, c; };
+      each_element(
+          N,
+          [&](int x, int y) {
+            return Three{Gt0[(size_t)x * ld + y], G0t[(size_t)x * ld + y], Gtt[(size_t)x * ld + y]};
+          },
+          [&](int x, int y, Three v) {
+            Gt0[(size_t)x * ld + y] = v.a * S.ev[x];
+            G0t[(size_t)x * ld + y] = v.b * S.hv[y];
+            Gtt[(size_t)x * ld + y] = v.c * (S.ev[x] * S.hv[y]);
+          });
       gemm_64<false, false>(S, N, N, N, C.E[s], ld, Gt0, ld, T1, ld, kCpEA, -1);
       { double* t_ = Gt0; Gt0 = T1; T1 = t_; }
       gemm_64<false, false>(S, N, N, N, G0t, ld, C.Einv[s], ld, T1, ld, -1, kCpEiB);
