@@ -53,7 +53,7 @@ typedef enum {
   DQMC_EUNSTABLE = 4, /* stabilisation failed, or max|G_wrap - G_fresh|
                          exceeded dqmc_run_opts.unstable_threshold             */
   DQMC_ETIMEOUT = 5,  /* a bounded device wait gave up (the tensor-core products
-                         of DQMC_PREC_MIXED_TC wait on their copies and MMAs) */
+                         wait on their copies and MMAs)                       */
   DQMC_ESTATE = 6     /* the call is not valid in the context's state          */
 } dqmc_status;
 
@@ -61,9 +61,13 @@ typedef enum { DQMC_FIELD_ISING = 1, DQMC_FIELD_HS4 = 2 } dqmc_field_type;
 
 /* Arithmetic of each precision mode.  The scales D of the UDV chains (which
  * reach e^100 and more) are FP64 in every mode.
- *   DQMC_PREC_FP64: everything in FP64: working G, wraps, delayed updates, the
- *     B-chain products, the pivoted QR, the T update, (1 + UDV)^-1 and log|det|
- *     (Sec. 2.3).
+ *   DQMC_PREC_FP64: working G, wraps, delayed updates, the B-chain products, the
+ *     pivoted QR, the T update, (1 + UDV)^-1 and log|det| (Sec. 2.3) are FP64.
+ *     From 32 sites the N x N x N products run on the tensor cores (tcgen05) as
+ *     exact-split BF16 products of FP64 operands: eight 8-bit digits each, 63 bits
+ *     under the largest entry of a row of the left and a column of the right
+ *     factor, recombined as one integer and rounded once to FP64.  Their error
+ *     against 64 bits is below that of a chain of FP64 multiply-adds.
  *   DQMC_PREC_FP32: working G, wraps and delayed updates in plain FP32; the
  *     stabilisation in FP64 as above.  Round-off grows by the condition number of
  *     the unstabilised slice product (Sec. 2.3), so at strong coupling the wrapped
@@ -71,9 +75,9 @@ typedef enum { DQMC_FIELD_ISING = 1, DQMC_FIELD_HS4 = 2 } dqmc_field_type;
  *   DQMC_PREC_MIXED: float pairs (hi + lo, about 48 significant bits, error-free
  *     transformations on the FP32 pipes) for the working G, the wraps and the
  *     delayed updates, and also for the stabilisation: the B-chain and T-update
- *     products, the Householder QR (pivot chosen in FP64 on the FP64-scaled column
- *     norms), Q^T Q, T T^T, the LU of the middle matrix and the solves, with the
- *     FP64 scales D kept apart.  This departs from an FP64 stabilisation: the
+ *     products, the Householder QR (in panels of 4 columns, pivots chosen on the
+ *     FP64-scaled column norms), Q^T Q, T T^T, the LU of the middle matrix and the
+ *     solves, with the FP64 scales D kept apart.  This departs from an FP64 stabilisation: the
  *     float-pair products accumulate about 42 bits, and the stable G then differs
  *     from an FP64 recompute by up to ~30x the FP64 round-off amplified by the
  *     conditioning (measured: 1e-9 at U = 4 - 6, beta = 4 - 8, n_wrap = 10 on
@@ -304,8 +308,9 @@ dqmc_status dqmc_measure_corr(dqmc_ctx* ctx, const int32_t* pair_class, const in
  *     grad_K  [n_cfg][n_flavors][N][N]: d/dK^s_xy with K_xy and K_yx varied
  *             together (x != y); d/dK_xx on the diagonal
  *     grad_U  [n_cfg][n_flavors]: d/dU through the couplings c(field).
- * The workspace (one FP64 chain per configuration) is allocated and freed by
- * the call, which waits for its work.  Errors: DQMC_EINVAL (model_index out of
+ * The workspace (one FP64 chain per configuration) stays with the context for the
+ * next call, up to 1 GiB, and is freed with it; a larger one is freed by the call.
+ * The call waits for its work.  Errors: DQMC_EINVAL (model_index out of
  * range, n_cfg < 1, a null pointer, an invalid field value), DQMC_ENOMEM,
  * DQMC_ECUDA, DQMC_EUNSTABLE (a singular matrix in the stabilisation of a
  * configuration). */
