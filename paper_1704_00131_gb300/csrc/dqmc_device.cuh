@@ -8,9 +8,9 @@
 // runs in the flavor's own CTA.
 //
 // Precision: the working Green function, the wraps and the delayed updates are
-// templated on `Real` (double for the plain FP64 path, float for the mixed
-// path); the stabilisation chain (B-products, pivoted QR, T update, the stable
-// (1 + UDV)^-1 and log|det|) is always FP64.
+// templated on `Real` (double, float, or float pairs); the stabilisation chain
+// (B-products, pivoted QR, T update, the stable (1 + UDV)^-1 and log|det|) is FP64
+// or, in the float-pair modes, float pairs with FP64 scales.
 //
 // Method (ALF 1.0 documentation, arXiv:1704.00131):
 //   B_tau = exp(-dtau K) exp(V_tau)                       Sec. 2.1, Eq. of B_tau
@@ -35,9 +35,10 @@
 #include "../../include/dqmc.h"
 #include "dqmc_internal.h"
 
-// DQMC_WITH_UMMA: 1 compiles the tensor-core product path into the float-pair
-// kernels (the unit of DQMC_PREC_MIXED_TC), 0 leaves it out (the unit of
-// DQMC_PREC_MIXED, whose kernels then keep their registers for the SIMT tiles).
+// DQMC_WITH_UMMA: 1 compiles the float pairs' tensor-core products into the
+// float-pair kernels (the unit of DQMC_PREC_MIXED_TC), 0 leaves them out (the unit of
+// DQMC_PREC_MIXED, whose kernels then keep their registers for the SIMT tiles).  The
+// FP64 products' are in every unit.
 #ifndef DQMC_WITH_UMMA
 #define DQMC_WITH_UMMA 1
 #endif
@@ -137,24 +138,6 @@ __device__ __forceinline__ double block_max(double v, double* red) {
   for (int w = 1; w < kThreads / 32; ++w) r = fmax(r, red[w]);
   return r;
 }
-// argmax of v over the block, ties to the lowest index; returns the index.
-__device__ __forceinline__ int block_argmax(double v, int idx, double* red, int* ired) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-    if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5] = v; ired[threadIdx.x >> 5] = idx; }
-  __syncthreads();
-  double bv = red[0];
-  int bi = ired[0];
-#pragma unroll
-  for (int w = 1; w < kThreads / 32; ++w)
-    if (red[w] > bv || (red[w] == bv && ired[w] < bi)) { bv = red[w]; bi = ired[w]; }
-  return bi;
-}
 
 // --------------------------------------------------------------------------
 // Float-float ("double-word") numbers: x = hi + lo with |lo| <= ulp(hi)/2,
@@ -236,7 +219,9 @@ __device__ __forceinline__ dd rsub(dd a, dd b) { return dd_add(a, {-b.hi, -b.lo}
 // Type of the acceptance ratios and of the diagonal they come from: float pairs
 // where G is held in float pairs (an FP64 instruction of a warp holds its
 // scheduler's FP64 unit for 65 cycles, a dependent float-pair operation takes
-// about 30), FP64 otherwise.
+// about 30), FP64 otherwise.  The ratios are then as exact as the diagonal they are
+// formed from: a pair rounds at 2^-47, the wrapped G between two stabilisations is
+// off by 1e-8 on average.
 template <typename Real>
 struct RatioOf { using type = double; };
 template <>
@@ -2318,10 +2303,10 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
 }
 
 // ---- stabilisation with float-float products (mixed path) ----------------
-// Same steps as chain_step / green_from_udv; the dense products (the B chain,
-// T = D^-1 R P^T T, Q_R^T Q_L, T_R T_L^T, Q_L Y) run as float-float GEMMs on the
-// FP32 pipes, the pivoted QR, Q accumulation, LU and triangular solves stay
-// FP64.  Storage matrices (Q, T) remain FP64.
+// Same steps as chain_step / green_from_udv in float pairs: the dense products (the B
+// chain, T = D^-1 R P^T T, Q_R^T Q_L, T_R T_L^T, Q_L Y), the pivoted QR, Q, LU and
+// triangular solves; the scales D and the pivots' norms are FP64, and the stored Q
+// and T are widened to FP64.
 __device__ int chain_step_mixed(const ChainDev& C, int s, int t1, int t2, bool left, UDV src, Smem& S,
                                              long long* det = nullptr) {
   long long t0 = clock64();

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads) fresh_green_noalloc_kernel(ChainDev 
   int* ibase = reinterpret_cast<int*>(ident + 2 * (size_t)N * ld + ld);
   Cl.slots[s] = slot;
   Cl.ident = ident;
-  Cl.iwork[s] = ibase;             // perm [ld], piv [ld]
+  Cl.iwork[s] = ibase;             // pivot order [ld]
   Cl.slot_detq[s] = ibase + 2 * ld;
   // the array keeps the previous call's contents: rebuild the identity UDV
   for (int e = threadIdx.x; e < N * N; e += kThreads) {

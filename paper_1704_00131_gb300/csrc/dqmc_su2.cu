@@ -85,13 +85,6 @@ __device__ __forceinline__ double2 block_zsum(double2 v, double* red) {
   return make_double2(re, im);
 }
 
-// a / b without the scaling of zdiv, for |b| of order one (ratios, pivots of Mid)
-__device__ __forceinline__ double2 zdiv_unit(double2 a, double2 b) {
-  return zscal(quick_div(1.0, zabs2(b)), zmul(a, zconj(b)));
-}
-// |a| where the squares neither overflow nor vanish
-__device__ __forceinline__ double zabs_unit(double2 a) { return sqrt(zabs2(a)); }
-
 // A warp's FP64 instruction holds its scheduler's FP64 unit for 65 cycles whatever its
 // active lanes: scalars that all threads need (reflector norms, pivots' inverses,
 // update factors) are formed by one warp and passed through shared memory, pivot
