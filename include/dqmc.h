@@ -126,7 +126,7 @@ typedef struct {
   int64_t spin_limit;         /* SM cycles before a bounded device wait gives up
                                  (DQMC_ETIMEOUT); 0: about one second            */
   int32_t tc_min_sites;       /* DQMC_PREC_MIXED_TC: chains of fewer sites use the
-                                 float-pair SIMT products (0: 96, where the tensor-
+                                 float-pair SIMT products (0: 72, where the tensor-
                                  core product overtakes them on GB300)            */
   int32_t dd_tile;            /* float-pair SIMT products: output tiles of 48 x 48
                                  (3) or 64 x 64 (4) per CTA; 0: the one that pads

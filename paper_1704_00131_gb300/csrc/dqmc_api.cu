@@ -27,8 +27,11 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 size_t pad_to(size_t n, size_t q) { return (n + q - 1) / q * q; }
 
 // Site count from which chains of a DQMC_PREC_MIXED_TC context run their N^3
-// products on the tensor cores (smaller ones keep the float-pair SIMT tiles).
-constexpr int kDefaultTcMinSites = 96;
+// products on the tensor cores (smaller ones keep the float-pair SIMT tiles).  Sweep of
+// 128 chains, L = 20, SIMT tiles against tensor cores: N = 49 11.2 and 10.7 ms, 64 13.6
+// and 13.3, 72 26.9 and 19.5, 90 34.8 and 25.7, 100 60.0 and 36.8; of 8 chains: 49 7.7 and
+// 8.3, 64 9.5 and 10.2, 72 17.4 and 14.9.
+constexpr int kDefaultTcMinSites = 72;
 int tc_min_sites(const dqmc_run_opts& o) { return o.tc_min_sites > 0 ? o.tc_min_sites : kDefaultTcMinSites; }
 // ... and from which FP64 products run on them, in every context (the FP64 kernels
 // serve all precisions): below it the FP64 pipe's N^3 / 1.65 cycles are less than
