@@ -638,6 +638,8 @@ __device__ __forceinline__ bool umma_begin(ChainDev& C, int s, Smem& S, bool wan
   S.ps = want_dd ? C.ps[s] : nullptr;
   S.ps64 = want_64 ? C.ps64[s] : nullptr;
   const bool on = S.ps != nullptr || S.ps64 != nullptr;
+  umma_acquire_maps(S.ps);
+  umma_acquire_maps(S.ps64);
   if (on) umma_alloc(S.um);
   return on;
 }

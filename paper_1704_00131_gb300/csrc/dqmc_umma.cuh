@@ -149,6 +149,11 @@ __device__ __forceinline__ void tma_load_block(void* dst, const CUtensorMap* tm,
       "l"(reinterpret_cast<uint64_t>(tm)), "r"(0), "r"(row), "r"(smem_u32(bar))
       : "memory");
 }
+// A tensor map in global memory that the host wrote (here by a copy, possibly over another
+// map at the same address): ordered before the block's tiled copies that use it.
+__device__ __forceinline__ void tensor_map_acquire(const CUtensorMap* tm) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
+}
 __device__ __forceinline__ void umma_bf16(uint32_t dtm, uint64_t ad, uint64_t bd, uint32_t id, uint32_t acc) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtm),
@@ -169,6 +174,15 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
   for (int q = 0; q < 4; ++q) v[q] = __uint_as_float(r[q]);
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The tensor maps of a plane set, acquired by the warp that issues the copies: a plane set
+// lies in memory that is written again (the adjoints' kept workspace, an arena that a
+// context before this one had), and a descriptor cached from then describes other planes.
+__device__ inline void umma_acquire_maps(const PlaneSet* ps) {
+  if (ps == nullptr || (threadIdx.x >> 5) != 1) return;
+  for (int q = 0; q < 2; ++q) tensor_map_acquire(&ps->tm_pl[q]);
+  for (int q = 0; q < kCpSets; ++q) tensor_map_acquire(&ps->tm_cp[q]);
+}
 
 // Tensor memory of the CTA: warp 0 allocates kUmmaCols columns (at most two
 // CTAs of a product kernel share an SM, so the 512 columns of an SM never run
