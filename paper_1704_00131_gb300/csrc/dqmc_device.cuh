@@ -786,18 +786,24 @@ __device__ __forceinline__ float log2_rough(double x) {
   const float m = __int_as_float(((hi & 0xfffff) << 3) | 0x3f800000);
   return ex == 0 ? -3.0e38f : (float)(ex - 1023) + __log2f(m);
 }
-// order of a column: log2 of its norm (from the square) and scale, NaN last
+// order of a column: log2 of its norm (from the square) and scale; zero and NaN columns
+// last, but finite: above the -Inf of a column that is no candidate
+constexpr float kLeastKey = -3.4e38f;
 __device__ __forceinline__ float column_key(float norm2, float lsc) {
-  const float k = 0.5f * log2f(norm2) + lsc;
-  return k == k ? k : -3.4e38f;
+  return fmaxf(0.5f * log2f(norm2) + lsc, kLeastKey);  // (fmaxf drops a NaN)
 }
 __device__ __forceinline__ float column_key(double norm2, float lsc) {
-  const float k = norm2 > 0.0 ? 0.5f * log2_rough(norm2) + lsc : -3.3e38f;
-  return k == k ? k : -3.4e38f;
+  return norm2 > 0.0 ? fmaxf(0.5f * log2_rough(norm2) + lsc, kLeastKey) : kLeastKey;
 }
 __device__ __forceinline__ float column_key(dd norm2, float lsc) { return column_key(fmaxf(norm2.hi, 0.f), lsc); }
 __device__ __forceinline__ float as_float(double x) { return (float)x; }
 __device__ __forceinline__ float as_float(dd x) { return x.hi; }
+// a downdated squared norm below 2^-26 of its last full value (or not positive)
+__device__ __forceinline__ bool norm_spent(double n, double full) {
+  const int a = __double2hiint(n), b = __double2hiint(full);
+  return a <= 0 || b - a > (26 << 20);
+}
+__device__ __forceinline__ bool norm_spent(dd n, dd full) { return !(n.hi > 1.4901161e-8f * full.hi); }
 
 // Keys (log2 of the scaled column norms, by list position) of the columns of M = X
 // diag(dsc), and log2 dsc (by column).  The sums of squares stay in FP32: X is a
@@ -996,7 +1002,9 @@ __device__ __forceinline__ T* panel_tri(const Smem& S) { return reinterpret_cast
 // Pivoting: a panel takes the columns of largest remaining scaled norm, renewed from the
 // updated matrix, and orders them by their downdated norms while it is factorised: the
 // order of Businger and Golub's pivoting but for a column that overtakes a panel's
-// last ones within the panel.  (Sorting the columns once before an unpivoted
+// last ones within the panel.  Norms that cancel below 2^-26 of the square they were
+// downdated from are formed again from the panel (LAPACK's xGEQPF rule): in float pairs
+// the rest is rounding error, of either sign.  (Sorting the columns once before an unpivoted
 // factorisation is cheaper still, but made the wrapped G's drift up to 3.5 times
 // larger: the first block of a chain has no graded scales to sort by.)
 //
@@ -1025,6 +1033,7 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
   int* rank = reinterpret_cast<int*>(S.spare);  // [N]
   int* pos_of = S.ired + 16;                    // [pw] position in the panel of its columns (-1: to come)
   int* next_p = S.ired;                         // [2] pivot of the next step
+  int* renew = S.ired + 2;                      // [1] the columns' norms are to be formed again
   int detq = 1;
   column_keys<T>(N, ld, X, dsc, key, lsc, S);
   for (int j = tid; j < N; j += kThreads) list[j] = j;
@@ -1079,8 +1088,9 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
     if (tid < pw) pos_of[tid] = -1;
     if (tid == 0) next_p[0] = 0;  // the selection is in order
     __syncthreads();
-    // squared norms of the panel's columns (warp 0, lane q), downdated step by step
-    T nrm2 = from_zero<T>();
+    // squared norms of the panel's columns (warp 0, lane q), downdated step by step, and
+    // their last full values
+    T nrm2 = from_zero<T>(), full2 = from_zero<T>();
     const float lscq = (q < nb) ? lsc[list[k0 + q]] : 0.f;
     auto over_groups = [](T v) {  // the sum over a warp's lanes of the same q
 #pragma unroll
@@ -1094,9 +1104,21 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
       a = over_groups(a);
       if (lane < pw) red[warp * pw + lane] = a;
       __syncthreads();
-      if (warp == 0) nrm2 = over_groups(red[lane]);
+      if (warp == 0) full2 = nrm2 = over_groups(red[lane]);
       __syncthreads();
     }
+    // the column to come of largest norm (ties: the lowest), for warp 0
+    auto next_pivot = [&](bool done) {
+      float k = done ? -INFINITY : column_key(nrm2, lscq);
+      int kp = q;
+#pragma unroll
+      for (int o = pw / 2; o; o >>= 1) {
+        const float ok = __shfl_xor_sync(0xffffffffu, k, o);
+        const int op = __shfl_xor_sync(0xffffffffu, kp, o);
+        if (ok > k || (ok == k && op < kp)) { k = ok; kp = op; }
+      }
+      return kp;
+    };
     for (int c = 0; c < nb; ++c) {
       const int p = next_p[c & 1];
       const T* x = Vp + p * ldp;
@@ -1127,16 +1149,11 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
         // the next pivot: largest downdated norm among the columns to come
         const T rc = rfma(w, v0, yc);
         nrm2 = rfma(rneg(rc), rc, nrm2);
-        float k = done ? -3.5e38f : column_key(nrm2, lscq);
-        int kp = q;
-#pragma unroll
-        for (int o = pw / 2; o; o >>= 1) {
-          const float ok = __shfl_xor_sync(0xffffffffu, k, o);
-          const int op = __shfl_xor_sync(0xffffffffu, kp, o);
-          if (ok > k || (ok == k && op < kp)) { k = ok; kp = op; }
-        }
+        const int kp = next_pivot(done);
+        const bool spent = __any_sync(0xffffffffu, !done && norm_spent(nrm2, full2));
         __syncwarp();
         if (lane == 0) {
+          *renew = spent;
           sc[(c & 1) * 2] = v0;
           sc[(c & 1) * 2 + 1] = beta;
           pos_of[p] = c;
@@ -1163,6 +1180,23 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
       }
       __syncthreads();
       if (tid == 0) Vp[p * ldp + c] = v0;
+      if (*renew) {
+        const bool done = q >= nb || pos_of[q] >= 0;
+        T a2 = from_zero<T>();
+        if (!done) {
+          const T* y = Vp + q * ldp;
+          for (int r = c + 1 + rg; r < rows; r += RG) a2 = rfma(y[r], y[r], a2);
+        }
+        a2 = over_groups(a2);
+        if (lane < pw) red[warp * pw + lane] = a2;
+        __syncthreads();
+        if (warp == 0) {
+          full2 = nrm2 = over_groups(red[lane]);
+          const int kp = next_pivot(done);
+          if (lane == 0) next_p[(c & 1) ^ 1] = kp;
+        }
+        __syncthreads();
+      }
     }
     __syncthreads();
     // R's strict upper part and the vectors back to X; V gets its zeros above the diagonal
