@@ -2066,6 +2066,7 @@ __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const d
 constexpr int kWin = 32;       // positions per window: one warp lane each
 constexpr int kWinAcc = 16;    // acceptances per window (the vectors' shared memory)
 constexpr int kVecChunk = 8;   // flips whose vectors one thread forms together
+static_assert(kMaxFlavors + 6 == kThreads / 32 && 6 * 6 >= kWin, "six warps renew a window's rows in six turns");
 constexpr int kWinLd = kWin + 1;  // row stride of a block: rows and columns without bank conflicts
 
 // Shared memory of a window: the idle product panels (S.gemm) and the QR's
@@ -2252,14 +2253,15 @@ __device__ void update_slice(ChainDev& C, int s, int tau, int dir, const SweepPa
           const Ratio df = shfl(delw, f), Rf = shfl(Rw, f);
           mf = rneg(ratio_to<Real>(quick_div(df, Rf)));
         }
-      } else if (last >= 0) {
-        // the other warps meanwhile: the rows after the last acceptance of both blocks
+      } else if (last >= 0 && warp >= kMaxFlavors) {
+        // the other warps meanwhile: the rows after the last acceptance of the flavors'
+        // blocks, each row by one of six warps (of a single flavor, warp 1 sits out)
         for (int r = 0; r < nfl; ++r) {
           const Real bc = w.b[r * kWin + lane];
           Real* blk = w.E + r * kWin * kWinLd + lane;
 #pragma unroll
           for (int j = 0; j < 6; ++j) {
-            const int row = last + 1 + (warp - 2) + 6 * j;
+            const int row = last + 1 + (warp - kMaxFlavors) + 6 * j;
             if (row < W) blk[row * kWinLd] = rfma(w.a[r * kWin + row], bc, blk[row * kWinLd]);
           }
         }
