@@ -805,10 +805,25 @@ __device__ __forceinline__ bool norm_spent(double n, double full) {
 }
 __device__ __forceinline__ bool norm_spent(dd n, dd full) { return !(n.hi > 1.4901161e-8f * full.hi); }
 
+// Squared norm of rows r0.. of column j, in FP64 (one thread).
+template <typename T>
+__device__ __noinline__ double column_norm2(int N, int ld, const T* X, int j, int r0) {
+  double a = 0.0;
+#pragma unroll 4
+  for (int i = r0; i < N; ++i) {
+    const double x = to_d(X[(size_t)i * ld + j]);
+    a = fma(x, x, a);
+  }
+  return a;
+}
+// Whether an FP32 sum of squares is good for a key: neither overflown nor (squares of
+// entries below 1e-19) underflown.
+__device__ __forceinline__ bool norm2_in_range(float a) { return a > 0x1.0p-100f && a < INFINITY; }
+
 // Keys (log2 of the scaled column norms, by list position) of the columns of M = X
-// diag(dsc), and log2 dsc (by column).  The sums of squares stay in FP32: X is a
-// product of n_wrap slices with an orthogonal matrix, far inside its range, and the
-// keys only order the columns (NaN last).
+// diag(dsc), and log2 dsc (by column).  The keys only order the columns, so the sums of
+// squares are formed in FP32; a column whose sum leaves its range is summed in FP64 (X is
+// a product of n_wrap slices with an orthogonal matrix, usually far inside).
 template <typename T>
 __device__ void column_keys(int N, int ld, const T* X, const double* dsc, float* key, float* lsc, Smem& S) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -836,7 +851,7 @@ __device__ void column_keys(int N, int ld, const T* X, const double* dsc, float*
 #pragma unroll
       for (int w = 0; w < nw; ++w) a += part[w * 32 + lane];
       lsc[j] = log2_rough(dsc[j]);
-      key[j] = column_key(a, lsc[j]);
+      key[j] = norm2_in_range(a) ? column_key(a, lsc[j]) : column_key(column_norm2<T>(N, ld, X, j, 0), lsc[j]);
     }
     __syncthreads();
   }
@@ -958,7 +973,8 @@ __device__ void panel_apply(int N, int ld, T* A, int r0, int j0, int nb, const T
       __syncthreads();
       if (act && g == 0) {
         for (int h = 1; h < G; ++h) n2 += part[h * cw + jj];
-        key[c0 + jj] = column_key(n2, lsc[j]);
+        key[c0 + jj] = norm2_in_range(n2) ? column_key(n2, lsc[j])
+                                          : column_key(column_norm2<T>(N, ld, A, j, r0 + nb), lsc[j]);
       }
       __syncthreads();
     }
@@ -988,6 +1004,19 @@ __device__ __forceinline__ void reflector_scalars(T x0, T xn2, T& alpha, T& v0, 
   beta = quick_div(unit<T>(true), rfma(rabs(x0), xn, xn2));  // v^T v = 2 (|x|^2 + |x_0| |x|)
 }
 
+// Power of two that brings a panel's column to a norm of about one, from the log2 of its
+// norm, so that squares of float pairs neither underflow (entries below 1e-19 would lose
+// their reflector, from 1e-16 bits of it) nor overflow.  Exact both ways; FP64 needs none.
+__device__ __forceinline__ int panel_shift(float log2_norm, double) { return 0; }
+__device__ __forceinline__ int panel_shift(float log2_norm, dd) {
+  return fabsf(log2_norm) < 150.f ? max(-120, min(120, __float2int_rn(log2_norm))) : 0;
+}
+__device__ __forceinline__ double times_pow2(double x, int) { return x; }
+__device__ __forceinline__ dd times_pow2(dd x, int e) {
+  const float f = __int_as_float((127 + e) << 23);
+  return {x.hi * f, x.lo * f};
+}
+
 // T of the panel at hand, behind qr_blocked's other entries of S.qred.
 template <typename T>
 __device__ __forceinline__ T* panel_tri(const Smem& S) { return reinterpret_cast<T*>(S.qred) + 256; }
@@ -995,7 +1024,8 @@ __device__ __forceinline__ T* panel_tri(const Smem& S) { return reinterpret_cast
 // Pivoted Householder QR of M = X diag(dsc), X N x N, in panels: reflections act on rows
 // and commute with the column scales, so the factors are X's, R_M = R_X diag(dsc[perm]).
 // Columns do not move: perm[k] is the column at position k, R_kj sits at X[k][perm[j]],
-// reflector k's vector below row k of column perm[k] (its leading entry in vk0[k]).
+// reflector k's vector below row k of column perm[k] (its leading entry in vk0[k]); in
+// float pairs each vector is that of its column scaled to norm one (panel_shift).
 // tri[panel][kPanel][kPanel]: the triangular factors T of the panels' products H_0 .. H_{nb-1} =
 // 1 - V T V^T (compact WY, Schreiber & Van Loan 1989).  Returns det(Q) = (-1)^#reflectors.
 //
@@ -1079,9 +1109,11 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
         }
       __syncthreads();
     }
+    // (a thread's panel column is q, here and below)
+    const int shift = (q < nb) ? panel_shift(key[k0 + q] - lsc[list[k0 + q]], T{}) : 0;
     for (int e = tid; e < rows * pw; e += kThreads) {
       const int r = e / pw, c = e - r * pw;
-      if (c < nb) Vp[c * ldp + r] = X[(size_t)(k0 + r) * ld + list[k0 + c]];
+      if (c < nb) Vp[c * ldp + r] = times_pow2(X[(size_t)(k0 + r) * ld + list[k0 + c]], -shift);
     }
     if (tid < pw * pw) Tm[tid] = from_zero<T>();
     if (tid < 2 * pw) zq[tid] = from_zero<T>();
@@ -1091,7 +1123,7 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
     // squared norms of the panel's columns (warp 0, lane q), downdated step by step, and
     // their last full values
     T nrm2 = from_zero<T>(), full2 = from_zero<T>();
-    const float lscq = (q < nb) ? lsc[list[k0 + q]] : 0.f;
+    const float lscq = (q < nb) ? lsc[list[k0 + q]] + (float)shift : 0.f;
     auto over_groups = [](T v) {  // the sum over a warp's lanes of the same q
 #pragma unroll
       for (int o = 16; o >= pw; o >>= 1) v = radd(v, shfl_xor(v, o));
@@ -1150,6 +1182,7 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
         const T rc = rfma(w, v0, yc);
         nrm2 = rfma(rneg(rc), rc, nrm2);
         const int kp = next_pivot(done);
+        const int shift_p = __shfl_sync(0xffffffffu, shift, p);
         const bool spent = __any_sync(0xffffffffu, !done && norm_spent(nrm2, full2));
         __syncwarp();
         if (lane == 0) {
@@ -1158,7 +1191,7 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
           sc[(c & 1) * 2 + 1] = beta;
           pos_of[p] = c;
           next_p[(c & 1) ^ 1] = kp;
-          X[(size_t)(k0 + c) * ld + list[k0 + p]] = alpha;  // R's diagonal
+          X[(size_t)(k0 + c) * ld + list[k0 + p]] = times_pow2(alpha, shift_p);  // R's diagonal
           vk0[k0 + c] = v0;
         }
       }
@@ -1202,7 +1235,8 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
     // R's strict upper part and the vectors back to X; V gets its zeros above the diagonal
     for (int e = tid; e < rows * pw; e += kThreads) {
       const int r = e / pw, c = e - r * pw;
-      if (c < nb && r != pos_of[c]) X[(size_t)(k0 + r) * ld + list[k0 + c]] = Vp[c * ldp + r];
+      if (c < nb && r != pos_of[c])
+        X[(size_t)(k0 + r) * ld + list[k0 + c]] = times_pow2(Vp[c * ldp + r], r < pos_of[c] ? shift : 0);
     }
     int col = 0, pc = 0;
     if (q < nb) { col = list[k0 + q]; pc = pos_of[q]; }
