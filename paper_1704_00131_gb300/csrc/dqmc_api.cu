@@ -81,6 +81,7 @@ struct dqmc_ctx {
   int ab_smem = 0;
   uint64_t sweep_counter = 0;
   int maxN = 0, maxld = 0, maxMV = 0;
+  std::vector<dqmc::PlaneSet> planes_h;
   double* scratch = nullptr;  // [nfl][maxN][maxN] FP64 for dqmc_greens
   unsigned char* grad_ws = nullptr;  // workspace of the adjoints, kept up to kKeptWorkspace bytes
   size_t grad_ws_bytes = 0;
@@ -210,11 +211,13 @@ int fill_plane_set(const ModelHost& M, int s, bool fp64, void* mem, dqmc::PlaneS
 
 // Plane sets of chains laid out over their scratch planes, copied to the device
 // memory `out` of plane_sets_bytes(chains); the chains get the device addresses
-// ([chain][flavor][float pairs, FP64]).
+// ([chain][flavor][float pairs, FP64]).  h: the host side of the copy, which may read it
+// until the stream has been waited for (a copy from pageable memory need not be staged
+// where the GPU reads host memory itself).
 size_t plane_sets_bytes(size_t chains) { return sizeof(dqmc::PlaneSet) * chains * dqmc::kMaxFlavors * 2; }
 dqmc_status plane_sets(dqmc_ctx* ctx, std::vector<ChainDev>& chains, const std::vector<int>& chain_model, bool pairs,
-                       dqmc::PlaneSet* out) {
-  std::vector<dqmc::PlaneSet> h(chains.size() * dqmc::kMaxFlavors * 2);
+                       dqmc::PlaneSet* out, std::vector<dqmc::PlaneSet>& h) {
+  h.assign(chains.size() * dqmc::kMaxFlavors * 2, dqmc::PlaneSet{});
   for (size_t c = 0; c < chains.size(); ++c) {
     const ModelHost& M = ctx->models[chain_model[c]];
     for (int s = 0; s < M.d.n_flavors; ++s)
@@ -579,7 +582,7 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   *out = ctx.release();
   c = *out;
   CUDA_TRY(c, cudaMalloc((void**)&c->planes_d, plane_sets_bytes(n_chains)));
-  if ((st = plane_sets(c, c->chains_h, c->chain_model, true, c->planes_d))) return st;
+  if ((st = plane_sets(c, c->chains_h, c->chain_model, true, c->planes_d, c->planes_h))) return st;
   CUDA_TRY(c, cudaMalloc((void**)&c->chains_d, sizeof(ChainDev) * n_chains));
   CUDA_TRY(c, cudaMemcpyAsync(c->chains_d, c->chains_h.data(), sizeof(ChainDev) * n_chains, cudaMemcpyHostToDevice,
                               c->stream));
@@ -799,6 +802,7 @@ dqmc_status build_class_lists(dqmc_ctx* ctx, const int32_t* pair_class, const in
 
 // Device copy of the class lists: one int buffer [csr | pairs | ccsr | cpairs | cncls].
 struct ClassListsDev {
+  std::vector<int> h;  // host side of the copy, until the stream has been waited for
   int* buf = nullptr;
   const int *csr = nullptr, *pairs = nullptr, *ccsr = nullptr, *cpairs = nullptr, *cncls = nullptr;
   ~ClassListsDev() { cudaFree(buf); }
@@ -812,7 +816,7 @@ dqmc_status upload_class_lists(dqmc_ctx* ctx, const ClassLists& L, ClassListsDev
     cudaGetLastError();
     return fail(ctx, DQMC_ENOMEM, "no device memory for the pair classes");
   }
-  std::vector<int> h;
+  std::vector<int>& h = D.h;
   h.reserve(n);
   h.insert(h.end(), L.csr.begin(), L.csr.end());
   h.insert(h.end(), L.pairs.begin(), L.pairs.end());
@@ -1081,7 +1085,12 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
     std::copy(M.eigval[s].begin(), M.eigval[s].end(), wh.begin() + (size_t)s * N);
   }
   dqmc_status st = DQMC_OK;
-  auto cleanup = [&]() { trim_grad_workspace(ctx); };
+  std::vector<dqmc::PlaneSet> planes_h;
+  // (on an error path copies from the call's host buffers may still be in flight)
+  auto cleanup = [&]() {
+    cudaStreamSynchronize(ctx->stream);
+    trim_grad_workspace(ctx);
+  };
 #define GRAD_TRY(expr)                                                                 \
   do {                                                                                 \
     cudaError_t e_ = (expr);                                                           \
@@ -1095,7 +1104,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   for (int c = 0; c < n_cfg; ++c)
     GRAD_TRY(cudaMemcpyAsync(ch[c].fields, fields + (size_t)c * L * MV, (size_t)L * MV, cudaMemcpyHostToDevice,
                              ctx->stream));
-  if ((st = plane_sets(ctx, ch, std::vector<int>(n_cfg, model_index), false, (dqmc::PlaneSet*)(ws + o_ps)))) {
+  if ((st = plane_sets(ctx, ch, std::vector<int>(n_cfg, model_index), false, (dqmc::PlaneSet*)(ws + o_ps), planes_h))) {
     cleanup();
     return st;
   }
@@ -1154,7 +1163,12 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
          *ew_d = (double*)(ws + o_ew), *gK_d = (double*)(ws + o_gK), *gU_d = (double*)(ws + o_gU),
          *ep_d = (double*)(ws + o_ep);
   dqmc_status st = DQMC_OK;
-  auto cleanup = [&]() { trim_grad_workspace(ctx); };
+  std::vector<dqmc::PlaneSet> planes_h;
+  // (on an error path copies from the call's host buffers may still be in flight)
+  auto cleanup = [&]() {
+    cudaStreamSynchronize(ctx->stream);
+    trim_grad_workspace(ctx);
+  };
 #define EGRAD_TRY(expr)                                                                \
   do {                                                                                 \
     cudaError_t e_ = (expr);                                                           \
@@ -1177,7 +1191,7 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
     std::copy(M.eigvec[s].begin(), M.eigvec[s].end(), Vh.begin() + (size_t)s * N * N);
     std::copy(M.eigval[s].begin(), M.eigval[s].end(), wh.begin() + (size_t)s * N);
   }
-  if ((st = plane_sets(ctx, ch, std::vector<int>(n_cfg, model_index), false, (dqmc::PlaneSet*)(ws + o_ps)))) {
+  if ((st = plane_sets(ctx, ch, std::vector<int>(n_cfg, model_index), false, (dqmc::PlaneSet*)(ws + o_ps), planes_h))) {
     cleanup();
     return st;
   }
