@@ -37,9 +37,6 @@ int tc_min_sites(const dqmc_run_opts& o) { return o.tc_min_sites > 0 ? o.tc_min_
 // serve all precisions): below it the FP64 pipe's N^3 / 1.65 cycles are less than
 // the split product's fixed cost.
 constexpr int kTc64MinSites = 32;
-bool pairs_on_tc(const dqmc_run_opts& o, int N) { return o.precision == DQMC_PREC_MIXED_TC && N >= tc_min_sites(o); }
-bool fp64_on_tc(int N) { return N >= kTc64MinSites; }
-
 
 struct ModelHost {
   dqmc_model_desc d;
@@ -82,6 +79,8 @@ struct dqmc_ctx {
   uint64_t sweep_counter = 0;
   int maxN = 0, maxld = 0, maxMV = 0;
   std::vector<dqmc::PlaneSet> planes_h;
+  // the split products' staging buffers fit the shared memory beside the largest model
+  bool pairs_fit = false, fp64_fit = false;
   double* scratch = nullptr;  // [nfl][maxN][maxN] FP64 for dqmc_greens
   unsigned char* grad_ws = nullptr;  // workspace of the adjoints, kept up to kKeptWorkspace bytes
   size_t grad_ws_bytes = 0;
@@ -170,6 +169,13 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
+// Whether a context's chains of N sites take the split products, for float pairs and for
+// FP64 operands.
+bool pairs_on_tc(const dqmc_ctx* ctx, int N) {
+  return ctx->opts.precision == DQMC_PREC_MIXED_TC && ctx->pairs_fit && N >= tc_min_sites(ctx->opts);
+}
+bool fp64_on_tc(const dqmc_ctx* ctx, int N) { return ctx->fp64_fit && N >= kTc64MinSites; }
+
 // Tensor map of a digit-plane buffer of `bytes` bytes for the split products: the 2D
 // view [rows][kPlaneRowElems] of bf16 with a box of one whole block (digits x
 // tile_rows x kPlaneK, contiguous, a multiple of a row's 512 bytes as tile_rows is
@@ -222,7 +228,7 @@ dqmc_status plane_sets(dqmc_ctx* ctx, std::vector<ChainDev>& chains, const std::
     const ModelHost& M = ctx->models[chain_model[c]];
     for (int s = 0; s < M.d.n_flavors; ++s)
       for (int t = 0; t < 2; ++t) {
-        if (!(t ? fp64_on_tc(M.d.n_sites) : (pairs && pairs_on_tc(ctx->opts, M.d.n_sites)))) continue;
+        if (!(t ? fp64_on_tc(ctx, M.d.n_sites) : (pairs && pairs_on_tc(ctx, M.d.n_sites)))) continue;
         const size_t at = (c * dqmc::kMaxFlavors + s) * 2 + t;
         const int em = fill_plane_set(M, s, t == 1, chains[c].planes[s], h[at]);
         if (em) return fail(ctx, DQMC_ECUDA, "tensor map of the digit-plane scratch (code %d)", em);
@@ -235,9 +241,7 @@ dqmc_status plane_sets(dqmc_ctx* ctx, std::vector<ChainDev>& chains, const std::
 
 dqmc_status setup_model(dqmc_ctx* ctx, ModelHost& M) {
   const dqmc_model_desc& d = M.d;
-  const int N = d.n_sites, nfl = d.n_flavors;
-  const int ld = (int)align_up(N, 4);
-  M.ld = ld;
+  const int N = d.n_sites, nfl = d.n_flavors, ld = M.ld;
   M.cscale = (d.field_type == DQMC_FIELD_ISING) ? std::acosh(std::exp(0.5 * d.dtau * d.U)) : std::sqrt(0.5 * d.dtau * d.U);
   M.hopping.assign(d.hopping, d.hopping + (size_t)nfl * N * N);
   M.vsign.assign(d.vertex_sign, d.vertex_sign + (size_t)nfl * d.n_vertices);
@@ -299,7 +303,7 @@ dqmc_status setup_model(dqmc_ctx* ctx, ModelHost& M) {
   dqmc::ConstPlaneJobs jobs{};
   int n_jobs = 0;
   for (int t = 0; t < 2; ++t) {
-    if (!(t ? fp64_on_tc(N) : pairs_on_tc(ctx->opts, N))) continue;
+    if (!(t ? fp64_on_tc(ctx, N) : pairs_on_tc(ctx, N))) continue;
     const int nd = t ? dqmc::kPlaneDigits64 : dqmc::kPlaneDigits;
     size_t bytes = 0, ints = 0;
     for (const auto& q : sets) {
@@ -331,7 +335,7 @@ dqmc_status setup_model(dqmc_ctx* ctx, ModelHost& M) {
 
 // Per-chain device memory, carved from one arena.  Returns the bytes needed
 // (ptrs filled when base != nullptr).
-size_t chain_layout(const ModelHost& M, int precision, int delay_k, unsigned char* base, ChainDev* C,
+size_t chain_layout(const ModelHost& M, int precision, int delay_k, unsigned char* base, ChainDev* C, bool fp64_tc,
                     bool pairs_tc = false) {
   const int N = M.d.n_sites, ld = M.ld, nfl = M.d.n_flavors, nst = M.d.L / M.d.n_wrap;
   const size_t rs = precision == DQMC_PREC_FP32 ? sizeof(float) : sizeof(double);  // FP64 or float pairs
@@ -363,7 +367,7 @@ size_t chain_layout(const ModelHost& M, int precision, int delay_k, unsigned cha
     if (C) C->iwork[s] = (int*)p;
     // BF16 digit planes of the split tensor-core products (N x N x N at most): both
     // operand types use the same memory, never at the same time
-    const int nd = fp64_on_tc(N) ? dqmc::kPlaneDigits64 : pairs_tc ? dqmc::kPlaneDigits : 0;
+    const int nd = fp64_tc ? dqmc::kPlaneDigits64 : pairs_tc ? dqmc::kPlaneDigits : 0;
     if (nd) {
       p = take(plane_bytes(nd, N, false) + plane_bytes(nd, N, true));
       if (C) C->planes[s] = p;
@@ -526,13 +530,16 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   }
   c->nfl = models[0].n_flavors;
   c->models.resize(n_models);
-  for (int m = 0; m < n_models && !st; ++m) {
+  for (int m = 0; m < n_models; ++m) {
     c->models[m].d = models[m];
-    st = setup_model(c, c->models[m]);
+    c->models[m].ld = (int)align_up(models[m].n_sites, 4);
     c->maxN = std::max(c->maxN, models[m].n_sites);
     c->maxld = std::max(c->maxld, c->models[m].ld);
     c->maxMV = std::max(c->maxMV, models[m].n_vertices);
   }
+  c->pairs_fit = dqmc::split_fits(c->maxld, c->maxMV, c->maxN, dqmc::kPlaneDigits);
+  c->fp64_fit = dqmc::split_fits(c->maxld, c->maxMV, c->maxN, dqmc::kPlaneDigits64);
+  for (int m = 0; m < n_models && !st; ++m) st = setup_model(c, c->models[m]);
   if (st) {
     *out = ctx.release();
     return st;
@@ -544,7 +551,7 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   for (int i = 0; i < n_chains; ++i) {
     offs[i] = total;
     total += chain_layout(c->models[chain_model[i]], opts->precision, opts->delay_k, nullptr, nullptr,
-                          pairs_on_tc(*opts, models[chain_model[i]].n_sites));
+                          fp64_on_tc(c, models[chain_model[i]].n_sites), pairs_on_tc(c, models[chain_model[i]].n_sites));
   }
   if (cudaMalloc((void**)&c->arena, total) != cudaSuccess) {
     *out = ctx.release();
@@ -556,7 +563,8 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
   for (int i = 0; i < n_chains; ++i) {
     ChainDev& C = c->chains_h[i];
     const ModelHost& M = c->models[chain_model[i]];
-    chain_layout(M, opts->precision, opts->delay_k, c->arena + offs[i], &C, pairs_on_tc(*opts, M.d.n_sites));
+    chain_layout(M, opts->precision, opts->delay_k, c->arena + offs[i], &C, fp64_on_tc(c, M.d.n_sites),
+                 pairs_on_tc(c, M.d.n_sites));
     fill_model_fields(M, C);
     C.chain_id = (uint32_t)i;
     C.sign = 1;
@@ -605,8 +613,8 @@ dqmc_status dqmc_init(const dqmc_model_desc* models, int32_t n_models, const int
     // fit beside the rest
     const size_t rs = c->kprec == DQMC_PREC_FP32 ? sizeof(float) : sizeof(double);
     const size_t ab = (size_t)2 * opts->delay_k * c->maxld * rs;
-    const int nd64 = fp64_on_tc(c->maxN) ? dqmc::kPlaneDigits64 : 0;
-    const int nd = c->kprec == DQMC_PREC_MIXED ? (pairs_on_tc(*opts, c->maxN) ? dqmc::kPlaneDigits : 0) : nd64;
+    const int nd64 = fp64_on_tc(c, c->maxN) ? dqmc::kPlaneDigits64 : 0;
+    const int nd = c->kprec == DQMC_PREC_MIXED ? (pairs_on_tc(c, c->maxN) ? dqmc::kPlaneDigits : 0) : nd64;
     c->smem = dqmc::smem_total(c->maxld, c->maxMV, 0, c->maxN, std::max(nd, nd64));
     c->ab_smem = (dqmc::smem_total(c->maxld, c->maxMV, ab, c->maxN, nd) <= 200 * 1024) ? 1 : 0;
     c->smem_sweep = dqmc::smem_total(c->maxld, c->maxMV, c->ab_smem ? ab : 0, c->maxN, nd);
@@ -1055,7 +1063,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
     const bool ok = (M.d.field_type == DQMC_FIELD_ISING) ? (f == 1 || f == -1) : (f == 1 || f == -1 || f == 2 || f == -2);
     if (!ok) return fail(ctx, DQMC_EINVAL, "invalid field value %d", (int)f);
   }
-  const size_t per = chain_layout(M, DQMC_PREC_FP64, 1, nullptr, nullptr);
+  const size_t per = chain_layout(M, DQMC_PREC_FP64, 1, nullptr, nullptr, fp64_on_tc(ctx, N));
   std::vector<double> Vh((size_t)nfl * N * N), wh((size_t)nfl * N);
   // one block: chains, their descriptions, plane sets, eigenpairs, outputs
   size_t bytes = 0;
@@ -1075,7 +1083,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
          *gU_d = (double*)(ws + o_gU);
   std::vector<ChainDev> ch(n_cfg, ChainDev{});
   for (int c = 0; c < n_cfg; ++c) {
-    chain_layout(M, DQMC_PREC_FP64, 1, arena + per * c, &ch[c]);
+    chain_layout(M, DQMC_PREC_FP64, 1, arena + per * c, &ch[c], fp64_on_tc(ctx, N));
     fill_model_fields(M, ch[c]);
     ch[c].chain_id = (uint32_t)c;
     ch[c].sign = 1;
@@ -1111,7 +1119,7 @@ dqmc_status dqmc_logdet_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   GRAD_TRY(cudaMemcpyAsync(ch_d, ch.data(), sizeof(ChainDev) * n_cfg, cudaMemcpyHostToDevice, ctx->stream));
   GRAD_TRY(cudaMemcpyAsync(V_d, Vh.data(), sizeof(double) * Vh.size(), cudaMemcpyHostToDevice, ctx->stream));
   GRAD_TRY(cudaMemcpyAsync(w_d, wh.data(), sizeof(double) * wh.size(), cudaMemcpyHostToDevice, ctx->stream));
-  dqmc::set_smem_bytes(dqmc::smem_total(M.ld, MV, 0, N, fp64_on_tc(N) ? dqmc::kPlaneDigits64 : 0));
+  dqmc::set_smem_bytes(dqmc::smem_total(M.ld, MV, 0, N, fp64_on_tc(ctx, N) ? dqmc::kPlaneDigits64 : 0));
   GRAD_TRY(dqmc::launch_logdet_grad(ch_d, n_cfg, nfl, V_d, w_d, gK_d, gU_d, nullptr, ctx->stream));
   GRAD_TRY(cudaMemcpyAsync(grad_K, gK_d, sizeof(double) * (size_t)n_cfg * nfl * N * N, cudaMemcpyDeviceToHost,
                            ctx->stream));
@@ -1141,7 +1149,7 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
     const bool ok = (M.d.field_type == DQMC_FIELD_ISING) ? (f == 1 || f == -1) : (f == 1 || f == -1 || f == 2 || f == -2);
     if (!ok) return fail(ctx, DQMC_EINVAL, "invalid field value %d", (int)f);
   }
-  const size_t per = chain_layout(M, DQMC_PREC_FP64, 1, nullptr, nullptr);
+  const size_t per = chain_layout(M, DQMC_PREC_FP64, 1, nullptr, nullptr, fp64_on_tc(ctx, N));
   const size_t mat = (size_t)N * ld;
   std::vector<double> Vh((size_t)nfl * N * N), wh((size_t)nfl * N);
   size_t bytes = 0;
@@ -1180,7 +1188,7 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   } while (0)
   EGRAD_TRY(cudaMemsetAsync(arena, 0, per * n_cfg, ctx->stream));
   for (int c = 0; c < n_cfg; ++c) {
-    chain_layout(M, DQMC_PREC_FP64, 1, arena + per * c, &ch[c]);
+    chain_layout(M, DQMC_PREC_FP64, 1, arena + per * c, &ch[c], fp64_on_tc(ctx, N));
     fill_model_fields(M, ch[c]);
     ch[c].chain_id = (uint32_t)c;
     ch[c].sign = 1;
@@ -1198,7 +1206,7 @@ dqmc_status dqmc_energy_backward(dqmc_ctx* ctx, int32_t model_index, const int8_
   EGRAD_TRY(cudaMemcpyAsync(ch_d, ch.data(), sizeof(ChainDev) * n_cfg, cudaMemcpyHostToDevice, ctx->stream));
   EGRAD_TRY(cudaMemcpyAsync(V_d, Vh.data(), sizeof(double) * Vh.size(), cudaMemcpyHostToDevice, ctx->stream));
   EGRAD_TRY(cudaMemcpyAsync(w_d, wh.data(), sizeof(double) * wh.size(), cudaMemcpyHostToDevice, ctx->stream));
-  dqmc::set_smem_bytes(dqmc::smem_total(ld, MV, 0, N, fp64_on_tc(N) ? dqmc::kPlaneDigits64 : 0));
+  dqmc::set_smem_bytes(dqmc::smem_total(ld, MV, 0, N, fp64_on_tc(ctx, N) ? dqmc::kPlaneDigits64 : 0));
   EGRAD_TRY(dqmc::launch_energy_grad(ch_d, n_cfg, nfl, V_d, w_d, G0_d, ew_d, gK_d, gU_d, ep_d, ctx->stream));
   std::vector<double> gU((size_t)n_cfg * nfl), ep((size_t)n_cfg * nfl * 3);
   EGRAD_TRY(cudaMemcpyAsync(grad_K, gK_d, sizeof(double) * (size_t)n_cfg * nfl * N * N, cudaMemcpyDeviceToHost,

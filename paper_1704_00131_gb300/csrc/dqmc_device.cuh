@@ -283,8 +283,6 @@ __device__ __forceinline__ T* as_shared(T* p) {
 // dimension; R is picked per size so that N = 16, 144 or 400 need no padding),
 // 16-deep K panels staged in shared memory.  C must not alias A or B.
 // --------------------------------------------------------------------------
-constexpr int kGemmMaxTile = 80;  // 16 * 5
-
 __host__ __device__ inline int gemm_pick_r(int n) {
   int best_r = 4, best = 1 << 30;
   for (int r = 5; r >= 1; --r) {
@@ -537,41 +535,6 @@ struct Smem {
   int dd_tile;      // register tile of the float-pair SIMT products (0: by padding, 3, 4)
 };
 
-// The first kSmemCounterBytes of the dynamic shared memory hold thread 0's
-// cycle counters of the sweep kernel (fixed addresses, no registers).
-constexpr int kSmemCounterBytes = 16 * 8;
-
-// exponent entries per operand of the split products: rows padded to whole tiles
-__host__ __device__ inline int exp_len(int ld) { return ld + kPlaneMaxRows; }
-
-// Layout: the vectors and barriers, then (128-byte aligned) the SIMT products'
-// panels and, in the sweep kernel, the delayed vectors.  The tensor-core products
-// stage their operands over both: neither is live inside a product (a flush has
-// cut its delayed vectors into digits before the first copy lands).
-// (The panels also hold the QR's, two of kPanel columns.)
-constexpr int kGemmRegionBytes = 2 * 16 * kGemmMaxTile * 8;
-__host__ __device__ inline size_t gemm_region_bytes(int ld) {
-  const size_t qr = (size_t)2 * 4 * (ld + 1) * 8;
-  return ((qr > (size_t)kGemmRegionBytes ? qr : (size_t)kGemmRegionBytes) + 127) / 128 * 128;
-}
-
-__host__ __device__ inline size_t smem_stage_offset(int ld, int MV) {
-  size_t b = kSmemCounterBytes;
-  b += 6 * (size_t)ld * 8;        // v, ev, d, hv, xdiag, spare
-  b += 3 * (size_t)MV * 8;        // u2, delta, gam
-  b += 8 * 8 + 32 * 8 + 32 * 4;   // xs, red, ired
-  b += (size_t)MV * 4;            // qsite
-  b += (size_t)ld * 4;            // qinv
-  b += 2 * (size_t)MV + 16;       // fnew, fslice
-  b = (b + 15) / 16 * 16;
-  b += 8 * 128 * 8;               // qred
-  b += 2 * (size_t)exp_len(ld) * 4;  // expA, expB
-  b = (b + 15) / 16 * 16;
-  b += 128;                       // mbarriers and the TMEM slot of the tensor-core products
-  return (b + 127) / 128 * 128 + 128;  // room to align the panels
-}
-__host__ __device__ inline size_t smem_bytes_for(int ld, int MV) { return smem_stage_offset(ld, MV) + gemm_region_bytes(ld); }
-
 __device__ inline Smem carve_smem(unsigned char* base, int ld, int MV) {
   Smem s;
   unsigned char* const start = base;
@@ -770,7 +733,8 @@ __device__ __forceinline__ int panel_ld(int N) { return N | 1; }
 // products of more reflectors lose the small rows of Q: with 16 columns the wrapped
 // G's drift on 4 x 4 lattices is four times the unblocked factorisation's, with 4
 // the same (FP64, U = 4: mean 1.4e-11, 3.7e-12 and 3.5e-12).
-constexpr int kPanel = 4;  // gemm_region_bytes counts two such panels
+// (kPanel; a matrix so large that the shared memory holds only narrower panels takes
+// qr_panel_cols of them.)
 // Columns per panel of the LU and the solves: the largest power of two <= 16 of which
 // two panels fit the product area.
 __device__ inline int panel_width(int N, const Smem& S) {
@@ -1046,12 +1010,13 @@ __device__ __forceinline__ T* panel_tri(const Smem& S) { return reinterpret_cast
 // is updated once per panel, from registers.
 template <typename T>
 __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* vk0, T* tri, Smem& S) {
+  // (pw: the arrays' strides; wide: the columns a panel takes)
   constexpr int pw = kPanel, RG = kThreads / pw, nwarp = kThreads / 32;
   static_assert(32 / pw == nwarp, "one lane group of the scalar warp per warp's partial products");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = tid % pw, rg = tid / pw;
-  const int ldp = panel_ld(N);
+  const int ldp = panel_ld(N), wide = qr_panel_cols(N, S.um.stage_bytes);
   T* Vp = reinterpret_cast<T*>(S.gemm);
-  T* Wp = Vp + pw * ldp;
+  T* Wp = Vp + wide * ldp;
   T* red = reinterpret_cast<T*>(S.qred);        // [nwarp][pw] partial products
   T* wq = red + nwarp * pw;                     // [pw] update coefficients of the columns to come
   T* zq = wq + pw;                              // [2][pw] products with the earlier vectors
@@ -1068,8 +1033,8 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
   column_keys<T>(N, ld, X, dsc, key, lsc, S);
   for (int j = tid; j < N; j += kThreads) list[j] = j;
   __syncthreads();
-  for (int k0 = 0; k0 < N; k0 += pw) {
-    const int nb = (N - k0 < pw) ? N - k0 : pw, rows = N - k0;
+  for (int k0 = 0; k0 < N; k0 += wide) {
+    const int nb = (N - k0 < wide) ? N - k0 : wide, rows = N - k0;
     // the panel's columns: the nb largest keys, in order; the others keep theirs
     for (int t = tid; t < rows; t += kThreads) {
       const float kt = key[k0 + t];
@@ -1247,7 +1212,7 @@ __device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* 
     if (q < nb && rg < pc) Vp[q * ldp + rg] = from_zero<T>();
     if (tid < nb) list[k0 + pc] = col;  // the panel's columns by position
     // T by position: in global memory, or in place for a single panel
-    T* tg = N > pw ? tri + (size_t)(k0 / pw) * pw * pw : Tm;
+    T* tg = N > pw ? tri + (size_t)(k0 / wide) * pw * pw : Tm;
     if (tid < pw * pw && tr < nb && q < nb) tg[pos_of[tr] * pw + pc] = tv;
     __syncthreads();
     if (k0 + nb < N) {
@@ -1267,23 +1232,23 @@ template <typename T>
 __device__ void form_q_blk(int N, int ld, const T* X, const int* perm, const T* vk0, const T* tri, T* Q, Smem& S) {
   const int tid = threadIdx.x;
   constexpr int pw = kPanel;
-  const int ldp = panel_ld(N);
+  const int ldp = panel_ld(N), wide = qr_panel_cols(N, S.um.stage_bytes);
   T* Vp = reinterpret_cast<T*>(S.gemm);
-  T* Wp = Vp + pw * ldp;
+  T* Wp = Vp + wide * ldp;
   for (int e = tid; e < N * N; e += kThreads) {
     const int x = e / N, y = e - x * N;
     Q[(size_t)x * ld + y] = unit<T>(x == y);
   }
   __syncthreads();
-  for (int k0 = (N - 1) / pw * pw; k0 >= 0; k0 -= pw) {
-    const int nb = (N - k0 < pw) ? N - k0 : pw, rows = N - k0;
+  for (int k0 = (N - 1) / wide * wide; k0 >= 0; k0 -= wide) {
+    const int nb = (N - k0 < wide) ? N - k0 : wide, rows = N - k0;
     for (int e = tid; e < rows * pw; e += kThreads) {
       const int r = e / pw, c = e - r * pw;
       if (c < nb)
         Vp[c * ldp + r] = r < c ? from_zero<T>() : r == c ? vk0[k0 + c] : X[(size_t)(k0 + r) * ld + perm[k0 + c]];
     }
     __syncthreads();
-    panel_times_t<T>(rows, ldp, nb, Vp, N > pw ? tri + (size_t)(k0 / pw) * pw * pw : panel_tri<T>(S), Wp);
+    panel_times_t<T>(rows, ldp, nb, Vp, N > pw ? tri + (size_t)(k0 / wide) * pw * pw : panel_tri<T>(S), Wp);
     panel_apply<T, true, false>(N, ld, Q, k0, k0, nb, Vp, Wp, S, nullptr, nullptr, nullptr);
   }
 }

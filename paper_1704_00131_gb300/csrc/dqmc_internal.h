@@ -5,30 +5,12 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "dqmc_layout.h"
+
 namespace dqmc {
 
 constexpr int kThreads = 256;      // threads per CTA of every kernel
 constexpr int kMaxFlavors = 2;
-// Digit planes of the split tensor-core products: blocks of digits x rows x kPlaneK
-// bf16, one block per (tile, 16-wide K chunk), copied to shared memory by one
-// tiled tensor copy each.  Float pairs have kPlaneDigits digits, FP64 operands
-// kPlaneDigits64; a right operand's tiles have kPlaneRowsB rows, a left operand's
-// umma_rows(N).
-constexpr int kPlaneDigits = 7, kPlaneDigits64 = 8, kPlaneMaxRows = 128, kPlaneRowsB = 32, kPlaneK = 16;
-constexpr int kPlaneRowElems = 256;  // bf16 per row of the copies' 2D view of a plane buffer
-// row tiles of an N-row left operand: equal, at most kPlaneMaxRows, rounded to 16
-__host__ __device__ inline int umma_row_tiles(int n) { return (n + kPlaneMaxRows - 1) / kPlaneMaxRows; }
-__host__ __device__ inline int umma_rows(int n) {
-  const int t = umma_row_tiles(n);
-  return ((n + t - 1) / t + 15) / 16 * 16;
-}
-// bf16 elements of the left and right operands' planes of N x K matrices
-__host__ __device__ inline size_t plane_elems(int digits, int n, int k, bool right) {
-  const size_t rows = right ? (size_t)(n + kPlaneRowsB - 1) / kPlaneRowsB * kPlaneRowsB
-                            : (size_t)umma_rows(n) * umma_row_tiles(n);
-  return (size_t)digits * rows * ((k + kPlaneK - 1) / kPlaneK * kPlaneK);
-}
-
 enum { kCpEA = 0, kCpEtA = 1, kCpEiA = 2, kCpEiB = 3, kCpEB = 4, kCpSets = 5 };
 
 // The split products' buffers of one (chain, flavor) and operand type: scratch
@@ -131,9 +113,6 @@ cudaError_t launch_fresh_green(ChainDev* chains, int n_chains, int nfl, int prec
                                double* out, int out_chain, cudaStream_t st);
 cudaError_t launch_sweep(ChainDev* chains, const SweepParams& p, int nfl, int precision, size_t smem,
                          cudaStream_t st);
-// dynamic shared memory with `ab_bytes` of delayed vectors; digits > 0: also room to
-// stage the split products of matrices of up to maxN sites
-size_t smem_total(int maxld, int maxMV, size_t ab_bytes, int maxN, int digits);
 // One constant operand's planes: an N x N FP64 or float-pair matrix as the left
 // (right = 0; tr = 1 for its transpose) or right factor.
 struct ConstPlaneJob {

@@ -111,26 +111,6 @@ __global__ void corr_kernel(ChainDev* chains, int n_chains, const int* csr_all, 
 // --------------------------------------------------------------------------
 // Launchers.
 // --------------------------------------------------------------------------
-// The split products want three stages; two where three would leave room for one
-// CTA per SM instead of two (a second CTA hides more than a third stage).
-size_t smem_total(int maxld, int maxMV, size_t ab_bytes, int maxN, int digits) {
-  const size_t plain = smem_bytes_for(maxld, maxMV) + ab_bytes;
-  if (!digits) return plain;
-  size_t stage = 0;  // the tile height is not monotonic in N
-  for (int n = 1; n <= maxN; ++n) {
-    const size_t b = (size_t)digits * kPlaneK * 2 * (umma_rows(n) + kPlaneRowsB);
-    stage = b > stage ? b : stage;
-  }
-  const size_t off = smem_stage_offset(maxld, maxMV), half = 113 * 1024;
-  const size_t two = off + 2 * stage > plain ? off + 2 * stage : plain;
-  const size_t three = off + 3 * stage > plain ? off + 3 * stage : plain;
-  // every CTA of these kernels holds half of the SM's tensor memory (256 of 512
-  // columns): at least 78 KB of shared memory per CTA keeps three of them from
-  // sharing an SM, so an allocation never waits
-  const size_t need = (three <= half || two > half) ? three : two;
-  return need > 78 * 1024 ? need : 78 * 1024;
-}
-
 // Digit planes and row exponents of a model's constant operands of the split
 // products, one CTA each: a left factor's rows (tiles of umma_rows(N)) or a right
 // factor's columns (tiles of kUmmaNT), laid out as gemm_umma stages them.
