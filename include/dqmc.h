@@ -123,16 +123,17 @@ typedef struct {
   int32_t meas_last;          /*   (upward tau = 1..L, downward tau-1 = L-1..0)    */
   uint64_t seed;              /* Philox key (seed_lo, seed_hi ^ chain)             */
   double unstable_threshold;  /* > 0: DQMC_EUNSTABLE when prec_green_max exceeds it*/
-  int64_t spin_limit;         /* SM cycles before a bounded device wait gives up
-                                 (DQMC_ETIMEOUT); 0: about one second            */
+  int64_t spin_limit;         /* SM cycles before a bounded wait of the float-pair
+                                 tensor-core products gives up (DQMC_ETIMEOUT); 0:
+                                 about one second, as always for the FP64 ones   */
   int32_t tc_min_sites;       /* DQMC_PREC_MIXED_TC: chains of fewer sites use the
                                  float-pair SIMT products (0: 72, where the tensor-
                                  core product overtakes them on GB300)            */
   int32_t dd_tile;            /* float-pair SIMT products: output tiles of 48 x 48
                                  (3) or 64 x 64 (4) per CTA; 0: the one that pads
                                  the matrix least                                 */
-  int32_t test_stall;         /* test hook, 0 in production: nonzero makes the
-                                 first bounded wait of every tensor-core product
+  int32_t test_stall;         /* test hook, 0 in production: nonzero makes the first
+                                 bounded wait of every float-pair tensor-core product
                                  wait on a barrier that nothing arrives on, so it
                                  gives up after spin_limit cycles; the call then
                                  reports DQMC_ETIMEOUT with the context usable    */

@@ -460,6 +460,13 @@ dqmc_status timeout_message(dqmc_ctx* ctx, const ChainDev& C) {
               m.c_str());
 }
 
+// What a chain's error word says.
+dqmc_status chain_status(dqmc_ctx* ctx, const ChainDev& C) {
+  if (C.error & 2) return timeout_message(ctx, C);
+  if (C.error) return fail(ctx, DQMC_EUNSTABLE, "chain %u: singular matrix in the stabilisation", C.chain_id);
+  return DQMC_OK;
+}
+
 // Fields in place -> left chain, G(0), sign of every chain.
 dqmc_status initial_fill(dqmc_ctx* ctx) {
   const int n = (int)ctx->chains_h.size();
@@ -469,10 +476,8 @@ dqmc_status initial_fill(dqmc_ctx* ctx) {
   CUDA_TRY(ctx, dqmc::launch_finalize_init(ctx->chains_d, n, ctx->stream));
   dqmc_status st = download_chains(ctx);
   if (st) return st;
-  for (const ChainDev& C : ctx->chains_h) {
-    if (C.error & 2) return timeout_message(ctx, C);
-    if (C.error) return fail(ctx, DQMC_EUNSTABLE, "chain %u: singular matrix in the stabilisation", C.chain_id);
-  }
+  for (const ChainDev& C : ctx->chains_h)
+    if ((st = chain_status(ctx, C))) return st;
   return DQMC_OK;
 }
 
@@ -720,7 +725,7 @@ dqmc_status dqmc_greens(dqmc_ctx* ctx, int32_t chain, int32_t flavor, int32_t fr
   dqmc_status st = download_chains(ctx);
   if (st) return st;
   const ChainDev& C = ctx->chains_h[chain];
-  if (C.error) return fail(ctx, DQMC_EUNSTABLE, "singular matrix in the stabilisation");
+  if ((st = chain_status(ctx, C))) return st;
   if (logdet_out) *logdet_out = C.logdet[flavor];
   if (sign_out) *sign_out = C.fresh_sign[flavor];
   return DQMC_OK;
@@ -741,8 +746,7 @@ dqmc_status dqmc_greens_tau(dqmc_ctx* ctx, int32_t chain, int32_t flavor, int32_
                                 out_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream));
   dqmc_status st = download_chains(ctx);
   if (st) return st;
-  if (ctx->chains_h[chain].error) return fail(ctx, DQMC_EUNSTABLE, "singular matrix in the stabilisation");
-  return DQMC_OK;
+  return chain_status(ctx, ctx->chains_h[chain]);
 }
 
 dqmc_status dqmc_measure(dqmc_ctx* ctx, double* out, double* sign_sum, int64_t* n_meas) {
@@ -900,11 +904,7 @@ dqmc_status run_tau_measure(dqmc_ctx* ctx, int32_t n_tau, const double* site_pha
     st = download_chains(ctx);
     if (st) break;
     for (const ChainDev& C : ctx->chains_h)
-      if (C.error) {
-        st = (C.error & 2) ? timeout_message(ctx, C)
-                           : fail(ctx, DQMC_EUNSTABLE, "chain %u: singular matrix in the stabilisation", C.chain_id);
-        break;
-      }
+      if ((st = chain_status(ctx, C))) break;
   } while (false);
   cleanup();
   if (st) return st;

@@ -633,6 +633,13 @@ __device__ void gemm_64(Smem& S, int M, int Nc, int Kd, const double* A, int lda
     cta_gemm<double, TA, TB>(M, Nc, Kd, A, lda, B, ldb, Cm, ldc, S.gemm);
 }
 
+// Bit 0 of the chain's error word.  (Beside bit 1 of a wait that gave up, which must stay:
+// the products after it are skipped, their barriers' phases are no longer known.  The
+// word is shared with the peer flavor's CTA.)
+__device__ __forceinline__ void numerical_failure(ChainDev& C) {
+  if (threadIdx.x == 0) atomicOr(&C.error, 1);
+}
+
 // Slice potential v^s_i of slice tau (1-based) from global fields.
 __device__ void slice_potential_global(const ChainDev& C, int s, int tau, double* v) {
   for (int x = threadIdx.x; x < C.N; x += kThreads) v[x] = 0.0;
@@ -1782,7 +1789,7 @@ __global__ void __launch_bounds__(kThreads) fresh_green_kernel(ChainDev* chains,
                               : fill_left_chain(C, s, S, logdet, sign);
   if (umma) umma_free(S.um);
   if (bad) {
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     return;
   }
   const double* Gf = wmat(C, s, 6);
@@ -1846,7 +1853,7 @@ __global__ void __launch_bounds__(kThreads) green_tau_kernel(ChainDev* chains, i
                         : green_from_udv(C, s, R, Lf, Gf, logdet, sg, S);
   if (bad) {
     if (umma) umma_free(S.um);
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     return;
   }
   Real* G = reinterpret_cast<Real*>(wmat(C, s, 7));
@@ -2468,7 +2475,7 @@ __device__ void stabilise(ChainDev& C, int s, int j, bool up, Real* G, Smem& S, 
   const int bad = mixed ? green_from_udv_mixed(C, s, R, Lf, Gf, logdet, sg, S)
                         : green_from_udv(C, s, R, Lf, Gf, logdet, sg, S);
   if (bad) {
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     sg = 1;
   }
   tick(det, 7, t0);

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(kThreads) green0_kernel(ChainDev* chains, int 
   double logdet;
   int sign;
   if (fill_left_chain(C, s, S, logdet, sign)) {
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     if (umma) umma_free(S.um);
     return;
   }
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
   double logdet;
   int sign;
   if (fill_left_chain(C, s, S, logdet, sign)) {  // storage slots: left chains; W6 = G(0)
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     if (umma) umma_free(S.um);
     return;
   }
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kThreads) energy_grad_kernel(ChainDev* chains,
       const int dq = chain_step(C, s, (j - 1) * nw, j * nw, false, src, S);
       const UDV Lf = (j == nst) ? ident_udv(C) : slot_udv(C, s, j);
       if (displaced_from_udv(C, s, work_udv(C, s, dq), Lf, T2, G0t, S)) {
-        if (threadIdx.x == 0) C.error = 1;
+        numerical_failure(C);
         if (umma) umma_free(S.um);
         return;
       }

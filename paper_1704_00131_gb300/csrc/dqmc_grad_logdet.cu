@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
   double logdet;
   int sign;
   if (fill_left_chain(C, s, S, logdet, sign)) {
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     if (umma) umma_free(S.um);
     return;
   }
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) logdet_grad_kernel(ChainDev* chains,
       double ldt;
       int sgt;
       if (green_from_udv(C, s, work_udv(C, s, dq), Lf, wmat(C, s, 6), ldt, sgt, S)) {
-        if (threadIdx.x == 0) C.error = 1;
+        numerical_failure(C);
         if (umma) umma_free(S.um);
         return;
       }

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
   int sg;
   double* Gf = wmat(C, s, 6);
   if (green_from_udv(C, s, ident_udv(C), slot_udv(C, s, 0), Gf, logdet, sg, S)) {
-    if (threadIdx.x == 0) C.error = 1;
+    numerical_failure(C);
     if (umma) umma_free(S.um);
     return;
   }
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kThreads) tau_measure_kernel(ChainDev* chains,
         int bad = displaced_from_udv(C, s, R, Lf, Ft0, F0t, S);
         if (!bad) bad = green_from_udv(C, s, R, Lf, Gf, logdet, sg, S);
         if (bad) {
-          if (threadIdx.x == 0) C.error = 1;
+          numerical_failure(C);
           if (umma) umma_free(S.um);
           return;
         }
