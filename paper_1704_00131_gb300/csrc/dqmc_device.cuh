@@ -2664,8 +2664,12 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(ChainDev* chains, Sw
 // --------------------------------------------------------------------------
 // Launch helpers (instantiated once per precision unit).
 // --------------------------------------------------------------------------
+// The kernel may be launched with up to the architecture's shared memory: the same value
+// in every call, as the attribute is the kernel's, not the launch's, and another thread
+// may be between its own call and its launch.
 static inline cudaError_t set_smem(const void* fn, size_t bytes) {
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (bytes > kMaxSmemBytes) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemBytes);
 }
 
 template <typename Real>

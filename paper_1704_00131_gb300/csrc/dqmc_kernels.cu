@@ -147,7 +147,9 @@ cudaError_t launch_init_fields(ChainDev* chains, int n_chains, uint64_t seed, in
   return cudaGetLastError();
 }
 
-static size_t g_smem_bytes = 0;
+// of the context that this host thread is launching for (contexts of other threads
+// have other sizes)
+static thread_local size_t g_smem_bytes = 0;
 
 cudaError_t launch_fresh_green(ChainDev* chains, int n_chains, int nfl, int precision, int write_working,
                                double* out, int out_chain, cudaStream_t st) {

@@ -141,9 +141,7 @@ extern "C" dqmc_status dqmc_green_fresh_noalloc(int32_t n_sites, int32_t n_flavo
   C.vsign = vertex_sign_dev;
   C.fields = const_cast<int8_t*>(fields_dev);
   const size_t smem = smem_bytes_for(n_sites, n_vertices);
-  if (cudaFuncSetAttribute((const void*)fresh_green_noalloc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
-    return DQMC_ECUDA;
+  if (set_smem((const void*)fresh_green_noalloc_kernel, smem) != cudaSuccess) return DQMC_ECUDA;
   fresh_green_noalloc_kernel<<<n_flavors, kThreads, smem, (cudaStream_t)cuda_stream>>>(
       C, g_noalloc_ptr[dev], G_out_dev, logdet_out_dev, sign_out_dev);
   return cudaGetLastError() == cudaSuccess ? DQMC_OK : DQMC_ECUDA;

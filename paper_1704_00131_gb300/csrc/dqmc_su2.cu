@@ -1319,10 +1319,6 @@ __global__ void su2_reset_stats_kernel(Su2Dev* chains, int n_chains, int clear_m
 
 size_t su2_smem_bytes(int maxN, int maxMV) { return su2_smem_layout(maxN, maxMV); }
 
-static cudaError_t su2_set_smem(const void* fn, size_t bytes) {
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 cudaError_t su2_launch_init_fields(Su2Dev* chains, int n_chains, uint64_t seed, cudaStream_t st) {
   su2_init_fields_kernel<<<n_chains, kThreads, 0, st>>>(chains, n_chains, seed);
   return cudaGetLastError();
@@ -1330,14 +1326,14 @@ cudaError_t su2_launch_init_fields(Su2Dev* chains, int n_chains, uint64_t seed, 
 
 cudaError_t su2_launch_fresh(Su2Dev* chains, int n_chains, int mode, int only, double2* out, size_t smem,
                              cudaStream_t st) {
-  cudaError_t e = su2_set_smem((const void*)su2_fresh_kernel, smem);
+  cudaError_t e = set_smem((const void*)su2_fresh_kernel, smem);
   if (e != cudaSuccess) return e;
   su2_fresh_kernel<<<n_chains, kThreads, smem, st>>>(chains, n_chains, mode, only, out);
   return cudaGetLastError();
 }
 
 cudaError_t su2_launch_sweep(Su2Dev* chains, const Su2SweepParams& p, size_t smem, cudaStream_t st) {
-  cudaError_t e = su2_set_smem((const void*)su2_sweep_kernel, smem);
+  cudaError_t e = set_smem((const void*)su2_sweep_kernel, smem);
   if (e != cudaSuccess) return e;
   su2_sweep_kernel<<<p.n_chains, kThreads, smem, st>>>(chains, p);
   return cudaGetLastError();
@@ -1356,7 +1352,7 @@ cudaError_t su2_launch_corr(const Su2Dev* chains, int n_chains, const int* const
 
 cudaError_t su2_launch_tau(Su2Dev* chains, int n_chains, int only, int n_tau, double2* out_a, double* out_prec,
                            double2* gt0, double2* g0t, size_t smem, cudaStream_t st) {
-  cudaError_t e = su2_set_smem((const void*)su2_tau_kernel, smem);
+  cudaError_t e = set_smem((const void*)su2_tau_kernel, smem);
   if (e != cudaSuccess) return e;
   su2_tau_kernel<<<n_chains, kThreads, smem, st>>>(chains, n_chains, only, n_tau, out_a, out_prec, gt0, g0t);
   return cudaGetLastError();
