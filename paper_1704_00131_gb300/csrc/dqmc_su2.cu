@@ -44,6 +44,13 @@ __device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -
 __device__ __forceinline__ double2 zscal(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
 __device__ __forceinline__ double zabs2(double2 a) { return fma(a.x, a.x, a.y * a.y); }
 __device__ __forceinline__ double zabs(double2 a) { return hypot(a.x, a.y); }
+// 1 / |a| (a != 0): from the square where that is far from the ends of the range (a
+// subnormal square holds few bits), else by the longer way
+__device__ __forceinline__ double zrabs(double2 a) {
+  const double a2 = zabs2(a);
+  const int e = __double2hiint(a2) >> 20;  // biased exponent
+  return (e > 64 && e < 2000) ? rsqrt(a2) : 1.0 / zabs(a);
+}
 __device__ __forceinline__ double2 zdiv(double2 a, double2 b) {
   // a conj(b) / |b|^2 with b rescaled by its larger component (Smith's idea)
   const double s = fmax(fabs(b.x), fabs(b.y));
@@ -104,9 +111,13 @@ __device__ __forceinline__ int block_argmax_key(int key, int idx, int N, int* ir
     if (ired[w] > bk || (ired[w] == bk && ired[8 + w] < bi)) { bk = ired[w]; bi = ired[8 + w]; }
   return bk < 0 ? N : bi;
 }
-// order of a nonnegative number / of a complex pivot's larger component (NaN: -1)
+// order of a nonnegative number / of a complex pivot's larger component (-1: a NaN, in
+// either component)
 __device__ __forceinline__ int top_bits(double x) { return x != x ? -1 : __double2hiint(x) & 0x7fffffff; }
-__device__ __forceinline__ int pivot_key(double2 a) { return max(pivot_key(a.x), pivot_key(a.y)); }
+__device__ __forceinline__ int pivot_key(double2 a) {
+  const int x = pivot_key(a.x), y = pivot_key(a.y);
+  return min(x, y) < 0 ? -1 : max(x, y);
+}
 
 // ---- shared memory of a chain's CTA ----------------------------------------
 constexpr int kZgTile = 32;  // C tile of the complex products
@@ -426,7 +437,7 @@ __device__ int zqr_pivoted(int N, int ld, double2* X, double* beta, double2* vk0
       double2 alpha = x0;
       if (xn2 > 0.0) {
         const double xnorm = sqrt(xn2), a2 = zabs2(x0);
-        alpha = (a2 > 0.0) ? zscal(-xnorm * rsqrt(a2), x0) : make_double2(-xnorm, 0.0);
+        alpha = (x0.x != 0.0 || x0.y != 0.0) ? zscal(-xnorm * zrabs(x0), x0) : make_double2(-xnorm, 0.0);
         const double2 v0 = zsub(x0, alpha);
         const double vhv = xn2 - a2 + zabs2(v0);
         bk = (vhv > 0.0) ? quick_div(2.0, vhv) : 0.0;
@@ -799,7 +810,7 @@ __device__ void z_update_slice(Su2Dev& C, int tau, int dir, const Su2SweepParams
         if (tid == 0) S.qred[0] = coef;
       } else {
         const double2 PR = zmul(Pc, zmul(S.gr[first], zmul(r1, r1)));
-        const double2 Pn = zscal(rsqrt(zabs2(PR)), PR);
+        const double2 Pn = zscal(zrabs(PR), PR);
         if (tid == 32) S.qred[1] = Pn;
       }
     }
