@@ -66,8 +66,15 @@ typedef enum { DQMC_FIELD_ISING = 1, DQMC_FIELD_HS4 = 2 } dqmc_field_type;
  *     From 32 sites the N x N x N products run on the tensor cores (tcgen05) as
  *     exact-split BF16 products of FP64 operands: eight 8-bit digits each, 63 bits
  *     under the largest entry of a row of the left and a column of the right
- *     factor, recombined as one integer and rounded once to FP64.  Their error
- *     against 64 bits is below that of a chain of FP64 multiply-adds.
+ *     factor, recombined as one integer and rounded once to FP64.  The error of an
+ *     element (i, j) is one rounding and at most N 2^-57 max_k |a_ik| max_k |b_kj|
+ *     (digits of either sign add up to about N^(1/2) 2^-61 of it): relative to the
+ *     largest entries of its row and column, where a chain of FP64 multiply-adds
+ *     errs by up to N 2^-53 sum_k |a_ik| |b_kj|.  It is the smaller one for entries
+ *     of similar size; what lies more than 2^63 below those largest entries is
+ *     lost.  The stable G is as accurate as with FP64 chains in norm, also where site
+ *     potentials spread a block of slices by 2^52; rows of G that are themselves far
+ *     below 1 (e^-28) keep fewer digits of their own.
  *   DQMC_PREC_FP32: working G, wraps and delayed updates in plain FP32; the
  *     stabilisation in FP64 as above.  Round-off grows by the condition number of
  *     the unstabilised slice product (Sec. 2.3), so at strong coupling the wrapped

@@ -19,9 +19,16 @@
 // are dropped (below 2^-56 and 2^-64 of the scale).  The diagonals are summed as
 // float pairs, or for FP64 as one integer that is rounded once.
 //
-// Largest error over |A||B| against 80-bit sums (normal A, log-normal B): FP64
-// operands 1.0e-16 at N = 64 and 5.6e-16 at N = 144, where a chain of FP64 FMAs has
-// 1.0e-15 and 1.4e-15.
+// Error: fixed-point under the largest entries of the row and the column, for FP64 at
+// most K 2^-57 max|a| max|b| (the dropped pairs, all of one sign) and one rounding;
+// an FP64 chain's is relative to each element's |A||B|, the smaller one where those
+// largest entries do not meet.  Largest error over |A||B| against 80-bit sums (normal
+// A, log-normal B): FP64 operands 1.0e-16 at N = 64 and 5.6e-16 at N = 144, where a chain
+// of FP64 FMAs has 1.0e-15 and 1.4e-15.  Of the stable G with site potentials, sorted,
+// that spread blocks of slices by 2^40 to 2^52 (N = 33, products of 63 bits and FP64
+// chains emulated on the CPU, against 70-digit decimals): 3.0e-16 to 3.2e-15 and 2.3e-16
+// to 6.8e-15.  Rows of G of the order of e^-28 have a relative error of 4e-10 where
+// chains leave 5e-12, of e^-56 1e-6 where chains leave 4e-10 to 9e-10.
 //
 // Cost per product on GB300 (one CTA of two per SM, cycles): FP64 N = 64 44k, 72 69k,
 // 144 298k, where the FP64 pipe's tiles need 159k, 280k and 1.8M per CTA and SM
