@@ -78,15 +78,14 @@ struct ChainDev {
   int test_stall;                 // test hook: tensor-core products wait on a barrier nothing arrives on
   int dd_tile;                    // register tile of the float-pair SIMT products (0 by padding, 3, 4)
   int wait_where[kMaxFlavors][6]; // first wait that gave up per flavor: kind (1 copy, 2 MMAs
-                                  // before a refill, 3 MMAs before the epilogue, 4 / 5 copy / MMAs
-                                  // at the end of a product; 9 a staging buffer not 128-byte
-                                  // aligned for the tensor copies), chunk (stage for 4, 5), chunks,
-                                  // product ordinal in the kernel, barrier word (low, high)
+                                  // before a refill, 3 MMAs before the epilogue; 9 a staging
+                                  // buffer not 128-byte aligned for the tensor copies), chunk,
+                                  // chunks, product ordinal in the kernel, barrier word (low, high)
   // SM cycles spent per phase during the current dqmc_sweep call, per flavor:
   // 0 updates, 1 wraps (V and T), 2 stabilisation, 3 measurement
   int64_t cyc[kMaxFlavors][4];
-  // finer split, per flavor: 0 ratio precompute, 1 acceptance scan (ratios,
-  // cluster barrier, first acceptance), 2 update vectors, 3 flushes,
+  // finer split, per flavor: 0 ratio precompute, 1 decisions (per window the exchange of the
+  // flavors' blocks, then its acceptances), 2 update vectors, 3 flushes,
   // 4 B-chain products, 5 QR and Q, 6 T update, 7 stable G
   int64_t cycd[kMaxFlavors][8];
 };
