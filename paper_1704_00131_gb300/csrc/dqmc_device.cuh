@@ -35,10 +35,20 @@
 #include "../../include/dqmc.h"
 #include "dqmc_internal.h"
 
+// DQMC_QR_CALL: how the panelled QR is called.  The sweep kernels' units say __noinline__:
+// held to 128 registers they spilled in it, with its renewed norms and scaled panels the
+// more (float pairs 480 bytes of spill loads, out of line 104; with split products 3220 and
+// 2144).  Sweeps of 9 x 7, 40 chains in float pairs: 23.3 ms inlined, 22.9 out of line
+// (22.4 before those corrections); 8 x 8, 64 chains in FP64: 35.5 and 34.7.  The
+// adjoints, at 255 registers, lose by the call (log|det| of 64 8 x 8: 8.75 and 8.89 ms).
+//
 // DQMC_WITH_UMMA: 1 compiles the float pairs' tensor-core products into the
 // float-pair kernels (the unit of DQMC_PREC_MIXED_TC), 0 leaves them out (the unit of
 // DQMC_PREC_MIXED, whose kernels then keep their registers for the SIMT tiles).  The
 // FP64 products' are in every unit.
+#ifndef DQMC_QR_CALL
+#define DQMC_QR_CALL
+#endif
 #ifndef DQMC_WITH_UMMA
 #define DQMC_WITH_UMMA 1
 #endif
@@ -1021,7 +1031,7 @@ __device__ __forceinline__ T* panel_tri(const Smem& S) { return reinterpret_cast
 // same square root and quotients cost most of a column before).  The rest of the matrix
 // is updated once per panel, from registers.
 template <typename T>
-__device__ int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* vk0, T* tri, Smem& S) {
+__device__ DQMC_QR_CALL int qr_blocked(int N, int ld, T* X, const double* dsc, int* perm, T* vk0, T* tri, Smem& S) {
   // (pw: the arrays' strides; wide: the columns a panel takes)
   constexpr int pw = kPanel, RG = kThreads / pw, nwarp = kThreads / 32;
   static_assert(32 / pw == nwarp, "one lane group of the scalar warp per warp's partial products");

@@ -1,4 +1,5 @@
 // Sweep and fresh-G kernels instantiated for the FP64 working Green function.
+#define DQMC_QR_CALL __noinline__
 #include "dqmc_device.cuh"
 
 namespace dqmc {

@@ -1,6 +1,7 @@
 // Sweep and fresh-G kernels instantiated for the float-pair working Green function
 // with the float-pair SIMT products only (DQMC_PREC_MIXED).
 #define DQMC_WITH_UMMA 0
+#define DQMC_QR_CALL __noinline__
 #include "dqmc_device.cuh"
 
 namespace dqmc {

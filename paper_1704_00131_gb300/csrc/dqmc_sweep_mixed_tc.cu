@@ -2,6 +2,7 @@
 // with the split tensor-core products (DQMC_PREC_MIXED_TC; chains below the
 // tensor-core size threshold use the SIMT products at run time).
 #define DQMC_WITH_UMMA 1
+#define DQMC_QR_CALL __noinline__
 #include "dqmc_device.cuh"
 
 namespace dqmc {
