@@ -256,7 +256,7 @@ SPLIT_PRODUCTS = 28.0
 # workload with the tensor-core products (34.54 GB read, 88.39 GB written).
 TRAFFIC_BYTES = {("mixed_tc", "square 8x8/12x12 x256 chains", 16): ("bdde3c910e225dba", 122932378368)}
 
-KERNEL_SOURCES = ["dqmc_device.cuh", "dqmc_umma.cuh", "dqmc_internal.h", "dqmc_sweep_fp64.cu",
+KERNEL_SOURCES = ["dqmc_device.cuh", "dqmc_umma.cuh", "dqmc_internal.h", "dqmc_layout.h", "dqmc_sweep_fp64.cu",
                   "dqmc_sweep_fp32.cu", "dqmc_sweep_mixed.cu", "dqmc_sweep_mixed_tc.cu"]
 
 
