@@ -2043,8 +2043,21 @@ __device__ void flush_delayed<float>(const ChainDev& C, float* G, const float* A
   else if (r == 5) cta_gemm_r<float, true, false, 5, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
   else cta_gemm_r<float, true, false, 4, true>(N, N, nacc, A, ld, B, ld, G, ld, sm);
 }
+// ... of vectors in the chain's arena, staged in shared memory panel by panel (out of line:
+// its registers are not the sweep's).
+__device__ __noinline__ void rank_update_staged_dd(int N, int ld, dd* G, const dd* A, const dd* B, int nacc, dd* sm,
+                                                   int dd_tile) {
+  gemm_dd_tiles<true, false, true>(N, N, nacc, A, ld, B, ld, G, ld, sm, dd_tile);
+}
 template <>
 __device__ void flush_delayed<dd>(const ChainDev& C, dd* G, const dd* A, const dd* B, int nacc, Smem& S) {
+  // Vectors that did not fit the shared memory (N = 400 from rank 32): read directly, every
+  // thread waits for L2 vector by vector.  20 x 20, L = 20, 4 chains: 2033 ms a sweep
+  // directly, 1578 staged; L = 200, 32 chains: flushes 9.6 and 3.3 s of 14.5 and 8.2 s.
+  if (!__isShared(A)) {
+    rank_update_staged_dd(C.N, C.ld, G, A, B, nacc, reinterpret_cast<dd*>(S.gemm), S.dd_tile);
+    return;
+  }
   // a rank-k update (k <= 64): the float-pair register tiles beat the split tensor-core
   // product, whose digit split and recombination cost O(N^2) whatever k
   int r = S.dd_tile;
