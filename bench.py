@@ -253,8 +253,8 @@ SPLIT_PRODUCTS = 28.0
 # change makes the lookup miss and the line report traffic null.  Capture:
 # `ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
 # --clock-control none -k regex:sweep_kernel -s 3 -c 1` on the full 256-chain
-# workload with the tensor-core products (34.54 GB read, 88.39 GB written).
-TRAFFIC_BYTES = {("mixed_tc", "square 8x8/12x12 x256 chains", 16): ("bdde3c910e225dba", 122932378368)}
+# workload with the tensor-core products (40.20 GB read, 98.41 GB written).
+TRAFFIC_BYTES = {("mixed_tc", "square 8x8/12x12 x256 chains", 16): ("1e934c61c55bd3c3", 138606576384)}
 
 KERNEL_SOURCES = ["dqmc_device.cuh", "dqmc_umma.cuh", "dqmc_internal.h", "dqmc_layout.h", "dqmc_sweep_fp64.cu",
                   "dqmc_sweep_fp32.cu", "dqmc_sweep_mixed.cu", "dqmc_sweep_mixed_tc.cu"]
